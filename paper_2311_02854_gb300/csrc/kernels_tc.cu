@@ -406,53 +406,136 @@ __device__ __forceinline__ void tma_piece(uint32_t dst, const CUtensorMap* map, 
     }
 }
 
-// Roles: warps 0-3 epilogue (as in tc_seg_gemm_kernel), warp 4 lane 0 TMA
-// producer, warp 5 lane 0 MMA issuer.
-constexpr int THREADS3 = (kEpiWarps + 2) * 32;
+// Roles (one CTA per SM): warps 0-7 epilogue in two groups of four that take
+// the CTA's tiles alternately, warp 8 TMA producer (all lanes), warp 9 lane 0
+// MMA issuer.
+constexpr int kEpiGroups = 2;
+constexpr int kProdWarp3 = 4 * kEpiGroups;
+constexpr int THREADS3 = (kProdWarp3 + 2) * 32;
+constexpr int HALF_BYTES = 64 * TK * 2;  // one 64 x 64 bf16 box
+constexpr uint32_t kAcc = 4;             // accumulators in tensor memory (4 x 128 of the 512 columns)
 
+// Shared memory is a ring of UNITS units.  A stage whose operands both end
+// within 64 rows / columns (most stages of a sigma: sectors are small) takes
+// one unit, [A pieces | B pieces] of 8 KB each; any other stage takes two, one
+// per operand, with 16 KB per piece.  So twice as many small stages are in
+// flight as a fixed 64 KB slot (BF16X3) would allow.
 template <int NSPLIT>
 struct Cfg3 {
-    static constexpr int STAGES = (NSPLIT == 1) ? 6 : (NSPLIT == 2 ? 3 : 2);
-    static constexpr int STAGE_BYTES = 2 * NSPLIT * PIECE_BYTES;
-    static constexpr int SMEM = STAGES * STAGE_BYTES + 1024;
+    static constexpr int UNITS = (NSPLIT == 1) ? 12 : (NSPLIT == 2 ? 6 : 4);
+    static constexpr int UNIT_BYTES = 2 * NSPLIT * HALF_BYTES;
+    static constexpr int SMEM = UNITS * UNIT_BYTES + 1024;
 };
 
-// stage record of the TMA kernel
-struct StageMeta3 {
-    uint8_t a_mn, b_mn, neg, flags;  // flags: 1 first stage of a tile, 2 last, 4 no MMA (empty tile)
+// stage record of the TMA kernel (one 8-byte word)
+struct __align__(8) StageMeta3 {
+    uint8_t a_mn, b_mn, neg, flags;  // flags: 1 first stage of a tile, 2 last, 4 no MMA (empty tile), 8 two units
     uint8_t k16, n16, pad[2];        // 16-deep K steps holding data; MMA N / 16
 };
 
 __device__ __forceinline__ uint32_t idesc_n(int a_mn, int b_mn, int neg, int n) { return idesc_mn(a_mn, b_mn, neg, n, TM); }
 
+// Epilogue of one tile by one group of four warps: the tile's columns 32 at a
+// time from tensor memory, then alpha * acc in the tile's mode.  Warps whose 32
+// rows lie outside the block only release the accumulator.
+template <int NSPLIT>
+__device__ __forceinline__ void epilogue_tma(const Tile& T, int v, uint32_t tacc, int w4, int lane, const TcBufs& B,
+                                             uint32_t tempty) {
+    const int r = T.m0 + w4 * 32 + lane;
+    const int ncol = min(T.tn, T.n - T.n0);
+    const bool any = T.nst > 0 && T.m0 + w4 * 32 < T.m;  // warp-uniform
+    const bool rok = r < T.m;
+    const float alpha = T.alpha;
+    const int64_t off = T.c_off + (int64_t)r * T.ldc + T.n0 + (int64_t)v * B.out_vstride[T.c_buf];
+    if (T.nst == 0 && T.mode == TC_STORE_SPLIT && rok) {  // a stored block without products is zero
+        for (int j0 = 0; j0 < ncol; j0 += 8) {
+            *(uint4*)((__nv_bfloat16*)B.out[T.c_buf] + off + j0) = make_uint4(0, 0, 0, 0);
+            if (NSPLIT >= 2) *(uint4*)((__nv_bfloat16*)B.out_lo[T.c_buf] + off + j0) = make_uint4(0, 0, 0, 0);
+            if (NSPLIT == 3)
+                *(uint4*)((__nv_bfloat16*)B.out_lo[T.c_buf] + B.out_pstride[T.c_buf] + off + j0) = make_uint4(0, 0, 0, 0);
+        }
+    }
+    if (any) {
+        for (int c0 = 0; c0 < ncol; c0 += 32) {
+            uint32_t acc[32];
+            __syncwarp();
+            tmem_ld32(tacc + ((uint32_t)(w4 * 32) << 16) + (uint32_t)c0, acc);
+            tmem_wait_ld();
+            if (c0 + 32 >= ncol) {  // the last columns are in registers: release the accumulator
+                tc_fence_before();
+                __syncwarp();
+                if (lane == 0) mbar_arrive(tempty);
+            }
+            if (!rok) continue;
+            if (T.mode == TC_ATOMIC_F64) {
+                double* o = (double*)B.out[T.c_buf] + off + c0;
+#pragma unroll
+                for (int j = 0; j < 32; ++j)
+                    if (c0 + j < ncol) atomicAdd(o + j, (double)alpha * (double)__uint_as_float(acc[j]));
+            } else {  // TC_STORE_SPLIT: chunks of 8 (rows padded to multiples of 8)
+                __nv_bfloat16* oh = (__nv_bfloat16*)B.out[T.c_buf] + off + c0;
+                __nv_bfloat16* ol = (__nv_bfloat16*)B.out_lo[T.c_buf] + off + c0;
+#pragma unroll
+                for (int j0 = 0; j0 < 32; j0 += 8) {
+                    if (c0 + j0 >= ncol) break;
+                    __align__(16) __nv_bfloat16 h8[8], l8[8], m8[8];
+#pragma unroll
+                    for (int j = 0; j < 8; ++j) {
+                        const float x = alpha * __uint_as_float(acc[j0 + j]);
+                        const __nv_bfloat16 h = __float2bfloat16_rn(x);
+                        h8[j] = h;
+                        const float d = x - __bfloat162float(h);
+                        l8[j] = __float2bfloat16_rn(d);
+                        m8[j] = __float2bfloat16_rn(d - __bfloat162float(l8[j]));
+                    }
+                    *(uint4*)(oh + j0) = *(const uint4*)h8;
+                    if (NSPLIT >= 2) *(uint4*)(ol + j0) = *(const uint4*)l8;
+                    if (NSPLIT == 3) *(uint4*)(ol + B.out_pstride[T.c_buf] + j0) = *(const uint4*)m8;
+                }
+            }
+        }
+    } else {
+        tc_fence_before();
+        __syncwarp();
+        if (lane == 0) mbar_arrive(tempty);
+    }
+}
+
+// The lanes of the producer warp each hold the record of one segment (and of
+// its tile): the tile / segment loads of 32 segments are in flight together,
+// one batch ahead of the copies, and the lanes then issue their stages in
+// order.  (One lane walking tile -> segment -> copies spent ~1 us per stage on
+// the dependent loads, whatever the stage held: K = 24, D = 500 ran 5 % of the
+// operand bytes per second that the same kernel reached on 400-wide sectors.)
+struct ProdRec {
+    int32_t a_map, b_map, a_z, b_z, k;
+    int32_t m0, n0, v;
+    uint8_t a_mn, b_mn, a_pv, b_pv, a_br, b_br, neg, flags;  // flags: 1 first segment of a tile, 2 last, 4 empty tile
+    uint8_t nA, nB, n16, valid;
+};
+
 template <int NSPLIT>
 __global__ void __launch_bounds__(THREADS3, 1)
     tc_tma_kernel(const Tile* __restrict__ tiles, int ntiles, int nvec, const TSeg* __restrict__ segs,
-                  const CUtensorMap* __restrict__ maps, TcBufs B) {
+                  const CUtensorMap* __restrict__ maps, int single, TcBufs B) {
     using C = Cfg3<NSPLIT>;
-    constexpr int S = C::STAGES;
+    constexpr uint32_t U = C::UNITS;
     extern __shared__ uint8_t smem_raw[];
-    __shared__ __align__(8) uint64_t full_bar[S], empty_bar[S], tfull_bar[2], tempty_bar[2], drain_bar;
-    __shared__ StageMeta3 meta[S];
+    __shared__ __align__(8) uint64_t full_bar[U], empty_bar[U], tfull_bar[kAcc], tempty_bar[kAcc], drain_bar;
+    __shared__ StageMeta3 meta[U];
     __shared__ uint32_t tmem_base_s;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const uint32_t sbase = (smem_u32(smem_raw) + 1023u) & ~1023u;
 
-    if (warp == 0) {
-        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;\n" ::"r"(
-                         smem_u32(&tmem_base_s)),
-                     "r"(2 * TMEM_COLS)
-                     : "memory");
-        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;\n" ::: "memory");
-    }
+    if (warp == 0) tmem_alloc(smem_u32(&tmem_base_s), kAcc * TMEM_COLS);
     if (tid == 0) {
-        for (int s = 0; s < S; ++s) {
+        for (uint32_t s = 0; s < U; ++s) {
             mbar_init(smem_u32(&full_bar[s]), 1);
             mbar_init(smem_u32(&empty_bar[s]), 1);
         }
-        for (int b = 0; b < 2; ++b) {
+        for (uint32_t b = 0; b < kAcc; ++b) {
             mbar_init(smem_u32(&tfull_bar[b]), 1);
-            mbar_init(smem_u32(&tempty_bar[b]), kEpiWarps);
+            mbar_init(smem_u32(&tempty_bar[b]), 4);
         }
         mbar_init(smem_u32(&drain_bar), 1);
         asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
@@ -461,70 +544,147 @@ __global__ void __launch_bounds__(THREADS3, 1)
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem = tmem_base_s;
-    const int total = ntiles * nvec;
+    const uint32_t total = (uint32_t)ntiles * (uint32_t)nvec, G = gridDim.x, NV = (uint32_t)nvec;  // total < 2^31
     bool failed = false;
 
-    if (warp == kEpiWarps) {
+    if (warp == kProdWarp3) {
         // ---------------- TMA producer ----------------
-        if (lane == 0) {
-            uint32_t q = 0;
-            for (int t = blockIdx.x; t < total && !failed; t += gridDim.x) {
-                const int v = t % nvec;
-                const Tile T = tiles[t / nvec];
-                const int nst = T.nst;
-                // a second 64-row (or 64-column) half only when the block extends past the first
-                const int ncol = min(T.tn, T.n - T.n0);  // columns of this tile
-                const int nA = (T.m - T.m0 > 64) ? 2 : 1, nB = (ncol > 64) ? 2 : 1;
-                const int n16 = (ncol + 15) / 16;
-                if (nst == 0) {
-                    if (q >= (uint32_t)S && !mbar_wait(smem_u32(&empty_bar[q % S]), ((q / S) - 1) & 1u)) {
-                        failed = true;
-                        break;
-                    }
-                    meta[q % S] = StageMeta3{0, 0, 0, 1 | 2 | 4, 0, 0, {0, 0}};
-                    mbar_arrive(smem_u32(&full_bar[q % S]));
-                    ++q;
-                    continue;
+        // cursor: the next tile (single: of lane 0) and, for lists whose tiles sum
+        // several segments, its record, the next segment and the record after it
+        uint32_t ct = blockIdx.x;
+        int cs = 0;
+        Tile cT{}, nT{};
+        if (!single) {
+            if (ct < total) {
+                cT = tiles[ct / NV];
+                cs = cT.seg_beg;
+            }
+            if (ct + G < total) nT = tiles[(ct + G) / NV];
+        }
+        auto fetch = [&]() {
+            ProdRec r{};
+            Tile T = cT;
+            int idx, v;
+            if (single) {
+                const uint32_t t = ct + (uint32_t)lane * G;
+                r.valid = t < total;
+                v = r.valid ? (int)(t % NV) : 0;
+                if (r.valid) T = tiles[t / NV];
+                idx = T.seg_beg;
+                r.flags = 1 | 2;
+                ct = min(total, ct + 32 * G);
+            } else {
+                idx = cs + lane;
+                v = (int)(ct % NV);
+                r.valid = ct < total && (idx < cT.seg_end || (lane == 0 && cT.seg_beg == cT.seg_end));
+                r.flags = (idx == cT.seg_beg ? 1 : 0) | (idx + 1 >= cT.seg_end ? 2 : 0);
+                cs += 32;
+                if (ct < total && cs >= cT.seg_end) {
+                    ct = min(total, ct + G);
+                    cT = nT;
+                    cs = cT.seg_beg;
+                    if (ct + G < total) nT = tiles[(ct + G) / NV];
                 }
-                int done = 0;
-                for (int s = T.seg_beg; s < T.seg_end && !failed; ++s) {
-                    const TSeg Sg = segs[s];
-                    const int a_mn = Sg.a_tr ? 1 : 0, b_mn = Sg.b_tr ? 0 : 1;
-                    const int aw = Sg.a_pv ? v : 0, bw = Sg.b_pv ? v : 0;
-                    const CUtensorMap* am = maps + 3 * Sg.a_map;
-                    const CUtensorMap* bm = maps + 3 * Sg.b_map;
-                    const uint32_t bytes = (uint32_t)NSPLIT * 128u * (uint32_t)(nA * Sg.a_br + nB * Sg.b_br);
-                    for (int k0 = 0; k0 < Sg.k; k0 += TK) {
-                        const uint32_t slot = q % S;
-                        if (q >= (uint32_t)S && !mbar_wait(smem_u32(&empty_bar[slot]), ((q / S) - 1) & 1u)) {
+            }
+            if (r.valid && idx < T.seg_end) {
+                const TSeg S = segs[idx];
+                r.a_map = S.a_map;
+                r.b_map = S.b_map;
+                r.a_z = S.a_z;
+                r.b_z = S.b_z;
+                r.k = S.k;
+                r.a_mn = S.a_tr ? 1 : 0;
+                r.b_mn = S.b_tr ? 0 : 1;
+                r.a_pv = S.a_pv;
+                r.b_pv = S.b_pv;
+                r.a_br = S.a_br;
+                r.b_br = S.b_br;
+                r.neg = S.sign < 0.f ? 1 : 0;
+            } else {
+                r.flags = 1 | 2 | 4;
+            }
+            // a second 64-row (or 64-column) half only when the block extends past the first
+            const int ncol = min(T.tn, T.n - T.n0);
+            r.m0 = T.m0;
+            r.n0 = T.n0;
+            r.v = v;
+            r.nA = (T.m - T.m0 > 64) ? 2 : 1;
+            r.nB = (ncol > 64) ? 2 : 1;
+            r.n16 = (uint8_t)((ncol + 15) / 16);
+            return r;
+        };
+        uint32_t q = 0;  // units handed out so far
+        ProdRec next = fetch();
+        while (!failed) {
+            const ProdRec R = next;
+            const unsigned live = __ballot_sync(0xffffffffu, R.valid);
+            if (!live) break;
+            next = fetch();
+            const int upst = (R.nA == 2 || R.nB == 2) ? 2 : 1;
+            const int nst = !R.valid ? 0 : ((R.flags & 4) ? 1 : (R.k + TK - 1) / TK);
+            uint32_t sum = (uint32_t)(nst * ((R.flags & 4) ? 1 : upst));
+            const uint32_t mine = sum;
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+                const uint32_t x = __shfl_up_sync(0xffffffffu, sum, o);
+                if (lane >= o) sum += x;
+            }
+            const uint32_t q0 = q + sum - mine;
+            q += __shfl_sync(0xffffffffu, sum, 31);
+            const int nl = __popc(live);  // the valid lanes are the first nl
+            for (int l = 0; l < nl; ++l) {
+                if (lane == l) {
+                    uint32_t u = q0;
+                    for (int st = 0; st < nst; ++st) {
+                        const uint32_t slot = u % U, slot1 = (u + 1) % U;
+                        if (u >= U && !mbar_wait(smem_u32(&empty_bar[slot]), ((u / U) - 1) & 1u)) {
                             failed = true;
                             break;
                         }
-                        const int kv = min(TK, Sg.k - k0);
-                        meta[slot] = StageMeta3{(uint8_t)a_mn, (uint8_t)b_mn, (uint8_t)(Sg.sign < 0.f ? 1 : 0),
-                                                (uint8_t)((done == 0 ? 1 : 0) | (done == nst - 1 ? 2 : 0)),
-                                                (uint8_t)((kv + 15) / 16), (uint8_t)n16, {0, 0}};
                         const uint32_t bar = smem_u32(&full_bar[slot]);
-                        mbar_arrive_tx(bar, bytes);
-                        const uint32_t sa = sbase + slot * C::STAGE_BYTES;
-                        const uint32_t sb = sa + NSPLIT * PIECE_BYTES;
+                        if (R.flags & 4) {
+                            meta[slot] = StageMeta3{0, 0, 0, 1 | 2 | 4, 0, 0, {0, 0}};
+                            mbar_arrive(bar);
+                            break;
+                        }
+                        if (upst == 2 && u + 1 >= U && !mbar_wait(smem_u32(&empty_bar[slot1]), (((u + 1) / U) - 1) & 1u)) {
+                            failed = true;
+                            break;
+                        }
+                        const int k0 = st * TK;
+                        meta[slot] = StageMeta3{R.a_mn, R.b_mn, R.neg,
+                                                (uint8_t)(((R.flags & 1) && st == 0 ? 1 : 0) |
+                                                          ((R.flags & 2) && st == nst - 1 ? 2 : 0) | (upst == 2 ? 8 : 0)),
+                                                (uint8_t)((min(TK, R.k - k0) + 15) / 16), R.n16, {0, 0}};
+                        // every unit's full barrier completes once per use: a second unit's at once (nobody waits on it)
+                        if (upst == 2) mbar_arrive(smem_u32(&full_bar[slot1]));
+                        mbar_arrive_tx(bar, (uint32_t)NSPLIT * 128u * (uint32_t)(R.nA * R.a_br + R.nB * R.b_br));
+                        const uint32_t ps = (uint32_t)upst * HALF_BYTES;  // bytes between the pieces of an operand
+                        const uint32_t sa = sbase + slot * C::UNIT_BYTES;
+                        const uint32_t sb = upst == 2 ? sbase + slot1 * C::UNIT_BYTES : sa + NSPLIT * HALF_BYTES;
+                        const CUtensorMap* am = maps + 3 * R.a_map;
+                        const CUtensorMap* bm = maps + 3 * R.b_map;
+                        const int aw = R.a_pv ? R.v : 0, bw = R.b_pv ? R.v : 0;
 #pragma unroll
                         for (int pc = 0; pc < NSPLIT; ++pc) {
-                            tma_piece(sa + pc * PIECE_BYTES, am + pc, a_mn, T.m0, k0, Sg.a_z, aw, bar, nA);
-                            tma_piece(sb + pc * PIECE_BYTES, bm + pc, b_mn, T.n0, k0, Sg.b_z, bw, bar, nB);
+                            tma_piece(sa + pc * ps, am + pc, R.a_mn, R.m0, k0, R.a_z, aw, bar, R.nA);
+                            tma_piece(sb + pc * ps, bm + pc, R.b_mn, R.n0, k0, R.b_z, bw, bar, R.nB);
                         }
-                        ++q;
-                        ++done;
+                        u += upst;
                     }
+                }
+                if (__any_sync(0xffffffffu, failed)) {
+                    failed = true;
+                    break;
                 }
             }
         }
-    } else if (warp == kEpiWarps + 1) {
+    } else if (warp == kProdWarp3 + 1) {
         // ---------------- MMA issuer ----------------
         if (lane == 0) {
             uint32_t q = 0, tc = 0;
-            for (int t = blockIdx.x; t < total && !failed; t += gridDim.x, ++tc) {
-                const uint32_t buf = tc & 1u, use = tc >> 1;
+            for (uint32_t t = blockIdx.x; t < total && !failed; t += G, ++tc) {
+                const uint32_t buf = tc % kAcc, use = tc / kAcc;
                 if (use > 0 && !mbar_wait(smem_u32(&tempty_bar[buf]), (use - 1) & 1u)) {
                     failed = true;
                     break;
@@ -532,34 +692,36 @@ __global__ void __launch_bounds__(THREADS3, 1)
                 tc_fence_after();
                 const uint32_t dt = tmem + buf * TMEM_COLS;
                 for (;;) {
-                    const uint32_t slot = q % S;
-                    if (!mbar_wait(smem_u32(&full_bar[slot]), (q / S) & 1u)) {
+                    const uint32_t slot = q % U, slot1 = (q + 1) % U;
+                    if (!mbar_wait(smem_u32(&full_bar[slot]), (q / U) & 1u)) {
                         failed = true;
                         break;
                     }
                     tc_fence_after();
                     const StageMeta3 M = meta[slot];
+                    const bool two = (M.flags & 8) != 0;
                     if (!(M.flags & 4)) {
-                        const uint32_t sa = sbase + slot * C::STAGE_BYTES;
-                        const uint32_t sb = sa + NSPLIT * PIECE_BYTES;
+                        const uint32_t ps = two ? 2u * HALF_BYTES : (uint32_t)HALF_BYTES;
+                        const uint32_t sa = sbase + slot * C::UNIT_BYTES;
+                        const uint32_t sb = two ? sbase + slot1 * C::UNIT_BYTES : sa + NSPLIT * HALF_BYTES;
                         const uint32_t id = idesc_n(M.a_mn, M.b_mn, M.neg, 16 * M.n16);
+                        // bits of a descriptor besides its address, and the address step of a 16-deep K step
+                        const uint64_t ab = M.a_mn ? sdesc(0, HALF_BYTES, 1024) : sdesc(0, 16, 1024);
+                        const uint64_t bb = M.b_mn ? sdesc(0, HALF_BYTES, 1024) : sdesc(0, 16, 1024);
+                        const uint32_t ak = M.a_mn ? 2048 : 32, bk = M.b_mn ? 2048 : 32;
                         for (int kk = 0; kk < M.k16; ++kk) {
 #pragma unroll
                             for (int pr = 0; pr < Prods<NSPLIT>::N; ++pr) {
-                                const int pa = prod_a(pr), pb = prod_b(pr);
-                                const uint32_t a_s = sa + pa * PIECE_BYTES;
-                                const uint32_t b_s = sb + pb * PIECE_BYTES;
-                                const uint64_t ad =
-                                    M.a_mn ? sdesc(a_s + kk * 2048, 8192, 1024) : sdesc(a_s + kk * 32, 16, 1024);
-                                const uint64_t bd =
-                                    M.b_mn ? sdesc(b_s + kk * 2048, 8192, 1024) : sdesc(b_s + kk * 32, 16, 1024);
+                                const uint32_t a_s = sa + prod_a(pr) * ps + kk * ak;
+                                const uint32_t b_s = sb + prod_b(pr) * ps + kk * bk;
                                 const uint32_t acc = ((M.flags & 1) && kk == 0 && pr == 0) ? 0u : 1u;
-                                mma_bf16(dt, ad, bd, id, acc);
+                                mma_bf16(dt, ab | ((a_s & 0x3FFFFu) >> 4), bb | ((b_s & 0x3FFFFu) >> 4), id, acc);
                             }
                         }
                     }
                     mma_commit(smem_u32(&empty_bar[slot]));
-                    ++q;
+                    if (two) mma_commit(smem_u32(&empty_bar[slot1]));
+                    q += two ? 2 : 1;
                     if (M.flags & 2) break;
                 }
                 if (failed) break;
@@ -570,13 +732,15 @@ __global__ void __launch_bounds__(THREADS3, 1)
         }
     } else {
         // ---------------- epilogue ----------------
-        uint32_t tc = 0;
+        const int grp = warp >> 2, w4 = warp & 3;
+        const uint32_t step = G * kEpiGroups;
+        uint32_t t = blockIdx.x + G * grp;
         Tile Tn{};
-        if (blockIdx.x < total) Tn = tiles[blockIdx.x / nvec];
-        for (int t = blockIdx.x; t < total && !failed; t += gridDim.x, ++tc) {
-            const uint32_t buf = tc & 1u, use = tc >> 1;
+        if (t < total) Tn = tiles[t / NV];
+        for (uint32_t tc = grp; t < total && !failed; t += step, tc += kEpiGroups) {
+            const uint32_t buf = tc % kAcc, use = tc / kAcc;
             const Tile T = Tn;  // fetched one tile ahead, while the MMAs of this one run
-            if (t + (int)gridDim.x < total) Tn = tiles[(t + gridDim.x) / nvec];
+            if (t + step < total) Tn = tiles[(t + step) / NV];
             int ok = 1;
             if (lane == 0) ok = mbar_wait(smem_u32(&tfull_bar[buf]), use & 1u) ? 1 : 0;
             ok = __shfl_sync(0xffffffffu, ok, 0);  // warp-uniform (tcgen05.ld is warp-collective)
@@ -586,18 +750,14 @@ __global__ void __launch_bounds__(THREADS3, 1)
             }
             __syncwarp();
             tc_fence_after();
-            epilogue_tile<NSPLIT>(T, t % nvec, T.nst, tmem + buf * TMEM_COLS, warp, lane, B,
-                                  smem_u32(&tempty_bar[buf]));
+            epilogue_tma<NSPLIT>(T, (int)(t % NV), tmem + buf * TMEM_COLS, w4, lane, B, smem_u32(&tempty_bar[buf]));
         }
     }
     if (failed) atomicExch(B.err, 1);
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
-    if (warp == 0) {
-        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;\n" ::"r"(tmem), "r"(2 * TMEM_COLS)
-                     : "memory");
-    }
+    if (warp == 0) tmem_dealloc(tmem, kAcc * TMEM_COLS);
 }
 
 // ---------------------------------------------------------------------------
@@ -760,6 +920,8 @@ void TmaWorkList::add_block(int64_t c_off, int c_buf, int m, int n, int ldc, con
 }
 
 void TmaWorkList::order_tiles() {
+    single = true;
+    for (const Tile& t : tiles) single = single && t.seg_end - t.seg_beg == 1;
     // longest tiles first: CTAs take tiles round-robin, so the short ones fill
     // in at the end of the launch instead of a few long ones trailing.  A
     // stable counting sort on the stage count (< 65536): two linear passes
@@ -907,15 +1069,16 @@ void launch_seg_gemm_tma(const TmaWorkList& w, const MapTable& maps, const TcBuf
     DMRG_REQUIRE(total < (1LL << 31), DMRG_EINVAL, "tensor-core work list too large");
     DMRG_REQUIRE(maps.d_maps != nullptr, DMRG_EINVAL, "tensor maps not uploaded");
     const int grid = (int)std::min<int64_t>(total, tc_num_sms());
+    const int single = w.single ? 1 : 0;
     if (nsplit == 3) {
         tc_tma_kernel<3><<<grid, THREADS3, Cfg3<3>::SMEM, st>>>(w.d_tiles, (int)w.tiles.size(), nvec, w.d_segs,
-                                                        maps.d_maps, b);
+                                                                maps.d_maps, single, b);
     } else if (nsplit == 2) {
         tc_tma_kernel<2><<<grid, THREADS3, Cfg3<2>::SMEM, st>>>(w.d_tiles, (int)w.tiles.size(), nvec, w.d_segs,
-                                                               maps.d_maps, b);
+                                                                maps.d_maps, single, b);
     } else {
         tc_tma_kernel<1><<<grid, THREADS3, Cfg3<1>::SMEM, st>>>(w.d_tiles, (int)w.tiles.size(), nvec, w.d_segs,
-                                                               maps.d_maps, b);
+                                                                maps.d_maps, single, b);
     }
     ++launch_counter();
     DMRG_CHECK_CUDA(cudaGetLastError());
