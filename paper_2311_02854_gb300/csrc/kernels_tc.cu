@@ -406,23 +406,30 @@ __device__ __forceinline__ void tma_piece(uint32_t dst, const CUtensorMap* map, 
     }
 }
 
-// Roles (one CTA per SM): warps 0-7 epilogue in two groups of four that take
-// the CTA's tiles alternately, warp 8 TMA producer (all lanes), warp 9 lane 0
-// MMA issuer.
+// Roles: warps 0-7 epilogue in two groups of four that take the CTA's tiles
+// alternately, warp 8 TMA producer (all lanes), warp 9 lane 0 MMA issuer.
+//
+// Bound: not by data.  The producer and the MMA lane are each busy ~1000 cycles
+// per stage with issuing (waits, descriptors, 4 to 12 copies, 6 to 12 MMAs,
+// commits), whatever the stage holds, so two CTAs share an SM, half of shared
+// and tensor memory each, and issue in parallel (one CTA with everything:
+// K = 24, D = 500, four vectors 20.4 ms, two: 11.6 ms; K = 36, D = 1000
+// 16.4 -> 13.5 ms).
+constexpr int kCtas3 = 2;
 constexpr int kEpiGroups = 2;
 constexpr int kProdWarp3 = 4 * kEpiGroups;
 constexpr int THREADS3 = (kProdWarp3 + 2) * 32;
 constexpr int HALF_BYTES = 64 * TK * 2;  // one 64 x 64 bf16 box
-constexpr uint32_t kAcc = 4;             // accumulators in tensor memory (4 x 128 of the 512 columns)
+constexpr uint32_t kAcc = 2;             // accumulators in tensor memory (2 x 128 of the 512 columns)
 
 // Shared memory is a ring of UNITS units.  A stage whose operands both end
 // within 64 rows / columns (most stages of a sigma: sectors are small) takes
 // one unit, [A pieces | B pieces] of 8 KB each; any other stage takes two, one
-// per operand, with 16 KB per piece.  So twice as many small stages are in
-// flight as a fixed 64 KB slot (BF16X3) would allow.
+// per operand, with 16 KB per piece (BF16X3), so three small stages are in
+// flight per CTA where a fixed 64 KB slot would allow one.
 template <int NSPLIT>
 struct Cfg3 {
-    static constexpr int UNITS = (NSPLIT == 1) ? 12 : (NSPLIT == 2 ? 6 : 4);
+    static constexpr int UNITS = (NSPLIT == 1) ? 6 : (NSPLIT == 2 ? 3 : 2);
     static constexpr int UNIT_BYTES = 2 * NSPLIT * HALF_BYTES;
     static constexpr int SMEM = UNITS * UNIT_BYTES + 1024;
 };
@@ -515,7 +522,7 @@ struct ProdRec {
 };
 
 template <int NSPLIT>
-__global__ void __launch_bounds__(THREADS3, 1)
+__global__ void __launch_bounds__(THREADS3, kCtas3)
     tc_tma_kernel(const Tile* __restrict__ tiles, int ntiles, int nvec, const TSeg* __restrict__ segs,
                   const CUtensorMap* __restrict__ maps, int single, TcBufs B) {
     using C = Cfg3<NSPLIT>;
@@ -1068,7 +1075,7 @@ void launch_seg_gemm_tma(const TmaWorkList& w, const MapTable& maps, const TcBuf
     const int64_t total = (int64_t)w.tiles.size() * nvec;
     DMRG_REQUIRE(total < (1LL << 31), DMRG_EINVAL, "tensor-core work list too large");
     DMRG_REQUIRE(maps.d_maps != nullptr, DMRG_EINVAL, "tensor maps not uploaded");
-    const int grid = (int)std::min<int64_t>(total, tc_num_sms());
+    const int grid = (int)std::min<int64_t>(total, kCtas3 * tc_num_sms());
     const int single = w.single ? 1 : 0;
     if (nsplit == 3) {
         tc_tma_kernel<3><<<grid, THREADS3, Cfg3<3>::SMEM, st>>>(w.d_tiles, (int)w.tiles.size(), nvec, w.d_segs,
