@@ -58,6 +58,11 @@ struct WorkList {
     size_t cap_tiles = 0, cap_segs = 0;
     double flops = 0.0;
     bool rank1 = false;  // every segment has K = 1 (run by the rank-1 kernel)
+    // FP64 units, set by upload: part of a tile per warp (16, 32, or 64 for four
+    // parts of 32 per tile); CTAs that share a part's term sum (0: one warp does
+    // it), by K-blocks of every segment (byk) or by segments
+    int part = 64, split = 0;
+    bool byk = false;
     // tile shape of add_block when nonzero (rows, columns); 128 x 64 lists run on
     // the FP64-accurate tensor-core engine (launch_seg_gemm_f64 dispatches on it)
     int tile_m = 0, tile_n = 0;

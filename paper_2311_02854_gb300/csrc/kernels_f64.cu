@@ -4,6 +4,7 @@
 // accumulator) and the vector / Jacobi kernels of Davidson and decimation.
 #include <cuda_bf16.h>
 
+#include <algorithm>
 #include <cmath>
 
 #include "engine.h"
@@ -67,25 +68,63 @@ void WorkList::add_block(int64_t c_off, int c_buf, int m, int n, int ldc, const 
     }
 }
 
+namespace {
+constexpr int kSplitWarps = 4;  // warps of a CTA that share a part's term sum (FP64 units)
+}
+
 void WorkList::upload(cudaStream_t st) {
-    if (tile_m == oz_tile_rows() && tiles.size() > 1) {
-        // the tensor-core engine's persistent CTAs take tiles round-robin: longest
-        // first (stable counting sort on the stage count), so that short tiles
-        // fill in at the end instead of a few long ones trailing
-        const int tk = oz_stage_depth();
-        std::vector<int> nst(tiles.size());
-        int maxn = 0;
-        for (size_t i = 0; i < tiles.size(); ++i) {
-            int64_t n = 0;
-            for (int s = tiles[i].seg_beg; s < tiles[i].seg_end; ++s) n += (segs[s].k + tk - 1) / tk;
-            nst[i] = (int)std::min<int64_t>(n, 1 << 20);
-            maxn = std::max(maxn, nst[i]);
-        }
+    // work of a tile: 64-deep (tensor-core engine: oz_stage_depth) K steps, for the
+    // FP64 units times its 8 x 8 groups
+    const bool oz = tile_m == oz_tile_rows();
+    const int tk = oz ? oz_stage_depth() : 64;
+    std::vector<int> cost(tiles.size());
+    int64_t total = 0;
+    int maxn = 0;
+    for (size_t i = 0; i < tiles.size(); ++i) {
+        const Tile& t = tiles[i];
+        int64_t n = 0;
+        for (int s = t.seg_beg; s < t.seg_end; ++s) n += (segs[s].k + tk - 1) / tk;
+        if (!oz) n *= (int64_t)((std::min(t.m - t.m0, 64) + 7) / 8) * ((std::min(t.n - t.n0, 64) + 7) / 8);
+        cost[i] = (int)std::min<int64_t>(n, 1 << 20);
+        total += cost[i];
+        maxn = std::max(maxn, cost[i]);
+    }
+    // FP64 units.  Part of a tile per warp: 16 or 32 square where every tile ends
+    // there, else 32 square, four per tile.  Several warps per part (split: CTAs of
+    // four) when there are fewer parts than two per warp slot (12 on each of the
+    // 152 SMs), or when the longest sum, on one warp, would take more than a
+    // quarter of the launch; eight CTAs where even four warps per part do not fill
+    // the slots and the sums are long (K = 10, D = 100: 250 outputs of ~300
+    // products; 2.0 ms with four warps per part, see seg_split_f64_kernel).
+    constexpr int64_t kSlots = 152 * 12;
+    int mmax = 0, nmax = 0;
+    int64_t parts = 0, segsum = 0, ksum = 0;
+    for (const Tile& t : tiles) {
+        const int m = std::min(t.m - t.m0, 64), n = std::min(t.n - t.n0, 64);
+        mmax = std::max(mmax, m);
+        nmax = std::max(nmax, n);
+        parts += (int64_t)((m + 31) / 32) * ((n + 31) / 32);
+        segsum += t.seg_end - t.seg_beg;
+    }
+    for (const Seg& g : segs) ksum += g.k;
+    part = std::max(mmax, nmax) <= 16 ? 16 : (std::max(mmax, nmax) <= 32 ? 32 : 64);
+    split = 0;
+    byk = false;
+    if (!oz && !rank1 && !tiles.empty() && !segs.empty()) {
+        const int64_t nt = (int64_t)tiles.size(), ns = (int64_t)segs.size();
+        const bool few = parts < 2 * kSlots, longest = (int64_t)maxn * kSlots > total;
+        byk = ksum / ns >= 32;  // a segment's K-blocks then feed four warps
+        if ((few || longest) && (byk || segsum >= 8 * nt)) split = 1;
+        if (split && !byk && parts * kSplitWarps < kSlots && segsum >= 64 * nt) split = 8;
+    }
+    if ((oz || split) && tiles.size() > 1) {
+        // longest first (stable counting sort), so that short tiles fill in at the
+        // end instead of a few long ones trailing
         std::vector<size_t> pos((size_t)maxn + 2, 0);
-        for (int n : nst) ++pos[(size_t)(maxn - n) + 1];
+        for (int n : cost) ++pos[(size_t)(maxn - n) + 1];
         for (size_t i = 1; i < pos.size(); ++i) pos[i] += pos[i - 1];
         std::vector<Tile> sorted(tiles.size());
-        for (size_t i = 0; i < tiles.size(); ++i) sorted[pos[(size_t)(maxn - nst[i])]++] = tiles[i];
+        for (size_t i = 0; i < tiles.size(); ++i) sorted[pos[(size_t)(maxn - cost[i])]++] = tiles[i];
         tiles.swap(sorted);
     }
     if (tiles.size() > cap_tiles) {
@@ -115,11 +154,22 @@ void WorkList::release() {
 }
 
 // ---------------------------------------------------------------------------
-// Segmented grouped GEMM, FP64 (64x64 tile, 256 threads, 4x4 per thread)
+// Segmented grouped GEMM on the FP64 units (64 x 64 tiles, 32 x 32 per warp)
 // ---------------------------------------------------------------------------
+//
+// Bound: the FP64 units (1.05 TFLOP/s measured, as FMA or as mma.m8n8k4: one
+// 8 x 8 x 4 product per ~140 cycles and SM).  The split follows from that:
+// work is cut in 8 x 8 x 4 products and the ones outside the block are not
+// issued (a 64 x 64 x 16 step computed in full spends 21 times a 10 x 10 x 10
+// product, the usual size at small bonds, and 2.3 times a 42 x 42 one), and
+// operands go from global memory to the fragments directly: at that rate the
+// loads cost nothing and neither shared memory nor barriers are needed.  A warp
+// owns a 32 x 32 part of a tile and is a CTA of its own, so that no warp's slot
+// waits for a larger neighbour (2 x 2 warps per 64 x 64 tile kept the units 79 %
+// busy, the ratio of the mean to the largest share of a 52 x 64 tile).
 
 namespace {
-constexpr int BM = 64, BN = 64, BK = 16, NT = 256;
+constexpr int PT = 32;  // part of a tile per warp: 4 x 4 groups of 8 x 8 (2 x 2 where all tiles end within 16 x 16)
 
 // element idx of buffer buf (FP64, or bf16 pieces read as hi + lo)
 __device__ __forceinline__ double ld_elem(const BufTable& bt, int buf, int64_t idx) {
@@ -136,147 +186,258 @@ __device__ __forceinline__ double ld_elem(const BufTable& bt, int buf, int64_t i
     return bt.p[buf][idx];
 }
 
-__global__ void __launch_bounds__(NT) seg_gemm_f64_kernel(const Tile* __restrict__ tiles,
-                                                          const Seg* __restrict__ segs, BufTable bt) {
-    const Tile T = tiles[blockIdx.x];
-    const int v = blockIdx.y;
-    __shared__ double As[BK][BM + 1];
-    __shared__ double Bs[BK][BN + 1];
-    const int tid = threadIdx.x;
-    const int tx = tid % 16, ty = tid / 16;
-    double acc[4][4];
-#pragma unroll
-    for (int i = 0; i < 4; ++i)
-#pragma unroll
-        for (int j = 0; j < 4; ++j) acc[i][j] = 0.0;
-    const int mrem = T.m - T.m0, nrem = T.n - T.n0;
-    for (int s = T.seg_beg; s < T.seg_end; ++s) {
-        const Seg S = segs[s];
-        int64_t A = S.a_off + (int64_t)v * bt.vstride[S.a_buf];
-        int64_t B = S.b_off + (int64_t)v * bt.vstride[S.b_buf];
-        A += S.a_tr ? (int64_t)T.m0 : (int64_t)T.m0 * S.lda;
-        B += S.b_tr ? (int64_t)T.n0 * S.ldb : (int64_t)T.n0;
-        for (int k0 = 0; k0 < S.k; k0 += BK) {
-#pragma unroll
-            for (int i = 0; i < 4; ++i) {
-                int m, kk;
-                if (!S.a_tr) {
-                    kk = tid % BK;
-                    m = tid / BK + 16 * i;
-                } else {
-                    m = tid % BM;
-                    kk = tid / BM + 4 * i;
-                }
-                double x = 0.0;
-                if (m < mrem && k0 + kk < S.k)
-                    x = ld_elem(bt, S.a_buf,
-                                A + (S.a_tr ? (int64_t)(k0 + kk) * S.lda + m : (int64_t)m * S.lda + k0 + kk));
-                As[kk][m] = x * S.alpha;
-            }
-#pragma unroll
-            for (int i = 0; i < 4; ++i) {
-                int n, kk;
-                if (!S.b_tr) {
-                    n = tid % BN;
-                    kk = tid / BN + 4 * i;
-                } else {
-                    kk = tid % BK;
-                    n = tid / BK + 16 * i;
-                }
-                double x = 0.0;
-                if (n < nrem && k0 + kk < S.k)
-                    x = ld_elem(bt, S.b_buf,
-                                B + (S.b_tr ? (int64_t)n * S.ldb + k0 + kk : (int64_t)(k0 + kk) * S.ldb + n));
-                Bs[kk][n] = x;
-            }
-            __syncthreads();
-#pragma unroll
-            for (int kk = 0; kk < BK; ++kk) {
-                double a[4], b[4];
-#pragma unroll
-                for (int i = 0; i < 4; ++i) a[i] = As[kk][ty + 16 * i];
-#pragma unroll
-                for (int j = 0; j < 4; ++j) b[j] = Bs[kk][tx + 16 * j];
-#pragma unroll
-                for (int i = 0; i < 4; ++i)
-#pragma unroll
-                    for (int j = 0; j < 4; ++j) acc[i][j] = fma(a[i], b[j], acc[i][j]);
-            }
-            __syncthreads();
-        }
-    }
+// D (8 x 8) += A (8 x 4) B (4 x 8): lane l holds A(l / 4, l % 4), B(l % 4, l / 4)
+// and D(l / 4, 2 (l % 4) + {0, 1})
+__device__ __forceinline__ void mma884(double (&d)[2], double a, double b) {
+    asm volatile("mma.sync.aligned.m8n8k4.row.col.f64.f64.f64.f64 {%0, %1}, {%2}, {%3}, {%0, %1};\n"
+                 : "+d"(d[0]), "+d"(d[1])
+                 : "d"(a), "d"(b));
+}
+
+// part `sub` (0: the only one of a tile within 32 x 32; else 2 x 2 per tile) of
+// tile T: its origin in the block and its extents (not positive: nothing there)
+struct Part {
+    int m0, n0, mr, nr;
+};
+__device__ __forceinline__ Part tile_part(const Tile& T, int sub) {
+    Part p;
+    p.m0 = T.m0 + (sub >> 1) * PT;
+    p.n0 = T.n0 + (sub & 1) * PT;
+    p.mr = min(PT, T.m - p.m0);
+    p.nr = min(PT, T.n - p.n0);
+    return p;
+}
+
+// Sums to the part's output.  TILE_ATOMIC outputs are added to without atomics:
+// one CTA owns each part, and the lists that add to the same output run one
+// after the other, so every element's sum has one order and two calls agree to
+// the bit.
+template <int GR>
+__device__ __forceinline__ void store_part(const Tile& T, const BufTable& bt, int v, const Part& p,
+                                           const double (&acc)[GR][GR][2]) {
+    const int lane = threadIdx.x & 31;
     double* C = bt.p[T.c_buf] + T.c_off + (int64_t)v * bt.vstride[T.c_buf];
 #pragma unroll
-    for (int i = 0; i < 4; ++i) {
-        const int r = T.m0 + ty + 16 * i;
-        if (r >= T.m) continue;
+    for (int i = 0; i < GR; ++i) {
+        const int r = 8 * i + (lane >> 2);
+        if (r >= p.mr) continue;
 #pragma unroll
-        for (int j = 0; j < 4; ++j) {
-            const int c = T.n0 + tx + 16 * j;
-            if (c >= T.n) continue;
-            double* dst = C + (int64_t)r * T.ldc + c;
-            if (T.mode == TILE_ATOMIC)
-                atomicAdd(dst, acc[i][j]);
-            else
-                *dst = acc[i][j];
+        for (int j = 0; j < GR; ++j)
+#pragma unroll
+            for (int e = 0; e < 2; ++e) {
+                const int c = 8 * j + 2 * (lane & 3) + e;
+                if (c >= p.nr) continue;
+                double* dst = C + (int64_t)(p.m0 + r) * T.ldc + p.n0 + c;
+                *dst = T.mode == TILE_ATOMIC ? *dst + acc[i][j][e] : acc[i][j][e];
+            }
+    }
+}
+
+// acc += the segments [sb, se) over part p; of each segment the K-blocks of
+// 4 KU that are kf, kf + ks, ... of its own
+template <int GR, int KU>
+__device__ __forceinline__ void part_sum(const Seg* __restrict__ segs, const BufTable& bt, int v, int sb, int se,
+                                         int kf, int ks, const Part& p, double (&acc)[GR][GR][2]) {
+    const int lane = threadIdx.x & 31;
+    const int lr = lane >> 2, lk = lane & 3;
+    Seg N{};
+    if (sb < se) N = segs[sb];
+    for (int s = sb; s < se; ++s) {
+        const Seg S = N;
+        if (s + 1 < se) N = segs[s + 1];  // in flight during this segment
+        // element (row, k) of op(A) at A + row * ra + k * ka, (k, col) of op(B) at B + k * kb + col * cb
+        const int64_t ra = S.a_tr ? 1 : S.lda, ka = S.a_tr ? S.lda : 1;
+        const int64_t cb = S.b_tr ? S.ldb : 1, kb = S.b_tr ? 1 : S.ldb;
+        const int64_t A = S.a_off + (int64_t)v * bt.vstride[S.a_buf] + (p.m0 + lr) * ra + lk * ka;
+        const int64_t B = S.b_off + (int64_t)v * bt.vstride[S.b_buf] + (p.n0 + lr) * cb + lk * kb;
+        for (int k0 = 4 * KU * kf; k0 < S.k; k0 += 4 * KU * ks) {
+            double a[KU][GR], b[KU][GR];
+#pragma unroll
+            for (int u = 0; u < KU; ++u) {
+                const bool kv = k0 + 4 * u + lk < S.k;
+#pragma unroll
+                for (int i = 0; i < GR; ++i) {
+                    a[u][i] = 0.0;
+                    b[u][i] = 0.0;
+                    if (kv && lr + 8 * i < p.mr) a[u][i] = ld_elem(bt, S.a_buf, A + 8 * i * ra + (k0 + 4 * u) * ka);
+                    if (kv && lr + 8 * i < p.nr) b[u][i] = ld_elem(bt, S.b_buf, B + 8 * i * cb + (k0 + 4 * u) * kb);
+                }
+            }
+            if (S.alpha != 1.0) {
+#pragma unroll
+                for (int u = 0; u < KU; ++u)
+#pragma unroll
+                    for (int i = 0; i < GR; ++i) a[u][i] *= S.alpha;
+            }
+#pragma unroll
+            for (int u = 0; u < KU; ++u) {
+                if (k0 + 4 * u >= S.k) break;
+#pragma unroll
+                for (int i = 0; i < GR; ++i)
+#pragma unroll
+                    for (int j = 0; j < GR; ++j)
+                        if (8 * i < p.mr && 8 * j < p.nr) mma884(acc[i][j], a[u][i], b[u][j]);
+            }
         }
     }
 }
-// The same product for lists whose segments all have K = 1 (rank-1 updates,
-// e.g. the diagonal of H_eff as sums of diag(O_L) diag(O_R)^T): each thread
-// reads its 4 + 4 operand elements straight from global memory (they stay in
-// L1 across the segments of a tile), no shared-memory staging or barriers.
-// Same accumulation order per element as seg_gemm_f64_kernel.
-__global__ void __launch_bounds__(NT) seg_outer_f64_kernel(const Tile* __restrict__ tiles,
-                                                           const Seg* __restrict__ segs, BufTable bt) {
-    const Tile T = tiles[blockIdx.x];
+
+template <int GR, int KU>
+__global__ void __launch_bounds__(32, GR == 2 ? 24 : 12)
+    seg_gemm_f64_kernel(const Tile* __restrict__ tiles, int subs, const Seg* __restrict__ segs, BufTable bt) {
+    const Tile T = tiles[blockIdx.x / subs];
+    const Part p = tile_part(T, (int)(blockIdx.x % subs));
+    if (p.mr <= 0 || p.nr <= 0) return;
     const int v = blockIdx.y;
-    const int tid = threadIdx.x;
-    const int tx = tid % 16, ty = tid / 16;
-    double acc[4][4];
+    double acc[GR][GR][2] = {};
+    part_sum<GR, KU>(segs, bt, v, T.seg_beg, T.seg_end, 0, 1, p, acc);
+    store_part<GR>(T, bt, v, p, acc);
+}
+
+// The same with several warps per part: kSplit in a CTA, and with a cluster of
+// CTAs that many times more.  Each takes a range of the tile's segments, or
+// (byk: segments of some depth) its share of every segment's K-blocks; the
+// partial sums are added in warp, then in rank order (through distributed
+// shared memory).  For lists with fewer parts than the chip has warps, or whose
+// longest term sums would outlast the rest of the launch: the sigma of a small
+// bond has a few hundred outputs, each the sum of hundreds to thousands of
+// products.
+constexpr int kSplit = kSplitWarps;
+template <int GR, int KU>
+__global__ void __launch_bounds__(32 * kSplit, GR == 2 ? 5 : 3)
+    seg_split_f64_kernel(const Tile* __restrict__ tiles, int subs, int nrank, int byk, const Seg* __restrict__ segs,
+                         BufTable bt) {
+    __shared__ double part[kSplit][GR * GR * 2][32];
+    const int rank = (int)(blockIdx.x % nrank);  // clusters are runs of nrank blocks
+    const uint32_t pi = blockIdx.x / nrank;
+    const Tile T = tiles[pi / subs];
+    const Part p = tile_part(T, (int)(pi % subs));
+    if (p.mr <= 0 || p.nr <= 0) return;  // the whole cluster leaves
+    const int v = blockIdx.y, warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int64_t ns = T.seg_end - T.seg_beg;
+    const int w = rank * kSplit + warp, nw = nrank * kSplit;
+    double acc[GR][GR][2] = {};
+    if (byk) part_sum<GR, KU>(segs, bt, v, T.seg_beg, T.seg_end, w, nw, p, acc);
+    else part_sum<GR, KU>(segs, bt, v, T.seg_beg + (int)(ns * w / nw), T.seg_beg + (int)(ns * (w + 1) / nw), 0, 1, p, acc);
 #pragma unroll
-    for (int i = 0; i < 4; ++i)
+    for (int i = 0; i < GR; ++i)
 #pragma unroll
-        for (int j = 0; j < 4; ++j) acc[i][j] = 0.0;
-    const int mrem = T.m - T.m0, nrem = T.n - T.n0;
-    for (int s = T.seg_beg; s < T.seg_end; ++s) {
-        const Seg S = segs[s];
-        int64_t A = S.a_off + (int64_t)v * bt.vstride[S.a_buf];
-        int64_t B = S.b_off + (int64_t)v * bt.vstride[S.b_buf];
-        A += S.a_tr ? (int64_t)T.m0 : (int64_t)T.m0 * S.lda;
-        B += S.b_tr ? (int64_t)T.n0 * S.ldb : (int64_t)T.n0;
-        double a[4], b[4];
+        for (int j = 0; j < GR; ++j)
 #pragma unroll
-        for (int i = 0; i < 4; ++i) {
-            const int m = ty + 16 * i;
-            a[i] = m < mrem ? ld_elem(bt, S.a_buf, A + (S.a_tr ? (int64_t)m : (int64_t)m * S.lda)) * S.alpha : 0.0;
+            for (int e = 0; e < 2; ++e) part[warp][(i * GR + j) * 2 + e][lane] = acc[i][j][e];
+    __syncthreads();
+    if (warp == 0) {
+#pragma unroll
+        for (int i = 0; i < GR; ++i)
+#pragma unroll
+            for (int j = 0; j < GR; ++j)
+#pragma unroll
+                for (int e = 0; e < 2; ++e)
+#pragma unroll
+                    for (int q = 1; q < kSplit; ++q) acc[i][j][e] += part[q][(i * GR + j) * 2 + e][lane];
+    }
+    if (nrank > 1) {
+        if (warp == 0) {
+#pragma unroll
+            for (int i = 0; i < GR; ++i)
+#pragma unroll
+                for (int j = 0; j < GR; ++j)
+#pragma unroll
+                    for (int e = 0; e < 2; ++e) part[0][(i * GR + j) * 2 + e][lane] = acc[i][j][e];
         }
+        __syncwarp();
+        asm volatile("barrier.cluster.arrive.release.aligned;\nbarrier.cluster.wait.acquire.aligned;\n" ::: "memory");
+        if (warp == 0 && rank == 0) {
 #pragma unroll
-        for (int j = 0; j < 4; ++j) {
-            const int n = tx + 16 * j;
-            b[j] = n < nrem ? ld_elem(bt, S.b_buf, B + (S.b_tr ? (int64_t)n * S.ldb : (int64_t)n)) : 0.0;
+            for (int i = 0; i < GR; ++i)
+#pragma unroll
+                for (int j = 0; j < GR; ++j)
+#pragma unroll
+                    for (int e = 0; e < 2; ++e) {
+                        const uint32_t a = (uint32_t)__cvta_generic_to_shared(&part[0][(i * GR + j) * 2 + e][lane]);
+                        for (int q = 1; q < nrank; ++q) {
+                            uint32_t ra;
+                            double x;
+                            asm volatile("mapa.shared::cluster.u32 %0, %1, %2;\n" : "=r"(ra) : "r"(a), "r"(q));
+                            asm volatile("ld.shared::cluster.f64 %0, [%1];\n" : "=d"(x) : "r"(ra) : "memory");
+                            acc[i][j][e] += x;
+                        }
+                    }
         }
+        // the partial sums stay until rank 0 has read them
+        __syncwarp();
+        asm volatile("barrier.cluster.arrive.release.aligned;\nbarrier.cluster.wait.acquire.aligned;\n" ::: "memory");
+    }
+    if (warp == 0 && rank == 0) store_part<GR>(T, bt, v, p, acc);
+}
+
+// The same product for lists whose segments all have K = 1 (rank-1 updates:
+// the diagonal of H_eff as sums of diag(O_L) diag(O_R)^T).  Bound: the latency
+// of the strided gathers (a diagonal is read with stride ld + 1) and, behind
+// it, the FP64 units.  A CTA gathers the elements of 64 segments into shared
+// memory with all its threads, one segment and operand each (32 loads in flight
+// per thread), and its four warps form the products, a quarter of the part's
+// 8 x 8 groups each, four segments per K-step and in segment order.
+constexpr int kOuter = 64;
+__global__ void __launch_bounds__(2 * kOuter)
+    seg_outer_f64_kernel(const Tile* __restrict__ tiles, int subs, const Seg* __restrict__ segs, BufTable bt) {
+    __shared__ double As[kOuter][PT + 4], Bs[kOuter][PT + 4];  // 36-double rows: fragment reads without conflicts
+    const Tile T = tiles[blockIdx.x / subs];
+    const Part p = tile_part(T, (int)(blockIdx.x % subs));
+    if (p.mr <= 0 || p.nr <= 0) return;
+    const int v = blockIdx.y, tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int lr = lane >> 2, lk = lane & 3;
+    const int gi = warp >> 1, gj = warp & 1;  // the warp's groups: rows gi, gi + 2, columns gj, gj + 2
+    const int ls = tid % kOuter;
+    const bool isb = tid >= kOuter;
+    double acc[2][2][2] = {};
+    for (int s0 = T.seg_beg; s0 < T.seg_end; s0 += kOuter) {
+        double x[PT];
+        const bool sv = s0 + ls < T.seg_end;
+        if (sv) {
+            const Seg S = segs[s0 + ls];
+            const int buf = isb ? S.b_buf : S.a_buf;
+            const int64_t st = isb ? (S.b_tr ? S.ldb : 1) : (S.a_tr ? 1 : S.lda);
+            const int64_t o = (isb ? S.b_off + p.n0 * st : S.a_off + p.m0 * st) + (int64_t)v * bt.vstride[buf];
+            const int nx = isb ? p.nr : p.mr;
+            const double al = isb ? 1.0 : S.alpha;
 #pragma unroll
-        for (int i = 0; i < 4; ++i)
+            for (int i = 0; i < PT; ++i) x[i] = i < nx ? ld_elem(bt, buf, o + i * st) * al : 0.0;
+        } else {
 #pragma unroll
-            for (int j = 0; j < 4; ++j) acc[i][j] = fma(a[i], b[j], acc[i][j]);
+            for (int i = 0; i < PT; ++i) x[i] = 0.0;
+        }
+        __syncthreads();  // the previous 64 segments have been used
+#pragma unroll
+        for (int i = 0; i < PT; ++i) (isb ? Bs : As)[ls][i] = x[i];
+        __syncthreads();
+        const int ne = min(kOuter, T.seg_end - s0);
+        for (int k = 0; k < ne; k += 4) {
+            double a[2], b[2];
+#pragma unroll
+            for (int i = 0; i < 2; ++i) {
+                a[i] = As[k + lk][8 * (gi + 2 * i) + lr];
+                b[i] = Bs[k + lk][8 * (gj + 2 * i) + lr];
+            }
+#pragma unroll
+            for (int i = 0; i < 2; ++i)
+#pragma unroll
+                for (int j = 0; j < 2; ++j)
+                    if (8 * (gi + 2 * i) < p.mr && 8 * (gj + 2 * j) < p.nr) mma884(acc[i][j], a[i], b[j]);
+        }
     }
     double* C = bt.p[T.c_buf] + T.c_off + (int64_t)v * bt.vstride[T.c_buf];
 #pragma unroll
-    for (int i = 0; i < 4; ++i) {
-        const int r = T.m0 + ty + 16 * i;
-        if (r >= T.m) continue;
+    for (int i = 0; i < 2; ++i)
 #pragma unroll
-        for (int j = 0; j < 4; ++j) {
-            const int c = T.n0 + tx + 16 * j;
-            if (c >= T.n) continue;
-            double* dst = C + (int64_t)r * T.ldc + c;
-            if (T.mode == TILE_ATOMIC)
-                atomicAdd(dst, acc[i][j]);
-            else
-                *dst = acc[i][j];
-        }
-    }
+        for (int j = 0; j < 2; ++j)
+#pragma unroll
+            for (int e = 0; e < 2; ++e) {
+                const int r = 8 * (gi + 2 * i) + lr, c = 8 * (gj + 2 * j) + 2 * lk + e;
+                if (r >= p.mr || c >= p.nr) continue;
+                double* dst = C + (int64_t)(p.m0 + r) * T.ldc + p.n0 + c;
+                *dst = T.mode == TILE_ATOMIC ? *dst + acc[i][j][e] : acc[i][j][e];
+            }
 }
 }  // namespace
 
@@ -286,25 +447,46 @@ void launch_seg_gemm_f64(const WorkList& w, const BufTable& bt, int nvec, cudaSt
         launch_seg_gemm_oz(w, bt, nvec, oz_error_word(), st);
         return;
     }
-    DMRG_REQUIRE(w.tile_m == 0 || w.tile_m == BM, DMRG_EINVAL, "work list tile shape not runnable on the FP64 engine");
-    const int64_t n = (int64_t)w.tiles.size();
-    const int64_t maxg = 2147483647LL;
-    DMRG_REQUIRE(n <= maxg && nvec <= 65535, DMRG_EINVAL, "work list too large for one launch");
-    dim3 grid((unsigned)n, (unsigned)nvec);
-    if (w.rank1)
-        seg_outer_f64_kernel<<<grid, NT, 0, st>>>(w.d_tiles, w.d_segs, bt);
-    else
-        seg_gemm_f64_kernel<<<grid, NT, 0, st>>>(w.d_tiles, w.d_segs, bt);
-    ++launch_counter();
+    DMRG_REQUIRE(w.tile_m == 0, DMRG_EINVAL, "work list tile shape not runnable on the FP64 engine");
+    DMRG_REQUIRE(nvec <= 65535, DMRG_EINVAL, "too many vectors for one launch");
+    const int subs = w.part == 64 ? 4 : 1;
+    const bool tiny = w.part == 16;
+    const int nrank = w.split ? w.split : 1;
+    const int64_t n = (int64_t)w.tiles.size(), maxt = 2147483647LL / (subs * nrank);
+    for (int64_t t0 = 0; t0 < n; t0 += maxt) {
+        const int64_t nt = std::min(n - t0, maxt);
+        const dim3 grid((unsigned)(nt * subs * nrank), (unsigned)nvec);
+        const Tile* tl = w.d_tiles + t0;
+        if (w.rank1) {
+            seg_outer_f64_kernel<<<grid, 2 * kOuter, 0, st>>>(tl, subs, w.d_segs, bt);
+        } else if (w.split) {
+            cudaLaunchConfig_t cfg{};
+            cfg.gridDim = grid;
+            cfg.blockDim = dim3(32 * kSplit);
+            cfg.stream = st;
+            cudaLaunchAttribute at{};
+            at.id = cudaLaunchAttributeClusterDimension;
+            at.val.clusterDim.x = (unsigned)nrank;
+            at.val.clusterDim.y = at.val.clusterDim.z = 1;
+            cfg.attrs = &at;
+            cfg.numAttrs = 1;
+            DMRG_CHECK_CUDA(cudaLaunchKernelEx(&cfg, tiny ? seg_split_f64_kernel<2, 4> : seg_split_f64_kernel<4, 2>, tl, subs,
+                                               nrank, (int)w.byk, (const Seg*)w.d_segs, bt));
+        } else {
+            (tiny ? seg_gemm_f64_kernel<2, 4> : seg_gemm_f64_kernel<4, 2>)<<<grid, 32, 0, st>>>(tl, subs, w.d_segs, bt);
+        }
+        ++launch_counter();
+    }
     DMRG_CHECK_CUDA(cudaGetLastError());
 }
 
 void launch_seg_gemm_f64_lists(const Tile* d_tiles, int64_t ntiles, const Seg* d_segs, const BufTable& bt,
                                cudaStream_t st) {
-    if (ntiles <= 0) return;
-    DMRG_REQUIRE(ntiles <= 2147483647LL, DMRG_EINVAL, "work list too large for one launch");
-    seg_gemm_f64_kernel<<<dim3((unsigned)ntiles, 1), NT, 0, st>>>(d_tiles, d_segs, bt);
-    ++launch_counter();
+    const int64_t maxt = 2147483647LL / 4;
+    for (int64_t t0 = 0; t0 < ntiles; t0 += maxt) {
+        seg_gemm_f64_kernel<4, 2><<<(unsigned)(4 * std::min(ntiles - t0, maxt)), 32, 0, st>>>(d_tiles + t0, 4, d_segs, bt);
+        ++launch_counter();
+    }
     DMRG_CHECK_CUDA(cudaGetLastError());
 }
 

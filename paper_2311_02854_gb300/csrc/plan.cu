@@ -397,7 +397,9 @@ void ProductList::lower(int8_t sbuf_, int8_t ibuf, int ild, int64_t cap, int64_t
         }
         for (int o : order) {
             const OutBlock& ob = outs[o];
-            p2.add_block(ob.off, ob.buf, ob.m, ob.n, ob.ldc, segs[o], TILE_ATOMIC, kchunk);
+            // the FP64 units' kernels share a long term sum among the CTAs of a cluster
+            // and add without atomics: one tile per output region, no K-chunks
+            p2.add_block(ob.off, ob.buf, ob.m, ob.n, ob.ldc, segs[o], TILE_ATOMIC, tile_m > 0 ? kchunk : 0);
         }
         scratch_elems = std::max(scratch_elems, used);
         chunks.emplace_back(std::move(p1), std::move(p2));
