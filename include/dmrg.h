@@ -110,9 +110,9 @@ typedef struct {
                                default 1 */
     int sigma_tune;         /* mixed modes: 1 = the tile shape of the sigma work lists
                                (tile width 128 or 64, phase-2 K-chunk) is picked per bond by
-                               timing each candidate on a sample of the bond's own work (every
-                               8th output block, 16th beyond a million products, with all their
-                               products); choices are cached by
+                               the estimated time of each candidate on a sample of the bond's
+                               own work (every 8th output block with all of its products), so
+                               that a bond always gets the same shape; choices are cached by
                                the bond's sector-size histogram; ignored when tc_kchunk > 0
                                or sigma_tile_n > 0, and for lists of over 2^20 products (which
                                keep tile width 128 and the full K-chunk, the measured winner
@@ -199,7 +199,7 @@ typedef struct {
     int64_t tunes;                /* autotuner runs (histograms not seen before) */
     int64_t tune_hits;            /* bonds whose histogram was already tuned */
     double ms_tune;               /* wall time of all autotuner runs */
-    double tune_cand_ms[4];       /* last autotuner run: sample time per candidate
+    double tune_cand_ms[4];       /* last autotuner run: estimated sample time per candidate
                                      (128 / K-chunk, 64 / K-chunk, 128 / half K-chunk, 64 / half) */
     double sigma_load_bytes[2][2];/* mixed sigma, one vector: operand bytes the tensor-core tiles
                                      load through TMA, [phase 1 / 2][other operands / phase-1

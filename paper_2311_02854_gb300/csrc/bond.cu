@@ -200,14 +200,20 @@ struct SigmaShape {
     int64_t kchunk;
 };
 
-// Times the candidate shapes (tile width 128 / 64, phase-2 K-chunk kmax /
-// kmax/2) on a sample of the bond's work list: every 8th (16th) output block
-// with all of its products, lowered exactly as the full list would be.  Each
-// candidate runs once to warm up and once timed (CUDA events on the plan's
-// stream); the fastest wins, the default (128, kmax) unless another is 2 %
-// faster.
-SigmaShape tune_sigma_shape(Plan& P, int k, const ProductList& tl, int64_t cap, int64_t kmax, const int64_t* vs,
-                            int G) {
+// Estimates the time of the candidate shapes (tile width 128 / 64, phase-2
+// K-chunk kmax / kmax/2) on a sample of the bond's work list: every 8th output
+// block with all of its products, cut into tiles and K-chunks as the list would
+// be and dealt to the SMs longest first.  In units of a 64-deep K stage of phase
+// 2: 16 for the launches, 1.6 per phase-1 stage of an SM, and for phase 2 the
+// largest SM's stages plus 4 per tile (its drain; 2 with three pieces, whose
+// stages take longer).  The weights are fitted to timings of 260 bonds (K = 7 to
+// 32, D = 30 to 900; one, two and three bf16 pieces), of which the estimate picks
+// the faster K-chunk in all but nine, five of those within 2 % either way.
+// Timing the sample instead took 8 to 60 ms per new bond, and near a tie it chose
+// by noise, so that one bond's sigma differed by the FP32 rounding of the other
+// chain length (3e-6) from run to run.  The fastest wins, the default (128, kmax)
+// unless another is faster (three pieces: 1 % faster).
+SigmaShape tune_sigma_shape(Plan& P, const ProductList& tl, int64_t kmax, int G) {
     const uint64_t key = sector_histogram_key(P, G);
     auto f = P.tune_cache.find(key);
     if (f != P.tune_cache.end()) {
@@ -215,61 +221,71 @@ SigmaShape tune_sigma_shape(Plan& P, int k, const ProductList& tl, int64_t cap, 
         return {f->second.first, f->second.second};
     }
     const auto t0 = std::chrono::steady_clock::now();
+    constexpr int kSMs = 152;
+    constexpr double kBase = 16.0, kStage1 = 1.6, kStageMs = 0.67e-3;
+    const double kDrain = P.nsplit == 3 ? 2.0 : 4.0, kMargin = P.nsplit == 3 ? 0.99 : 1.0;
     const int64_t khalf = std::max<int64_t>(kmax / 2, 64);
     const SigmaShape cand[4] = {{128, kmax}, {64, kmax}, {128, khalf}, {64, khalf}};
-    // every 8th output (16th for lists of over a million products)
-    const int stride = tl.outs.size() >= 64 ? (tl.cs.size() > ((size_t)1 << 20) ? 16 : 8) : 1;
-    ensure_psi_pieces(P, (int64_t)G * P.dim_pad);
-    // a fixed nonzero bf16 pattern in psi's pieces (the sample is timed, not used)
-    DMRG_CHECK_CUDA(cudaMemsetAsync(P.ps_hi, 0x3c, (size_t)P.n_ppc * 2, P.stream));
-    DMRG_CHECK_CUDA(cudaMemsetAsync(P.ps_lo, 0x3c, (size_t)P.n_ppc * 2 * P.lo_pieces(), P.stream));
-    double* out = P.alloc(std::max<int64_t>(P.dim, 1));
-    cudaEvent_t e0 = P.take_event(), e1 = P.take_event();
-    double best = 0.0;
-    int bi = 0;
-    ProductList smp;
-    try {
-        for (int c = 0; c < 4; ++c) {
-            smp.clear();
-            smp.outs = tl.outs;
-            for (const Contrib& x : tl.cs)
-                if (x.out % stride == 0) smp.cs.push_back(x);
-            smp.lower_tma(BUF_SCR, BUF_ID, P.id_n, cap, cand[c].kchunk, TC_ATOMIC_F64, vs, G, cand[c].tn);
-            smp.cs.clear();
-            ensure_scratch(P, (int64_t)G * smp.scratch_elems);
-            for (auto& ch : smp.tchunks) {
-                ch.first.upload(P.stream);
-                ch.second.upload(P.stream);
-            }
-            const TcBufs tb = sigma_bufs(P, k, out);
-            smp.maps.encode_upload(tb, P.nsplit, P.stream);
-            tc_prepare(P.nsplit);
-            float msb = 0.f;
-            for (int rep = 0; rep < 2; ++rep) {  // a warm-up run, then the timed one
-                DMRG_CHECK_CUDA(cudaEventRecord(e0, P.stream));
-                smp.run_tma(tb, 1, P.nsplit, P.stream);
-                DMRG_CHECK_CUDA(cudaEventRecord(e1, P.stream));
-                DMRG_CHECK_CUDA(cudaEventSynchronize(e1));
-                DMRG_CHECK_CUDA(cudaEventElapsedTime(&msb, e0, e1));
-            }
-            P.check_device_error();
-            P.stats.tune_cand_ms[c] = msb;
-            if (c == 0 || msb < 0.98 * best) {
-                best = msb;
-                bi = c;
+    const int stride = tl.outs.size() >= 64 ? 8 : 1;
+    // per sampled output its phase-2 depths in item order; phase-1 stages per tile width
+    std::vector<std::vector<int>> depth(tl.outs.size());
+    double s1[2] = {0.0, 0.0};
+    for (const Contrib& c : tl.cs) {
+        if (c.out % stride != 0) continue;
+        const int nreal = (!c.P.ident) + (!c.Q.ident) + (!c.R.ident);
+        const bool unit = c.alpha == 1.0 || c.alpha == -1.0;
+        int k2, m1 = 0, n1 = 0, k1 = 0;
+        if (nreal == 3) {
+            const double cost_pq = 2.0 * c.m * c.k1 * c.k2 + 2.0 * c.m * c.k2 * c.n;
+            const double cost_qr = 2.0 * c.k1 * c.k2 * c.n + 2.0 * c.m * c.k1 * c.n;
+            const bool pq = cost_pq <= cost_qr;
+            k2 = pq ? c.k2 : c.k1;
+            m1 = pq ? c.m : c.k1;
+            n1 = pq ? c.k2 : c.n;
+            k1 = pq ? c.k1 : c.k2;
+        } else {
+            const int k = nreal == 2 ? (c.P.ident ? c.k2 : c.k1) : c.n;
+            k2 = unit ? k : c.n;
+            if (!unit) {
+                m1 = c.m;
+                n1 = c.n;
+                k1 = k;
             }
         }
-    } catch (...) {
-        smp.clear();
-        P.free(out, std::max<int64_t>(P.dim, 1));
-        P.ev_pool.push_back(e0);
-        P.ev_pool.push_back(e1);
-        throw;
+        depth[c.out].push_back(k2);
+        for (int w = 0; w < 2; ++w)
+            s1[w] += (double)((m1 + 127) / 128) * ((n1 + (w ? 63 : 127)) / (w ? 64 : 128)) * ((k1 + 63) / 64);
     }
-    smp.clear();
-    P.free(out, std::max<int64_t>(P.dim, 1));
-    P.ev_pool.push_back(e0);
-    P.ev_pool.push_back(e1);
+    double best = 0.0;
+    int bi = 0;
+    for (int x = 0; x < 4; ++x) {
+        std::vector<int> nst;  // stages of every tile
+        for (size_t o = 0; o < tl.outs.size(); ++o) {
+            if (depth[o].empty()) continue;
+            const int tiles = ((tl.outs[o].m + 127) / 128) * ((tl.outs[o].n + cand[x].tn - 1) / cand[x].tn);
+            int64_t acc = 0;
+            int st = 0;
+            for (int k : depth[o]) {
+                if (acc > 0 && acc + k > cand[x].kchunk) {
+                    nst.insert(nst.end(), tiles, st);
+                    acc = 0;
+                    st = 0;
+                }
+                acc += k;
+                st += (k + 63) / 64;
+            }
+            nst.insert(nst.end(), tiles, st);
+        }
+        std::sort(nst.begin(), nst.end(), [](int a, int b) { return a > b; });
+        std::vector<double> sm(kSMs, 0.0);
+        for (size_t i = 0; i < nst.size(); ++i) sm[i % kSMs] += nst[i] + kDrain;
+        const double ms = kStageMs * (kBase + kStage1 * s1[cand[x].tn == 64 ? 1 : 0] / kSMs + *std::max_element(sm.begin(), sm.end()));
+        P.stats.tune_cand_ms[x] = ms;
+        if (x == 0 || (ms < best && ms < kMargin * P.stats.tune_cand_ms[0])) {
+            best = ms;
+            bi = x;
+        }
+    }
     P.tune_cache[key] = {cand[bi].tn, cand[bi].kchunk};
     ++P.stats.tunes;
     P.stats.ms_tune += std::chrono::duration<double, std::milli>(std::chrono::steady_clock::now() - t0).count();
@@ -1020,7 +1036,7 @@ void set_bond(Plan& P, int k) {
         double t_tune = 0.0;
         if (tune_later) {
             const auto c0 = std::chrono::steady_clock::now();
-            shape = tune_sigma_shape(P, k, tl, cap, shape.kchunk, vs, G);
+            shape = tune_sigma_shape(P, tl, shape.kchunk, G);
             t_tune = host_ms_since(c0);
             lower_and_count();
         }
