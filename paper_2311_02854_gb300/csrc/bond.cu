@@ -886,11 +886,11 @@ void set_bond(Plan& P, int k) {
                 c.mma += 2.0 * 128 * 128 * (double)kk;
                 // operand bytes the TMA loads for this tile (boxes of 128-byte
                 // rows, one per piece), split into scratch and everything else
-                const int nA = (t.m - t.m0 > 64) ? 2 : 1, nB = (std::min(t.tn, t.n - t.n0) > 64) ? 2 : 1;
+                const int nA = (t.m - t.m0 > 64 && !t.sn) ? 2 : 1, nB = (std::min<int>(t.tn, t.n - t.n0) > 64) ? 2 : 1;
                 for (int q = t.seg_beg; q < t.seg_end; ++q) {
                     const TSeg& g = w.segs[q];
                     const double st = (double)((g.k + 63) / 64) * P.nsplit * 128.0;
-                    c.load[tl.maps.keys[g.a_map].buf == BUF_SCR ? 1 : 0] += st * nA * g.a_br;
+                    c.load[tl.maps.keys[g.a_map].buf == BUF_SCR ? 1 : 0] += st * nA * g.a_bz * g.a_br;
                     c.load[tl.maps.keys[g.b_map].buf == BUF_SCR ? 1 : 0] += st * nB * g.b_br;
                 }
             }

@@ -32,7 +32,10 @@ struct Tile {
     uint8_t c_buf, mode;
     uint16_t nst;         // tensor-core engine: 64-deep K stages of the tile (set by the TMA work list)
     float alpha;          // epilogue scale (tensor-core engine; the FP64 engine scales per segment)
-    int32_t tn;           // TMA tensor-core engine: tile width (64 or 128 columns)
+    // TMA tensor-core engine: tile width (64 or 128 columns); products stacked along
+    // the rows (0: none; else product i holds accumulator rows i * 16 * sb ..., and
+    // its m x n block lies i * m * ldc elements behind c_off)
+    uint8_t tn, sn, sb, pad;
 };
 static_assert(sizeof(Tile) == 48, "Tile keeps its 48-byte record");
 

@@ -149,7 +149,7 @@ __device__ __forceinline__ void epilogue_tile(const Tile& T, int v, int nst, uin
     __syncwarp();
     if (lane == 0) mbar_arrive(tempty);
     if (!rok || (nst == 0 && (T.mode == TC_ATOMIC_F64 || T.mode == TC_ATOMIC_F32))) return;
-    const int ncol = min(T.tn > 0 ? T.tn : TN, T.n - T.n0);  // the FP64-engine work list leaves tn 0
+    const int ncol = min(TN, T.n - T.n0);
     const int64_t off = T.c_off + (int64_t)r * T.ldc + T.n0 + (int64_t)v * B.out_vstride[T.c_buf];
     if (T.mode == TC_ATOMIC_F64) {
         double* o = (double*)B.out[T.c_buf] + off;
@@ -437,7 +437,8 @@ struct Cfg3 {
 // stage record of the TMA kernel (one 8-byte word)
 struct __align__(8) StageMeta3 {
     uint8_t a_mn, b_mn, neg, flags;  // flags: 1 first stage of a tile, 2 last, 4 no MMA (empty tile), 8 two units
-    uint8_t k16, n16, pad[2];        // 16-deep K steps holding data; MMA N / 16
+    uint8_t k16, n16;                // 16-deep K steps holding data; MMA N / 16
+    uint8_t a_lb, swap;              // MN-major A: 2 KB steps between its 64-wide halves; cross terms swapped
 };
 
 __device__ __forceinline__ uint32_t idesc_n(int a_mn, int b_mn, int neg, int n) { return idesc_mn(a_mn, b_mn, neg, n, TM); }
@@ -448,12 +449,23 @@ __device__ __forceinline__ uint32_t idesc_n(int a_mn, int b_mn, int neg, int n) 
 template <int NSPLIT>
 __device__ __forceinline__ void epilogue_tma(const Tile& T, int v, uint32_t tacc, int w4, int lane, const TcBufs& B,
                                              uint32_t tempty) {
-    const int r = T.m0 + w4 * 32 + lane;
-    const int ncol = min(T.tn, T.n - T.n0);
-    const bool any = T.nst > 0 && T.m0 + w4 * 32 < T.m;  // warp-uniform
-    const bool rok = r < T.m;
+    const int row = w4 * 32 + lane;
+    const int ncol = min((int)T.tn, T.n - T.n0);
+    // row of the output: of stacked products (m * ldc apart) the rows run on
+    bool any, rok;
+    int64_t r;
+    if (T.sn) {
+        const int i = row / (16 * T.sb), ri = row - i * 16 * T.sb;
+        any = w4 * 32 < T.sn * 16 * T.sb;
+        rok = i < T.sn && ri < T.m;
+        r = (int64_t)i * T.m + ri;
+    } else {
+        any = T.nst > 0 && T.m0 + w4 * 32 < T.m;
+        r = T.m0 + row;
+        rok = r < T.m;
+    }
     const float alpha = T.alpha;
-    const int64_t off = T.c_off + (int64_t)r * T.ldc + T.n0 + (int64_t)v * B.out_vstride[T.c_buf];
+    const int64_t off = T.c_off + r * T.ldc + T.n0 + (int64_t)v * B.out_vstride[T.c_buf];
     if (T.nst == 0 && T.mode == TC_STORE_SPLIT && rok) {  // a stored block without products is zero
         for (int j0 = 0; j0 < ncol; j0 += 8) {
             *(uint4*)((__nv_bfloat16*)B.out[T.c_buf] + off + j0) = make_uint4(0, 0, 0, 0);
@@ -518,7 +530,7 @@ struct ProdRec {
     int32_t a_map, b_map, a_z, b_z, k;
     int32_t m0, n0, v;
     uint8_t a_mn, b_mn, a_pv, b_pv, a_br, b_br, neg, flags;  // flags: 1 first segment of a tile, 2 last, 4 empty tile
-    uint8_t nA, nB, n16, valid;
+    uint8_t nA, nB, n16, valid, a_bz, swap;
 };
 
 template <int NSPLIT>
@@ -606,16 +618,18 @@ __global__ void __launch_bounds__(THREADS3, kCtas3)
                 r.b_pv = S.b_pv;
                 r.a_br = S.a_br;
                 r.b_br = S.b_br;
+                r.a_bz = S.a_bz;
+                r.swap = S.swap;
                 r.neg = S.sign < 0.f ? 1 : 0;
             } else {
                 r.flags = 1 | 2 | 4;
             }
             // a second 64-row (or 64-column) half only when the block extends past the first
-            const int ncol = min(T.tn, T.n - T.n0);
+            const int ncol = min((int)T.tn, T.n - T.n0);
             r.m0 = T.m0;
             r.n0 = T.n0;
             r.v = v;
-            r.nA = (T.m - T.m0 > 64) ? 2 : 1;
+            r.nA = (T.m - T.m0 > 64 && !T.sn) ? 2 : 1;
             r.nB = (ncol > 64) ? 2 : 1;
             r.n16 = (uint8_t)((ncol + 15) / 16);
             return r;
@@ -627,7 +641,7 @@ __global__ void __launch_bounds__(THREADS3, kCtas3)
             const unsigned live = __ballot_sync(0xffffffffu, R.valid);
             if (!live) break;
             next = fetch();
-            const int upst = (R.nA == 2 || R.nB == 2) ? 2 : 1;
+            const int upst = (R.nA == 2 || R.nB == 2 || R.a_bz * R.a_br > 64) ? 2 : 1;
             const int nst = !R.valid ? 0 : ((R.flags & 4) ? 1 : (R.k + TK - 1) / TK);
             uint32_t sum = (uint32_t)(nst * ((R.flags & 4) ? 1 : upst));
             const uint32_t mine = sum;
@@ -650,7 +664,7 @@ __global__ void __launch_bounds__(THREADS3, kCtas3)
                         }
                         const uint32_t bar = smem_u32(&full_bar[slot]);
                         if (R.flags & 4) {
-                            meta[slot] = StageMeta3{0, 0, 0, 1 | 2 | 4, 0, 0, {0, 0}};
+                            meta[slot] = StageMeta3{0, 0, 0, 1 | 2 | 4, 0, 0, 0, 0};
                             mbar_arrive(bar);
                             break;
                         }
@@ -662,10 +676,11 @@ __global__ void __launch_bounds__(THREADS3, kCtas3)
                         meta[slot] = StageMeta3{R.a_mn, R.b_mn, R.neg,
                                                 (uint8_t)(((R.flags & 1) && st == 0 ? 1 : 0) |
                                                           ((R.flags & 2) && st == nst - 1 ? 2 : 0) | (upst == 2 ? 8 : 0)),
-                                                (uint8_t)((min(TK, R.k - k0) + 15) / 16), R.n16, {0, 0}};
+                                                (uint8_t)((min(TK, R.k - k0) + 15) / 16), R.n16,
+                                                (uint8_t)(R.a_bz > 1 ? R.a_br / 16 : 4), R.swap};
                         // every unit's full barrier completes once per use: a second unit's at once (nobody waits on it)
                         if (upst == 2) mbar_arrive(smem_u32(&full_bar[slot1]));
-                        mbar_arrive_tx(bar, (uint32_t)NSPLIT * 128u * (uint32_t)(R.nA * R.a_br + R.nB * R.b_br));
+                        mbar_arrive_tx(bar, (uint32_t)NSPLIT * 128u * (uint32_t)(R.nA * R.a_bz * R.a_br + R.nB * R.b_br));
                         const uint32_t ps = (uint32_t)upst * HALF_BYTES;  // bytes between the pieces of an operand
                         const uint32_t sa = sbase + slot * C::UNIT_BYTES;
                         const uint32_t sb = upst == 2 ? sbase + slot1 * C::UNIT_BYTES : sa + NSPLIT * HALF_BYTES;
@@ -713,14 +728,14 @@ __global__ void __launch_bounds__(THREADS3, kCtas3)
                         const uint32_t sb = two ? sbase + slot1 * C::UNIT_BYTES : sa + NSPLIT * HALF_BYTES;
                         const uint32_t id = idesc_n(M.a_mn, M.b_mn, M.neg, 16 * M.n16);
                         // bits of a descriptor besides its address, and the address step of a 16-deep K step
-                        const uint64_t ab = M.a_mn ? sdesc(0, HALF_BYTES, 1024) : sdesc(0, 16, 1024);
+                        const uint64_t ab = M.a_mn ? sdesc(0, M.a_lb * 2048u, 1024) : sdesc(0, 16, 1024);
                         const uint64_t bb = M.b_mn ? sdesc(0, HALF_BYTES, 1024) : sdesc(0, 16, 1024);
                         const uint32_t ak = M.a_mn ? 2048 : 32, bk = M.b_mn ? 2048 : 32;
                         for (int kk = 0; kk < M.k16; ++kk) {
 #pragma unroll
                             for (int pr = 0; pr < Prods<NSPLIT>::N; ++pr) {
-                                const uint32_t a_s = sa + prod_a(pr) * ps + kk * ak;
-                                const uint32_t b_s = sb + prod_b(pr) * ps + kk * bk;
+                                const uint32_t a_s = sa + (M.swap ? prod_b(pr) : prod_a(pr)) * ps + kk * ak;
+                                const uint32_t b_s = sb + (M.swap ? prod_a(pr) : prod_b(pr)) * ps + kk * bk;
                                 const uint32_t acc = ((M.flags & 1) && kk == 0 && pr == 0) ? 0u : 1u;
                                 mma_bf16(dt, ab | ((a_s & 0x3FFFFu) >> 4), bb | ((b_s & 0x3FFFFu) >> 4), id, acc);
                             }
@@ -908,7 +923,7 @@ void TmaWorkList::add_block(int64_t c_off, int c_buf, int m, int n, int ldc, con
         for (int m0 = 0; m0 < m; m0 += TM)
             for (int n0 = 0; n0 < n; n0 += tn) {
                 Tile t{};
-                t.tn = tn;
+                t.tn = (uint8_t)tn;
                 t.alpha = alpha;
                 t.c_off = c_off;
                 t.ldc = ldc;
@@ -923,6 +938,31 @@ void TmaWorkList::add_block(int64_t c_off, int c_buf, int m, int n, int ldc, con
                 t.nst = (uint16_t)nst;
                 tiles.push_back(t);
             }
+    }
+}
+
+void TmaWorkList::add_stack(int64_t c_off, int c_buf, int m, int n, int ldc, const TSeg& s, float alpha, int sn, int sb,
+                            int tn) {
+    if (m <= 0 || n <= 0 || sn <= 0) return;
+    const int sbeg = (int)segs.size();
+    segs.push_back(s);
+    for (int n0 = 0; n0 < n; n0 += tn) {
+        Tile t{};
+        t.tn = (uint8_t)tn;
+        t.sn = (uint8_t)sn;
+        t.sb = (uint8_t)sb;
+        t.alpha = alpha;
+        t.c_off = c_off;
+        t.ldc = ldc;
+        t.m = m;
+        t.n = n;
+        t.n0 = n0;
+        t.seg_beg = sbeg;
+        t.seg_end = sbeg + 1;
+        t.c_buf = (uint8_t)c_buf;
+        t.mode = TC_STORE_SPLIT;
+        t.nst = (uint16_t)((s.k + TK - 1) / TK);
+        tiles.push_back(t);
     }
 }
 
@@ -1017,7 +1057,7 @@ void MapTable::encode_upload(const TcBufs& tb, int nsplit, cudaStream_t st) {
             DMRG_REQUIRE(base != nullptr, DMRG_EINVAL, "tensor map over an unset buffer");
             const cuuint64_t dims[4] = {(cuuint64_t)k.cols, (cuuint64_t)k.rows, (cuuint64_t)k.nz, (cuuint64_t)k.nv};
             const cuuint64_t strides[3] = {(cuuint64_t)k.ld * 2, (cuuint64_t)k.zstride * 2, (cuuint64_t)k.vstride * 2};
-            const cuuint32_t box[4] = {64, (cuuint32_t)box_rows(k.rows), 1, 1};
+            const cuuint32_t box[4] = {64, (cuuint32_t)box_rows(k.rows), (cuuint32_t)k.bz, 1};
             const cuuint32_t estr[4] = {1, 1, 1, 1};
             const CUresult r = fn(&h[3 * i + pc], CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, (void*)(base + k.off), dims,
                                   strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,

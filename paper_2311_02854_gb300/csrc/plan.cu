@@ -614,11 +614,13 @@ MapKey view_key(const View& V, int64_t rows, int64_t cols, const int64_t* vstrid
     return k;
 }
 
-// out (m x n) += sign * op(A) (m x k) * op(B) (k x n) through tensor maps
+// out (m x n) += sign * op(A) (m x k) * op(B) (k x n) through tensor maps; bz > 1:
+// A's boxes hold bz operators of its family from number A.z on
 TSeg make_tseg(MapTable& mt, const View& A, const View& B, int m, int n, int k, double sign, const int64_t* vstride,
-               int nv) {
+               int nv, int bz = 1) {
     TSeg s{};
-    const MapKey ka = view_key(A, A.tr ? k : m, A.tr ? m : k, vstride, nv);
+    MapKey ka = view_key(A, A.tr ? k : m, A.tr ? m : k, vstride, nv);
+    ka.bz = bz;
     const MapKey kb = view_key(B, B.tr ? n : k, B.tr ? k : n, vstride, nv);
     s.a_map = mt.get(ka);
     s.b_map = mt.get(kb);
@@ -631,6 +633,7 @@ TSeg make_tseg(MapTable& mt, const View& A, const View& B, int m, int n, int k, 
     s.b_tr = B.tr;
     s.a_pv = (vstride && vstride[A.buf] > 0) ? 1 : 0;
     s.b_pv = (vstride && vstride[B.buf] > 0) ? 1 : 0;
+    s.a_bz = (uint8_t)bz;
     s.sign = sign < 0.0 ? -1.0f : 1.0f;
     return s;
 }
@@ -659,6 +662,7 @@ void ProductList::lower_tma(int8_t sbuf_, int8_t ibuf, int ild, int64_t cap, int
     struct Item {
         int kind = 0;  // 3: three factors; 2: scaled two-factor product; 1: direct segment
         bool pq_first = true;
+        bool neg = false;     // kind 3: the stored product has the other sign (its stack's first item's alpha)
         int tr = 0, tcl = 0;  // phase-1 product rows / columns
         int grp = -1, z = 0;
         View X, Y;            // direct / scaled two-factor operands
@@ -678,7 +682,6 @@ void ProductList::lower_tma(int8_t sbuf_, int8_t ibuf, int ild, int64_t cap, int
     while (i < cs.size()) {
         ChunkPlan cp;
         cp.i = i;
-        std::unordered_map<int64_t, int> gidx;  // (rows << 32 | cols) -> scratch group
         size_t j = i;
         for (; j < cs.size(); ++j) {
             const Contrib& c = cs[j];
@@ -691,8 +694,10 @@ void ProductList::lower_tma(int8_t sbuf_, int8_t ibuf, int ild, int64_t cap, int
                 const double cost_qr = 2.0 * c.k1 * c.k2 * c.n + 2.0 * c.m * c.k1 * c.n;
                 it.kind = 3;
                 it.pq_first = cost_pq <= cost_qr;
-                it.tr = it.pq_first ? c.m : c.k1;
-                it.tcl = it.pq_first ? c.k2 : c.n;
+                // the operator is the product's left factor: O Psi, or R^T Psi^T (the
+                // transpose of Psi R), so that operators can be stacked along its rows
+                it.tr = it.pq_first ? c.m : c.n;
+                it.tcl = it.pq_first ? c.k2 : c.k1;
             } else {
                 if (nreal == 2) {
                     if (c.P.ident) {
@@ -722,29 +727,153 @@ void ProductList::lower_tma(int8_t sbuf_, int8_t ibuf, int ild, int64_t cap, int
                 }
             }
             int64_t need = 0;
-            if (it.kind >= 2) need = (int64_t)it.tr * round_up(it.tcl, 8);
+            if (it.kind >= 2) need = it.kind == 2 || it.pq_first ? (int64_t)it.tr * round_up(it.tcl, 8) : (int64_t)c.k1 * round_up(c.n, 8);
             if (cp.used + need > cap && cp.used > 0) break;
-            if (it.kind >= 2) {
-                const int64_t key = ((int64_t)it.tr << 32) | (int64_t)it.tcl;
-                auto g = gidx.find(key);
-                if (g == gidx.end()) {
-                    g = gidx.emplace(key, (int)cp.groups.size()).first;
-                    cp.groups.push_back({(int64_t)it.tr, (int64_t)it.tcl, 0, 0});
-                }
-                it.grp = g->second;
-                it.z = (int)cp.groups[it.grp][2]++;
-            }
             cp.used += need;
             cp.items.push_back(it);
         }
+        cp.j = j;
+        plans.push_back(std::move(cp));
+        i = j;
+    }
+    // pass 1b: the phase-1 products of every chunk.  Items with the same operator,
+    // sector and |alpha| share one product (a sign is the MMA's negate bit); the
+    // products of consecutive operators of a family with one sector are stacked
+    // along the rows of a tile, as many as fit its 128 rows, and get consecutive
+    // scratch slots.  Tiles of one 21 x 21 product each (K = 24, D = 500) used a
+    // sixth of a tile's rows and loaded the sector once per operator.
+    struct Stack {
+        size_t item;  // the first product's item (index in the chunk)
+        int n;        // products
+    };
+    std::vector<std::vector<Stack>> stacks(plans.size());
+    auto op_view = [&](const Contrib& c, const Item& it) { return it.pq_first ? c.P : c.R.T(); };
+    // operators per tile: K-major rows are stacked 16 * sb rows apart, MN-major
+    // ones in 64-wide halves
+    auto stack_rows = [](const View& A, int m) { return A.tr ? 64 : box_rows(m); };
+    auto stack_max = [&](const View& A, int m) { return m > 64 ? 1 : (A.tr ? 2 : 128 / stack_rows(A, m)); };
+    for (size_t ch = 0; ch < plans.size(); ++ch) {
+        ChunkPlan& cp = plans[ch];
+        const size_t ni = cp.items.size();
+        struct Key {
+            uint64_t h;
+            int64_t off, alpha;  // family block (without the operator number) and |alpha|
+            int32_t buf, sec;
+            bool operator==(const Key& o) const {
+                return off == o.off && alpha == o.alpha && buf == o.buf && sec == o.sec;
+            }
+        };
+        struct KeyHash {
+            size_t operator()(const Key& k) const { return (size_t)k.h; }
+        };
+        std::vector<Key> keys(ni);
+        const size_t kPart = ni < 4096 ? 1 : 16;
+        const size_t nb = (ni + 4095) / 4096;
+        parallel_for(nb, [&](size_t b) {
+            for (size_t q = b * 4096; q < std::min(ni, (b + 1) * 4096); ++q) {
+                const Item& it = cp.items[q];
+                if (it.kind != 3) continue;
+                const Contrib& c = cs[cp.i + q];
+                const View A = op_view(c, it);
+                Key& k = keys[q];
+                const double aa = std::fabs(c.alpha);
+                std::memcpy(&k.alpha, &aa, 8);
+                k.off = A.off - (int64_t)A.z * A.zstride;
+                k.buf = A.buf * 4 + (A.tr ? 2 : 0) + (it.pq_first ? 1 : 0);
+                k.sec = c.qsec;
+                uint64_t h = 0x9e3779b97f4a7c15ull;
+                for (uint64_t x : {(uint64_t)k.off, (uint64_t)k.alpha, ((uint64_t)(uint32_t)k.buf << 32) | (uint32_t)k.sec}) {
+                    h ^= x + 0x9e3779b97f4a7c15ull + (h << 6) + (h >> 2);
+                    h *= 0xff51afd7ed558ccdull;
+                }
+                k.h = h ^ (h >> 33);
+            }
+        });
+        // partitions of the keys on host threads: per key its items by operator
+        // number, one product per number, runs of consecutive numbers cut to tiles
+        struct Prod {
+            int32_t z;
+            uint32_t item;
+        };
+        std::vector<std::vector<Stack>> pst(kPart);
+        std::vector<std::vector<std::pair<uint32_t, uint32_t>>> same(kPart);  // (item, item whose product it uses)
+        parallel_for(kPart, [&](size_t pt) {
+            std::unordered_map<Key, int, KeyHash> idx;
+            std::vector<std::vector<Prod>> lists;
+            for (size_t q = 0; q < ni; ++q) {
+                if (cp.items[q].kind != 3 || (keys[q].h >> 40) % kPart != pt) continue;
+                auto f = idx.emplace(keys[q], (int)lists.size());
+                if (f.second) lists.emplace_back();
+                lists[f.first->second].push_back({op_view(cs[cp.i + q], cp.items[q]).z, (uint32_t)q});
+            }
+            for (auto& l : lists) {
+                std::stable_sort(l.begin(), l.end(), [](const Prod& a, const Prod& b) { return a.z < b.z; });
+                const Item& it0 = cp.items[l[0].item];
+                const int most = stack_max(op_view(cs[cp.i + l[0].item], it0), it0.tr);
+                int last = -2;
+                uint32_t first = 0;
+                for (const Prod& x : l) {
+                    if (x.z == last) {  // the same product
+                        same[pt].push_back({x.item, first});
+                        continue;
+                    }
+                    if (!pst[pt].empty() && last >= 0 && x.z == last + 1 && pst[pt].back().n < most) ++pst[pt].back().n;
+                    else pst[pt].push_back({x.item, 1});
+                    // slot of the product, relative to its stack's first for now
+                    cp.items[x.item].z = pst[pt].back().n - 1;
+                    cp.items[x.item].neg = (cs[cp.i + x.item].alpha < 0.0) != (cs[cp.i + pst[pt].back().item].alpha < 0.0);
+                    cp.items[x.item].grp = (int)(pst[pt].size() - 1);
+                    last = x.z;
+                    first = x.item;
+                }
+            }
+        });
+        // scratch slots: groups of equal shape, a stack's products consecutive
+        std::unordered_map<int64_t, int> gidx;  // (rows << 32 | cols) -> scratch group
+        auto group_of = [&](const Item& it) {
+            const int64_t key = ((int64_t)it.tr << 32) | (int64_t)it.tcl;
+            auto g = gidx.find(key);
+            if (g == gidx.end()) {
+                g = gidx.emplace(key, (int)cp.groups.size()).first;
+                cp.groups.push_back({(int64_t)it.tr, (int64_t)it.tcl, 0, 0});
+            }
+            return g->second;
+        };
+        std::vector<std::vector<std::pair<int, int>>> at(kPart);  // stack -> (group, first slot)
+        for (size_t pt = 0; pt < kPart; ++pt) {
+            at[pt].resize(pst[pt].size());
+            for (size_t x = 0; x < pst[pt].size(); ++x) {
+                const int g = group_of(cp.items[pst[pt][x].item]);
+                at[pt][x] = {g, (int)cp.groups[g][2]};
+                cp.groups[g][2] += pst[pt][x].n;
+            }
+        }
+        for (Item& it : cp.items)
+            if (it.kind == 2) {
+                it.grp = group_of(it);
+                it.z = (int)cp.groups[it.grp][2]++;
+            }
+        parallel_for(kPart, [&](size_t pt) {
+            for (size_t q = 0; q < ni; ++q) {
+                Item& it = cp.items[q];
+                if (it.kind != 3 || (keys[q].h >> 40) % kPart != pt || it.grp < 0) continue;
+                const auto& a = at[pt][it.grp];
+                it.grp = a.first;
+                it.z += a.second;
+            }
+            for (const auto& d : same[pt]) {
+                cp.items[d.first].grp = cp.items[d.second].grp;
+                cp.items[d.first].z = cp.items[d.second].z;
+                cp.items[d.first].neg = cp.items[d.second].neg != ((cs[cp.i + d.first].alpha < 0.0) != (cs[cp.i + d.second].alpha < 0.0));
+            }
+        });
         int64_t base = 0;
         for (auto& g : cp.groups) {
             g[3] = base;
             base += g[2] * g[0] * round_up(g[1], 8);
         }
-        cp.j = j;
-        plans.push_back(std::move(cp));
-        i = j;
+        cp.used = base;
+        for (auto& l : pst) stacks[ch].insert(stacks[ch].end(), l.begin(), l.end());
     }
     // pass 2: the work lists.  Each chunk's items are cut into units of at
     // most kUnit items that run on host threads, each with a tensor-map table
@@ -795,16 +924,13 @@ void ProductList::lower_tma(int8_t sbuf_, int8_t ibuf, int ild, int64_t cap, int
                 T.off = g[3] + (int64_t)it.z * T.zstride;
             }
             if (it.kind == 3) {
+                const double sg = it.neg ? -1.0 : 1.0;
                 if (it.pq_first) {
                     fl += 2.0 * c.m * c.k1 * c.k2 + 2.0 * c.m * c.k2 * c.n;
-                    p1.add_block(T.off, sbuf, c.m, c.k2, T.ld, {make_tseg(lm, c.P, c.Q, c.m, c.k2, c.k1, 1.0, vstride, nv)},
-                                 TC_STORE_SPLIT, 0, (float)c.alpha, tile_n);
-                    u.osegs.push_back({c.out, make_tseg(lm, T, c.R, c.m, c.n, c.k2, 1.0, vstride, nv)});
+                    u.osegs.push_back({c.out, make_tseg(lm, T, c.R, c.m, c.n, c.k2, sg, vstride, nv)});
                 } else {
                     fl += 2.0 * c.k1 * c.k2 * c.n + 2.0 * c.m * c.k1 * c.n;
-                    p1.add_block(T.off, sbuf, c.k1, c.n, T.ld, {make_tseg(lm, c.Q, c.R, c.k1, c.n, c.k2, 1.0, vstride, nv)},
-                                 TC_STORE_SPLIT, 0, (float)c.alpha, tile_n);
-                    u.osegs.push_back({c.out, make_tseg(lm, c.P, T, c.m, c.n, c.k1, 1.0, vstride, nv)});
+                    u.osegs.push_back({c.out, make_tseg(lm, c.P, T.T(), c.m, c.n, c.k1, sg, vstride, nv)});
                 }
             } else if (it.kind == 2) {
                 fl += it.fl;
@@ -815,6 +941,23 @@ void ProductList::lower_tma(int8_t sbuf_, int8_t ibuf, int ild, int64_t cap, int
                 fl += it.fl;
                 u.osegs.push_back({c.out, make_tseg(lm, it.X, it.Y, c.m, c.n, it.k, c.alpha, vstride, nv)});
             }
+        }
+        // the unit's share of the chunk's stacks
+        const std::vector<Stack>& sk = stacks[u.ch];
+        const size_t nu = unit_beg[u.ch + 1] - unit_beg[u.ch], un = ui - unit_beg[u.ch];
+        for (size_t x = sk.size() * un / nu; x < sk.size() * (un + 1) / nu; ++x) {
+            const Contrib& c = cs[cp.i + sk[x].item];
+            const Item& it = cp.items[sk[x].item];
+            const auto& g = cp.groups[it.grp];
+            const int ld = (int)round_up(g[1], 8);
+            const int64_t off = g[3] + (int64_t)it.z * g[0] * ld;
+            const View A = op_view(c, it), Q = it.pq_first ? c.Q : c.Q.T();
+            const int k = it.pq_first ? c.k1 : c.k2;
+            const int most = stack_max(A, it.tr);
+            TSeg s = make_tseg(lm, A, Q, it.tr, it.tcl, k, 1.0, vstride, nv, most);
+            s.swap = it.pq_first ? 0 : 1;
+            if (most > 1) p1.add_stack(off, sbuf, it.tr, it.tcl, ld, s, (float)c.alpha, sk[x].n, stack_rows(A, it.tr) / 16, tile_n);
+            else p1.add_block(off, sbuf, it.tr, it.tcl, ld, {s}, TC_STORE_SPLIT, 0, (float)c.alpha, tile_n);
         }
         u.fl = fl;
     });

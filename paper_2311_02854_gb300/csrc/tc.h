@@ -58,7 +58,8 @@ struct TSeg {
     uint8_t a_tr, b_tr;    // a_tr: A held as K x M (MN-major); b_tr: B held as N x K (K-major)
     uint8_t a_pv, b_pv;    // 1: the operand's w coordinate is the vector index
     uint8_t a_br, b_br;    // rows of the maps' boxes (min(64, rows rounded up to 16))
-    uint8_t pad[2];
+    uint8_t a_bz;          // operator rows of A's boxes (stacked products: up to 8, else 1)
+    uint8_t swap;          // the factors of the product trade sides: its cross terms run in the other order
     float sign;            // +1 or -1 (MMA negate bit)
 };
 
@@ -73,6 +74,9 @@ struct TmaWorkList {
     // 128), split into K-chunks of at most kchunk (atomic modes only)
     void add_block(int64_t c_off, int c_buf, int m, int n, int ldc, const std::vector<TSeg>& s, uint8_t mode,
                    int64_t kchunk, float alpha, int tn = 128);
+    // sn stored products (m x n, ld ldc, m * ldc apart from c_off on) of one tile
+    // row: product i in accumulator rows i * 16 * sb ...
+    void add_stack(int64_t c_off, int c_buf, int m, int n, int ldc, const TSeg& s, float alpha, int sn, int sb, int tn);
     void order_tiles();  // longest tiles first (stable)
     void upload(cudaStream_t st);
     void release();
@@ -80,21 +84,22 @@ struct TmaWorkList {
 
 // A matrix as a tensor-map key: element (z, y, x) of vector w of buffer `buf`
 // lives at off + w*vstride + z*zstride + y*ld + x (elements), x < cols, y < rows.
-// Its boxes are 64 columns x box_rows(rows) rows.
+// Its boxes are 64 columns x box_rows(rows) rows x bz operator rows.
 inline int box_rows(int64_t rows) { return rows >= 64 ? 64 : (int)((rows + 15) / 16 * 16); }
 struct MapKey {
     int buf;
     int64_t off;
     int64_t cols, rows, ld, nz, zstride, nv, vstride;
-    auto tie() const { return std::tie(buf, off, cols, rows, ld, nz, zstride, nv, vstride); }
+    int bz = 1;  // operator rows of a box
+    auto tie() const { return std::tie(buf, off, cols, rows, ld, nz, zstride, nv, vstride, bz); }
     bool operator<(const MapKey& o) const { return tie() < o.tie(); }
 };
 
 struct MapKeyHash {
     size_t operator()(const MapKey& k) const {
         uint64_t h = 0x9e3779b97f4a7c15ull ^ (uint64_t)k.buf;
-        const int64_t v[9] = {k.off, k.cols, k.rows, k.ld, k.nz, k.zstride, k.nv, k.vstride, 0};
-        for (int i = 0; i < 8; ++i) {
+        const int64_t v[9] = {k.off, k.cols, k.rows, k.ld, k.nz, k.zstride, k.nv, k.vstride, k.bz};
+        for (int i = 0; i < 9; ++i) {
             h ^= (uint64_t)v[i] + 0x9e3779b97f4a7c15ull + (h << 6) + (h >> 2);
             h *= 0xff51afd7ed558ccdull;
         }
