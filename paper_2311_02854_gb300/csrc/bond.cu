@@ -322,7 +322,7 @@ void ensure_ident(Plan& P, int n) {
         const int64_t nn = (int64_t)P.id_n * P.id_n;
         P.id_hi = P.alloc_bf16(nn);
         P.id_lo = P.alloc_lo(nn);
-        dev_split_f64(P.d_ident, 1, (int)nn, nn, P.id_hi, P.id_lo, nn, P.stream, P.lo2(P.id_lo, nn));
+        dev_split_f64_flat(P.d_ident, nn, P.id_hi, P.id_lo, P.stream, P.lo2(P.id_lo, nn));
     }
 }
 
@@ -434,7 +434,7 @@ void form_interms(Plan& P, Interms& im, const Block* blocks[2], IntermStore& S, 
             P.w_hi = P.alloc_bf16(wn);
             P.w_lo = P.alloc_lo(wn);
         }
-        dev_split_f64(P.d_wcoef, 1, (int)wn, wn, P.w_hi, P.w_lo, wn, P.stream, P.lo2(P.w_lo, P.n_wpc));
+        dev_split_f64_flat(P.d_wcoef, wn, P.w_hi, P.w_lo, P.stream, P.lo2(P.w_lo, P.n_wpc));
         // FP32 sum of the K-chunks, then split into the bf16 pieces
         double* acc = P.alloc(S.n);  // FP64 sum of the K-chunks, then split into the pieces
         DMRG_CHECK_CUDA(cudaMemsetAsync(acc, 0, S.n * 8, P.stream));
@@ -536,7 +536,7 @@ static SiteDev upload_site(Plan& P, int k) {
     if (P.mixed()) {
         S.h = P.alloc_bf16(S.n);
         S.l = P.alloc_lo(S.n);
-        dev_split_f64(S.d, 1, (int)S.n, S.n, S.h, S.l, S.n, P.stream, P.lo2(S.l, S.n));
+        dev_split_f64_flat(S.d, S.n, S.h, S.l, P.stream, P.lo2(S.l, S.n));
     }
     DMRG_CHECK_CUDA(cudaStreamSynchronize(P.stream));
     return S;

@@ -96,8 +96,8 @@ dmrg_status grouped_gemm_tc(int nsplit, int n_out, const int* m, const int* n, c
     DMRG_CHECK_CUDA(cudaMalloc(&ctr, 2 * sizeof(int)));
     DMRG_CHECK_CUDA(cudaMemsetAsync(ctr, 0, 2 * sizeof(int), st));
     DMRG_REQUIRE(ea < 2147483647 && eb < 2147483647, DMRG_EINVAL, "operand too large");
-    dev_split_f64(a, 1, (int)ea_n, ea_n, ha, la, ea, st, nsplit == 3 ? la + ea : nullptr);
-    dev_split_f64(b, 1, (int)eb_n, eb_n, hb, lb, eb, st, nsplit == 3 ? lb + eb : nullptr);
+    dev_split_f64_flat(a, ea_n, ha, la, st, nsplit == 3 ? la + ea : nullptr, ea);
+    dev_split_f64_flat(b, eb_n, hb, lb, st, nsplit == 3 ? lb + eb : nullptr, eb);
     if (ec > 0) DMRG_CHECK_CUDA(cudaMemsetAsync(c, 0, ec * 8, st));
     wl.upload(st);
     TcBufs tb{};

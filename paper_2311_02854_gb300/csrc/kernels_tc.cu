@@ -786,49 +786,91 @@ __global__ void __launch_bounds__(THREADS3, kCtas3)
 // conversions
 // ---------------------------------------------------------------------------
 
-// x -> hi (+ lo (+ lo2)): each piece is the bf16 rounding of what the previous ones leave
-__device__ __forceinline__ void split3(double xd, __nv_bfloat16* hi, __nv_bfloat16* lo, __nv_bfloat16* lo2,
-                                      int64_t i) {
-    const __nv_bfloat16 h = __float2bfloat16_rn((float)xd);
-    hi[i] = h;
-    if (lo) {
-        const double r = xd - (double)__bfloat162float(h);
-        const __nv_bfloat16 l = __float2bfloat16_rn((float)r);
-        lo[i] = l;
-        if (lo2) lo2[i] = __float2bfloat16_rn((float)(r - (double)__bfloat162float(l)));
+// x -> hi + lo + lo2: each piece is the bf16 rounding (through FP32) of what the
+// previous ones leave.  Bound: HBM (14 bytes per element with two pieces) once
+// the FP64 pipe is out of the way: conversions between FP64 and FP32 run there
+// at ~2 per cycle and SM, and four of them per element took 180 us for 26
+// million elements (79 us at the copy rate).  So x is rounded to FP32 by integer
+// operations on its bits, and what that leaves, an integer of 29 bits in units
+// of x's last place, is converted as an integer; the sums below are then those
+// of FP32 numbers, exact but for their own rounding.
+struct Pieces {
+    __nv_bfloat16 h, l, m;
+};
+__device__ __forceinline__ Pieces split_pieces(double xd) {
+    const uint32_t hi = (uint32_t)__double2hiint(xd), lo = (uint32_t)__double2loint(xd);
+    const int eb = (int)((hi >> 20) & 0x7FFu);
+    Pieces p;
+    if (eb >= 1023 - 90 && eb < 1023 + 126) {
+        uint32_t f = (hi & 0x80000000u) | ((uint32_t)(eb - 896) << 23) | ((hi & 0xFFFFFu) << 3) | (lo >> 29);
+        const uint32_t rem = lo & 0x1FFFFFFFu;
+        const uint32_t up = (rem > 0x10000000u || (rem == 0x10000000u && (f & 1u))) ? 1u : 0u;  // to nearest even
+        f += up;
+        int left = (int)rem - (up ? 0x20000000 : 0);  // |x| - |f| in units of 2^(eb - 1075)
+        if (hi >> 31) left = -left;
+        const float xf = __uint_as_float(f);
+        const float e = __int2float_rn(left) * 0x1p-52f * __uint_as_float((uint32_t)(eb - 896) << 23);
+        p.h = __float2bfloat16_rn(xf);
+        const float d = __fsub_rn(xf, __bfloat162float(p.h));
+        p.l = __float2bfloat16_rn(__fadd_rn(d, e));
+        p.m = __float2bfloat16_rn(__fadd_rn(__fsub_rn(d, __bfloat162float(p.l)), e));
+    } else if ((hi << 1 | lo) == 0u) {
+        p.h = __ushort_as_bfloat16((unsigned short)(hi >> 16));
+        p.l = p.m = __ushort_as_bfloat16((unsigned short)0);
+    } else {  // outside FP32's comfortable range, infinities, NaN
+        p.h = __float2bfloat16_rn((float)xd);
+        const double r = xd - (double)__bfloat162float(p.h);
+        p.l = __float2bfloat16_rn((float)r);
+        p.m = __float2bfloat16_rn((float)(r - (double)__bfloat162float(p.l)));
+    }
+    return p;
+}
+__device__ __forceinline__ uint32_t pack2(__nv_bfloat16 a, __nv_bfloat16 b) {
+    return (uint32_t)__bfloat16_as_ushort(a) | ((uint32_t)__bfloat16_as_ushort(b) << 16);
+}
+
+// n elements, then zeros up to ldd; VEC: four elements per thread and step
+// (src 16-byte, pieces 8-byte aligned)
+template <bool VEC>
+__global__ void split_f64_flat_kernel(const double* __restrict__ src, int64_t n, int64_t ldd,
+                                      __nv_bfloat16* __restrict__ hi, __nv_bfloat16* __restrict__ lo,
+                                      __nv_bfloat16* __restrict__ lo2) {
+    const int64_t t0 = (int64_t)blockIdx.x * blockDim.x + threadIdx.x, nt = (int64_t)gridDim.x * blockDim.x;
+    const int64_t nv = VEC ? n / 4 : 0;
+    if (VEC) {
+        for (int64_t i = t0; i < nv; i += nt) {
+            const double2 a = ((const double2*)src)[2 * i], b = ((const double2*)src)[2 * i + 1];
+            const Pieces p[4] = {split_pieces(a.x), split_pieces(a.y), split_pieces(b.x), split_pieces(b.y)};
+            ((uint2*)hi)[i] = make_uint2(pack2(p[0].h, p[1].h), pack2(p[2].h, p[3].h));
+            if (lo) ((uint2*)lo)[i] = make_uint2(pack2(p[0].l, p[1].l), pack2(p[2].l, p[3].l));
+            if (lo2) ((uint2*)lo2)[i] = make_uint2(pack2(p[0].m, p[1].m), pack2(p[2].m, p[3].m));
+        }
+    }
+    for (int64_t i = 4 * nv + t0; i < ldd; i += nt) {
+        const Pieces p = split_pieces(i < n ? src[i] : 0.0);
+        hi[i] = p.h;
+        if (lo) lo[i] = p.l;
+        if (lo2) lo2[i] = p.m;
     }
 }
 
-__global__ void split_f64_kernel(const double* __restrict__ src, int64_t rows, int n, int64_t lds,
-                                 __nv_bfloat16* __restrict__ hi, __nv_bfloat16* __restrict__ lo, int64_t ldd,
-                                 __nv_bfloat16* __restrict__ lo2) {
-    const int64_t tot = rows * ldd;
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < tot; i += (int64_t)gridDim.x * blockDim.x) {
-        const int64_t r = i / ldd, c = i % ldd;
-        split3((c < n) ? src[r * lds + c] : 0.0, hi, lo, lo2, i);
-    }
-}
-
-__global__ void split_f64_flat_kernel(const double* __restrict__ src, int64_t n, __nv_bfloat16* __restrict__ hi,
-                                      __nv_bfloat16* __restrict__ lo, __nv_bfloat16* __restrict__ lo2) {
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
-        split3(src[i], hi, lo, lo2, i);
-}
-
-__global__ void split_f32_kernel(const float* __restrict__ src, int64_t n, __nv_bfloat16* __restrict__ hi,
-                                 __nv_bfloat16* __restrict__ lo, __nv_bfloat16* __restrict__ lo2) {
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
-        split3((double)src[i], hi, lo, lo2, i);
-}
-
+// one job per blockIdx.x, its rows dealt to the warps of gridDim.y blocks (one
+// block per job left most SMs idle: K = 14, D = 600 has sectors of 13 000
+// elements on 1.8 waves of blocks, 104 us for 0.6 million elements)
 __global__ void split_blocks_kernel(const double* __restrict__ src, const SplitJob* __restrict__ jobs,
                                     __nv_bfloat16* __restrict__ hi, __nv_bfloat16* __restrict__ lo,
                                     __nv_bfloat16* __restrict__ lo2) {
     const SplitJob J = jobs[blockIdx.x];
-    const int64_t tot = (int64_t)J.rows * J.ld_dst;
-    for (int64_t i = threadIdx.x; i < tot; i += blockDim.x) {
-        const int r = (int)(i / J.ld_dst), c = (int)(i % J.ld_dst);
-        split3((c < J.cols) ? src[J.src_off + (int64_t)r * J.ld_src + c] : 0.0, hi, lo, lo2, J.dst_off + i);
+    const int nw = blockDim.x / 32, lane = threadIdx.x & 31;
+    for (int r = blockIdx.y * nw + threadIdx.x / 32; r < J.rows; r += gridDim.y * nw) {
+        const double* q = src + J.src_off + (int64_t)r * J.ld_src;
+        const int64_t o = J.dst_off + (int64_t)r * J.ld_dst;  // offsets and leading dimensions are multiples of 8
+        for (int c = 2 * lane; c < J.ld_dst; c += 64) {
+            const Pieces a = split_pieces(c < J.cols ? q[c] : 0.0), b = split_pieces(c + 1 < J.cols ? q[c + 1] : 0.0);
+            *(uint32_t*)(hi + o + c) = pack2(a.h, b.h);
+            if (lo) *(uint32_t*)(lo + o + c) = pack2(a.l, b.l);
+            if (lo2) *(uint32_t*)(lo2 + o + c) = pack2(a.m, b.m);
+        }
     }
 }
 
@@ -1131,26 +1173,13 @@ void launch_seg_gemm_tma(const TmaWorkList& w, const MapTable& maps, const TcBuf
     DMRG_CHECK_CUDA(cudaGetLastError());
 }
 
-void dev_split_f64(const double* src, int64_t rows, int n, int64_t ld_src, __nv_bfloat16* hi, __nv_bfloat16* lo,
-                   int64_t ld_dst, cudaStream_t st, __nv_bfloat16* lo2) {
-    if (rows <= 0) return;
-    split_f64_kernel<<<grid_for(rows * ld_dst), 256, 0, st>>>(src, rows, n, ld_src, hi, lo, ld_dst, lo2);
-    ++launch_counter();
-    DMRG_CHECK_CUDA(cudaGetLastError());
-}
-
 void dev_split_f64_flat(const double* src, int64_t n, __nv_bfloat16* hi, __nv_bfloat16* lo, cudaStream_t st,
-                        __nv_bfloat16* lo2) {
-    if (n <= 0) return;
-    split_f64_flat_kernel<<<grid_for(n), 256, 0, st>>>(src, n, hi, lo, lo2);
-    ++launch_counter();
-    DMRG_CHECK_CUDA(cudaGetLastError());
-}
-
-void dev_split_f32(const float* src, int64_t n, __nv_bfloat16* hi, __nv_bfloat16* lo, cudaStream_t st,
-                   __nv_bfloat16* lo2) {
-    if (n <= 0) return;
-    split_f32_kernel<<<grid_for(n), 256, 0, st>>>(src, n, hi, lo, lo2);
+                        __nv_bfloat16* lo2, int64_t n_pad) {
+    n_pad = std::max(n, n_pad);
+    if (n_pad <= 0) return;
+    const bool vec = ((uintptr_t)src & 15) == 0 && (((uintptr_t)hi | (uintptr_t)lo | (uintptr_t)lo2) & 7) == 0;
+    if (vec) split_f64_flat_kernel<true><<<grid_for((n_pad + 3) / 4), 256, 0, st>>>(src, n, n_pad, hi, lo, lo2);
+    else split_f64_flat_kernel<false><<<grid_for(n_pad), 256, 0, st>>>(src, n, n_pad, hi, lo, lo2);
     ++launch_counter();
     DMRG_CHECK_CUDA(cudaGetLastError());
 }
@@ -1158,7 +1187,7 @@ void dev_split_f32(const float* src, int64_t n, __nv_bfloat16* hi, __nv_bfloat16
 void dev_split_blocks(const double* src, const SplitJob* d_jobs, int njobs, __nv_bfloat16* hi, __nv_bfloat16* lo,
                       cudaStream_t st, __nv_bfloat16* lo2) {
     if (njobs <= 0) return;
-    split_blocks_kernel<<<njobs, 256, 0, st>>>(src, d_jobs, hi, lo, lo2);
+    split_blocks_kernel<<<dim3(njobs, 16), 256, 0, st>>>(src, d_jobs, hi, lo, lo2);
     ++launch_counter();
     DMRG_CHECK_CUDA(cudaGetLastError());
 }

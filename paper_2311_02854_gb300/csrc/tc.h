@@ -131,16 +131,10 @@ struct MapTable {
 void launch_seg_gemm_tma(const TmaWorkList& w, const MapTable& maps, const TcBufs& b, int nvec, int nsplit,
                          cudaStream_t st);
 
-// FP64 (unpadded rows of length n, ld_src) -> bf16 pieces (rows padded to ld_dst);
-// lo2 (optional) receives the third piece x - hi - lo
-void dev_split_f64(const double* src, int64_t rows, int n, int64_t ld_src, __nv_bfloat16* hi,
-                   __nv_bfloat16* lo, int64_t ld_dst, cudaStream_t st, __nv_bfloat16* lo2 = nullptr);
-// FP64 -> bf16 pieces, same layout, n elements
+// FP64 -> bf16 pieces (hi, lo, optionally lo2), same layout, n elements, then
+// zeros up to n_pad (0: none); lo2 receives the third piece x - hi - lo
 void dev_split_f64_flat(const double* src, int64_t n, __nv_bfloat16* hi, __nv_bfloat16* lo, cudaStream_t st,
-                        __nv_bfloat16* lo2 = nullptr);
-// FP32 -> bf16 pieces, same layout, n elements
-void dev_split_f32(const float* src, int64_t n, __nv_bfloat16* hi, __nv_bfloat16* lo, cudaStream_t st,
-                   __nv_bfloat16* lo2 = nullptr);
+                        __nv_bfloat16* lo2 = nullptr, int64_t n_pad = 0);
 // batched block copy FP64 -> pieces: for each job (src_off, dst_off, rows, cols, ld_src, ld_dst)
 struct SplitJob {
     int64_t src_off, dst_off;
