@@ -129,6 +129,12 @@ void dev_fill(double* x, double v, int64_t n, cudaStream_t st);
 void dev_perturb(double* x, int64_t n, uint32_t seed, double amp, cudaStream_t st);
 void dev_identity(double* x, int n, cudaStream_t st);
 int64_t& launch_counter();
+// Pool of the grouped products' device memory on the current device: it keeps up
+// to kPoolKeep bytes between calls (any stream, any thread) and gives them back
+// when an allocation of a plan fails (trim_product_pool)
+constexpr uint64_t kPoolKeep = 1ull << 30;
+cudaMemPool_t product_pool();
+void trim_product_pool();
 // selftest.cu: one bounded mbarrier wait (arrived on or not); false if it gave up
 bool wait_selftest(double seconds, bool arrive, cudaStream_t st);
 

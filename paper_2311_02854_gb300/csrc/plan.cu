@@ -9,6 +9,7 @@
 #include <cmath>
 #include <cstring>
 #include <fstream>
+#include <mutex>
 #include <unordered_map>
 
 #include "bond.h"
@@ -132,6 +133,38 @@ bool MPSHost::write(const std::string& path) const {
 // Device memory
 // ---------------------------------------------------------------------------
 
+namespace {
+constexpr int kMaxDevices = 64;
+std::mutex g_pool_mu;
+cudaMemPool_t g_pools[kMaxDevices] = {};
+}  // namespace
+
+cudaMemPool_t product_pool() {
+    int dev = 0;
+    DMRG_CHECK_CUDA(cudaGetDevice(&dev));
+    DMRG_REQUIRE(dev >= 0 && dev < kMaxDevices, DMRG_ECUDA, "device number out of range");
+    std::lock_guard<std::mutex> lk(g_pool_mu);
+    if (!g_pools[dev]) {
+        cudaMemPoolProps props{};
+        props.allocType = cudaMemAllocationTypePinned;
+        props.location.type = cudaMemLocationTypeDevice;
+        props.location.id = dev;
+        cudaMemPool_t pool = nullptr;
+        DMRG_CHECK_CUDA(cudaMemPoolCreate(&pool, &props));
+        uint64_t keep = kPoolKeep;
+        DMRG_CHECK_CUDA(cudaMemPoolSetAttribute(pool, cudaMemPoolAttrReleaseThreshold, &keep));
+        g_pools[dev] = pool;
+    }
+    return g_pools[dev];
+}
+
+void trim_product_pool() {
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kMaxDevices) return;
+    std::lock_guard<std::mutex> lk(g_pool_mu);
+    if (g_pools[dev]) cudaMemPoolTrimTo(g_pools[dev], 0);
+}
+
 double* Plan::alloc(int64_t n) {
     if (n <= 0) return nullptr;
     int64_t bytes = n * 8;
@@ -139,6 +172,11 @@ double* Plan::alloc(int64_t n) {
                  "device budget exceeded (" + std::to_string((dev_bytes + bytes) >> 20) + " MiB)");
     void* p = nullptr;
     cudaError_t e = cudaMalloc(&p, bytes);
+    if (e != cudaSuccess) {  // once more without what the grouped products keep
+        cudaGetLastError();
+        trim_product_pool();
+        e = cudaMalloc(&p, bytes);
+    }
     if (e != cudaSuccess) {
         cudaGetLastError();
         throw Error(DMRG_ENOMEM, "cudaMalloc of " + std::to_string(bytes >> 20) + " MiB failed");
@@ -165,6 +203,11 @@ __nv_bfloat16* Plan::alloc_bf16(int64_t n) {
                  "device budget exceeded (" + std::to_string((dev_bytes + bytes) >> 20) + " MiB)");
     void* p = nullptr;
     cudaError_t e = cudaMalloc(&p, bytes);
+    if (e != cudaSuccess) {  // once more without what the grouped products keep
+        cudaGetLastError();
+        trim_product_pool();
+        e = cudaMalloc(&p, bytes);
+    }
     if (e != cudaSuccess) {
         cudaGetLastError();
         throw Error(DMRG_ENOMEM, "cudaMalloc of " + std::to_string(bytes >> 20) + " MiB failed");
