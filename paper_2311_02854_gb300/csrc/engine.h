@@ -31,10 +31,14 @@ struct Tile {
     int32_t seg_beg, seg_end;
     uint8_t c_buf, mode;
     uint16_t nst;         // tensor-core engine: 64-deep K stages of the tile (set by the TMA work list)
-    float alpha;          // epilogue scale (tensor-core engine; the FP64 engine scales per segment)
-    // TMA tensor-core engine: tile width (64 or 128 columns); products stacked along
-    // the rows (0: none; else product i holds accumulator rows i * 16 * sb ..., and
-    // its m x n block lies i * m * ldc elements behind c_off)
+    union {
+        float alpha;      // epilogue scale (bf16-piece engines; the FP64 engines scale per segment)
+        int32_t astride;  // FP64-accurate tensor-core engine: elements between the A of stacked products
+    };
+    // TMA tensor-core engine: tile width (64 or 128 columns).  Both tensor-core
+    // engines of sigma: products stacked along the rows (0: none; else product i
+    // holds accumulator rows i * 16 * sb ..., and its m x n block lies i * m * ldc
+    // elements behind c_off)
     uint8_t tn, sn, sb, pad;
 };
 static_assert(sizeof(Tile) == 48, "Tile keeps its 48-byte record");
@@ -78,6 +82,10 @@ struct WorkList {
     // K-chunks of at most kchunk when the block is atomically accumulated).
     void add_block(int64_t c_off, int c_buf, int m, int n, int ldc, const std::vector<Seg>& s,
                    uint8_t mode, int64_t kchunk = 0, int tile = 64, float alpha = 1.0f);
+    // FP64-accurate tensor-core engine: sn products (m x n, ld ldc, m * ldc apart from
+    // c_off on) whose first factor is `s`'s A, astride elements apart; product i in
+    // accumulator rows i * 16 * sb ... (16 * sb >= m, 16 * sb * sn <= 128)
+    void add_stack(int64_t c_off, int c_buf, int m, int n, int ldc, const Seg& s, int64_t astride, int sn, int sb);
     void upload(cudaStream_t st);
     void release();
 };

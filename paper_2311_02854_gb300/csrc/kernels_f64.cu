@@ -68,6 +68,30 @@ void WorkList::add_block(int64_t c_off, int c_buf, int m, int n, int ldc, const 
     }
 }
 
+void WorkList::add_stack(int64_t c_off, int c_buf, int m, int n, int ldc, const Seg& s, int64_t astride, int sn, int sb) {
+    if (m <= 0 || n <= 0 || sn <= 0) return;
+    DMRG_REQUIRE(std::abs(astride) < (1LL << 31), DMRG_EINVAL, "operators too far apart to be stacked");
+    const int sbeg = (int)segs.size();
+    segs.push_back(s);
+    flops += 2.0 * sn * m * n * (double)s.k;
+    for (int n0 = 0; n0 < n; n0 += tile_n) {
+        Tile t{};
+        t.astride = (int32_t)astride;
+        t.sn = (uint8_t)sn;
+        t.sb = (uint8_t)sb;
+        t.c_off = c_off;
+        t.ldc = ldc;
+        t.m = m;
+        t.n = n;
+        t.n0 = n0;
+        t.seg_beg = sbeg;
+        t.seg_end = sbeg + 1;
+        t.c_buf = (uint8_t)c_buf;
+        t.mode = TILE_STORE;
+        tiles.push_back(t);
+    }
+}
+
 namespace {
 constexpr int kSplitWarps = 4;  // warps of a CTA that share a part's term sum (FP64 units)
 }

@@ -7,14 +7,14 @@
 // transformations of matrix multiplication by using fast routines of matrix
 // multiplication", Numer. Algorithms 59, 2012):
 //
-//  * every 32-deep K stage of a 128 x 64 output tile is converted by loader
-//    warps: row r of A and column c of B get a power-of-two scale 2^E from the
+//  * every 32-deep K stage of an output tile of up to 128 x 64 is converted by
+//    loader warps: row r of A and column c of B get a power-of-two scale 2^E from the
 //    largest magnitude in their 32 elements, the element is rounded to a
 //    48-bit integer Q = round(|x| 2^(48-E)), and Q is cut into six 8-bit
 //    slices q_0..q_5 (q_0 <= 256) stored as bf16 (exact: at most 9 significant
 //    bits), so that x = sign * sum_i q_i 2^(E - 8(i+1)) up to 2^(E-49);
 //  * the slice products with i + j = g <= 5 are issued as tcgen05.mma
-//    (M = 128, N = 64, K = 16 per instruction) into one FP32 accumulator per
+//    (M = 128, K = 16 per instruction) into one FP32 accumulator per
 //    order g in tensor memory.  Every product is an integer below 2^16 and
 //    each order's sum over the 32-deep stage stays below 2^24 for g <= 5, so
 //    the accumulations are exact whatever the order of the additions;
@@ -25,15 +25,31 @@
 //    FP64 result.
 //
 // The work list is the FP64 engine's (Tile / Seg records over FP64 buffers of
-// a BufTable), lowered with 128 x 64 tiles and uploaded longest first.
-// Persistent CTAs, one per SM, walk (tile, vector) items with the vectors
-// innermost, so the CTAs that run at the same time share their operator tiles
-// in L2.  Slices are kept in 128B-swizzled rows 64 deep that hold two stages,
-// so stage q+1 is converted into the other half while the tensor cores consume
-// stage q.  Warps 0-7 epilogue (warp w: tile rows 32 (w % 4) .., columns
-// 32 (w / 4) ..), warps 8-11 loaders (A rows one per thread, B columns two
-// threads each), warp 12 lane 0 issues the MMAs.  Every wait is bounded; a
-// timeout sets the device error word.
+// a BufTable), lowered with 128 x 64 tiles (stacked products: Tile::sn) and
+// uploaded longest first.  Persistent CTAs, one per SM, walk (tile, vector)
+// items with the vectors innermost, so the CTAs that run at the same time share
+// their operator tiles in L2.  Slices are kept in 128B-swizzled rows 64 deep
+// that hold two stages, so stage q+1 is converted into the other half while the
+// tensor cores consume stage q.
+//
+// Bound: the instruction streams of the conversion and of the combination (and
+// FP64-pipe instructions: one takes a scheduler ~74 cycles), not the tensor
+// pipe.  Hence the split: two groups of three loader warps convert alternate
+// stages, each thread eight values of one row that it keeps in registers from
+// the scale to the slices (two to four lanes share a row, by the depth of the
+// stage); rows and columns outside the block are neither loaded nor converted;
+// the slices of B follow each other along N, so that one instruction multiplies
+// a slice of A with all the slices of B it meets (6 instructions per 16-deep
+// step instead of 21); a tile of up to 32 columns has two sets of accumulators,
+// and only its columns are combined, by two warps per 32 rows.  A warp reads
+// the tensor memory of its own scheduler's quarter only, so tiles of up to 32
+// rows keep one of the four schedulers busy: the loaders stay off the first
+// scheduler, and lists stack up to four such products in a tile.  (Four warps
+// that converted all 128 rows of every stage, one row per thread, and 42
+// instructions per stage took ~7 us per stage.)
+// Warps 0-7 epilogue (warp w: tile rows 32 (w % 4) .., half w / 4 of the
+// columns), warp 8 lane 0 issues the MMAs, warps 9-11 and 13-15 loaders.  Every
+// wait is bounded; a timeout sets the device error word.
 #include <cuda_bf16.h>
 
 #include <algorithm>
@@ -47,95 +63,78 @@ namespace {
 using namespace ptx;
 
 constexpr int OTM = 128, OTN = 64, OTK = 32;   // tile rows, columns, stage depth
-constexpr int ROWK = 64;                       // K of a swizzled slice row (two stages)
+constexpr int ROWB = 128;                      // bytes of a swizzled slice row (64 deep: two stages)
 constexpr int NSL = 6;                         // slices per operand
 constexpr int NORD = 6;                        // accumulated orders g = i + j = 0..5
-constexpr int A_SLICE = OTM * ROWK * 2;        // 16 KB
-constexpr int B_SLICE = OTN * ROWK * 2;        // 8 KB
-constexpr int SLICE_BYTES = NSL * (A_SLICE + B_SLICE);
-constexpr int EXP_SLOTS = 4;
-constexpr uint32_t TMEM_COLS = 512;            // 6 orders x 64 columns, rounded to a power of two
-// warps 0-7 epilogue (warp w: tile rows 32 (w % 4) .., columns 32 (w / 4) ..),
-// warps 8-11 loaders, warp 12 lane 0 MMA issuer; 13 warps keep 4 per SM
-// sub-partition, i.e. up to 128 registers per thread
-constexpr int NEPI = 8;
-constexpr int OZ_THREADS = (NEPI + 4 + 1) * 32;
-constexpr int NLOAD = 128;
+constexpr int A_SLICE = OTM * ROWB;            // 16 KB
+constexpr int SLICE_BYTES = NSL * (OTM + OTN) * ROWB;
+constexpr int NREC = 4;
+constexpr uint32_t TMEM_COLS = 512;            // 6 orders x 64 columns (or twice 6 x 32), rounded to a power of two
+constexpr int NEPI = 8;                        // epilogue warps
+constexpr int MMA_WARP = NEPI, IDLE_WARP = NEPI + 4;
+constexpr int NLDW = 3;                        // loader warps of a group
+constexpr int OZ_THREADS = (NEPI + 8) * 32;
 constexpr int EPI_COLS = OTN / 2;
 
-// per-stage record shared by loaders (write) and epilogue (read)
+// per-stage record shared by loaders (write), MMA issuer and epilogue (read)
 struct OzStage {
     int32_t ea[OTM];   // row scales of A (exponent E: |x| < 2^E), -1000 for a zero row
     int32_t eb[OTN];   // column scales of B
     float ah, al;      // alpha as a double-float pair
-    int32_t flags;     // 1 first stage of the tile, 2 last, 4 no MMA (tile without stages)
+    int32_t flags;     // 2 last stage of the tile, 4 no MMA (tile without products)
+    int32_t ksteps;    // 16-deep MMA steps
+    int32_t n16;       // MMA N / 16
     int32_t pad;
 };
 // the low parts of the epilogue's double-float accumulators live in shared
 // memory ([column][thread], conflict-free), the high parts in registers
 constexpr int ACL_BYTES = NEPI * 32 * EPI_COLS * 4;
-constexpr int OZ_SMEM = 1024 + SLICE_BYTES + EXP_SLOTS * (int)sizeof(OzStage) + ACL_BYTES;
+constexpr int OZ_SMEM = 1024 + SLICE_BYTES + NREC * (int)sizeof(OzStage) + ACL_BYTES;
 
-// biased exponent field of a double from its high 32-bit word (0 for zero and subnormals)
-__device__ __forceinline__ int exp_field_hi(int hi) { return (hi >> 20) & 0x7FF; }
+// biased exponent field of a double (0 for zero and subnormals)
+__device__ __forceinline__ int exp_field(double x) { return (__double2hiint(x) >> 20) & 0x7FF; }
 
 // 48-bit integer magnitude of |x| 2^(48-E) (rounded half up), with E = ebias - 1023
 __device__ __forceinline__ uint64_t q48(double x, int ebias) {
     const uint64_t bits = (uint64_t)__double_as_longlong(x);
     const int eb = (int)((bits >> 52) & 0x7FF);
-    if (eb == 0) return 0;  // zero / subnormal: below every scale used here
     const uint64_t m = (bits & 0x000FFFFFFFFFFFFFull) | 0x0010000000000000ull;
     const int sh = ebias + 4 - eb;  // right shift, >= 5
-    if (sh >= 54) return 0;
+    if (eb == 0 || sh >= 54) return 0;  // zero / subnormal: below every scale used here
     return (m + (1ull << (sh - 1))) >> sh;
 }
 
-// bf16 bit pattern of the integer q (0..256) with the given sign bit
-__device__ __forceinline__ uint32_t bf16_of_int(uint32_t q, uint32_t sign) {
-    const float f = __uint_as_float(0x4B000000u | q) - 8388608.0f;
-    return (__float_as_uint(f) >> 16) | (sign << 15);
-}
-
-// Convert N values (read by ld(kk), kk = 0..N-1) into the six slices at
-// dst + s * slice_bytes: row `row` of a 128B-swizzled K-major tile, 16-byte
-// chunks cbase .. cbase + N/8 - 1 of the row.
-template <int N, class Ld>
-__device__ __forceinline__ void store_slices(const Ld& ld, int ebias, uint32_t dst, int slice_bytes, int row,
-                                             int cbase) {
-    const uint32_t rowoff = (uint32_t)((row >> 3) * 1024 + (row & 7) * 128);
+// Slices of eight values at 16-byte column c of row `row` of the six slice tiles
+// at dst + i * slice (128B-swizzled, K-major)
+__device__ __forceinline__ void store_slices(const double (&x)[8], int ebias, uint32_t dst, uint32_t slice, int row,
+                                             int c) {
+    uint32_t w[NSL][4];
 #pragma unroll
-    for (int cl = 0; cl < N / 8; ++cl) {
-        uint32_t w[NSL][4];
+    for (int p = 0; p < 4; ++p) {
+        uint32_t f[2][NSL];
 #pragma unroll
-        for (int p = 0; p < 4; ++p) {
-            uint32_t b16[2][NSL];
+        for (int h = 0; h < 2; ++h) {
+            const uint64_t Q = q48(x[2 * p + h], ebias);
+            const uint32_t ql = (uint32_t)Q, qh = (uint32_t)(Q >> 32);
+            // 2^23 + slice as FP32 bits, minus 2^23: the slice (0..256), exact in bf16
+            const uint32_t t[NSL] = {0x4B000000u | (qh >> 8), __byte_perm(qh, 0x4B000000u, 0x7650),
+                                     __byte_perm(ql, 0x4B000000u, 0x7653), __byte_perm(ql, 0x4B000000u, 0x7652),
+                                     __byte_perm(ql, 0x4B000000u, 0x7651), __byte_perm(ql, 0x4B000000u, 0x7650)};
 #pragma unroll
-            for (int h = 0; h < 2; ++h) {
-                const double v = ld(cl * 8 + 2 * p + h);
-                const uint32_t sign = (uint32_t)(__double2hiint(v) >> 31) & 1u;
-                const uint64_t Q = q48(v, ebias);
-                const uint32_t ql = (uint32_t)Q, qh = (uint32_t)(Q >> 32);
-                b16[h][0] = bf16_of_int(qh >> 8, sign);
-                b16[h][1] = bf16_of_int(qh & 255u, sign);
-                b16[h][2] = bf16_of_int(ql >> 24, sign);
-                b16[h][3] = bf16_of_int((ql >> 16) & 255u, sign);
-                b16[h][4] = bf16_of_int((ql >> 8) & 255u, sign);
-                b16[h][5] = bf16_of_int(ql & 255u, sign);
-            }
-#pragma unroll
-            for (int s = 0; s < NSL; ++s) w[s][p] = b16[0][s] | (b16[1][s] << 16);
+            for (int i = 0; i < NSL; ++i) f[h][i] = __float_as_uint(__uint_as_float(t[i]) - 8388608.0f);
         }
-        const int c = cbase + cl;
-        const uint32_t off = rowoff + (uint32_t)(((c ^ (row & 7)) & 7) << 4);
+        const uint32_t sign = (((uint32_t)__double2hiint(x[2 * p]) >> 16) & 0x8000u) |
+                              ((uint32_t)__double2hiint(x[2 * p + 1]) & 0x80000000u);
 #pragma unroll
-        for (int s = 0; s < NSL; ++s)
-            asm volatile("st.shared.v4.u32 [%0], {%1, %2, %3, %4};\n" ::"r"(dst + s * slice_bytes + off), "r"(w[s][0]),
-                         "r"(w[s][1]), "r"(w[s][2]), "r"(w[s][3])
-                         : "memory");
+        for (int i = 0; i < NSL; ++i) w[i][p] = __byte_perm(f[0][i], f[1][i], 0x7632) | sign;
     }
+    const uint32_t off = dst + (uint32_t)((row >> 3) * 1024 + (row & 7) * ROWB + (((c ^ (row & 7)) & 7) << 4));
+#pragma unroll
+    for (int i = 0; i < NSL; ++i)
+        asm volatile("st.shared.v4.u32 [%0], {%1, %2, %3, %4};\n" ::"r"(off + i * slice), "r"(w[i][0]), "r"(w[i][1]),
+                     "r"(w[i][2]), "r"(w[i][3])
+                     : "memory");
 }
-
-__device__ __forceinline__ void loaders_sync() { asm volatile("bar.sync 1, 128;\n" ::: "memory"); }
 
 __device__ __forceinline__ void two_sum(float a, float b, float& s, float& e) {
     s = a + b;
@@ -150,10 +149,13 @@ __device__ __forceinline__ float pow2f(int k) {
     return __uint_as_float((uint32_t)(k + 127) << 23);
 }
 
-__device__ __forceinline__ int tile_nst(const Tile& T, const Seg* __restrict__ segs) {
-    int nst = 0;
-    for (int s = T.seg_beg; s < T.seg_end; ++s) nst += (segs[s].k + OTK - 1) / OTK;
-    return nst;
+// (double)f by its bits for zeros and normal numbers (the conversion is an
+// FP64-pipe instruction)
+__device__ __forceinline__ double widen(float f) {
+    const uint32_t u = __float_as_uint(f), e = (u >> 23) & 0xFFu;
+    if (e - 1u < 254u) return __hiloint2double((int)((u & 0x80000000u) | (((u & 0x7FFFFFFFu) >> 3) + 0x38000000u)), (int)(u << 29));
+    if ((u << 1) == 0u) return __hiloint2double((int)u, 0);
+    return (double)f;
 }
 
 __global__ void __launch_bounds__(OZ_THREADS, 1)
@@ -161,27 +163,24 @@ __global__ void __launch_bounds__(OZ_THREADS, 1)
                    int* err) {
     extern __shared__ uint8_t smem_raw[];
     // full[h]: loaders -> MMA (slices of K half h and the stage record written);
-    // stage: MMA -> epilogue (stage record visible; arrived after the previous
-    // accumulators were read); mma[h]: MMA completion -> loaders (half h free)
-    // and epilogue (orders ready); free: epilogue -> MMA (accumulators read)
-    __shared__ __align__(8) uint64_t full_bar[2], mma_bar[2], stage_bar, free_bar, drain_bar;
+    // rec[h]: MMA -> epilogue (record visible); done[h]: MMA completion -> loaders
+    // (half h free) and epilogue (orders ready); free[h]: epilogue -> MMA (orders read)
+    __shared__ __align__(8) uint64_t full_bar[2], rec_bar[2], done_bar[2], free_bar[2], drain_bar;
     __shared__ uint32_t tmem_base_s;
-    __shared__ int32_t ebp[2][OTN];  // per-part column exponent fields of B (loaders)
-    __shared__ int32_t load_ok;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const uint32_t sbase = (smem_u32(smem_raw) + 1023u) & ~1023u;
     const uint32_t sA = sbase, sB = sbase + NSL * A_SLICE;
-    OzStage* stages = reinterpret_cast<OzStage*>(smem_raw + (sbase - smem_u32(smem_raw)) + SLICE_BYTES);
-    float* acl_s = reinterpret_cast<float*>(stages + EXP_SLOTS);
+    OzStage* recs = reinterpret_cast<OzStage*>(smem_raw + (sbase - smem_u32(smem_raw)) + SLICE_BYTES);
+    float* acl_s = reinterpret_cast<float*>(recs + NREC);
 
     if (warp == 0) tmem_alloc(smem_u32(&tmem_base_s), TMEM_COLS);
     if (tid == 0) {
         for (int h = 0; h < 2; ++h) {
-            mbar_init(smem_u32(&full_bar[h]), NLOAD);
-            mbar_init(smem_u32(&mma_bar[h]), 1);
+            mbar_init(smem_u32(&full_bar[h]), NLDW);
+            mbar_init(smem_u32(&rec_bar[h]), 1);
+            mbar_init(smem_u32(&done_bar[h]), 1);
+            mbar_init(smem_u32(&free_bar[h]), NEPI);
         }
-        mbar_init(smem_u32(&stage_bar), 1);
-        mbar_init(smem_u32(&free_bar), NEPI);
         mbar_init(smem_u32(&drain_bar), 1);
         asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
     }
@@ -189,190 +188,247 @@ __global__ void __launch_bounds__(OZ_THREADS, 1)
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem = tmem_base_s;
-    const int total = ntiles * nvec;
+    const uint32_t total = (uint32_t)ntiles * (uint32_t)nvec, NV = (uint32_t)nvec;  // total < 2^31
     bool failed = false;
 
-    if (warp >= NEPI && warp < NEPI + 4) {
+    if (warp > MMA_WARP && warp != IDLE_WARP) {
         // ---------------- loaders / converters ----------------
-        const int t = tid - NEPI * 32;
-        uint32_t q = 0;
-        // K half (q & 1) of the slices is free once the MMAs of stage q - 2
-        // completed; one thread waits and the decision is shared, so the loaders
-        // stay uniform
-        auto begin = [&]() -> bool {
-            if (t == 0)
-                load_ok = (q < 2 || mbar_wait(smem_u32(&mma_bar[q & 1u]), ((q >> 1) - 1) & 1u)) ? 1 : 0;
-            loaders_sync();
-            const bool ok = load_ok != 0;
-            loaders_sync();
-            return ok;
+        const uint32_t grp = warp > IDLE_WARP ? 1u : 0u;
+        const int gw = warp - (grp ? IDLE_WARP : MMA_WARP) - 1;
+        uint32_t d = 0;  // stages so far (all tiles, both groups)
+        // the next tile and its first segment are in flight while a tile is converted
+        struct Place {
+            int m0, n0, m, n, seg_beg, seg_end, astride;
+            int sn, srows;  // stacked products and the rows between them (0: none)
         };
-        for (int it = blockIdx.x; it < total && !failed; it += gridDim.x) {
-            const Tile T = tiles[it / nvec];
-            const int v = it % nvec;
-            const int nst = tile_nst(T, segs);
-            int done = 0;
-            if (nst == 0) {
-                if (!begin()) { failed = true; break; }
-                OzStage& S = stages[q % EXP_SLOTS];
-                if (t == 0) {
-                    S.flags = 1 | 2 | 4;
-                    S.ah = S.al = 0.f;
+        auto place = [&](uint32_t i) {
+            Place p{};
+            if (i < total) {
+                const Tile& t = tiles[i / NV];
+                p = Place{t.m0, t.n0, t.m, t.n, t.seg_beg, t.seg_end, t.astride, t.sn, 16 * t.sb};
+            }
+            return p;
+        };
+        Seg S{};
+        const uint32_t G = gridDim.x;
+        Place T = place(blockIdx.x), nT = place(blockIdx.x + G);
+        if (T.seg_beg < T.seg_end) S = segs[T.seg_beg];
+        for (uint32_t it = blockIdx.x; it < total && !failed; it += G) {
+            const int v = (int)(it % NV);
+            const int mrem = min(OTM, T.m - T.m0), nrem = min(OTN, T.n - T.n0), n16 = (nrem + 15) / 16;
+            const uint32_t b_slice = (uint32_t)n16 * 16u * ROWB;  // the slices of B follow each other along N
+            Seg nS{};
+            if (nT.seg_beg < nT.seg_end) nS = segs[nT.seg_beg];
+            const Place nnT = place(it + 2 * G);
+            int s = T.seg_beg;
+            while (s < T.seg_end && S.k <= 0)
+                if (++s < T.seg_end) S = segs[s];
+            int k0 = 0;
+            bool more = true;
+            while (more) {
+                // the stage: k0 .. k0 + kn of segment s (kn = 0: a tile without products)
+                const int kn = s < T.seg_end ? min(OTK, S.k - k0) : 0;
+                const Seg Sc = S;
+                const int kb = k0;
+                k0 += kn;
+                while (s < T.seg_end && k0 >= S.k) {  // the next segment with products
+                    k0 = 0;
+                    if (++s < T.seg_end) S = segs[s];
+                }
+                more = s < T.seg_end;
+                const uint32_t slot = d & 1u, use = d >> 1;
+                OzStage& R = recs[d % NREC];
+                ++d;
+                if (slot != grp) continue;
+                const int steps = (kn + 15) / 16;
+                // a task: rt rows of one product's A or columns of B, 32 / rt K groups of eight
+                const int lg = kn > 16 ? 3 : 4, rt = 1 << lg;
+                const int lr = lane & (rt - 1), cg = lane >> lg;
+                const int nap = (mrem + rt - 1) >> lg;  // tasks of a product
+                const int na = kn > 0 ? nap * max(T.sn, 1) : 0, nb = kn > 0 ? (nrem + rt - 1) >> lg : 0;
+                const int64_t ak = Sc.a_tr ? Sc.lda : 1, ar = Sc.a_tr ? 1 : Sc.lda;
+                const int64_t bk = Sc.b_tr ? 1 : Sc.ldb, br = Sc.b_tr ? Sc.ldb : 1;
+                const double* A = bt.p[Sc.a_buf] + Sc.a_off + (int64_t)v * bt.vstride[Sc.a_buf] + T.m0 * ar + (kb + 8 * cg) * ak;
+                const double* B = bt.p[Sc.b_buf] + Sc.b_off + (int64_t)v * bt.vstride[Sc.b_buf] + T.n0 * br + (kb + 8 * cg) * bk;
+                const int kv = kn - 8 * cg;  // K values of this lane's group that exist
+                int ok = 1;
+                bool waited = false;
+                for (int t0 = gw; t0 < na + nb || !waited; t0 += 2 * NLDW) {
+                    double x[2][8];  // two tasks' loads in flight together
+                    int rows[2];
+#pragma unroll
+                    for (int h = 0; h < 2; ++h) {
+                        const int t = t0 + h * NLDW;
+                        const bool isb = t >= na;
+                        const int pi = isb || T.sn == 0 ? 0 : t / nap;  // stacked product
+                        const int row = ((isb ? t - na : t - pi * nap) << lg) + lr;
+                        const double* q = isb ? B + row * br : A + (int64_t)pi * T.astride + row * ar;
+                        const int64_t st = isb ? bk : ak;
+                        const int n = t < na + nb && row < (isb ? nrem : mrem) ? kv : 0;
+                        rows[h] = row + pi * T.srows;
+#pragma unroll
+                        for (int j = 0; j < 8; ++j) x[h][j] = j < n ? q[j * st] : 0.0;
+                    }
+                    if (!waited) {  // half free: the MMAs of stage d - 2 completed
+                        waited = true;
+                        if (lane == 0 && use > 0) ok = mbar_wait(smem_u32(&done_bar[slot]), (use - 1) & 1u) ? 1 : 0;
+                        ok = __shfl_sync(0xffffffffu, ok, 0);
+                        if (!ok) break;
+                    }
+#pragma unroll
+                    for (int h = 0; h < 2; ++h) {
+                        const int t = t0 + h * NLDW;
+                        if (t >= na + nb) break;
+                        const bool isb = t >= na;
+                        const int row = rows[h];
+                        int emax = 0;
+#pragma unroll
+                        for (int j = 0; j < 8; ++j) emax = max(emax, exp_field(x[h][j]));
+                        for (int o = rt; o < 32; o *= 2) emax = max(emax, __shfl_xor_sync(0xffffffffu, emax, o));
+                        const bool in = row < (isb ? 16 * n16 : OTM);  // (a task's last rows may lie beyond the buffers)
+                        if (cg == 0 && in) (isb ? R.eb : R.ea)[row] = emax ? emax + 1 - 1023 : -1000;
+                        if (cg < 2 * steps && in)
+                            store_slices(x[h], emax + 1, isb ? sB : sA, isb ? b_slice : (uint32_t)A_SLICE, row,
+                                         (int)slot * (OTK / 8) + cg);
+                    }
+                }
+                if (!ok) {
+                    failed = true;
+                    break;
+                }
+                if (gw == 0 && lane == 0) {
+                    R.ah = (float)Sc.alpha;
+                    R.al = (float)(Sc.alpha - (double)R.ah);
+                    R.flags = (more ? 0 : 2) | (kn == 0 ? 4 : 0);
+                    R.ksteps = steps;
+                    R.n16 = n16;
                 }
                 fence_proxy_async();
-                mbar_arrive(smem_u32(&full_bar[q & 1u]));
-                ++q;
-                continue;
+                __syncwarp();
+                if (lane == 0) mbar_arrive(smem_u32(&full_bar[slot]));
             }
-            for (int s = T.seg_beg; s < T.seg_end && !failed; ++s) {
-                const Seg Sg = segs[s];
-                const double* A = bt.p[Sg.a_buf] + Sg.a_off + (int64_t)v * bt.vstride[Sg.a_buf];
-                const double* B = bt.p[Sg.b_buf] + Sg.b_off + (int64_t)v * bt.vstride[Sg.b_buf];
-                for (int k0 = 0; k0 < Sg.k; k0 += OTK) {
-                    if (!begin()) { failed = true; break; }
-                    OzStage& S = stages[q % EXP_SLOTS];
-                    const int cbase = (int)(q & 1u) * (OTK / 8);
-                    // A: thread t converts row m0 + t over k0 .. k0+31: the row's scale
-                    // from the high words (32 loads in flight), then the values
-                    {
-                        const int gi = T.m0 + t;
-                        const bool rv = gi < T.m;
-                        const int kn = rv ? min(OTK, Sg.k - k0) : 0;
-                        auto idx = [&](int kk) -> int64_t {
-                            const int k = k0 + kk;
-                            return Sg.a_tr ? (int64_t)k * Sg.lda + gi : (int64_t)gi * Sg.lda + k;
-                        };
-                        int emax = 0;
-#pragma unroll
-                        for (int kk = 0; kk < OTK; ++kk)
-                            if (kk < kn) emax = max(emax, exp_field_hi(reinterpret_cast<const int*>(A + idx(kk))[1]));
-                        const int ebias = emax + 1;  // |x| < 2^(ebias - 1023)
-                        S.ea[t] = emax ? ebias - 1023 : -1000;
-                        auto lda = [&](int kk) -> double { return kk < kn ? A[idx(kk)] : 0.0; };
-                        store_slices<OTK>(lda, ebias, sA, A_SLICE, t, cbase);
-                    }
-                    // B: threads t and t + 64 convert column (t & 63), K parts of 16
-                    {
-                        const int c = t & 63, part = t >> 6;
-                        const int gj = T.n0 + c;
-                        const int kb = k0 + 16 * part;
-                        const int kn = gj < T.n ? max(0, min(16, Sg.k - kb)) : 0;
-                        auto idx = [&](int kk) -> int64_t {
-                            const int k = kb + kk;
-                            return Sg.b_tr ? (int64_t)gj * Sg.ldb + k : (int64_t)k * Sg.ldb + gj;
-                        };
-                        int emax = 0;
-#pragma unroll
-                        for (int kk = 0; kk < 16; ++kk)
-                            if (kk < kn) emax = max(emax, exp_field_hi(reinterpret_cast<const int*>(B + idx(kk))[1]));
-                        ebp[part][c] = emax;
-                        loaders_sync();
-                        emax = max(ebp[0][c], ebp[1][c]);
-                        const int ebias = emax + 1;
-                        if (part == 0) S.eb[c] = emax ? ebias - 1023 : -1000;
-                        auto ldb = [&](int kk) -> double { return kk < kn ? B[idx(kk)] : 0.0; };
-                        store_slices<16>(ldb, ebias, sB, B_SLICE, c, cbase + 2 * part);
-                    }
-                    if (t == 0) {
-                        const float ah = (float)Sg.alpha;
-                        S.ah = ah;
-                        S.al = (float)(Sg.alpha - (double)ah);
-                        S.flags = (done == 0 ? 1 : 0) | (done == nst - 1 ? 2 : 0);
-                    }
-                    fence_proxy_async();
-                    mbar_arrive(smem_u32(&full_bar[q & 1u]));
-                    ++q;
-                    ++done;
-                }
-            }
+            T = nT;
+            S = nS;
+            nT = nnT;
         }
-    } else if (warp == NEPI + 4) {
+    } else if (warp == MMA_WARP) {
         // ---------------- MMA issuer ----------------
         if (lane == 0) {
-            uint32_t q = 0;
-            const uint32_t id = idesc_mn(0, 0, 0, OTN, OTM);
-            for (int it = blockIdx.x; it < total && !failed; it += gridDim.x) {
-                const Tile T = tiles[it / nvec];
-                int nst = tile_nst(T, segs);
-                if (nst == 0) nst = 1;
-                for (int st = 0; st < nst; ++st, ++q) {
-                    const uint32_t h = q & 1u;
-                    if (!mbar_wait(smem_u32(&full_bar[h]), (q >> 1) & 1u)) { failed = true; break; }
-                    if (q >= 1 && !mbar_wait(smem_u32(&free_bar), (q - 1) & 1u)) { failed = true; break; }
-                    mbar_arrive(smem_u32(&stage_bar));
+            uint32_t d = 0;
+            bool wide = false;  // the previous stage used all the accumulators
+            for (uint32_t it = blockIdx.x; it < total && !failed; it += gridDim.x) {
+                for (;;) {
+                    const uint32_t slot = d & 1u, use = d >> 1;
+                    if (!mbar_wait(smem_u32(&full_bar[slot]), use & 1u)) { failed = true; break; }
+                    const OzStage& R = recs[d % NREC];
+                    const int flags = R.flags, steps = R.ksteps, n16 = R.n16;
+                    // accumulators: the set of the stage's parity (up to 32 columns), or all
+                    const bool w = n16 > 2;
+                    if (use > 0 && !mbar_wait(smem_u32(&free_bar[slot]), (use - 1) & 1u)) { failed = true; break; }
+                    if ((w || wide) && d >= 1 && !mbar_wait(smem_u32(&free_bar[slot ^ 1u]), ((d - 1) >> 1) & 1u)) {
+                        failed = true;
+                        break;
+                    }
+                    wide = w;
+                    mbar_arrive(smem_u32(&rec_bar[slot]));
                     tc_fence_after();
-                    const OzStage& S = stages[q % EXP_SLOTS];
-                    if (!(S.flags & 4)) {
+                    if (!(flags & 4)) {
+                        // slice i of A times the slices 0 .. 5 - i of B adds to the orders
+                        // i .. 5: one instruction of N = (6 - i) cs (two above 256)
+                        const uint32_t cs = 16u * (uint32_t)n16, dt0 = tmem + (w ? 0u : slot * 256u);
+                        const uint32_t most = 256u / cs;  // slices of B per instruction
+                        const uint32_t khalf = slot * (OTK * 2);
+                        const uint64_t ad0 = sdesc(sA + khalf, 16, 1024), bd0 = sdesc(sB + khalf, 16, 1024);
+                        for (int kk = 0; kk < steps; ++kk) {
 #pragma unroll
-                        for (int g = 0; g < NORD; ++g) {
-                            const uint32_t dt = tmem + (uint32_t)(g * OTN);
-#pragma unroll
-                            for (int i = 0; i <= g; ++i) {
-                                const int j = g - i;
-#pragma unroll
-                                for (int kk = 0; kk < OTK / 16; ++kk) {
-                                    const uint32_t koff = (h * (OTK / 16) + kk) * 32;
-                                    const uint64_t ad = sdesc(sA + i * A_SLICE + koff, 16, 1024);
-                                    const uint64_t bd = sdesc(sB + j * B_SLICE + koff, 16, 1024);
-                                    mma_bf16(dt, ad, bd, id, (i == 0 && kk == 0) ? 0u : 1u);
-                                }
+                            for (uint32_t i = 0; i < NSL; ++i) {
+                                const uint64_t ad = ad0 + (uint64_t)((i * A_SLICE) >> 4) + 2u * kk;
+                                const uint32_t n0 = min((uint32_t)NSL - i, most), n1 = NSL - i - n0;
+                                const uint32_t acc = (i == 0 && kk == 0) ? 0u : 1u;
+                                mma_bf16(dt0 + i * cs, ad, bd0 + 2u * kk, idesc_mn(0, 0, 0, (int)(n0 * cs), OTM), acc);
+                                if (n1 > 0)
+                                    mma_bf16(dt0 + (i + n0) * cs, ad, bd0 + 2u * kk + (uint64_t)((n0 * cs * ROWB) >> 4),
+                                             idesc_mn(0, 0, 0, (int)(n1 * cs), OTM), acc);
                             }
                         }
                     }
-                    mma_commit(smem_u32(&mma_bar[h]));
+                    mma_commit(smem_u32(&done_bar[slot]));
+                    ++d;
+                    if (flags & 2) break;
                 }
             }
             mma_commit(smem_u32(&drain_bar));
             if (!mbar_wait(smem_u32(&drain_bar), 0)) failed = true;
         }
-    } else {
+    } else if (warp < NEPI) {
         // ---------------- epilogue ----------------
         const int quarter = warp & 3, chalf = warp >> 2;
         const int row = quarter * 32 + lane;
-        uint32_t q = 0;
-        for (int it = blockIdx.x; it < total && !failed; it += gridDim.x) {
-            const Tile T = tiles[it / nvec];
-            const int v = it % nvec;
-            int nst = tile_nst(T, segs);
-            if (nst == 0) nst = 1;
-            float ach[EPI_COLS];
-            float* acl = acl_s + tid;  // acl[c * NEPI * 32]
-#pragma unroll
-            for (int c = 0; c < EPI_COLS; ++c) {
-                ach[c] = 0.f;
-                acl[c * NEPI * 32] = 0.f;
+        float* acl = acl_s + tid;  // acl[c * NEPI * 32]
+        uint32_t d = 0;
+        Tile nT{};
+        if (blockIdx.x < total) nT = tiles[blockIdx.x / NV];
+        for (uint32_t it = blockIdx.x; it < total && !failed; it += gridDim.x) {
+            const Tile T = nT;
+            if (it + gridDim.x < total) nT = tiles[(it + gridDim.x) / NV];
+            const int v = (int)(it % NV);
+            const int nrem = min(OTN, T.n - T.n0);
+            // this thread's output row (stacked products: m * ldc apart, their rows run on)
+            int64_t orow = T.m0 + row;
+            bool rok = orow < T.m, any = T.m0 + quarter * 32 < T.m;
+            if (T.sn) {
+                const int sr = 16 * T.sb, i = row / sr;
+                rok = i < T.sn && row - i * sr < T.m;
+                any = quarter * 32 < T.sn * sr;
+                orow = (int64_t)i * T.m + row - i * sr;
             }
-            for (int st = 0; st < nst; ++st, ++q) {
+            // columns of this half (a multiple of four apart), none for rows outside
+            const int hc = ((nrem + 1) / 2 + 3) & ~3, c0 = chalf * hc;
+            const int ncol = any ? min(hc, nrem - c0) : 0;
+            const uint32_t cs = (uint32_t)((nrem + 15) / 16) * 16u;  // columns of an order
+            float ach[EPI_COLS];
+#pragma unroll
+            for (int c = 0; c < EPI_COLS; ++c) ach[c] = 0.f;
+            for (int c = 0; c < ncol; ++c) acl[c * NEPI * 32] = 0.f;
+            for (;;) {
+                const uint32_t slot = d & 1u, use = d >> 1;
                 int ok = 1;
                 if (lane == 0)
-                    ok = (mbar_wait(smem_u32(&stage_bar), q & 1u) &&
-                          mbar_wait(smem_u32(&mma_bar[q & 1u]), (q >> 1) & 1u))
+                    ok = (mbar_wait(smem_u32(&rec_bar[slot]), use & 1u) && mbar_wait(smem_u32(&done_bar[slot]), use & 1u))
                              ? 1
                              : 0;
                 ok = __shfl_sync(0xffffffffu, ok, 0);
                 if (!ok) { failed = true; break; }
                 __syncwarp();
                 tc_fence_after();
-                const OzStage& S = stages[q % EXP_SLOTS];
-                if (S.flags & 4) {
+                const OzStage& R = recs[d % NREC];
+                const int flags = R.flags;
+                ++d;
+                if ((flags & 4) || ncol <= 0) {
+                    tc_fence_before();
                     __syncwarp();
-                    if (lane == 0) mbar_arrive(smem_u32(&free_bar));
+                    if (lane == 0) mbar_arrive(smem_u32(&free_bar[slot]));
+                    if (flags & 2) break;
                     continue;
                 }
-                const int er = S.ea[row];
-                const float ah = S.ah, al = S.al;
+                const int er = R.ea[row];
+                const float ah = R.ah, al = R.al;
                 const bool unit = (ah == 1.f || ah == -1.f) && al == 0.f;  // alpha = +-1: a sign only
-                const uint32_t tbase = tmem + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(chalf * EPI_COLS);
+                const uint32_t tb = tmem + ((uint32_t)(quarter * 32) << 16) + (cs > 32u ? 0u : slot * 256u) + (uint32_t)c0;
 #pragma unroll
                 for (int cc = 0; cc < EPI_COLS / 4; ++cc) {
+                    if (cc * 4 >= ncol) break;
                     uint32_t a[NORD][4];
 #pragma unroll
-                    for (int g = 0; g < NORD; ++g) tmem_ld4(tbase + (uint32_t)(g * OTN + cc * 4), a[g]);
+                    for (int g = 0; g < NORD; ++g) tmem_ld4(tb + (uint32_t)g * cs + (uint32_t)(cc * 4), a[g]);
+                    int ec[4];
+#pragma unroll
+                    for (int j = 0; j < 4; ++j) ec[j] = R.eb[min(c0 + cc * 4 + j, OTN - 1)];
                     tmem_wait_ld();
-                    if (cc == EPI_COLS / 4 - 1) {  // every order of this stage is in registers: release the accumulators
+                    if (cc * 4 + 4 >= ncol) {  // every order and scale of this stage is in registers: release them
                         tc_fence_before();
                         __syncwarp();
-                        if (lane == 0) mbar_arrive(smem_u32(&free_bar));
+                        if (lane == 0) mbar_arrive(smem_u32(&free_bar[slot]));
                     }
 #pragma unroll
                     for (int j = 0; j < 4; ++j) {
@@ -385,7 +441,7 @@ __global__ void __launch_bounds__(OZ_THREADS, 1)
                             sl += e;
                         }
                         // unit of order 0: 2^(E_r - 8) 2^(E_c - 8)
-                        const float sc = pow2f(er + S.eb[chalf * EPI_COLS + c] - 16);
+                        const float sc = pow2f(er + ec[j] - 16);
                         sh *= sc;
                         sl *= sc;
                         float p, pe;
@@ -404,23 +460,19 @@ __global__ void __launch_bounds__(OZ_THREADS, 1)
                         acl[c * NEPI * 32] += e + pe;
                     }
                 }
+                if (flags & 2) break;
             }
             if (failed) break;
             // the tile's FP64 result
-            const int r = T.m0 + row;
-            const int c0 = T.n0 + chalf * EPI_COLS;
-            if (r < T.m && c0 < T.n) {
-                const int ncol = min(EPI_COLS, T.n - c0);
-                double* C = bt.p[T.c_buf] + T.c_off + (int64_t)v * bt.vstride[T.c_buf] + (int64_t)r * T.ldc + c0;
-                if (T.mode == TILE_ATOMIC) {
+            if (rok && ncol > 0) {
+                double* C = bt.p[T.c_buf] + T.c_off + (int64_t)v * bt.vstride[T.c_buf] + orow * T.ldc + T.n0 + c0;
 #pragma unroll
-                    for (int c = 0; c < EPI_COLS; ++c)
-                        if (c < ncol) atomicAdd(C + c, (double)ach[c] + (double)acl[c * NEPI * 32]);
-                } else {
-#pragma unroll
-                    for (int c = 0; c < EPI_COLS; ++c)
-                        if (c < ncol) C[c] = (double)ach[c] + (double)acl[c * NEPI * 32];
-                }
+                for (int c = 0; c < EPI_COLS; ++c)
+                    if (c < ncol) {
+                        const double r = widen(ach[c]) + widen(acl[c * NEPI * 32]);
+                        if (T.mode == TILE_ATOMIC) atomicAdd(C + c, r);
+                        else C[c] = r;
+                    }
             }
         }
     }

@@ -368,6 +368,138 @@ static Seg make_seg(const View& A, const View& B, int k, double alpha) {
     return s;
 }
 
+namespace {
+
+// First products of a chunk of three-factor items: items with the same factors
+// share one product, and the products of consecutive operators of a family with
+// one other factor form stacks (runs of at most `most`), which the tensor-core
+// engines compute as one tile.
+struct ProdKey {
+    int64_t a_off, b_off;  // operator family block (without the operator's number), other factor
+    int64_t alpha;         // bits of |alpha| where it is part of the product, else 0
+    int32_t form;          // buffers, orders, which factors
+    bool operator==(const ProdKey& o) const {
+        return a_off == o.a_off && b_off == o.b_off && alpha == o.alpha && form == o.form;
+    }
+    uint64_t hash() const {
+        uint64_t h = 0x9e3779b97f4a7c15ull;
+        for (uint64_t x : {(uint64_t)a_off, (uint64_t)b_off, (uint64_t)alpha, (uint64_t)form}) {
+            h ^= x + 0x9e3779b97f4a7c15ull + (h << 6) + (h >> 2);
+            h *= 0xff51afd7ed558ccdull;
+        }
+        return h ^ (h >> 33);
+    }
+};
+struct ProdStack {
+    uint32_t item;  // the item of its first product
+    int n;          // products
+};
+struct Products {
+    std::vector<ProdStack> stacks;
+    std::vector<int32_t> stack;  // per item: its stack (-1: not a three-factor item) ...
+    std::vector<uint8_t> pos;    // ... and its product's place there
+};
+// get(item, key, z, most): false for items that are not three-factor products;
+// z the operator's number in its family.  Runs on host threads; the result does
+// not depend on their number.
+template <typename Get>
+Products share_products(size_t ni, const Get& get) {
+    Products pr;
+    pr.stack.assign(ni, -1);
+    pr.pos.assign(ni, 0);
+    const size_t np = ni < 4096 ? 1 : 16;  // partitions of the keys
+    std::vector<uint64_t> hash(ni, 0);     // 0: no product
+    parallel_for((ni + 4095) / 4096, [&](size_t b) {
+        for (size_t q = b * 4096; q < std::min(ni, (b + 1) * 4096); ++q) {
+            ProdKey k{};
+            int z, most;
+            if (get(q, k, z, most)) hash[q] = k.hash() | 1;
+        }
+    });
+    std::vector<std::vector<ProdStack>> st(np);
+    parallel_for(np, [&](size_t pt) {
+        struct KeyHash {
+            size_t operator()(const ProdKey& k) const { return (size_t)k.hash(); }
+        };
+        std::unordered_map<ProdKey, int, KeyHash> idx;
+        std::vector<std::vector<std::pair<int32_t, uint32_t>>> lists;  // per key: (z, item)
+        std::vector<int> mosts;
+        for (size_t q = 0; q < ni; ++q) {
+            if (!hash[q] || (hash[q] >> 40) % np != pt) continue;
+            ProdKey k{};
+            int z = 0, most = 1;
+            get(q, k, z, most);
+            auto f = idx.emplace(k, (int)lists.size());
+            if (f.second) {
+                lists.emplace_back();
+                mosts.push_back(most);
+            }
+            lists[f.first->second].push_back({z, (uint32_t)q});
+        }
+        for (size_t x = 0; x < lists.size(); ++x) {
+            auto& l = lists[x];
+            std::stable_sort(l.begin(), l.end(), [](const auto& a, const auto& b) { return a.first < b.first; });
+            for (size_t y = 0; y < l.size(); ++y) {
+                const bool same = y > 0 && l[y].first == l[y - 1].first;
+                if (!same) {
+                    if (y > 0 && l[y].first == l[y - 1].first + 1 && st[pt].back().n < mosts[x]) ++st[pt].back().n;
+                    else st[pt].push_back({l[y].second, 1});
+                }
+                pr.stack[l[y].second] = (int32_t)st[pt].size() - 1;  // within the partition for now
+                pr.pos[l[y].second] = (uint8_t)(st[pt].back().n - 1);
+            }
+        }
+    });
+    std::vector<int32_t> first(np, 0);
+    for (size_t pt = 0; pt < np; ++pt) {
+        first[pt] = (int32_t)pr.stacks.size();
+        pr.stacks.insert(pr.stacks.end(), st[pt].begin(), st[pt].end());
+    }
+    for (size_t q = 0; q < ni; ++q)
+        if (pr.stack[q] >= 0) pr.stack[q] += first[(hash[q] >> 40) % np];
+    return pr;
+}
+
+int64_t bits_of(double x) {
+    int64_t r;
+    std::memcpy(&r, &x, 8);
+    return r;
+}
+
+// The first product of a three-factor item as op(A) (rows x k) op(B) (k x cols).
+// A is the factor that is one of a family, where one is, so that products can be
+// stacked along its rows; `tr`: that makes it the transpose of the item's product.
+struct FirstProduct {
+    View A, B;
+    int rows, cols, k;
+    bool tr;
+};
+FirstProduct first_product(const Contrib& c, bool pq, bool family_left) {
+    if (pq) {
+        if (family_left && c.P.nz <= 1 && c.Q.nz > 1) return {c.Q.T(), c.P.T(), c.k2, c.m, c.k1, true};
+        return {c.P, c.Q, c.m, c.k2, c.k1, false};
+    }
+    if (family_left && c.R.nz > 1) return {c.R.T(), c.Q.T(), c.n, c.k1, c.k2, true};
+    return {c.Q, c.R, c.k1, c.n, c.k2, false};
+}
+ProdKey product_key(const FirstProduct& f, bool pq, int64_t alpha) {
+    ProdKey k{};
+    k.a_off = f.A.off - (int64_t)f.A.z * f.A.zstride;
+    k.b_off = f.B.off;
+    k.alpha = alpha;
+    k.form = f.A.buf | (f.B.buf << 4) | (f.A.tr << 8) | (f.B.tr << 9) | ((int)pq << 10) | (f.tr << 11);
+    return k;
+}
+bool pq_is_first(const Contrib& c, double* cost) {
+    const double cost_pq = 2.0 * c.m * c.k1 * c.k2 + 2.0 * c.m * c.k2 * c.n;
+    const double cost_qr = 2.0 * c.k1 * c.k2 * c.n + 2.0 * c.m * c.k1 * c.n;
+    if (cost) *cost = std::min(cost_pq, cost_qr);
+    return cost_pq <= cost_qr;
+}
+int real_factors(const Contrib& c) { return (!c.P.ident) + (!c.Q.ident) + (!c.R.ident); }
+
+}  // namespace
+
 void ProductList::lower(int8_t sbuf_, int8_t ibuf, int ild, int64_t cap, int64_t kchunk) {
     const int8_t sbuf = sbuf_;
     this->sbuf = sbuf_;
@@ -375,57 +507,75 @@ void ProductList::lower(int8_t sbuf_, int8_t ibuf, int ild, int64_t cap, int64_t
     chunks.clear();
     flops = 0.0;
     scratch_elems = 0;
+    const bool oz = tile_m > 0;  // the FP64-accurate tensor-core engine: products stacked along a tile's rows
+    View I;
+    I.buf = ibuf;
+    I.off = 0;
+    I.ld = ild;
     size_t i = 0;
-    auto ident_view = [&](void) {
-        View v;
-        v.buf = ibuf;
-        v.off = 0;
-        v.ld = ild;
-        return v;
-    };
     while (i < cs.size()) {
+        // the chunk's items: their first products fit the scratch one by one
+        size_t j = i;
+        int64_t room = 0;
+        for (; j < cs.size(); ++j) {
+            const Contrib& c = cs[j];
+            int64_t need = 0;
+            if (real_factors(c) == 3)
+                need = round_up(pq_is_first(c, nullptr) ? (int64_t)c.m * c.k2 : (int64_t)c.k1 * c.n, 4);
+            if (room + need > cap && room > 0) break;
+            room += need;
+        }
         WorkList p1, p2;
         p1.tile_m = p2.tile_m = tile_m;
         p1.tile_n = p2.tile_n = tile_n;
+        const Products pr = share_products(j - i, [&](size_t q, ProdKey& k, int& z, int& most) {
+            const Contrib& c = cs[i + q];
+            if (real_factors(c) != 3) return false;
+            const bool pq = pq_is_first(c, nullptr);
+            const FirstProduct f = first_product(c, pq, oz);
+            k = product_key(f, pq, 0);
+            z = f.A.z;
+            most = !oz || f.rows > 64 || f.A.zstride >= (1LL << 31) ? 1 : (f.rows > 32 ? 2 : 4);
+            return true;
+        });
+        // phase 1: the stacks in the order of their first items, their products one behind another
+        std::vector<int64_t> base(pr.stacks.size(), -1);
+        int64_t used = 0;
+        for (size_t q = 0; q < j - i; ++q) {
+            const int x = pr.stack[q];
+            if (x < 0 || base[x] >= 0) continue;
+            const ProdStack& ps = pr.stacks[x];
+            const Contrib& c = cs[i + ps.item];
+            const FirstProduct f = first_product(c, pq_is_first(c, nullptr), oz);
+            base[x] = used;
+            const Seg sg = make_seg(f.A, f.B, f.k, 1.0);
+            if (ps.n > 1) p1.add_stack(used, sbuf, f.rows, f.cols, f.cols, sg, f.A.zstride, ps.n, f.rows > 32 ? 4 : 2);
+            else p1.add_block(used, sbuf, f.rows, f.cols, f.cols, {sg}, TILE_STORE);
+            used = round_up(used + (int64_t)ps.n * f.rows * f.cols, 4);
+        }
+        // phase 2: every output's segments in item order
         std::vector<std::vector<Seg>> segs(outs.size());
         std::vector<char> seen(outs.size(), 0);
         std::vector<int> order;
-        int64_t used = 0;
-        for (; i < cs.size(); ++i) {
-            const Contrib& c = cs[i];
-            int nreal = (!c.P.ident) + (!c.Q.ident) + (!c.R.ident);
-            int64_t need = 0;
-            bool pq_first = true;
-            if (nreal == 3) {
-                double cost_pq = 2.0 * c.m * c.k1 * c.k2 + 2.0 * c.m * c.k2 * c.n;
-                double cost_qr = 2.0 * c.k1 * c.k2 * c.n + 2.0 * c.m * c.k1 * c.n;
-                pq_first = cost_pq <= cost_qr;
-                need = pq_first ? (int64_t)c.m * c.k2 : (int64_t)c.k1 * c.n;
-                need = round_up(need, 4);
-                if (used + need > cap && used > 0) break;
-                flops += std::min(cost_pq, cost_qr);
-            }
+        for (size_t q = 0; q < j - i; ++q) {
+            const Contrib& c = cs[i + q];
+            const int nreal = real_factors(c);
             if (!seen[c.out]) {
                 seen[c.out] = 1;
                 order.push_back(c.out);
             }
             std::vector<Seg>& sv = segs[c.out];
             if (nreal == 3) {
+                double cost = 0.0;
+                const bool pq = pq_is_first(c, &cost);
+                const FirstProduct f = first_product(c, pq, oz);
+                flops += cost;
                 View T;
                 T.buf = sbuf;
-                T.off = used;
-                if (pq_first) {
-                    T.ld = c.k2;
-                    std::vector<Seg> one{make_seg(c.P, c.Q, c.k1, 1.0)};
-                    p1.add_block(used, sbuf, c.m, c.k2, c.k2, one, TILE_STORE);
-                    sv.push_back(make_seg(T, c.R, c.k2, c.alpha));
-                } else {
-                    T.ld = c.n;
-                    std::vector<Seg> one{make_seg(c.Q, c.R, c.k2, 1.0)};
-                    p1.add_block(used, sbuf, c.k1, c.n, c.n, one, TILE_STORE);
-                    sv.push_back(make_seg(c.P, T, c.k1, c.alpha));
-                }
-                used += need;
+                T.off = base[pr.stack[q]] + (int64_t)pr.pos[q] * f.rows * f.cols;
+                T.ld = f.cols;
+                T.tr = f.tr;
+                sv.push_back(pq ? make_seg(T, c.R, c.k2, c.alpha) : make_seg(c.P, T, c.k1, c.alpha));
             } else if (nreal == 2) {
                 if (c.P.ident) sv.push_back(make_seg(c.Q, c.R, c.k2, c.alpha));
                 else if (c.R.ident) sv.push_back(make_seg(c.P, c.Q, c.k1, c.alpha));
@@ -433,8 +583,8 @@ void ProductList::lower(int8_t sbuf_, int8_t ibuf, int ild, int64_t cap, int64_t
                 flops += 2.0 * c.m * c.n * (c.P.ident ? c.k2 : c.k1);
             } else {
                 const View& F = !c.P.ident ? c.P : (!c.Q.ident ? c.Q : c.R);
-                if (nreal == 1) sv.push_back(make_seg(F, ident_view(), c.n, c.alpha));
-                else sv.push_back(make_seg(ident_view(), ident_view(), c.n, c.alpha));
+                if (nreal == 1) sv.push_back(make_seg(F, I, c.n, c.alpha));
+                else sv.push_back(make_seg(I, I, c.n, c.alpha));
                 flops += 2.0 * c.m * c.n;
             }
         }
@@ -442,10 +592,11 @@ void ProductList::lower(int8_t sbuf_, int8_t ibuf, int ild, int64_t cap, int64_t
             const OutBlock& ob = outs[o];
             // the FP64 units' kernels share a long term sum among the CTAs of a cluster
             // and add without atomics: one tile per output region, no K-chunks
-            p2.add_block(ob.off, ob.buf, ob.m, ob.n, ob.ldc, segs[o], TILE_ATOMIC, tile_m > 0 ? kchunk : 0);
+            p2.add_block(ob.off, ob.buf, ob.m, ob.n, ob.ldc, segs[o], TILE_ATOMIC, oz ? kchunk : 0);
         }
         scratch_elems = std::max(scratch_elems, used);
         chunks.emplace_back(std::move(p1), std::move(p2));
+        i = j;
     }
 }
 
@@ -785,11 +936,8 @@ void ProductList::lower_tma(int8_t sbuf_, int8_t ibuf, int ild, int64_t cap, int
     // along the rows of a tile, as many as fit its 128 rows, and get consecutive
     // scratch slots.  Tiles of one 21 x 21 product each (K = 24, D = 500) used a
     // sixth of a tile's rows and loaded the sector once per operator.
-    struct Stack {
-        size_t item;  // the first product's item (index in the chunk)
-        int n;        // products
-    };
-    std::vector<std::vector<Stack>> stacks(plans.size());
+    std::vector<std::vector<ProdStack>> stacks(plans.size());
+    // the operator is the product's left factor: O Psi, or R^T Psi^T (the transpose of Psi R)
     auto op_view = [&](const Contrib& c, const Item& it) { return it.pq_first ? c.P : c.R.T(); };
     // operators per tile: K-major rows are stacked 16 * sb rows apart, MN-major
     // ones in 64-wide halves
@@ -798,78 +946,15 @@ void ProductList::lower_tma(int8_t sbuf_, int8_t ibuf, int ild, int64_t cap, int
     for (size_t ch = 0; ch < plans.size(); ++ch) {
         ChunkPlan& cp = plans[ch];
         const size_t ni = cp.items.size();
-        struct Key {
-            uint64_t h;
-            int64_t off, alpha;  // family block (without the operator number) and |alpha|
-            int32_t buf, sec;
-            bool operator==(const Key& o) const {
-                return off == o.off && alpha == o.alpha && buf == o.buf && sec == o.sec;
-            }
-        };
-        struct KeyHash {
-            size_t operator()(const Key& k) const { return (size_t)k.h; }
-        };
-        std::vector<Key> keys(ni);
-        const size_t kPart = ni < 4096 ? 1 : 16;
-        const size_t nb = (ni + 4095) / 4096;
-        parallel_for(nb, [&](size_t b) {
-            for (size_t q = b * 4096; q < std::min(ni, (b + 1) * 4096); ++q) {
-                const Item& it = cp.items[q];
-                if (it.kind != 3) continue;
-                const Contrib& c = cs[cp.i + q];
-                const View A = op_view(c, it);
-                Key& k = keys[q];
-                const double aa = std::fabs(c.alpha);
-                std::memcpy(&k.alpha, &aa, 8);
-                k.off = A.off - (int64_t)A.z * A.zstride;
-                k.buf = A.buf * 4 + (A.tr ? 2 : 0) + (it.pq_first ? 1 : 0);
-                k.sec = c.qsec;
-                uint64_t h = 0x9e3779b97f4a7c15ull;
-                for (uint64_t x : {(uint64_t)k.off, (uint64_t)k.alpha, ((uint64_t)(uint32_t)k.buf << 32) | (uint32_t)k.sec}) {
-                    h ^= x + 0x9e3779b97f4a7c15ull + (h << 6) + (h >> 2);
-                    h *= 0xff51afd7ed558ccdull;
-                }
-                k.h = h ^ (h >> 33);
-            }
-        });
-        // partitions of the keys on host threads: per key its items by operator
-        // number, one product per number, runs of consecutive numbers cut to tiles
-        struct Prod {
-            int32_t z;
-            uint32_t item;
-        };
-        std::vector<std::vector<Stack>> pst(kPart);
-        std::vector<std::vector<std::pair<uint32_t, uint32_t>>> same(kPart);  // (item, item whose product it uses)
-        parallel_for(kPart, [&](size_t pt) {
-            std::unordered_map<Key, int, KeyHash> idx;
-            std::vector<std::vector<Prod>> lists;
-            for (size_t q = 0; q < ni; ++q) {
-                if (cp.items[q].kind != 3 || (keys[q].h >> 40) % kPart != pt) continue;
-                auto f = idx.emplace(keys[q], (int)lists.size());
-                if (f.second) lists.emplace_back();
-                lists[f.first->second].push_back({op_view(cs[cp.i + q], cp.items[q]).z, (uint32_t)q});
-            }
-            for (auto& l : lists) {
-                std::stable_sort(l.begin(), l.end(), [](const Prod& a, const Prod& b) { return a.z < b.z; });
-                const Item& it0 = cp.items[l[0].item];
-                const int most = stack_max(op_view(cs[cp.i + l[0].item], it0), it0.tr);
-                int last = -2;
-                uint32_t first = 0;
-                for (const Prod& x : l) {
-                    if (x.z == last) {  // the same product
-                        same[pt].push_back({x.item, first});
-                        continue;
-                    }
-                    if (!pst[pt].empty() && last >= 0 && x.z == last + 1 && pst[pt].back().n < most) ++pst[pt].back().n;
-                    else pst[pt].push_back({x.item, 1});
-                    // slot of the product, relative to its stack's first for now
-                    cp.items[x.item].z = pst[pt].back().n - 1;
-                    cp.items[x.item].neg = (cs[cp.i + x.item].alpha < 0.0) != (cs[cp.i + pst[pt].back().item].alpha < 0.0);
-                    cp.items[x.item].grp = (int)(pst[pt].size() - 1);
-                    last = x.z;
-                    first = x.item;
-                }
-            }
+        Products pr = share_products(ni, [&](size_t q, ProdKey& k, int& z, int& most) {
+            const Item& it = cp.items[q];
+            if (it.kind != 3) return false;
+            const Contrib& c = cs[cp.i + q];
+            const View A = op_view(c, it);
+            k = product_key({A, c.Q, it.tr, it.tcl, 0, !it.pq_first}, it.pq_first, bits_of(std::fabs(c.alpha)));
+            z = A.z;
+            most = stack_max(A, it.tr);
+            return true;
         });
         // scratch slots: groups of equal shape, a stack's products consecutive
         std::unordered_map<int64_t, int> gidx;  // (rows << 32 | cols) -> scratch group
@@ -882,41 +967,31 @@ void ProductList::lower_tma(int8_t sbuf_, int8_t ibuf, int ild, int64_t cap, int
             }
             return g->second;
         };
-        std::vector<std::vector<std::pair<int, int>>> at(kPart);  // stack -> (group, first slot)
-        for (size_t pt = 0; pt < kPart; ++pt) {
-            at[pt].resize(pst[pt].size());
-            for (size_t x = 0; x < pst[pt].size(); ++x) {
-                const int g = group_of(cp.items[pst[pt][x].item]);
-                at[pt][x] = {g, (int)cp.groups[g][2]};
-                cp.groups[g][2] += pst[pt][x].n;
-            }
+        std::vector<std::pair<int, int>> at(pr.stacks.size());  // stack -> (group, first slot)
+        for (size_t x = 0; x < pr.stacks.size(); ++x) {
+            const int g = group_of(cp.items[pr.stacks[x].item]);
+            at[x] = {g, (int)cp.groups[g][2]};
+            cp.groups[g][2] += pr.stacks[x].n;
         }
-        for (Item& it : cp.items)
+        for (size_t q = 0; q < ni; ++q) {
+            Item& it = cp.items[q];
             if (it.kind == 2) {
                 it.grp = group_of(it);
                 it.z = (int)cp.groups[it.grp][2]++;
+            } else if (it.kind == 3) {
+                const int x = pr.stack[q];
+                it.grp = at[x].first;
+                it.z = at[x].second + pr.pos[q];
+                it.neg = (cs[cp.i + q].alpha < 0.0) != (cs[cp.i + pr.stacks[x].item].alpha < 0.0);
             }
-        parallel_for(kPart, [&](size_t pt) {
-            for (size_t q = 0; q < ni; ++q) {
-                Item& it = cp.items[q];
-                if (it.kind != 3 || (keys[q].h >> 40) % kPart != pt || it.grp < 0) continue;
-                const auto& a = at[pt][it.grp];
-                it.grp = a.first;
-                it.z += a.second;
-            }
-            for (const auto& d : same[pt]) {
-                cp.items[d.first].grp = cp.items[d.second].grp;
-                cp.items[d.first].z = cp.items[d.second].z;
-                cp.items[d.first].neg = cp.items[d.second].neg != ((cs[cp.i + d.first].alpha < 0.0) != (cs[cp.i + d.second].alpha < 0.0));
-            }
-        });
+        }
         int64_t base = 0;
         for (auto& g : cp.groups) {
             g[3] = base;
             base += g[2] * g[0] * round_up(g[1], 8);
         }
         cp.used = base;
-        for (auto& l : pst) stacks[ch].insert(stacks[ch].end(), l.begin(), l.end());
+        stacks[ch] = std::move(pr.stacks);
     }
     // pass 2: the work lists.  Each chunk's items are cut into units of at
     // most kUnit items that run on host threads, each with a tensor-map table
@@ -986,7 +1061,7 @@ void ProductList::lower_tma(int8_t sbuf_, int8_t ibuf, int ild, int64_t cap, int
             }
         }
         // the unit's share of the chunk's stacks
-        const std::vector<Stack>& sk = stacks[u.ch];
+        const std::vector<ProdStack>& sk = stacks[u.ch];
         const size_t nu = unit_beg[u.ch + 1] - unit_beg[u.ch], un = ui - unit_beg[u.ch];
         for (size_t x = sk.size() * un / nu; x < sk.size() * (un + 1) / nu; ++x) {
             const Contrib& c = cs[cp.i + sk[x].item];
