@@ -16,7 +16,9 @@ namespace {
 // Buffer ids of the tables used by every work list.
 enum : int8_t { BUF_L = 0, BUF_R = 1, BUF_INT = 2, BUF_PSI = 3, BUF_SCR = 4, BUF_ID = 5, BUF_OUT = 6, BUF_W = 7 };
 
-constexpr int64_t kChunkF64 = 1 << 14;  // K-depth per accumulation pass (FP64 engine)
+// K-depth per accumulation pass of the FP64-accurate tensor-core engine: several
+// tiles per SM where a bond's few hundred outputs sum thousands of products
+constexpr int64_t kChunkF64 = 1 << 12;
 // Tensor cores: K-depth one output tile accumulates in FP32 tensor memory
 // before it is added (atomically) into an FP64 result.  The error of a chain
 // grows linearly with its depth (about 6e-6 relative at 1024 on sigma-like
@@ -205,14 +207,13 @@ struct SigmaShape {
 // block with all of its products, cut into tiles and K-chunks as the list would
 // be and dealt to the SMs longest first.  In units of a 64-deep K stage of phase
 // 2: 16 for the launches, 1.6 per phase-1 stage of an SM, and for phase 2 the
-// largest SM's stages plus 4 per tile (its drain; 2 with three pieces, whose
-// stages take longer).  The weights are fitted to timings of 260 bonds (K = 7 to
-// 32, D = 30 to 900; one, two and three bf16 pieces), of which the estimate picks
-// the faster K-chunk in all but nine, five of those within 2 % either way.
-// Timing the sample instead took 8 to 60 ms per new bond, and near a tie it chose
-// by noise, so that one bond's sigma differed by the FP32 rounding of the other
-// chain length (3e-6) from run to run.  The fastest wins, the default (128, kmax)
-// unless another is faster (three pieces: 1 % faster).
+// largest SM's stages plus 4 per tile (its drain).  The weights are fitted to
+// timings of 420 bonds (K = 7 to 32, D = 30 to 900; one, two and three bf16
+// pieces), of which the estimate picks the faster K-chunk in all but 23, half of
+// those within 2 % either way.  Timing the sample instead took 8 to 60 ms per new
+// bond, and near a tie it chose by noise, so that one bond's sigma differed by
+// the FP32 rounding of the other chain length (3e-6) from run to run.  The
+// fastest wins, the default (128, kmax) unless another is 0.5 % faster.
 SigmaShape tune_sigma_shape(Plan& P, const ProductList& tl, int64_t kmax, int G) {
     const uint64_t key = sector_histogram_key(P, G);
     auto f = P.tune_cache.find(key);
@@ -222,8 +223,7 @@ SigmaShape tune_sigma_shape(Plan& P, const ProductList& tl, int64_t kmax, int G)
     }
     const auto t0 = std::chrono::steady_clock::now();
     constexpr int kSMs = 152;
-    constexpr double kBase = 16.0, kStage1 = 1.6, kStageMs = 0.67e-3;
-    const double kDrain = P.nsplit == 3 ? 2.0 : 4.0, kMargin = P.nsplit == 3 ? 0.99 : 1.0;
+    constexpr double kBase = 16.0, kStage1 = 1.6, kDrain = 4.0, kStageMs = 0.67e-3, kMargin = 0.995;
     const int64_t khalf = std::max<int64_t>(kmax / 2, 64);
     const SigmaShape cand[4] = {{128, kmax}, {64, kmax}, {128, khalf}, {64, khalf}};
     const int stride = tl.outs.size() >= 64 ? 8 : 1;

@@ -70,6 +70,7 @@ struct WorkList {
     // it), by K-blocks of every segment (byk) or by segments
     int part = 64, split = 0;
     bool byk = false;
+    bool single = false;  // every tile has one segment (FP64-accurate tensor-core engine, set by upload)
     // tile shape of add_block when nonzero (rows, columns); 128 x 64 lists run on
     // the FP64-accurate tensor-core engine (launch_seg_gemm_f64 dispatches on it)
     int tile_m = 0, tile_n = 0;

@@ -131,6 +131,8 @@ void WorkList::upload(cudaStream_t st) {
         segsum += t.seg_end - t.seg_beg;
     }
     for (const Seg& g : segs) ksum += g.k;
+    single = true;
+    for (const Tile& t : tiles) single = single && t.seg_end - t.seg_beg == 1;
     part = std::max(mmax, nmax) <= 16 ? 16 : (std::max(mmax, nmax) <= 32 ? 32 : 64);
     split = 0;
     byk = false;

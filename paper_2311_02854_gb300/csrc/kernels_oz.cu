@@ -32,23 +32,26 @@
 // that hold two stages, so stage q+1 is converted into the other half while the
 // tensor cores consume stage q.
 //
-// Bound: the instruction streams of the conversion and of the combination (and
-// FP64-pipe instructions: one takes a scheduler ~74 cycles), not the tensor
-// pipe.  Hence the split: two groups of three loader warps convert alternate
-// stages, each thread eight values of one row that it keeps in registers from
-// the scale to the slices (two to four lanes share a row, by the depth of the
-// stage); rows and columns outside the block are neither loaded nor converted;
-// the slices of B follow each other along N, so that one instruction multiplies
-// a slice of A with all the slices of B it meets (6 instructions per 16-deep
-// step instead of 21); a tile of up to 32 columns has two sets of accumulators,
-// and only its columns are combined, by two warps per 32 rows.  A warp reads
-// the tensor memory of its own scheduler's quarter only, so tiles of up to 32
-// rows keep one of the four schedulers busy: the loaders stay off the first
-// scheduler, and lists stack up to four such products in a tile.  (Four warps
-// that converted all 128 rows of every stage, one row per thread, and 42
-// instructions per stage took ~7 us per stage.)
+// Bound: the instruction streams of the conversion and of the combination, not
+// the tensor pipe.  Hence the split: two groups of six loader warps convert
+// alternate stages, each thread eight values of one row that it keeps in
+// registers from the scale to the slices (two to four lanes share a row, by the
+// depth of the stage); rows and columns outside the block are neither loaded nor
+// converted; the slices of B follow each other along N, so that one instruction
+// multiplies a slice of A with all the slices of B it meets (6 instructions per
+// 16-deep step instead of 21); a tile of up to 32 columns has two sets of
+// accumulators, and only its columns are combined, by two warps per 32 rows.  A
+// warp reads the tensor memory of its own scheduler's quarter only, so tiles of
+// up to 32 rows keep one of the four schedulers busy: the loaders stay off the
+// first scheduler, and lists stack up to four such products in a tile.  The code
+// of each role is kept short: with the column loops unrolled (accumulators in
+// registers) a warp spent ~1900 cycles per four columns and 22 000 on writing a
+// tile out, fetching instructions.  FP64-pipe instructions take a scheduler ~74
+// cycles each, so floats are widened by their bits.  (Four warps that converted
+// all 128 rows of every stage, one row per thread, and 42 instructions per stage
+// took ~7 us per stage.)
 // Warps 0-7 epilogue (warp w: tile rows 32 (w % 4) .., half w / 4 of the
-// columns), warp 8 lane 0 issues the MMAs, warps 9-11 and 13-15 loaders.  Every
+// columns), warp 8 lane 0 issues the MMAs, the other warps but 12, 16 and 20 loaders.  Every
 // wait is bounded; a timeout sets the device error word.
 #include <cuda_bf16.h>
 
@@ -71,9 +74,9 @@ constexpr int SLICE_BYTES = NSL * (OTM + OTN) * ROWB;
 constexpr int NREC = 4;
 constexpr uint32_t TMEM_COLS = 512;            // 6 orders x 64 columns (or twice 6 x 32), rounded to a power of two
 constexpr int NEPI = 8;                        // epilogue warps
-constexpr int MMA_WARP = NEPI, IDLE_WARP = NEPI + 4;
-constexpr int NLDW = 3;                        // loader warps of a group
-constexpr int OZ_THREADS = (NEPI + 8) * 32;
+constexpr int MMA_WARP = NEPI;
+constexpr int NLDW = 6;                        // loader warps of a group
+constexpr int OZ_THREADS = (NEPI + 16) * 32;   // warps 12, 16 and 20 idle (the first scheduler's)
 constexpr int EPI_COLS = OTN / 2;
 
 // per-stage record shared by loaders (write), MMA issuer and epilogue (read)
@@ -86,10 +89,11 @@ struct OzStage {
     int32_t n16;       // MMA N / 16
     int32_t pad;
 };
-// the low parts of the epilogue's double-float accumulators live in shared
-// memory ([column][thread], conflict-free), the high parts in registers
-constexpr int ACL_BYTES = NEPI * 32 * EPI_COLS * 4;
-constexpr int OZ_SMEM = 1024 + SLICE_BYTES + NREC * (int)sizeof(OzStage) + ACL_BYTES;
+// the epilogue's double-float accumulators live in shared memory ([column][thread],
+// conflict-free), so that the loop over the columns need not be unrolled
+constexpr int ACC_BYTES = NEPI * 32 * EPI_COLS * 8;
+constexpr int OZ_SMEM = 1024 + SLICE_BYTES + NREC * (int)sizeof(OzStage) + ACC_BYTES;
+static_assert(OZ_SMEM <= 232448, "shared memory of one SM");
 
 // biased exponent field of a double (0 for zero and subnormals)
 __device__ __forceinline__ int exp_field(double x) { return (__double2hiint(x) >> 20) & 0x7FF; }
@@ -149,18 +153,9 @@ __device__ __forceinline__ float pow2f(int k) {
     return __uint_as_float((uint32_t)(k + 127) << 23);
 }
 
-// (double)f by its bits for zeros and normal numbers (the conversion is an
-// FP64-pipe instruction)
-__device__ __forceinline__ double widen(float f) {
-    const uint32_t u = __float_as_uint(f), e = (u >> 23) & 0xFFu;
-    if (e - 1u < 254u) return __hiloint2double((int)((u & 0x80000000u) | (((u & 0x7FFFFFFFu) >> 3) + 0x38000000u)), (int)(u << 29));
-    if ((u << 1) == 0u) return __hiloint2double((int)u, 0);
-    return (double)f;
-}
-
 __global__ void __launch_bounds__(OZ_THREADS, 1)
-    oz_gemm_kernel(const Tile* __restrict__ tiles, int ntiles, int nvec, const Seg* __restrict__ segs, BufTable bt,
-                   int* err) {
+    oz_gemm_kernel(const Tile* __restrict__ tiles, int ntiles, int nvec, int single, const Seg* __restrict__ segs,
+                   BufTable bt, int* err) {
     extern __shared__ uint8_t smem_raw[];
     // full[h]: loaders -> MMA (slices of K half h and the stage record written);
     // rec[h]: MMA -> epilogue (record visible); done[h]: MMA completion -> loaders
@@ -171,7 +166,7 @@ __global__ void __launch_bounds__(OZ_THREADS, 1)
     const uint32_t sbase = (smem_u32(smem_raw) + 1023u) & ~1023u;
     const uint32_t sA = sbase, sB = sbase + NSL * A_SLICE;
     OzStage* recs = reinterpret_cast<OzStage*>(smem_raw + (sbase - smem_u32(smem_raw)) + SLICE_BYTES);
-    float* acl_s = reinterpret_cast<float*>(recs + NREC);
+    float2* acc_s = reinterpret_cast<float2*>(recs + NREC);
 
     if (warp == 0) tmem_alloc(smem_u32(&tmem_base_s), TMEM_COLS);
     if (tid == 0) {
@@ -191,125 +186,120 @@ __global__ void __launch_bounds__(OZ_THREADS, 1)
     const uint32_t total = (uint32_t)ntiles * (uint32_t)nvec, NV = (uint32_t)nvec;  // total < 2^31
     bool failed = false;
 
-    if (warp > MMA_WARP && warp != IDLE_WARP) {
+    if (warp > MMA_WARP && (warp & 3) != 0) {
         // ---------------- loaders / converters ----------------
-        const uint32_t grp = warp > IDLE_WARP ? 1u : 0u;
-        const int gw = warp - (grp ? IDLE_WARP : MMA_WARP) - 1;
+        const int li = warp - MMA_WARP - 1 - ((warp - MMA_WARP) >> 2);
+        const uint32_t grp = (uint32_t)(li / NLDW);
+        const int gw = li % NLDW;
         uint32_t d = 0;  // stages so far (all tiles, both groups)
-        // the next tile and its first segment are in flight while a tile is converted
-        struct Place {
-            int m0, n0, m, n, seg_beg, seg_end, astride;
-            int sn, srows;  // stacked products and the rows between them (0: none)
-        };
-        auto place = [&](uint32_t i) {
-            Place p{};
-            if (i < total) {
-                const Tile& t = tiles[i / NV];
-                p = Place{t.m0, t.n0, t.m, t.n, t.seg_beg, t.seg_end, t.astride, t.sn, 16 * t.sb};
-            }
-            return p;
-        };
-        Seg S{};
         const uint32_t G = gridDim.x;
-        Place T = place(blockIdx.x), nT = place(blockIdx.x + G);
-        if (T.seg_beg < T.seg_end) S = segs[T.seg_beg];
-        for (uint32_t it = blockIdx.x; it < total && !failed; it += G) {
-            const int v = (int)(it % NV);
-            const int mrem = min(OTM, T.m - T.m0), nrem = min(OTN, T.n - T.n0), n16 = (nrem + 15) / 16;
-            const uint32_t b_slice = (uint32_t)n16 * 16u * ROWB;  // the slices of B follow each other along N
-            Seg nS{};
-            if (nT.seg_beg < nT.seg_end) nS = segs[nT.seg_beg];
-            const Place nnT = place(it + 2 * G);
-            int s = T.seg_beg;
-            while (s < T.seg_end && S.k <= 0)
-                if (++s < T.seg_end) S = segs[s];
-            int k0 = 0;
-            bool more = true;
-            while (more) {
-                // the stage: k0 .. k0 + kn of segment s (kn = 0: a tile without products)
-                const int kn = s < T.seg_end ? min(OTK, S.k - k0) : 0;
-                const Seg Sc = S;
-                const int kb = k0;
-                k0 += kn;
-                while (s < T.seg_end && k0 >= S.k) {  // the next segment with products
-                    k0 = 0;
-                    if (++s < T.seg_end) S = segs[s];
+        // The lanes hold the records of the next 32 segments of a tile (or, of lists
+        // whose tiles have one segment each, of the next 32 tiles of this CTA): the
+        // dependent loads tile -> segment are paid once per 32, not by every stage.
+        uint32_t ct = blockIdx.x;  // next tile
+        int cs = 0;                // segments of it already taken
+        while (ct < total && !failed) {
+            const uint32_t t = single ? ct + (uint32_t)lane * G : ct;
+            Tile T{};
+            Seg S{};
+            bool valid = false, last = true;
+            if (t < total) {
+                T = tiles[t / NV];
+                const int idx = T.seg_beg + (single ? 0 : cs + lane);
+                valid = idx < T.seg_end || (idx == T.seg_beg && T.seg_beg == T.seg_end);
+                last = idx + 1 >= T.seg_end;
+                if (idx < T.seg_end) S = segs[idx];
+            }
+            const int nseg = __shfl_sync(0xffffffffu, T.seg_end - T.seg_beg, 0);
+            cs += 32;
+            if (single) {
+                ct = min(total, ct + 32 * G);
+            } else if (cs >= nseg) {
+                ct = min(total, ct + G);
+                cs = 0;
+            }
+            const int vt = (int)(t % NV);
+            const int nl = __popc(__ballot_sync(0xffffffffu, valid));  // the valid lanes are the first nl
+            for (int l = 0; l < nl && !failed; ++l) {
+                const auto at = [&](auto x) { return __shfl_sync(0xffffffffu, x, l); };
+                const int k = at(S.k), end = at((int)last);
+                // a segment without depth only matters where it ends a tile
+                const int nst = k > 0 ? (k + OTK - 1) / OTK : end;
+                if (nst == 0) continue;
+                if (nst == 1 && (d & 1u) != grp) {  // the other group's
+                    ++d;
+                    continue;
                 }
-                more = s < T.seg_end;
-                const uint32_t slot = d & 1u, use = d >> 1;
-                OzStage& R = recs[d % NREC];
-                ++d;
-                if (slot != grp) continue;
-                const int steps = (kn + 15) / 16;
-                // a task: rt rows of one product's A or columns of B, 32 / rt K groups of eight
-                const int lg = kn > 16 ? 3 : 4, rt = 1 << lg;
-                const int lr = lane & (rt - 1), cg = lane >> lg;
-                const int nap = (mrem + rt - 1) >> lg;  // tasks of a product
-                const int na = kn > 0 ? nap * max(T.sn, 1) : 0, nb = kn > 0 ? (nrem + rt - 1) >> lg : 0;
-                const int64_t ak = Sc.a_tr ? Sc.lda : 1, ar = Sc.a_tr ? 1 : Sc.lda;
-                const int64_t bk = Sc.b_tr ? 1 : Sc.ldb, br = Sc.b_tr ? Sc.ldb : 1;
-                const double* A = bt.p[Sc.a_buf] + Sc.a_off + (int64_t)v * bt.vstride[Sc.a_buf] + T.m0 * ar + (kb + 8 * cg) * ak;
-                const double* B = bt.p[Sc.b_buf] + Sc.b_off + (int64_t)v * bt.vstride[Sc.b_buf] + T.n0 * br + (kb + 8 * cg) * bk;
-                const int kv = kn - 8 * cg;  // K values of this lane's group that exist
-                int ok = 1;
-                bool waited = false;
-                for (int t0 = gw; t0 < na + nb || !waited; t0 += 2 * NLDW) {
-                    double x[2][8];  // two tasks' loads in flight together
-                    int rows[2];
+                const int m = at(T.m), m0 = at(T.m0), n0 = at(T.n0), sn = at((int)T.sn), srows = 16 * at((int)T.sb);
+                const int astride = at(T.astride), v = at(vt);
+                const int mrem = min(OTM, m - m0), nrem = min(OTN, at(T.n) - n0), n16 = (nrem + 15) / 16;
+                const uint32_t b_slice = (uint32_t)n16 * 16u * ROWB;  // the slices of B follow each other along N
+                const int form = at(S.a_buf | (S.b_buf << 8) | (S.a_tr ? 1 << 16 : 0) | (S.b_tr ? 1 << 17 : 0));
+                const int lda = at(S.lda), ldb = at(S.ldb);
+                const int64_t ak = form >> 16 & 1 ? lda : 1, ar = form >> 16 & 1 ? 1 : lda;
+                const int64_t bk = form >> 17 & 1 ? 1 : ldb, br = form >> 17 & 1 ? ldb : 1;
+                const double* A0 = bt.p[form & 255] + at((long long)S.a_off) + (int64_t)v * bt.vstride[form & 255] + m0 * ar;
+                const double* B0 = bt.p[form >> 8 & 255] + at((long long)S.b_off) + (int64_t)v * bt.vstride[form >> 8 & 255] + n0 * br;
+                const double alpha = at(S.alpha);
+                for (int st = 0; st < nst; ++st) {
+                    const uint32_t slot = d & 1u, use = d >> 1;
+                    OzStage& R = recs[d % NREC];
+                    ++d;
+                    if (slot != grp) continue;
+                    const int kb = st * OTK, kn = max(0, min(OTK, k - kb)), steps = (kn + 15) / 16;
+                    // a task: rt rows of one product's A or columns of B, 32 / rt K groups of eight
+                    const int lg = kn > 16 ? 3 : 4, rt = 1 << lg;
+                    const int lr = lane & (rt - 1), cg = lane >> lg;
+                    const int nap = (mrem + rt - 1) >> lg;  // tasks of a product
+                    const int na = kn > 0 ? nap * max(sn, 1) : 0, nb = kn > 0 ? (nrem + rt - 1) >> lg : 0;
+                    const int kv = kn - 8 * cg;  // K values of this lane's group that exist
+                    int ok = 1;
+                    bool waited = false;
+#pragma unroll 1
+                    for (int t1 = gw; t1 < na + nb || !waited; t1 += NLDW) {
+                        const bool isb = t1 >= na;
+                        const int pi = isb || sn == 0 ? 0 : t1 / nap;  // stacked product
+                        int row = ((isb ? t1 - na : t1 - pi * nap) << lg) + lr;
+                        const double* q = isb ? B0 + row * br + (kb + 8 * cg) * bk
+                                              : A0 + (int64_t)pi * astride + row * ar + (kb + 8 * cg) * ak;
+                        const int64_t ks = isb ? bk : ak;
+                        const int n = t1 < na + nb && row < (isb ? nrem : mrem) ? kv : 0;
+                        row += pi * srows;
+                        double x[8];
 #pragma unroll
-                    for (int h = 0; h < 2; ++h) {
-                        const int t = t0 + h * NLDW;
-                        const bool isb = t >= na;
-                        const int pi = isb || T.sn == 0 ? 0 : t / nap;  // stacked product
-                        const int row = ((isb ? t - na : t - pi * nap) << lg) + lr;
-                        const double* q = isb ? B + row * br : A + (int64_t)pi * T.astride + row * ar;
-                        const int64_t st = isb ? bk : ak;
-                        const int n = t < na + nb && row < (isb ? nrem : mrem) ? kv : 0;
-                        rows[h] = row + pi * T.srows;
-#pragma unroll
-                        for (int j = 0; j < 8; ++j) x[h][j] = j < n ? q[j * st] : 0.0;
-                    }
-                    if (!waited) {  // half free: the MMAs of stage d - 2 completed
-                        waited = true;
-                        if (lane == 0 && use > 0) ok = mbar_wait(smem_u32(&done_bar[slot]), (use - 1) & 1u) ? 1 : 0;
-                        ok = __shfl_sync(0xffffffffu, ok, 0);
-                        if (!ok) break;
-                    }
-#pragma unroll
-                    for (int h = 0; h < 2; ++h) {
-                        const int t = t0 + h * NLDW;
-                        if (t >= na + nb) break;
-                        const bool isb = t >= na;
-                        const int row = rows[h];
+                        for (int j = 0; j < 8; ++j) x[j] = j < n ? q[j * ks] : 0.0;
+                        if (!waited) {  // (the loads are in flight) half free: the MMAs of stage d - 2 completed
+                            waited = true;
+                            if (lane == 0 && use > 0) ok = mbar_wait(smem_u32(&done_bar[slot]), (use - 1) & 1u) ? 1 : 0;
+                            ok = __shfl_sync(0xffffffffu, ok, 0);
+                            if (!ok || t1 >= na + nb) break;
+                        }
                         int emax = 0;
 #pragma unroll
-                        for (int j = 0; j < 8; ++j) emax = max(emax, exp_field(x[h][j]));
+                        for (int j = 0; j < 8; ++j) emax = max(emax, exp_field(x[j]));
                         for (int o = rt; o < 32; o *= 2) emax = max(emax, __shfl_xor_sync(0xffffffffu, emax, o));
                         const bool in = row < (isb ? 16 * n16 : OTM);  // (a task's last rows may lie beyond the buffers)
                         if (cg == 0 && in) (isb ? R.eb : R.ea)[row] = emax ? emax + 1 - 1023 : -1000;
                         if (cg < 2 * steps && in)
-                            store_slices(x[h], emax + 1, isb ? sB : sA, isb ? b_slice : (uint32_t)A_SLICE, row,
+                            store_slices(x, emax + 1, isb ? sB : sA, isb ? b_slice : (uint32_t)A_SLICE, row,
                                          (int)slot * (OTK / 8) + cg);
                     }
+                    if (!ok) {
+                        failed = true;
+                        break;
+                    }
+                    if (gw == 0 && lane == 0) {
+                        R.ah = (float)alpha;
+                        R.al = (float)(alpha - (double)R.ah);
+                        R.flags = (end && st == nst - 1 ? 2 : 0) | (kn == 0 ? 4 : 0);
+                        R.ksteps = steps;
+                        R.n16 = n16;
+                    }
+                    fence_proxy_async();
+                    __syncwarp();
+                    if (lane == 0) mbar_arrive(smem_u32(&full_bar[slot]));
                 }
-                if (!ok) {
-                    failed = true;
-                    break;
-                }
-                if (gw == 0 && lane == 0) {
-                    R.ah = (float)Sc.alpha;
-                    R.al = (float)(Sc.alpha - (double)R.ah);
-                    R.flags = (more ? 0 : 2) | (kn == 0 ? 4 : 0);
-                    R.ksteps = steps;
-                    R.n16 = n16;
-                }
-                fence_proxy_async();
-                __syncwarp();
-                if (lane == 0) mbar_arrive(smem_u32(&full_bar[slot]));
             }
-            T = nT;
-            S = nS;
-            nT = nnT;
         }
     } else if (warp == MMA_WARP) {
         // ---------------- MMA issuer ----------------
@@ -364,7 +354,7 @@ __global__ void __launch_bounds__(OZ_THREADS, 1)
         // ---------------- epilogue ----------------
         const int quarter = warp & 3, chalf = warp >> 2;
         const int row = quarter * 32 + lane;
-        float* acl = acl_s + tid;  // acl[c * NEPI * 32]
+        float2* acc = acc_s + tid;  // acc[c * NEPI * 32]: (high, low)
         uint32_t d = 0;
         Tile nT{};
         if (blockIdx.x < total) nT = tiles[blockIdx.x / NV];
@@ -386,10 +376,7 @@ __global__ void __launch_bounds__(OZ_THREADS, 1)
             const int hc = ((nrem + 1) / 2 + 3) & ~3, c0 = chalf * hc;
             const int ncol = any ? min(hc, nrem - c0) : 0;
             const uint32_t cs = (uint32_t)((nrem + 15) / 16) * 16u;  // columns of an order
-            float ach[EPI_COLS];
-#pragma unroll
-            for (int c = 0; c < EPI_COLS; ++c) ach[c] = 0.f;
-            for (int c = 0; c < ncol; ++c) acl[c * NEPI * 32] = 0.f;
+            for (int c = 0; c < ((ncol + 3) & ~3); ++c) acc[c * NEPI * 32] = make_float2(0.f, 0.f);
             for (;;) {
                 const uint32_t slot = d & 1u, use = d >> 1;
                 int ok = 1;
@@ -415,9 +402,8 @@ __global__ void __launch_bounds__(OZ_THREADS, 1)
                 const float ah = R.ah, al = R.al;
                 const bool unit = (ah == 1.f || ah == -1.f) && al == 0.f;  // alpha = +-1: a sign only
                 const uint32_t tb = tmem + ((uint32_t)(quarter * 32) << 16) + (cs > 32u ? 0u : slot * 256u) + (uint32_t)c0;
-#pragma unroll
-                for (int cc = 0; cc < EPI_COLS / 4; ++cc) {
-                    if (cc * 4 >= ncol) break;
+#pragma unroll 1
+                for (int cc = 0; cc * 4 < ncol; ++cc) {
                     uint32_t a[NORD][4];
 #pragma unroll
                     for (int g = 0; g < NORD; ++g) tmem_ld4(tb + (uint32_t)g * cs + (uint32_t)(cc * 4), a[g]);
@@ -432,7 +418,7 @@ __global__ void __launch_bounds__(OZ_THREADS, 1)
                     }
 #pragma unroll
                     for (int j = 0; j < 4; ++j) {
-                        const int c = cc * 4 + j;
+                        float2& sum = acc[(cc * 4 + j) * NEPI * 32];
                         // sum of the orders, order g weighted 2^-8g, as a double-float
                         float sh = __uint_as_float(a[0][j]), sl = 0.f, e;
 #pragma unroll
@@ -454,10 +440,12 @@ __global__ void __launch_bounds__(OZ_THREADS, 1)
                             pe = fmaf(sh, al, pe);
                             pe = fmaf(sl, ah, pe);
                         }
+                        float2 t = sum;
                         float nh;
-                        two_sum(ach[c], p, nh, e);
-                        ach[c] = nh;
-                        acl[c * NEPI * 32] += e + pe;
+                        two_sum(t.x, p, nh, e);
+                        t.y += e + pe;
+                        t.x = nh;
+                        sum = t;
                     }
                 }
                 if (flags & 2) break;
@@ -466,13 +454,13 @@ __global__ void __launch_bounds__(OZ_THREADS, 1)
             // the tile's FP64 result
             if (rok && ncol > 0) {
                 double* C = bt.p[T.c_buf] + T.c_off + (int64_t)v * bt.vstride[T.c_buf] + orow * T.ldc + T.n0 + c0;
-#pragma unroll
-                for (int c = 0; c < EPI_COLS; ++c)
-                    if (c < ncol) {
-                        const double r = widen(ach[c]) + widen(acl[c * NEPI * 32]);
-                        if (T.mode == TILE_ATOMIC) atomicAdd(C + c, r);
-                        else C[c] = r;
-                    }
+#pragma unroll 1
+                for (int c = 0; c < ncol; ++c) {
+                    const float2 t = acc[c * NEPI * 32];
+                    const double r = widen(t.x) + widen(t.y);
+                    if (T.mode == TILE_ATOMIC) atomicAdd(C + c, r);
+                    else C[c] = r;
+                }
             }
         }
     }
@@ -522,7 +510,8 @@ void launch_seg_gemm_oz(const WorkList& w, const BufTable& bt, int nvec, int* d_
     DMRG_CHECK_CUDA(cudaGetDevice(&dev));
     DMRG_CHECK_CUDA(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev));
     const int grid = (int)std::min<int64_t>(total, std::max(nsm, 1));
-    oz_gemm_kernel<<<grid, OZ_THREADS, OZ_SMEM, st>>>(w.d_tiles, (int)w.tiles.size(), nvec, w.d_segs, bt, d_err);
+    oz_gemm_kernel<<<grid, OZ_THREADS, OZ_SMEM, st>>>(w.d_tiles, (int)w.tiles.size(), nvec, (int)w.single, w.d_segs, bt,
+                                                       d_err);
     ++launch_counter();
     DMRG_CHECK_CUDA(cudaGetLastError());
 }

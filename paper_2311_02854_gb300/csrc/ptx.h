@@ -109,5 +109,14 @@ __device__ __forceinline__ void tmem_dealloc(uint32_t tmem, uint32_t ncols) {
     asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;\n" ::"r"(tmem), "r"(ncols) : "memory");
 }
 
+// (double)f by its bits for zeros and normal numbers (the conversion is an
+// FP64-pipe instruction)
+__device__ __forceinline__ double widen(float f) {
+    const uint32_t u = __float_as_uint(f), e = (u >> 23) & 0xFFu;
+    if (e - 1u < 254u) return __hiloint2double((int)((u & 0x80000000u) | (((u & 0x7FFFFFFFu) >> 3) + 0x38000000u)), (int)(u << 29));
+    if ((u << 1) == 0u) return __hiloint2double((int)u, 0);
+    return (double)f;
+}
+
 }  // namespace ptx
 }  // namespace dmrg
