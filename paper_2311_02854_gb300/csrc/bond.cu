@@ -127,11 +127,9 @@ void set_out_pieces(const Plan& P, TcBufs& tb, int b, __nv_bfloat16* hi, __nv_bf
 // bf16 pieces of the padded wavefunction copy for n elements (all vectors of a launch)
 void ensure_psi_pieces(Plan& P, int64_t n) {
     if (n <= P.n_ppc) return;
-    P.free_bf16(P.ps_hi, P.n_ppc);
-    P.free_lo(P.ps_lo, P.n_ppc);
+    P.free_pieces(P.ps_hi, P.ps_lo, P.n_ppc);
     P.n_ppc = n;
-    P.ps_hi = P.alloc_bf16(n);
-    P.ps_lo = P.alloc_lo(n);
+    P.alloc_pieces(n, P.ps_hi, P.ps_lo);
 }
 
 // Buffers of the mixed sigma at bond k (out: FP64 result of vector 0)
@@ -298,8 +296,7 @@ void free_block(Plan& P, std::unique_ptr<Block>& b) {
     if (!b) return;
     tier_release(P, *b);
     P.free(b->d, b->n);
-    P.free_bf16(b->h, b->n);
-    P.free_lo(b->l, b->n);
+    P.free_pieces(b->h, b->l, b->n);
     b.reset();
 }
 
@@ -316,12 +313,10 @@ void ensure_ident(Plan& P, int n) {
         dev_identity(P.d_ident, n, P.stream);
     }
     if (P.mixed() && P.id_n != P.ident_n) {
-        P.free_bf16(P.id_hi, (int64_t)P.id_n * P.id_n);
-        P.free_lo(P.id_lo, (int64_t)P.id_n * P.id_n);
+        P.free_pieces(P.id_hi, P.id_lo, (int64_t)P.id_n * P.id_n);
         P.id_n = P.ident_n;
         const int64_t nn = (int64_t)P.id_n * P.id_n;
-        P.id_hi = P.alloc_bf16(nn);
-        P.id_lo = P.alloc_lo(nn);
+        P.alloc_pieces(nn, P.id_hi, P.id_lo);
         dev_split_f64_flat(P.d_ident, nn, P.id_hi, P.id_lo, P.stream, P.lo2(P.id_lo, nn));
     }
 }
@@ -329,11 +324,9 @@ void ensure_ident(Plan& P, int n) {
 void ensure_scratch(Plan& P, int64_t n) {
     if (P.mixed()) {
         if (n <= P.n_spc) return;
-        P.free_bf16(P.s_hi, P.n_spc);
-        P.free_lo(P.s_lo, P.n_spc);
+        P.free_pieces(P.s_hi, P.s_lo, P.n_spc);
         P.n_spc = n;
-        P.s_hi = P.alloc_bf16(n);
-        P.s_lo = P.alloc_lo(n);
+        P.alloc_pieces(n, P.s_hi, P.s_lo);
         return;
     }
     if (n <= P.n_scratch) return;
@@ -388,8 +381,7 @@ void form_interms(Plan& P, Interms& im, const Block* blocks[2], IntermStore& S, 
     S.n = std::max<int64_t>(total, 32);
     flops = 0.0;
     if (P.mixed()) {
-        S.h = P.alloc_bf16(S.n);
-        S.l = P.alloc_lo(S.n);
+        P.alloc_pieces(S.n, S.h, S.l);
     }
     if (P.f64_store()) S.d = P.alloc(S.n);
     if (im.fams.empty()) return;
@@ -428,11 +420,9 @@ void form_interms(Plan& P, Interms& im, const Block* blocks[2], IntermStore& S, 
     wl.upload(P.stream);
     if (P.tc_store()) {
         if (wn > P.n_wpc) {
-            P.free_bf16(P.w_hi, P.n_wpc);
-            P.free_lo(P.w_lo, P.n_wpc);
+            P.free_pieces(P.w_hi, P.w_lo, P.n_wpc);
             P.n_wpc = wn;
-            P.w_hi = P.alloc_bf16(wn);
-            P.w_lo = P.alloc_lo(wn);
+            P.alloc_pieces(wn, P.w_hi, P.w_lo);
         }
         dev_split_f64_flat(P.d_wcoef, wn, P.w_hi, P.w_lo, P.stream, P.lo2(P.w_lo, P.n_wpc));
         // FP32 sum of the K-chunks, then split into the bf16 pieces
@@ -465,8 +455,7 @@ void form_interms(Plan& P, Interms& im, const Block* blocks[2], IntermStore& S, 
 
 void free_interms(Plan& P, IntermStore& S) {
     P.free(S.d, S.n);
-    P.free_bf16(S.h, S.n);
-    P.free_lo(S.l, S.n);
+    P.free_pieces(S.h, S.l, S.n);
     S.n = 0;
 }
 
@@ -482,8 +471,7 @@ std::unique_ptr<Block> make_vacuum(Plan& P, bool right_end) {
     B->lay.build(b, lo, lo, P.n_so);
     B->n = std::max<int64_t>(B->lay.total, 32);
     if (P.mixed()) {
-        B->h = P.alloc_bf16(B->n);
-        B->l = P.alloc_lo(B->n);
+        P.alloc_pieces(B->n, B->h, B->l);
         DMRG_CHECK_CUDA(cudaMemsetAsync(B->h, 0, B->n * 2, P.stream));
         DMRG_CHECK_CUDA(cudaMemsetAsync(B->l, 0, P.lo_pieces() * B->n * 2, P.stream));
     }
@@ -534,8 +522,7 @@ static SiteDev upload_site(Plan& P, int k) {
     S.d = P.alloc(S.n);
     DMRG_CHECK_CUDA(cudaMemcpyAsync(S.d, host.data(), S.n * 8, cudaMemcpyHostToDevice, P.stream));
     if (P.mixed()) {
-        S.h = P.alloc_bf16(S.n);
-        S.l = P.alloc_lo(S.n);
+        P.alloc_pieces(S.n, S.h, S.l);
         dev_split_f64_flat(S.d, S.n, S.h, S.l, P.stream, P.lo2(S.l, S.n));
     }
     DMRG_CHECK_CUDA(cudaStreamSynchronize(P.stream));
@@ -544,8 +531,7 @@ static SiteDev upload_site(Plan& P, int k) {
 
 static void free_site(Plan& P, SiteDev& S) {
     P.free(S.d, S.n);
-    P.free_bf16(S.h, S.n);
-    P.free_lo(S.l, S.n);
+    P.free_pieces(S.h, S.l, S.n);
 }
 
 // Grow block X by site m (forward: X = sites 1..m-1 -> sites 1..m) or
@@ -704,8 +690,7 @@ std::unique_ptr<Block> renormalise(Plan& P, const Block& X, int m, bool forward)
         set_out_pieces(P, tb, BUF_SCR, P.s_hi, P.s_lo, P.n_spc);
         pl.run_tc(tb, 1, P.nsplit, P.stream);
         P.check_device_error();
-        out->h = P.alloc_bf16(out->n);
-        out->l = P.alloc_lo(out->n);
+        P.alloc_pieces(out->n, out->h, out->l);
         dev_split_f64_flat(acc, out->n, out->h, out->l, P.stream, P.lo2(out->l, out->n));
         DMRG_CHECK_CUDA(cudaStreamSynchronize(P.stream));
         P.free(acc, out->n);
@@ -727,8 +712,7 @@ std::unique_ptr<Block> renormalise(Plan& P, const Block& X, int m, bool forward)
         bt.p[BUF_ID] = P.d_ident;
         pl.run(bt, 1, P.stream);
         if (P.mixed()) {  // bf16 pieces of the FP64 store for the tensor-core sigma
-            out->h = P.alloc_bf16(out->n);
-            out->l = P.alloc_lo(out->n);
+            P.alloc_pieces(out->n, out->h, out->l);
             dev_split_f64_flat(out->d, out->n, out->h, out->l, P.stream, P.lo2(out->l, out->n));
         }
     }

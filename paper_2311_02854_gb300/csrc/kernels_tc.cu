@@ -377,32 +377,40 @@ __global__ void __launch_bounds__(THREADS2, 1)
 __device__ __forceinline__ void mbar_arrive_tx(uint32_t addr, uint32_t bytes) {
     asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;\n" ::"r"(addr), "r"(bytes) : "memory");
 }
-// 64 x 64 box of a 4-D tensor map into shared memory, completion on an mbarrier
-__device__ __forceinline__ void tma_load4(uint32_t dst, const CUtensorMap* map, int x, int y, int z, int w,
+// box of a 5-D tensor map (all its pieces) into shared memory, completion on an mbarrier
+__device__ __forceinline__ void tma_load5(uint32_t dst, const CUtensorMap* map, int x, int y, int z, int w,
                                           uint32_t bar) {
     asm volatile(
-        "cp.async.bulk.tensor.4d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3, %4, "
-        "%5}], [%6];\n" ::"r"(dst),
-        "l"(reinterpret_cast<uint64_t>(map)), "r"(x), "r"(y), "r"(z), "r"(w), "r"(bar)
+        "cp.async.bulk.tensor.5d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3, %4, "
+        "%5, %6}], [%7];\n" ::"r"(dst),
+        "l"(reinterpret_cast<uint64_t>(map)), "r"(x), "r"(y), "r"(z), "r"(w), "r"(0), "r"(bar)
         : "memory");
 }
 
+// Rows of 128 bytes that one piece of an operand takes in shared memory: one box,
+// of 128 rows for a K-major operand beyond 64 rows; an MN-major one beyond 64
+// columns (halves = 2) has two boxes, every piece's halves NSPLIT * rows apart.
+__device__ __forceinline__ int piece_rows(int mn, int halves, int box) { return !mn && halves == 2 ? 128 : box; }
 
-// One 128 x 64 operand piece as (up to) two 64-row boxes.  K-major (mn = 0):
-// rows r0.. of the map at x = k0; MN-major (mn = 1): columns r0.. of the map
-// at rows k0..  Shared layout: K-major rows at 128 B (8-row groups 1 KB
-// apart); MN-major 64-element halves 8 KB apart, 8-row K groups 1 KB apart.
-// With halves = 1 the second half is not loaded (the block ends within the
-// first 64 rows / columns; the MMA reads don't-care data there, which only
-// reaches output rows / columns the epilogue drops).
-__device__ __forceinline__ void tma_piece(uint32_t dst, const CUtensorMap* map, int mn, int r0, int k0, int z, int w,
-                                          uint32_t bar, int halves) {
+// One operand (all pieces) of a stage.  K-major (mn = 0): rows r0.. of the map at
+// x = k0; MN-major (mn = 1): columns r0.. of the map at rows k0..  With halves = 1
+// the block ends within the first 64 rows / columns: the MMA reads don't-care
+// data beyond, which only reaches output rows / columns the epilogue drops.
+template <int NSPLIT>
+__device__ __forceinline__ void tma_operand(uint32_t dst, const CUtensorMap* key, int mn, int r0, int k0, int z, int w,
+                                            uint32_t bar, int halves, int box) {
+    const uint32_t ps = (uint32_t)piece_rows(mn, halves, box) * 128u;
+    const CUtensorMap* map = key + (!mn && halves == 2 ? 2 : 0);
     if (!mn) {
-        tma_load4(dst, map, k0, r0, z, w, bar);
-        if (halves == 2) tma_load4(dst + 8192, map, k0, r0 + 64, z, w, bar);
+        tma_load5(dst, map, k0, r0, z, w, bar);
+        if (NSPLIT == 3) tma_load5(dst + ps, map + 1, k0, r0, z, w, bar);
     } else {
-        tma_load4(dst, map, r0, k0, z, w, bar);
-        if (halves == 2) tma_load4(dst + 8192, map, r0 + 64, k0, z, w, bar);
+        tma_load5(dst, map, r0, k0, z, w, bar);
+        if (NSPLIT == 3) tma_load5(dst + ps, map + 1, r0, k0, z, w, bar);
+        if (halves == 2) {
+            tma_load5(dst + NSPLIT * ps, map, r0 + 64, k0, z, w, bar);
+            if (NSPLIT == 3) tma_load5(dst + 4 * ps, map + 1, r0 + 64, k0, z, w, bar);
+        }
     }
 }
 
@@ -410,11 +418,12 @@ __device__ __forceinline__ void tma_piece(uint32_t dst, const CUtensorMap* map, 
 // alternately, warp 8 TMA producer (all lanes), warp 9 lane 0 MMA issuer.
 //
 // Bound: not by data.  The producer and the MMA lane are each busy ~1000 cycles
-// per stage with issuing (waits, descriptors, 4 to 12 copies, 6 to 12 MMAs,
+// per stage with issuing (waits, descriptors, copies, 6 to 12 MMAs,
 // commits), whatever the stage holds, so two CTAs share an SM, half of shared
 // and tensor memory each, and issue in parallel (one CTA with everything:
 // K = 24, D = 500, four vectors 20.4 ms, two: 11.6 ms; K = 36, D = 1000
-// 16.4 -> 13.5 ms).
+// 16.4 -> 13.5 ms), and one copy brings all pieces of an operand (two per small
+// stage instead of four: K = 8, D = 64 233 -> 185 us, K = 24 8.5 -> 7.7 ms).
 constexpr int kCtas3 = 2;
 constexpr int kEpiGroups = 2;
 constexpr int kProdWarp3 = 4 * kEpiGroups;
@@ -436,9 +445,11 @@ struct Cfg3 {
 
 // stage record of the TMA kernel (one 8-byte word)
 struct __align__(8) StageMeta3 {
-    uint8_t a_mn, b_mn, neg, flags;  // flags: 1 first stage of a tile, 2 last, 4 no MMA (empty tile), 8 two units
-    uint8_t k16, n16;                // 16-deep K steps holding data; MMA N / 16
-    uint8_t a_lb, swap;              // MN-major A: 2 KB steps between its 64-wide halves; cross terms swapped
+    uint8_t form, flags;  // form: 1 A MN-major, 2 B MN-major, 4 negate A, 8 cross terms swapped
+                          // flags: 1 first stage of a tile, 2 last, 4 no MMA (empty tile), 8 two units
+    uint8_t k16, n16;     // 16-deep K steps holding data; MMA N / 16
+    uint8_t a_ps, b_ps;   // 2 KB steps between the pieces of an operand ...
+    uint8_t a_lb, b_lb;   // ... and between the 64-wide halves of an MN-major one
 };
 
 __device__ __forceinline__ uint32_t idesc_n(int a_mn, int b_mn, int neg, int n) { return idesc_mn(a_mn, b_mn, neg, n, TM); }
@@ -664,7 +675,7 @@ __global__ void __launch_bounds__(THREADS3, kCtas3)
                         }
                         const uint32_t bar = smem_u32(&full_bar[slot]);
                         if (R.flags & 4) {
-                            meta[slot] = StageMeta3{0, 0, 0, 1 | 2 | 4, 0, 0, 0, 0};
+                            meta[slot] = StageMeta3{0, 1 | 2 | 4, 0, 0, 0, 0, 0, 0};
                             mbar_arrive(bar);
                             break;
                         }
@@ -673,25 +684,26 @@ __global__ void __launch_bounds__(THREADS3, kCtas3)
                             break;
                         }
                         const int k0 = st * TK;
-                        meta[slot] = StageMeta3{R.a_mn, R.b_mn, R.neg,
-                                                (uint8_t)(((R.flags & 1) && st == 0 ? 1 : 0) |
-                                                          ((R.flags & 2) && st == nst - 1 ? 2 : 0) | (upst == 2 ? 8 : 0)),
-                                                (uint8_t)((min(TK, R.k - k0) + 15) / 16), R.n16,
-                                                (uint8_t)(R.a_bz > 1 ? R.a_br / 16 : 4), R.swap};
                         // every unit's full barrier completes once per use: a second unit's at once (nobody waits on it)
                         if (upst == 2) mbar_arrive(smem_u32(&full_bar[slot1]));
-                        mbar_arrive_tx(bar, (uint32_t)NSPLIT * 128u * (uint32_t)(R.nA * R.a_bz * R.a_br + R.nB * R.b_br));
-                        const uint32_t ps = (uint32_t)upst * HALF_BYTES;  // bytes between the pieces of an operand
+                        const int abox = R.a_bz * R.a_br;
+                        const int arows = piece_rows(R.a_mn, R.nA, abox), brows = piece_rows(R.b_mn, R.nB, R.b_br);
+                        meta[slot] = StageMeta3{(uint8_t)(R.a_mn | R.b_mn << 1 | R.neg << 2 | R.swap << 3),
+                                                (uint8_t)(((R.flags & 1) && st == 0 ? 1 : 0) |
+                                                          ((R.flags & 2) && st == nst - 1 ? 2 : 0) | (upst == 2 ? 8 : 0)),
+                                                (uint8_t)((min(TK, R.k - k0) + 15) / 16), R.n16, (uint8_t)(arows / 16),
+                                                (uint8_t)(brows / 16),
+                                                // (stacked MN-major operators lie one box apart)
+                                                (uint8_t)(R.a_bz > 1 ? R.a_br / 16 : NSPLIT * arows / 16),
+                                                (uint8_t)(NSPLIT * brows / 16)};
+                        mbar_arrive_tx(bar, (uint32_t)NSPLIT * 128u *
+                                                (uint32_t)(arows * (R.a_mn ? R.nA : 1) + brows * (R.b_mn ? R.nB : 1)));
                         const uint32_t sa = sbase + slot * C::UNIT_BYTES;
                         const uint32_t sb = upst == 2 ? sbase + slot1 * C::UNIT_BYTES : sa + NSPLIT * HALF_BYTES;
-                        const CUtensorMap* am = maps + 3 * R.a_map;
-                        const CUtensorMap* bm = maps + 3 * R.b_map;
-                        const int aw = R.a_pv ? R.v : 0, bw = R.b_pv ? R.v : 0;
-#pragma unroll
-                        for (int pc = 0; pc < NSPLIT; ++pc) {
-                            tma_piece(sa + pc * ps, am + pc, R.a_mn, R.m0, k0, R.a_z, aw, bar, R.nA);
-                            tma_piece(sb + pc * ps, bm + pc, R.b_mn, R.n0, k0, R.b_z, bw, bar, R.nB);
-                        }
+                        tma_operand<NSPLIT>(sa, maps + kMapsPerKey * R.a_map, R.a_mn, R.m0, k0, R.a_z, R.a_pv ? R.v : 0,
+                                            bar, R.nA, abox);
+                        tma_operand<NSPLIT>(sb, maps + kMapsPerKey * R.b_map, R.b_mn, R.n0, k0, R.b_z, R.b_pv ? R.v : 0,
+                                            bar, R.nB, R.b_br);
                         u += upst;
                     }
                 }
@@ -723,19 +735,20 @@ __global__ void __launch_bounds__(THREADS3, kCtas3)
                     const StageMeta3 M = meta[slot];
                     const bool two = (M.flags & 8) != 0;
                     if (!(M.flags & 4)) {
-                        const uint32_t ps = two ? 2u * HALF_BYTES : (uint32_t)HALF_BYTES;
                         const uint32_t sa = sbase + slot * C::UNIT_BYTES;
                         const uint32_t sb = two ? sbase + slot1 * C::UNIT_BYTES : sa + NSPLIT * HALF_BYTES;
-                        const uint32_t id = idesc_n(M.a_mn, M.b_mn, M.neg, 16 * M.n16);
+                        const int a_mn = M.form & 1, b_mn = M.form >> 1 & 1, swap = M.form >> 3 & 1;
+                        const uint32_t aps = M.a_ps * 2048u, bps = M.b_ps * 2048u;
+                        const uint32_t id = idesc_n(a_mn, b_mn, M.form >> 2 & 1, 16 * M.n16);
                         // bits of a descriptor besides its address, and the address step of a 16-deep K step
-                        const uint64_t ab = M.a_mn ? sdesc(0, M.a_lb * 2048u, 1024) : sdesc(0, 16, 1024);
-                        const uint64_t bb = M.b_mn ? sdesc(0, HALF_BYTES, 1024) : sdesc(0, 16, 1024);
-                        const uint32_t ak = M.a_mn ? 2048 : 32, bk = M.b_mn ? 2048 : 32;
+                        const uint64_t ab = a_mn ? sdesc(0, M.a_lb * 2048u, 1024) : sdesc(0, 16, 1024);
+                        const uint64_t bb = b_mn ? sdesc(0, M.b_lb * 2048u, 1024) : sdesc(0, 16, 1024);
+                        const uint32_t ak = a_mn ? 2048 : 32, bk = b_mn ? 2048 : 32;
                         for (int kk = 0; kk < M.k16; ++kk) {
 #pragma unroll
                             for (int pr = 0; pr < Prods<NSPLIT>::N; ++pr) {
-                                const uint32_t a_s = sa + (M.swap ? prod_b(pr) : prod_a(pr)) * ps + kk * ak;
-                                const uint32_t b_s = sb + (M.swap ? prod_a(pr) : prod_b(pr)) * ps + kk * bk;
+                                const uint32_t a_s = sa + (swap ? prod_b(pr) : prod_a(pr)) * aps + kk * ak;
+                                const uint32_t b_s = sb + (swap ? prod_a(pr) : prod_b(pr)) * bps + kk * bk;
                                 const uint32_t acc = ((M.flags & 1) && kk == 0 && pr == 0) ? 0u : 1u;
                                 mma_bf16(dt, ab | ((a_s & 0x3FFFFu) >> 4), bb | ((b_s & 0x3FFFFu) >> 4), id, acc);
                             }
@@ -1084,24 +1097,31 @@ EncodeTiledFn encode_fn() {
 }  // namespace
 
 void MapTable::encode_upload(const TcBufs& tb, int nsplit, cudaStream_t st) {
-    const size_t n = 3 * keys.size();
+    const size_t n = kMapsPerKey * keys.size();
     std::vector<CUtensorMap> h(std::max<size_t>(n, 1));
     EncodeTiledFn fn = encode_fn();
     for (size_t i = 0; i < keys.size(); ++i) {
         const MapKey& k = keys[i];
-        for (int pc = 0; pc < 3; ++pc) {
-            const __nv_bfloat16* base =
-                pc == 0 ? tb.hi[k.buf] : (pc == 1 ? tb.lo[k.buf] : (tb.lo[k.buf] ? tb.lo[k.buf] + tb.pstride[k.buf] : nullptr));
-            if (pc >= nsplit || !base) {  // unused piece: a copy of the hi map
-                h[3 * i + pc] = h[3 * i];
+        for (int m = 0; m < kMapsPerKey; ++m) {
+            const bool tall = m >= 2, rest = m & 1;
+            if ((tall && (k.rows <= 64 || k.bz > 1)) || (rest && nsplit != 3)) {  // unused: a copy of the first map
+                h[kMapsPerKey * i + m] = h[kMapsPerKey * i];
                 continue;
             }
-            DMRG_REQUIRE(base != nullptr, DMRG_EINVAL, "tensor map over an unset buffer");
-            const cuuint64_t dims[4] = {(cuuint64_t)k.cols, (cuuint64_t)k.rows, (cuuint64_t)k.nz, (cuuint64_t)k.nv};
-            const cuuint64_t strides[3] = {(cuuint64_t)k.ld * 2, (cuuint64_t)k.zstride * 2, (cuuint64_t)k.vstride * 2};
-            const cuuint32_t box[4] = {64, (cuuint32_t)box_rows(k.rows), (cuuint32_t)k.bz, 1};
-            const cuuint32_t estr[4] = {1, 1, 1, 1};
-            const CUresult r = fn(&h[3 * i + pc], CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, (void*)(base + k.off), dims,
+            const __nv_bfloat16 *hi = tb.hi[k.buf], *lo = tb.lo[k.buf];
+            const __nv_bfloat16* base = rest ? lo : hi;
+            const int pieces = rest || nsplit == 2 ? 2 : 1;
+            DMRG_REQUIRE(base && (nsplit == 1 || lo), DMRG_EINVAL, "tensor map over an unset buffer");
+            const int64_t pst = pieces == 1 ? k.vstride : (rest ? tb.pstride[k.buf] : (int64_t)(lo - hi));
+            DMRG_REQUIRE(pst > 0 && pst % 8 == 0 && pst * 2 < (1LL << 40), DMRG_EINVAL, "pieces not in one allocation");
+            const cuuint64_t dims[5] = {(cuuint64_t)k.cols, (cuuint64_t)k.rows, (cuuint64_t)k.nz, (cuuint64_t)k.nv,
+                                        (cuuint64_t)pieces};
+            const cuuint64_t strides[4] = {(cuuint64_t)k.ld * 2, (cuuint64_t)k.zstride * 2, (cuuint64_t)k.vstride * 2,
+                                           (cuuint64_t)pst * 2};
+            const cuuint32_t box[5] = {64, tall ? 128u : (cuuint32_t)box_rows(k.rows), (cuuint32_t)k.bz, 1,
+                                       (cuuint32_t)pieces};
+            const cuuint32_t estr[5] = {1, 1, 1, 1, 1};
+            const CUresult r = fn(&h[kMapsPerKey * i + m], CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 5, (void*)(base + k.off), dims,
                                   strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
                                   CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
             DMRG_REQUIRE(r == CUDA_SUCCESS, DMRG_ECUDA, "cuTensorMapEncodeTiled failed (" + std::to_string((int)r) + ")");

@@ -296,26 +296,20 @@ Plan::~Plan() {
                 } catch (...) {
                 }
                 if (b->d) free(b->d, b->n);
-                free_bf16(b->h, b->n);
-                free_lo(b->l, b->n);
+                free_pieces(b->h, b->l, b->n);
             }
     tier_destroy(*this);
-    free_bf16(s_hi, n_spc);
-    free_lo(s_lo, n_spc);
-    free_bf16(ps_hi, n_ppc);
-    free_lo(ps_lo, n_ppc);
-    free_bf16(id_hi, (int64_t)id_n * id_n);
-    free_lo(id_lo, (int64_t)id_n * id_n);
-    free_bf16(w_hi, n_wpc);
-    free_lo(w_lo, n_wpc);
+    free_pieces(s_hi, s_lo, n_spc);
+    free_pieces(ps_hi, ps_lo, n_ppc);
+    free_pieces(id_hi, id_lo, (int64_t)id_n * id_n);
+    free_pieces(w_hi, w_lo, n_wpc);
     if (d_psi_jobs) cudaFree(d_psi_jobs);
     mlp.release();
     if (d_mlp_feat) cudaFree(d_mlp_feat);
     if (d_ctr) cudaFree(d_ctr);
     sigma_tc.release();
     free(interm.d, interm.n);
-    free_bf16(interm.h, interm.n);
-    free_lo(interm.l, interm.n);
+    free_pieces(interm.h, interm.l, interm.n);
     free(d_scratch, n_scratch);
     free(d_ident, (int64_t)ident_n * ident_n);
     free(d_wcoef, n_wcoef);

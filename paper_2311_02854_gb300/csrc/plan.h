@@ -274,8 +274,18 @@ struct Plan {
     void free(double*& p, int64_t n);
     __nv_bfloat16* alloc_bf16(int64_t n);
     void free_bf16(__nv_bfloat16*& p, int64_t n);
-    __nv_bfloat16* alloc_lo(int64_t n) { return alloc_bf16(lo_pieces() * n); }
-    void free_lo(__nv_bfloat16*& p, int64_t n) { free_bf16(p, lo_pieces() * n); }
+    // the pieces of n elements in one allocation, hi first (so that one tensor map
+    // covers both: its piece stride is the same wherever the allocation lies)
+    int64_t pieces_lo_at(int64_t n) const { return round_up(n * 2, 256) / 2; }
+    int64_t pieces_len(int64_t n) const { return pieces_lo_at(n) + round_up(lo_pieces() * n * 2, 256) / 2; }
+    void alloc_pieces(int64_t n, __nv_bfloat16*& hi, __nv_bfloat16*& lo) {
+        hi = n > 0 ? alloc_bf16(pieces_len(n)) : nullptr;
+        lo = hi ? hi + pieces_lo_at(n) : nullptr;
+    }
+    void free_pieces(__nv_bfloat16*& hi, __nv_bfloat16*& lo, int64_t n) {
+        free_bf16(hi, pieces_len(n));
+        lo = nullptr;
+    }
     // piece 2 of a lo array of n elements per piece (null unless three pieces)
     __nv_bfloat16* lo2(__nv_bfloat16* lo, int64_t n) const { return (nsplit == 3 && lo) ? lo + n : nullptr; }
     void check_device_error();

@@ -47,10 +47,12 @@ void tc_prepare(int nsplit);
 // TMA-staged variant: every operand is addressed through a tensor map.
 // ---------------------------------------------------------------------------
 
-// A segment whose operands are read through tensor maps.  Each map is 4-D over
-// one bf16 piece: x = column, y = row, z = operator row of a stored family
-// (0 otherwise), w = vector index (for per-vector buffers).  The maps of a key
-// come in piece order (hi, lo, lo2) at 3 * key + piece.
+// A segment whose operands are read through tensor maps.  Each map is 5-D:
+// x = column, y = row, z = operator row of a stored family (0 otherwise), w =
+// vector index (for per-vector buffers), then the bf16 piece, so that one copy
+// brings both pieces.  A key has kMapsPerKey maps: boxes of up to 64 rows and, at
+// 2, of 128 rows; with three pieces hi alone and, one further, (lo, lo2).
+constexpr int kMapsPerKey = 4;
 struct TSeg {
     int32_t a_map, b_map;  // map keys
     int32_t a_z, b_z;      // z coordinates
@@ -118,7 +120,7 @@ struct MapTable {
     const void* enc_ptr[kMaxBufs][3] = {};  // piece pointers the device maps were encoded with
     int get(const MapKey& k);  // validates alignment; returns the key index
     bool stale(const TcBufs& tb) const;  // a piece pointer moved since the last encode
-    // encode 3 maps per key (pieces hi, lo, lo + pstride) and copy them to the device
+    // encode the maps of every key and copy them to the device
     void encode_upload(const TcBufs& tb, int nsplit, cudaStream_t st);
     void clear() {
         keys.clear();

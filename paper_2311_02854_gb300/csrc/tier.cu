@@ -59,8 +59,7 @@ char* host_take(Plan& P, int64_t n, int64_t& cap) {
 
 void free_dev(Plan& P, Block& b) {
     P.free(b.d, b.n);
-    P.free_bf16(b.h, b.n);
-    P.free_lo(b.l, b.n);
+    P.free_pieces(b.h, b.l, b.n);
     b.dev = false;
     b.evicting = false;
 }
@@ -132,8 +131,7 @@ void tier_in(Plan& P, Block& b) {
     if (b.dev) return;
     DMRG_REQUIRE(b.host_valid, DMRG_EINVAL, "environment block has neither a device nor a host copy");
     if (b.has_d) b.d = P.alloc(b.n);
-    if (b.has_h) b.h = P.alloc_bf16(b.n);
-    if (b.has_l) b.l = P.alloc_lo(b.n);
+    if (b.has_h) P.alloc_pieces(b.n, b.h, b.l);  // (a block has both pieces or none)
     b.dev = true;
     cudaStream_t cs = copy_stream(P);
     // the eviction's copy wrote the host buffer (long done: its device arrays were freed after it)
