@@ -401,15 +401,18 @@ Products share_products(size_t ni, const Get& get) {
     Products pr;
     pr.stack.assign(ni, -1);
     pr.pos.assign(ni, 0);
-    const size_t np = ni < 4096 ? 1 : 16;  // partitions of the keys
-    std::vector<uint64_t> hash(ni, 0);     // 0: no product
-    parallel_for((ni + 4095) / 4096, [&](size_t b) {
-        for (size_t q = b * 4096; q < std::min(ni, (b + 1) * 4096); ++q) {
-            ProdKey k{};
-            int z, most;
-            if (get(q, k, z, most)) hash[q] = k.hash() | 1;
-        }
-    });
+    // partitions of the keys, one per host thread; short lists are done at once
+    // (starting the threads takes as long)
+    const size_t np = ni < 16384 ? 1 : 16;
+    std::vector<uint64_t> hash(np > 1 ? ni : 0, 0);  // 0: no product
+    if (np > 1)
+        parallel_for((ni + 8191) / 8192, [&](size_t b) {
+            for (size_t q = b * 8192; q < std::min(ni, (b + 1) * 8192); ++q) {
+                ProdKey k{};
+                int z, most;
+                if (get(q, k, z, most)) hash[q] = k.hash() | 1;
+            }
+        });
     std::vector<std::vector<ProdStack>> st(np);
     parallel_for(np, [&](size_t pt) {
         struct KeyHash {
@@ -419,10 +422,10 @@ Products share_products(size_t ni, const Get& get) {
         std::vector<std::vector<std::pair<int32_t, uint32_t>>> lists;  // per key: (z, item)
         std::vector<int> mosts;
         for (size_t q = 0; q < ni; ++q) {
-            if (!hash[q] || (hash[q] >> 40) % np != pt) continue;
+            if (np > 1 && (!hash[q] || (hash[q] >> 40) % np != pt)) continue;
             ProdKey k{};
             int z = 0, most = 1;
-            get(q, k, z, most);
+            if (!get(q, k, z, most)) continue;
             auto f = idx.emplace(k, (int)lists.size());
             if (f.second) {
                 lists.emplace_back();
@@ -450,7 +453,7 @@ Products share_products(size_t ni, const Get& get) {
         pr.stacks.insert(pr.stacks.end(), st[pt].begin(), st[pt].end());
     }
     for (size_t q = 0; q < ni; ++q)
-        if (pr.stack[q] >= 0) pr.stack[q] += first[(hash[q] >> 40) % np];
+        if (np > 1 && pr.stack[q] >= 0) pr.stack[q] += first[(hash[q] >> 40) % np];
     return pr;
 }
 
