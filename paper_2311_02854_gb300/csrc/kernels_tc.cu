@@ -392,25 +392,19 @@ __device__ __forceinline__ void tma_load5(uint32_t dst, const CUtensorMap* map, 
 // columns (halves = 2) has two boxes, every piece's halves NSPLIT * rows apart.
 __device__ __forceinline__ int piece_rows(int mn, int halves, int box) { return !mn && halves == 2 ? 128 : box; }
 
-// One operand (all pieces) of a stage.  K-major (mn = 0): rows r0.. of the map at
-// x = k0; MN-major (mn = 1): columns r0.. of the map at rows k0..  With halves = 1
-// the block ends within the first 64 rows / columns: the MMA reads don't-care
-// data beyond, which only reaches output rows / columns the epilogue drops.
+// One operand (all pieces) of a stage from coordinates (x, y) of its map.  K-major
+// (mn = 0): rows of the block at x = k0; MN-major (mn = 1): its columns at rows k0..
+// (two: 128 of them).  A block that ends within the first 64 rows / columns brings
+// no more: the MMA reads don't-care data beyond, which only reaches output rows /
+// columns the epilogue drops.
 template <int NSPLIT>
-__device__ __forceinline__ void tma_operand(uint32_t dst, const CUtensorMap* key, int mn, int r0, int k0, int z, int w,
-                                            uint32_t bar, int halves, int box) {
-    const uint32_t ps = (uint32_t)piece_rows(mn, halves, box) * 128u;
-    const CUtensorMap* map = key + (!mn && halves == 2 ? 2 : 0);
-    if (!mn) {
-        tma_load5(dst, map, k0, r0, z, w, bar);
-        if (NSPLIT == 3) tma_load5(dst + ps, map + 1, k0, r0, z, w, bar);
-    } else {
-        tma_load5(dst, map, r0, k0, z, w, bar);
-        if (NSPLIT == 3) tma_load5(dst + ps, map + 1, r0, k0, z, w, bar);
-        if (halves == 2) {
-            tma_load5(dst + NSPLIT * ps, map, r0 + 64, k0, z, w, bar);
-            if (NSPLIT == 3) tma_load5(dst + 4 * ps, map + 1, r0 + 64, k0, z, w, bar);
-        }
+__device__ __forceinline__ void tma_operand(uint32_t dst, const CUtensorMap* map, int x, int y, int z, int w, uint32_t bar,
+                                            uint32_t ps, bool two) {
+    tma_load5(dst, map, x, y, z, w, bar);
+    if (NSPLIT == 3) tma_load5(dst + ps, map + 1, x, y, z, w, bar);
+    if (two) {
+        tma_load5(dst + NSPLIT * ps, map, x + 64, y, z, w, bar);
+        if (NSPLIT == 3) tma_load5(dst + 4 * ps, map + 1, x + 64, y, z, w, bar);
     }
 }
 
@@ -424,32 +418,37 @@ __device__ __forceinline__ void tma_operand(uint32_t dst, const CUtensorMap* key
 // K = 24, D = 500, four vectors 20.4 ms, two: 11.6 ms; K = 36, D = 1000
 // 16.4 -> 13.5 ms), and one copy brings all pieces of an operand (two per small
 // stage instead of four: K = 8, D = 64 233 -> 185 us, K = 24 8.5 -> 7.7 ms).
+// Large sectors come near what L2 hands to the SMs (K = 14 and K = 36: 8 to 10
+// TB/s of operands while it runs), small ones stay with the issuing lanes.
 constexpr int kCtas3 = 2;
 constexpr int kEpiGroups = 2;
 constexpr int kProdWarp3 = 4 * kEpiGroups;
 constexpr int THREADS3 = (kProdWarp3 + 2) * 32;
-constexpr int HALF_BYTES = 64 * TK * 2;  // one 64 x 64 bf16 box
 constexpr uint32_t kAcc = 2;             // accumulators in tensor memory (2 x 128 of the 512 columns)
 
-// Shared memory is a ring of UNITS units.  A stage whose operands both end
-// within 64 rows / columns (most stages of a sigma: sectors are small) takes
-// one unit, [A pieces | B pieces] of 8 KB each; any other stage takes two, one
-// per operand, with 16 KB per piece (BF16X3), so three small stages are in
-// flight per CTA where a fixed 64 KB slot would allow one.
+// Shared memory is a ring of UNITS units of 2 KB (16 rows of 128 bytes).  A stage
+// takes the units that its boxes fill, [A pieces | B pieces] in one stretch, and
+// up to SLOTS stages are in flight.  With fixed units of 32 KB (one for a stage
+// within 64 x 64, else two) a stage of 48 x 48 or of 128 x 16 took 32 or 64 KB
+// instead of 24 or 36, and two or three of them filled the ring: K = 14, D = 600
+// 1.81 -> 1.52 ms, K = 36, D = 1000 11.0 -> 10.0, K = 24, D = 500, four vectors
+// 7.7 -> 7.35.  (Tiny stages, which never filled it, pay for the bookkeeping:
+// K = 8, D = 64 189 -> 197 us.  More than four slots gave nothing more there.)
 template <int NSPLIT>
 struct Cfg3 {
-    static constexpr int UNITS = (NSPLIT == 1) ? 6 : (NSPLIT == 2 ? 3 : 2);
-    static constexpr int UNIT_BYTES = 2 * NSPLIT * HALF_BYTES;
-    static constexpr int SMEM = UNITS * UNIT_BYTES + 1024;
+    static constexpr int UNITS = 55;
+    static constexpr int SLOTS = 16;
+    static constexpr int SMEM = UNITS * 2048 + 1024;
 };
 
 // stage record of the TMA kernel (one 8-byte word)
 struct __align__(8) StageMeta3 {
-    uint8_t form, flags;  // form: 1 A MN-major, 2 B MN-major, 4 negate A, 8 cross terms swapped
-                          // flags: 1 first stage of a tile, 2 last, 4 no MMA (empty tile), 8 two units
-    uint8_t k16, n16;     // 16-deep K steps holding data; MMA N / 16
-    uint8_t a_ps, b_ps;   // 2 KB steps between the pieces of an operand ...
-    uint8_t a_lb, b_lb;   // ... and between the 64-wide halves of an MN-major one
+    uint8_t form;        // 1 A MN-major, 2 B MN-major, 4 negate A, 8 cross terms swapped,
+                         // 16 first stage of a tile, 32 last, 64 no MMA (empty tile)
+    uint8_t kn;          // 16-deep K steps holding data | 16 * (MMA N / 16)
+    uint8_t a_ps, b_ps;  // units between the pieces of an operand ...
+    uint8_t a_lb, b_lb;  // ... and between the 64-wide halves of an MN-major one
+    uint8_t a_at, b_at;  // first unit of each operand
 };
 
 __device__ __forceinline__ uint32_t idesc_n(int a_mn, int b_mn, int neg, int n) { return idesc_mn(a_mn, b_mn, neg, n, TM); }
@@ -549,17 +548,17 @@ __global__ void __launch_bounds__(THREADS3, kCtas3)
     tc_tma_kernel(const Tile* __restrict__ tiles, int ntiles, int nvec, const TSeg* __restrict__ segs,
                   const CUtensorMap* __restrict__ maps, int single, TcBufs B) {
     using C = Cfg3<NSPLIT>;
-    constexpr uint32_t U = C::UNITS;
+    constexpr uint32_t U = C::UNITS, SL = C::SLOTS;
     extern __shared__ uint8_t smem_raw[];
-    __shared__ __align__(8) uint64_t full_bar[U], empty_bar[U], tfull_bar[kAcc], tempty_bar[kAcc], drain_bar;
-    __shared__ StageMeta3 meta[U];
+    __shared__ __align__(8) uint64_t full_bar[SL], empty_bar[SL], tfull_bar[kAcc], tempty_bar[kAcc], drain_bar;
+    __shared__ StageMeta3 meta[SL];
     __shared__ uint32_t tmem_base_s;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const uint32_t sbase = (smem_u32(smem_raw) + 1023u) & ~1023u;
 
     if (warp == 0) tmem_alloc(smem_u32(&tmem_base_s), kAcc * TMEM_COLS);
     if (tid == 0) {
-        for (uint32_t s = 0; s < U; ++s) {
+        for (uint32_t s = 0; s < SL; ++s) {
             mbar_init(smem_u32(&full_bar[s]), 1);
             mbar_init(smem_u32(&empty_bar[s]), 1);
         }
@@ -645,71 +644,83 @@ __global__ void __launch_bounds__(THREADS3, kCtas3)
             r.n16 = (uint8_t)((ncol + 15) / 16);
             return r;
         };
-        uint32_t q = 0;  // units handed out so far
+        // The same in all lanes: stages issued, stages known to be free again, units
+        // handed out (or skipped) and given back, and the ring position of head.
+        // Lane i holds where the stage in slot i ends.
+        uint32_t si = 0, tail = 0, head = 0, back = 0, pos = 0, end = 0;
         ProdRec next = fetch();
         while (!failed) {
             const ProdRec R = next;
             const unsigned live = __ballot_sync(0xffffffffu, R.valid);
             if (!live) break;
             next = fetch();
-            const int upst = (R.nA == 2 || R.nB == 2 || R.a_bz * R.a_br > 64) ? 2 : 1;
-            const int nst = !R.valid ? 0 : ((R.flags & 4) ? 1 : (R.k + TK - 1) / TK);
-            uint32_t sum = (uint32_t)(nst * ((R.flags & 4) ? 1 : upst));
-            const uint32_t mine = sum;
-#pragma unroll
-            for (int o = 1; o < 32; o <<= 1) {
-                const uint32_t x = __shfl_up_sync(0xffffffffu, sum, o);
-                if (lane >= o) sum += x;
-            }
-            const uint32_t q0 = q + sum - mine;
-            q += __shfl_sync(0xffffffffu, sum, 31);
+            const bool none = (R.flags & 4) != 0;
+            const int nst = !R.valid ? 0 : (none ? 1 : (R.k + TK - 1) / TK);
+            const int abox = R.a_bz * R.a_br;
+            const int arows = piece_rows(R.a_mn, R.nA, abox), brows = piece_rows(R.b_mn, R.nB, R.b_br);
+            const int au = NSPLIT * arows * (R.a_mn ? R.nA : 1) / 16, bu = NSPLIT * brows * (R.b_mn ? R.nB : 1) / 16;
+            const uint32_t n = none ? 0 : au + bu;
+            // the MMAs read 128 rows of A whatever the box holds: those units lie in the ring too
+            // (but for stacked MN-major operators, whose two boxes are those 128 rows)
+            const int areach = !R.a_mn ? (NSPLIT - 1) * arows / 16 + 8 : (R.a_bz > 1 ? au : 2 * NSPLIT * arows / 16);
+            const uint32_t reach = none ? 0 : max((int)n, areach);
+            const uint32_t need_l = n | reach << 8 | (uint32_t)nst << 16;
+            // this segment's StageMeta3 but for the flags of first and last, the K steps
+            // of its last stage and the ring position (the record is two words)
+            const uint32_t form = R.a_mn | R.b_mn << 1 | R.neg << 2 | R.swap << 3;
+            const uint32_t m0 = form | (uint32_t)(4 | R.n16 << 4) << 8 | (uint32_t)arows / 16 << 16 | (uint32_t)brows / 16 << 24;
+            const uint32_t a_lb = R.a_bz > 1 ? R.a_br / 16 : NSPLIT * arows / 16;  // (stacked MN-major: one box apart)
+            const uint32_t m1 = a_lb | (uint32_t)(NSPLIT * brows / 16) << 8 | (uint32_t)au << 24;
+            const uint32_t klast = (uint32_t)(4 - (R.k - TK * (nst - 1) + 15) / 16) << 8;
+            const CUtensorMap* am = maps + kMapsPerKey * R.a_map + (!R.a_mn && R.nA == 2 ? 2 : 0);
+            const CUtensorMap* bm = maps + kMapsPerKey * R.b_map + (!R.b_mn && R.nB == 2 ? 2 : 0);
+            const int av = R.a_pv ? R.v : 0, bv = R.b_pv ? R.v : 0;
+            const bool a2 = R.a_mn && R.nA == 2, b2 = R.b_mn && R.nB == 2;
             const int nl = __popc(live);  // the valid lanes are the first nl
-            for (int l = 0; l < nl; ++l) {
-                if (lane == l) {
-                    uint32_t u = q0;
-                    for (int st = 0; st < nst; ++st) {
-                        const uint32_t slot = u % U, slot1 = (u + 1) % U;
-                        if (u >= U && !mbar_wait(smem_u32(&empty_bar[slot]), ((u / U) - 1) & 1u)) {
-                            failed = true;
-                            break;
-                        }
-                        const uint32_t bar = smem_u32(&full_bar[slot]);
-                        if (R.flags & 4) {
-                            meta[slot] = StageMeta3{0, 1 | 2 | 4, 0, 0, 0, 0, 0, 0};
-                            mbar_arrive(bar);
-                            break;
-                        }
-                        if (upst == 2 && u + 1 >= U && !mbar_wait(smem_u32(&empty_bar[slot1]), (((u + 1) / U) - 1) & 1u)) {
-                            failed = true;
-                            break;
-                        }
-                        const int k0 = st * TK;
-                        // every unit's full barrier completes once per use: a second unit's at once (nobody waits on it)
-                        if (upst == 2) mbar_arrive(smem_u32(&full_bar[slot1]));
-                        const int abox = R.a_bz * R.a_br;
-                        const int arows = piece_rows(R.a_mn, R.nA, abox), brows = piece_rows(R.b_mn, R.nB, R.b_br);
-                        meta[slot] = StageMeta3{(uint8_t)(R.a_mn | R.b_mn << 1 | R.neg << 2 | R.swap << 3),
-                                                (uint8_t)(((R.flags & 1) && st == 0 ? 1 : 0) |
-                                                          ((R.flags & 2) && st == nst - 1 ? 2 : 0) | (upst == 2 ? 8 : 0)),
-                                                (uint8_t)((min(TK, R.k - k0) + 15) / 16), R.n16, (uint8_t)(arows / 16),
-                                                (uint8_t)(brows / 16),
-                                                // (stacked MN-major operators lie one box apart)
-                                                (uint8_t)(R.a_bz > 1 ? R.a_br / 16 : NSPLIT * arows / 16),
-                                                (uint8_t)(NSPLIT * brows / 16)};
-                        mbar_arrive_tx(bar, (uint32_t)NSPLIT * 128u *
-                                                (uint32_t)(arows * (R.a_mn ? R.nA : 1) + brows * (R.b_mn ? R.nB : 1)));
-                        const uint32_t sa = sbase + slot * C::UNIT_BYTES;
-                        const uint32_t sb = upst == 2 ? sbase + slot1 * C::UNIT_BYTES : sa + NSPLIT * HALF_BYTES;
-                        tma_operand<NSPLIT>(sa, maps + kMapsPerKey * R.a_map, R.a_mn, R.m0, k0, R.a_z, R.a_pv ? R.v : 0,
-                                            bar, R.nA, abox);
-                        tma_operand<NSPLIT>(sb, maps + kMapsPerKey * R.b_map, R.b_mn, R.n0, k0, R.b_z, R.b_pv ? R.v : 0,
-                                            bar, R.nB, R.b_br);
-                        u += upst;
+            for (int l = 0; l < nl && !failed; ++l) {
+                const uint32_t w = __shfl_sync(0xffffffffu, need_l, l), un = w & 255u, ur = w >> 8 & 255u, us = w >> 16;
+                for (uint32_t st = 0; st < us; ++st) {
+                    if (pos + ur > U) {
+                        head += U - pos;
+                        pos = 0;
                     }
-                }
-                if (__any_sync(0xffffffffu, failed)) {
-                    failed = true;
-                    break;
+                    // units before head + un - U must be free (with no stage in flight all are)
+                    while (si - tail >= SL || (tail != si && (int)(back + U - un - head) < 0)) {
+                        const uint32_t t = tail % SL;
+                        if (!__all_sync(0xffffffffu, mbar_wait(smem_u32(&empty_bar[t]), (tail / SL) & 1u))) {
+                            failed = true;
+                            break;
+                        }
+                        back = __shfl_sync(0xffffffffu, end, t);
+                        ++tail;
+                    }
+                    if (failed) break;
+                    const uint32_t slot = si % SL;
+                    if (lane == l) {
+                        const uint32_t bar = smem_u32(&full_bar[slot]);
+                        uint2* rec = reinterpret_cast<uint2*>(&meta[slot]);
+                        if (none) {
+                            *rec = make_uint2(16 | 32 | 64, 0);
+                            mbar_arrive(bar);
+                        } else {
+                            const bool last = st + 1 == us;
+                            *rec = make_uint2(m0 + ((R.flags & 1) && st == 0 ? 16 : 0) + ((R.flags & 2) && last ? 32 : 0) -
+                                                  (last ? klast : 0),
+                                              m1 + pos * 0x01010000u);
+                            mbar_arrive_tx(bar, 2048u * n);
+                            const uint32_t sa = sbase + 2048u * pos;
+                            const int k0 = (int)st * TK;
+                            tma_operand<NSPLIT>(sa, am, R.a_mn ? R.m0 : k0, R.a_mn ? k0 : R.m0, R.a_z, av, bar,
+                                                128u * arows, a2);
+                            tma_operand<NSPLIT>(sa + 2048u * au, bm, R.b_mn ? R.n0 : k0, R.b_mn ? k0 : R.n0, R.b_z, bv, bar,
+                                                128u * brows, b2);
+                        }
+                    }
+                    __syncwarp();
+                    head += un;
+                    pos += un;
+                    if (lane == (int)slot) end = head;
+                    ++si;
                 }
             }
         }
@@ -726,38 +737,35 @@ __global__ void __launch_bounds__(THREADS3, kCtas3)
                 tc_fence_after();
                 const uint32_t dt = tmem + buf * TMEM_COLS;
                 for (;;) {
-                    const uint32_t slot = q % U, slot1 = (q + 1) % U;
-                    if (!mbar_wait(smem_u32(&full_bar[slot]), (q / U) & 1u)) {
+                    const uint32_t slot = q % SL;
+                    if (!mbar_wait(smem_u32(&full_bar[slot]), (q / SL) & 1u)) {
                         failed = true;
                         break;
                     }
                     tc_fence_after();
                     const StageMeta3 M = meta[slot];
-                    const bool two = (M.flags & 8) != 0;
-                    if (!(M.flags & 4)) {
-                        const uint32_t sa = sbase + slot * C::UNIT_BYTES;
-                        const uint32_t sb = two ? sbase + slot1 * C::UNIT_BYTES : sa + NSPLIT * HALF_BYTES;
+                    if (!(M.form & 64)) {
+                        const uint32_t sa = sbase + M.a_at * 2048u, sb = sbase + M.b_at * 2048u;
                         const int a_mn = M.form & 1, b_mn = M.form >> 1 & 1, swap = M.form >> 3 & 1;
                         const uint32_t aps = M.a_ps * 2048u, bps = M.b_ps * 2048u;
-                        const uint32_t id = idesc_n(a_mn, b_mn, M.form >> 2 & 1, 16 * M.n16);
+                        const uint32_t id = idesc_n(a_mn, b_mn, M.form >> 2 & 1, M.kn & 0xF0);
                         // bits of a descriptor besides its address, and the address step of a 16-deep K step
                         const uint64_t ab = a_mn ? sdesc(0, M.a_lb * 2048u, 1024) : sdesc(0, 16, 1024);
                         const uint64_t bb = b_mn ? sdesc(0, M.b_lb * 2048u, 1024) : sdesc(0, 16, 1024);
                         const uint32_t ak = a_mn ? 2048 : 32, bk = b_mn ? 2048 : 32;
-                        for (int kk = 0; kk < M.k16; ++kk) {
+                        for (int kk = 0; kk < (M.kn & 15); ++kk) {
 #pragma unroll
                             for (int pr = 0; pr < Prods<NSPLIT>::N; ++pr) {
                                 const uint32_t a_s = sa + (swap ? prod_b(pr) : prod_a(pr)) * aps + kk * ak;
                                 const uint32_t b_s = sb + (swap ? prod_a(pr) : prod_b(pr)) * bps + kk * bk;
-                                const uint32_t acc = ((M.flags & 1) && kk == 0 && pr == 0) ? 0u : 1u;
+                                const uint32_t acc = ((M.form & 16) && kk == 0 && pr == 0) ? 0u : 1u;
                                 mma_bf16(dt, ab | ((a_s & 0x3FFFFu) >> 4), bb | ((b_s & 0x3FFFFu) >> 4), id, acc);
                             }
                         }
                     }
                     mma_commit(smem_u32(&empty_bar[slot]));
-                    if (two) mma_commit(smem_u32(&empty_bar[slot1]));
-                    q += two ? 2 : 1;
-                    if (M.flags & 2) break;
+                    ++q;
+                    if (M.form & 32) break;
                 }
                 if (failed) break;
                 mma_commit(smem_u32(&tfull_bar[buf]));
