@@ -65,12 +65,12 @@ struct WorkList {
     size_t cap_tiles = 0, cap_segs = 0;
     double flops = 0.0;
     bool rank1 = false;  // every segment has K = 1 (run by the rank-1 kernel)
-    // FP64 units, set by upload: part of a tile per warp (16, 32, or 64 for four
+    // FP64 units, set by arrange: part of a tile per warp (16, 32, or 64 for four
     // parts of 32 per tile); CTAs that share a part's term sum (0: one warp does
     // it), by K-blocks of every segment (byk) or by segments
     int part = 64, split = 0;
     bool byk = false;
-    bool single = false;  // every tile has one segment (FP64-accurate tensor-core engine, set by upload)
+    bool single = false;  // every tile has one segment (FP64-accurate tensor-core engine, set by arrange)
     // tile shape of add_block when nonzero (rows, columns); 128 x 64 lists run on
     // the FP64-accurate tensor-core engine (launch_seg_gemm_f64 dispatches on it)
     int tile_m = 0, tile_n = 0;
@@ -87,6 +87,7 @@ struct WorkList {
     // c_off on) whose first factor is `s`'s A, astride elements apart; product i in
     // accumulator rows i * 16 * sb ... (16 * sb >= m, 16 * sb * sn <= 128)
     void add_stack(int64_t c_off, int c_buf, int m, int n, int ldc, const Seg& s, int64_t astride, int sn, int sb);
+    void arrange();  // order of the tiles and the split above
     void upload(cudaStream_t st);
     void release();
 };
@@ -104,11 +105,8 @@ int* oz_error_word();
 bool oz_take_error(cudaStream_t st);
 // FP64 grouped GEMM with the work list in a static device array (noalloc.cu);
 // a, b, c as buffers 0, 1, 2 of the work list
-void grouped_gemm_f64_noalloc(const WorkList& host_wl, const double* a, const double* b, double* c, cudaStream_t st);
+void grouped_gemm_f64_noalloc(WorkList& host_wl, const double* a, const double* b, double* c, cudaStream_t st);
 int64_t noalloc_scratch_bytes();
-// the same kernel on device tile / segment lists owned by the caller (one vector)
-void launch_seg_gemm_f64_lists(const Tile* d_tiles, int64_t ntiles, const Seg* d_segs, const BufTable& bt,
-                               cudaStream_t st);
 
 // --- small FP64 kernels (Davidson / decimation) ---------------------------
 // out[i] = sum_k X[i*ldx + k] * y[k], i < m   (deterministic two-pass)

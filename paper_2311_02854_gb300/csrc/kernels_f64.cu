@@ -96,7 +96,7 @@ namespace {
 constexpr int kSplitWarps = 4;  // warps of a CTA that share a part's term sum (FP64 units)
 }
 
-void WorkList::upload(cudaStream_t st) {
+void WorkList::arrange() {
     // work of a tile: 64-deep (tensor-core engine: oz_stage_depth) K steps, for the
     // FP64 units times its 8 x 8 groups
     const bool oz = tile_m == oz_tile_rows();
@@ -153,6 +153,10 @@ void WorkList::upload(cudaStream_t st) {
         for (size_t i = 0; i < tiles.size(); ++i) sorted[pos[(size_t)(maxn - cost[i])]++] = tiles[i];
         tiles.swap(sorted);
     }
+}
+
+void WorkList::upload(cudaStream_t st) {
+    arrange();
     if (tiles.size() > cap_tiles) {
         if (d_tiles) cudaFree(d_tiles);
         cap_tiles = tiles.size() + tiles.size() / 4 + 16;
@@ -501,16 +505,6 @@ void launch_seg_gemm_f64(const WorkList& w, const BufTable& bt, int nvec, cudaSt
         } else {
             (tiny ? seg_gemm_f64_kernel<2, 4> : seg_gemm_f64_kernel<4, 2>)<<<grid, 32, 0, st>>>(tl, subs, w.d_segs, bt);
         }
-        ++launch_counter();
-    }
-    DMRG_CHECK_CUDA(cudaGetLastError());
-}
-
-void launch_seg_gemm_f64_lists(const Tile* d_tiles, int64_t ntiles, const Seg* d_segs, const BufTable& bt,
-                               cudaStream_t st) {
-    const int64_t maxt = 2147483647LL / 4;
-    for (int64_t t0 = 0; t0 < ntiles; t0 += maxt) {
-        seg_gemm_f64_kernel<4, 2><<<(unsigned)(4 * std::min(ntiles - t0, maxt)), 32, 0, st>>>(d_tiles + t0, 4, d_segs, bt);
         ++launch_counter();
     }
     DMRG_CHECK_CUDA(cudaGetLastError());

@@ -55,7 +55,7 @@ unsigned char* scratch_for_current_device() {
 int64_t noalloc_scratch_bytes() { return kScratchBytes; }
 
 // Work list of the product (host side) -> static scratch -> FP64 segmented GEMM.
-void grouped_gemm_f64_noalloc(const WorkList& host_wl, const double* a, const double* b, double* c, cudaStream_t st) {
+void grouped_gemm_f64_noalloc(WorkList& host_wl, const double* a, const double* b, double* c, cudaStream_t st) {
     if (host_wl.tiles.empty()) return;
     const int64_t tile_bytes = (int64_t)(host_wl.tiles.size() * sizeof(Tile));
     const int64_t seg_off = round_up(tile_bytes, 256);
@@ -74,6 +74,7 @@ void grouped_gemm_f64_noalloc(const WorkList& host_wl, const double* a, const do
     DMRG_REQUIRE(cap == cudaStreamCaptureStatusNone, DMRG_EINVAL,
                  "dmrg_grouped_gemm_noalloc called on a stream that is being captured");
     unsigned char* base = scratch_for_current_device();
+    host_wl.arrange();  // the kernel and the order of the sums of dmrg_grouped_gemm
     DMRG_CHECK_CUDA(cudaMemcpyAsync(base, host_wl.tiles.data(), tile_bytes, cudaMemcpyHostToDevice, st));
     if (seg_bytes > 0)
         DMRG_CHECK_CUDA(cudaMemcpyAsync(base + seg_off, host_wl.segs.data(), seg_bytes, cudaMemcpyHostToDevice, st));
@@ -81,7 +82,11 @@ void grouped_gemm_f64_noalloc(const WorkList& host_wl, const double* a, const do
     bt.p[0] = const_cast<double*>(a);
     bt.p[1] = const_cast<double*>(b);
     bt.p[2] = c;
-    launch_seg_gemm_f64_lists((const Tile*)base, (int64_t)host_wl.tiles.size(), (const Seg*)(base + seg_off), bt, st);
+    host_wl.d_tiles = (Tile*)base;
+    host_wl.d_segs = (Seg*)(base + seg_off);
+    launch_seg_gemm_f64(host_wl, bt, 1, st);
+    host_wl.d_tiles = nullptr;
+    host_wl.d_segs = nullptr;
 }
 
 }  // namespace dmrg
