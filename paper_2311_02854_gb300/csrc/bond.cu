@@ -1,8 +1,8 @@
 // Environments and the current bond: vacuum blocks, renormalisation
 // (Eq. Renorm / Eqs. renorm12-renormFinal), the bond's intermediates (the
 // "intermediates" step of Sec. 2.2) and the sigma / diag(H_eff) work lists
-// (Eqs. sigmablk56-sigmablk).  Two engines share the planning: FP64 (SIMT
-// kernel, 64x64 tiles) and the tcgen05 engine on bf16 pieces (mixed precision).
+// (Eqs. sigmablk56-sigmablk).  Three engines share the planning: the FP64 units,
+// the FP64-accurate one on the tensor cores, and bf16 pieces (mixed precision).
 #include <algorithm>
 #include <chrono>
 #include <cmath>

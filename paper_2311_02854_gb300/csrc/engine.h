@@ -23,7 +23,8 @@ struct Seg {
 
 enum TileMode : uint8_t { TILE_STORE = 0, TILE_ATOMIC = 1 };
 
-// One output tile (at most 64 x 64) of an output block C (m x n, leading dim ldc).
+// One output tile (FP64 units 64 x 64, tensor cores 128 x 64 or 128) of an output
+// block C (m x n, leading dim ldc).
 struct Tile {
     int64_t c_off;        // block origin in buffer c_buf
     int32_t ldc, m, n;    // block leading dim and extents

@@ -97,8 +97,9 @@ constexpr int kSplitWarps = 4;  // warps of a CTA that share a part's term sum (
 }
 
 void WorkList::arrange() {
-    // work of a tile: 64-deep (tensor-core engine: oz_stage_depth) K steps, for the
-    // FP64 units times its 8 x 8 groups
+    // work of a tile: 64-deep (FP64-accurate engine: oz_stage_depth) K steps, times
+    // its rows and columns to convert plus a constant (by stages alone K = 24,
+    // D = 500 took 18.8 ms instead of 17.8) or its 8 x 8 groups (FP64 units)
     const bool oz = tile_m == oz_tile_rows();
     const int tk = oz ? oz_stage_depth() : 64;
     std::vector<int> cost(tiles.size());
@@ -108,7 +109,9 @@ void WorkList::arrange() {
         const Tile& t = tiles[i];
         int64_t n = 0;
         for (int s = t.seg_beg; s < t.seg_end; ++s) n += (segs[s].k + tk - 1) / tk;
-        if (!oz) n *= (int64_t)((std::min(t.m - t.m0, 64) + 7) / 8) * ((std::min(t.n - t.n0, 64) + 7) / 8);
+        const int rows = t.sn ? t.sn * 16 * t.sb : std::min(t.m - t.m0, 128);
+        if (oz) n = (n * (32 + rows + std::min(t.n - t.n0, 128)) + 31) / 32;
+        else n *= (int64_t)((std::min(t.m - t.m0, 64) + 7) / 8) * ((std::min(t.n - t.n0, 64) + 7) / 8);
         cost[i] = (int)std::min<int64_t>(n, 1 << 20);
         total += cost[i];
         maxn = std::max(maxn, cost[i]);

@@ -184,6 +184,9 @@ __global__ void __launch_bounds__(OZ_THREADS, 1)
     tc_fence_after();
     const uint32_t tmem = tmem_base_s;
     const uint32_t total = (uint32_t)ntiles * (uint32_t)nvec, NV = (uint32_t)nvec;  // total < 2^31
+    // the CTA's r-th item: dealt back and forth, since the items are ordered longest first
+    const uint32_t G = gridDim.x;
+    auto item = [&](uint32_t r) { return r * G + ((r & 1u) ? G - 1u - blockIdx.x : blockIdx.x); };
     bool failed = false;
 
     if (warp > MMA_WARP && (warp & 3) != 0) {
@@ -192,14 +195,13 @@ __global__ void __launch_bounds__(OZ_THREADS, 1)
         const uint32_t grp = (uint32_t)(li / NLDW);
         const int gw = li % NLDW;
         uint32_t d = 0;  // stages so far (all tiles, both groups)
-        const uint32_t G = gridDim.x;
         // The lanes hold the records of the next 32 segments of a tile (or, of lists
         // whose tiles have one segment each, of the next 32 tiles of this CTA): the
         // dependent loads tile -> segment are paid once per 32, not by every stage.
-        uint32_t ct = blockIdx.x;  // next tile
-        int cs = 0;                // segments of it already taken
-        while (ct < total && !failed) {
-            const uint32_t t = single ? ct + (uint32_t)lane * G : ct;
+        uint32_t cr = 0;  // round of the next tile
+        int cs = 0;       // segments of it already taken
+        while (item(cr) < total && !failed) {
+            const uint32_t t = item(single ? cr + (uint32_t)lane : cr);
             Tile T{};
             Seg S{};
             bool valid = false, last = true;
@@ -213,9 +215,9 @@ __global__ void __launch_bounds__(OZ_THREADS, 1)
             const int nseg = __shfl_sync(0xffffffffu, T.seg_end - T.seg_beg, 0);
             cs += 32;
             if (single) {
-                ct = min(total, ct + 32 * G);
+                cr += 32;
             } else if (cs >= nseg) {
-                ct = min(total, ct + G);
+                ++cr;
                 cs = 0;
             }
             const int vt = (int)(t % NV);
@@ -306,7 +308,7 @@ __global__ void __launch_bounds__(OZ_THREADS, 1)
         if (lane == 0) {
             uint32_t d = 0;
             bool wide = false;  // the previous stage used all the accumulators
-            for (uint32_t it = blockIdx.x; it < total && !failed; it += gridDim.x) {
+            for (uint32_t r = 0; item(r) < total && !failed; ++r) {
                 for (;;) {
                     const uint32_t slot = d & 1u, use = d >> 1;
                     if (!mbar_wait(smem_u32(&full_bar[slot]), use & 1u)) { failed = true; break; }
@@ -358,9 +360,10 @@ __global__ void __launch_bounds__(OZ_THREADS, 1)
         uint32_t d = 0;
         Tile nT{};
         if (blockIdx.x < total) nT = tiles[blockIdx.x / NV];
-        for (uint32_t it = blockIdx.x; it < total && !failed; it += gridDim.x) {
+        for (uint32_t round = 0; item(round) < total && !failed; ++round) {
+            const uint32_t it = item(round), in = item(round + 1);
             const Tile T = nT;
-            if (it + gridDim.x < total) nT = tiles[(it + gridDim.x) / NV];
+            if (in < total) nT = tiles[in / NV];
             const int v = (int)(it % NV);
             const int nrem = min(OTN, T.n - T.n0);
             // this thread's output row (stacked products: m * ldc apart, their rows run on)
