@@ -820,7 +820,7 @@ __global__ void __launch_bounds__(THREADS3, kCtas3)
 struct Pieces {
     __nv_bfloat16 h, l, m;
 };
-__device__ __forceinline__ Pieces split_pieces(double xd) {
+__device__ __forceinline__ Pieces split_pieces(double xd, bool three) {
     const uint32_t hi = (uint32_t)__double2hiint(xd), lo = (uint32_t)__double2loint(xd);
     const int eb = (int)((hi >> 20) & 0x7FFu);
     Pieces p;
@@ -836,7 +836,20 @@ __device__ __forceinline__ Pieces split_pieces(double xd) {
         p.h = __float2bfloat16_rn(xf);
         const float d = __fsub_rn(xf, __bfloat162float(p.h));
         p.l = __float2bfloat16_rn(__fadd_rn(d, e));
-        p.m = __float2bfloat16_rn(__fadd_rn(__fsub_rn(d, __bfloat162float(p.l)), e));
+        p.m = __ushort_as_bfloat16((unsigned short)0);
+        if (three) {
+            const float t = __fadd_rn(__fsub_rn(d, __bfloat162float(p.l)), e);
+            p.m = __float2bfloat16_rn(t);
+            // e is off by up to 2^-25 of itself where left has more than 24 bits: too
+            // little to matter unless t is close to the middle of two pieces or tiny
+            // (0.1 % of random values; without this 7 third pieces in 10 million were
+            // rounded the other way, enough to move a BF16X6 store by 1e-7)
+            const uint32_t tb = __float_as_uint(t);
+            if (abs(left) >= 1 << 24 && ((tb & 0xFFFFu) - 0x7FF8u <= 0x10u || (int)(tb >> 23 & 0xFFu) < eb - 896 - 28)) {
+                const double r = xd - (double)__bfloat162float(p.h);
+                p.m = __float2bfloat16_rn((float)(r - (double)__bfloat162float(p.l)));
+            }
+        }
     } else if ((hi << 1 | lo) == 0u) {
         p.h = __ushort_as_bfloat16((unsigned short)(hi >> 16));
         p.l = p.m = __ushort_as_bfloat16((unsigned short)0);
@@ -860,17 +873,19 @@ __global__ void split_f64_flat_kernel(const double* __restrict__ src, int64_t n,
                                       __nv_bfloat16* __restrict__ lo2) {
     const int64_t t0 = (int64_t)blockIdx.x * blockDim.x + threadIdx.x, nt = (int64_t)gridDim.x * blockDim.x;
     const int64_t nv = VEC ? n / 4 : 0;
+    const bool three = lo2 != nullptr;
     if (VEC) {
         for (int64_t i = t0; i < nv; i += nt) {
             const double2 a = ((const double2*)src)[2 * i], b = ((const double2*)src)[2 * i + 1];
-            const Pieces p[4] = {split_pieces(a.x), split_pieces(a.y), split_pieces(b.x), split_pieces(b.y)};
+            const Pieces p[4] = {split_pieces(a.x, three), split_pieces(a.y, three), split_pieces(b.x, three),
+                                 split_pieces(b.y, three)};
             ((uint2*)hi)[i] = make_uint2(pack2(p[0].h, p[1].h), pack2(p[2].h, p[3].h));
             if (lo) ((uint2*)lo)[i] = make_uint2(pack2(p[0].l, p[1].l), pack2(p[2].l, p[3].l));
             if (lo2) ((uint2*)lo2)[i] = make_uint2(pack2(p[0].m, p[1].m), pack2(p[2].m, p[3].m));
         }
     }
     for (int64_t i = 4 * nv + t0; i < ldd; i += nt) {
-        const Pieces p = split_pieces(i < n ? src[i] : 0.0);
+        const Pieces p = split_pieces(i < n ? src[i] : 0.0, three);
         hi[i] = p.h;
         if (lo) lo[i] = p.l;
         if (lo2) lo2[i] = p.m;
@@ -885,11 +900,13 @@ __global__ void split_blocks_kernel(const double* __restrict__ src, const SplitJ
                                     __nv_bfloat16* __restrict__ lo2) {
     const SplitJob J = jobs[blockIdx.x];
     const int nw = blockDim.x / 32, lane = threadIdx.x & 31;
+    const bool three = lo2 != nullptr;
     for (int r = blockIdx.y * nw + threadIdx.x / 32; r < J.rows; r += gridDim.y * nw) {
         const double* q = src + J.src_off + (int64_t)r * J.ld_src;
         const int64_t o = J.dst_off + (int64_t)r * J.ld_dst;  // offsets and leading dimensions are multiples of 8
         for (int c = 2 * lane; c < J.ld_dst; c += 64) {
-            const Pieces a = split_pieces(c < J.cols ? q[c] : 0.0), b = split_pieces(c + 1 < J.cols ? q[c + 1] : 0.0);
+            const Pieces a = split_pieces(c < J.cols ? q[c] : 0.0, three),
+                         b = split_pieces(c + 1 < J.cols ? q[c + 1] : 0.0, three);
             *(uint32_t*)(hi + o + c) = pack2(a.h, b.h);
             if (lo) *(uint32_t*)(lo + o + c) = pack2(a.l, b.l);
             if (lo2) *(uint32_t*)(lo2 + o + c) = pack2(a.m, b.m);
