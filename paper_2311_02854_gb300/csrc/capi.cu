@@ -269,19 +269,22 @@ dmrg_status dmrg_plan(const double* h, const double* chol, int n_chol, double e_
         double* dL = P.alloc(n_chol * K2);
         double* dE = P.alloc(K2 * K2);
         DMRG_CHECK_CUDA(cudaMemcpy(dL, chol, n_chol * K2 * 8, cudaMemcpyHostToDevice));
+        // one segment per Cholesky vector: every integral is one chain of fused
+        // multiply-adds, whatever the list's shape (see seg_outer_f64_kernel)
         WorkList wl;
-        Seg s{};
-        s.a_off = 0;
-        s.lda = (int)K2;
-        s.a_tr = 1;  // A(pq, X) = L[X][pq]
-        s.b_off = 0;
-        s.ldb = (int)K2;
-        s.b_tr = 0;  // B(X, rs) = L[X][rs]
-        s.k = n_chol;
-        s.a_buf = 0;
-        s.b_buf = 0;
-        s.alpha = 1.0;
-        wl.add_block(0, 1, (int)K2, (int)K2, (int)K2, {s}, TILE_STORE);
+        wl.rank1 = true;
+        std::vector<Seg> sum(n_chol);
+        for (int x = 0; x < n_chol; ++x) {
+            Seg& s = sum[x];
+            s.a_off = s.b_off = x * K2;  // A(pq, 0) = B(0, pq) = L[x][pq]
+            s.lda = s.ldb = (int)K2;
+            s.a_tr = 1;
+            s.b_tr = 0;
+            s.k = 1;
+            s.a_buf = s.b_buf = 0;
+            s.alpha = 1.0;
+        }
+        wl.add_block(0, 1, (int)K2, (int)K2, (int)K2, sum, TILE_STORE);
         wl.upload(nullptr);
         BufTable bt{};
         bt.p[0] = dL;

@@ -405,25 +405,29 @@ __global__ void __launch_bounds__(32 * kSplit, GR == 2 ? 5 : 3)
 }
 
 // The same product for lists whose segments all have K = 1 (rank-1 updates:
-// the diagonal of H_eff as sums of diag(O_L) diag(O_R)^T).  Bound: the latency
-// of the strided gathers (a diagonal is read with stride ld + 1) and, behind
-// it, the FP64 units.  A CTA gathers the elements of 64 segments into shared
-// memory with all its threads, one segment and operand each (32 loads in flight
-// per thread), and its four warps form the products, a quarter of the part's
-// 8 x 8 groups each, four segments per K-step and in segment order.
+// the diagonal of H_eff as sums of diag(O_L) diag(O_R)^T, the two-electron
+// integrals as a sum over Cholesky vectors).  Every element is one chain of fused
+// multiply-adds in segment order: the correction step of Davidson divides by
+// theta - H_ii, so a last place of the diagonal, or of the integrals behind it,
+// can end up as any figure of its vector.  (Integrals summed by four warps each and
+// a diagonal on mma.m8n8k4 moved the last place of one element in 14 000 at K = 14,
+// D = 600, and took 396 us instead of 370 at K = 24, D = 500.)  Bound: the latency of the strided gathers (a diagonal is
+// read with stride ld + 1) and, behind it, the FP64 units.  A CTA gathers the
+// elements of 64 segments into shared memory with all its threads, one segment
+// and operand each (32 loads in flight per thread); a thread then sums two rows,
+// 16 apart, of four columns, 8 apart.
 constexpr int kOuter = 64;
 __global__ void __launch_bounds__(2 * kOuter)
     seg_outer_f64_kernel(const Tile* __restrict__ tiles, int subs, const Seg* __restrict__ segs, BufTable bt) {
-    __shared__ double As[kOuter][PT + 4], Bs[kOuter][PT + 4];  // 36-double rows: fragment reads without conflicts
+    __shared__ double As[kOuter][PT + 1], Bs[kOuter][PT + 1];  // odd rows: a gathering warp writes without conflicts
     const Tile T = tiles[blockIdx.x / subs];
     const Part p = tile_part(T, (int)(blockIdx.x % subs));
     if (p.mr <= 0 || p.nr <= 0) return;
-    const int v = blockIdx.y, tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    const int lr = lane >> 2, lk = lane & 3;
-    const int gi = warp >> 1, gj = warp & 1;  // the warp's groups: rows gi, gi + 2, columns gj, gj + 2
+    const int v = blockIdx.y, tid = threadIdx.x;
+    const int r0 = tid >> 3, c0 = tid & 7;  // the thread's first row and column
     const int ls = tid % kOuter;
     const bool isb = tid >= kOuter;
-    double acc[2][2][2] = {};
+    double acc[2][4] = {};
     for (int s0 = T.seg_beg; s0 < T.seg_end; s0 += kOuter) {
         double x[PT];
         const bool sv = s0 + ls < T.seg_end;
@@ -445,32 +449,31 @@ __global__ void __launch_bounds__(2 * kOuter)
         for (int i = 0; i < PT; ++i) (isb ? Bs : As)[ls][i] = x[i];
         __syncthreads();
         const int ne = min(kOuter, T.seg_end - s0);
-        for (int k = 0; k < ne; k += 4) {
-            double a[2], b[2];
+        if ((r0 & ~3) < p.mr) {  // (a warp has four consecutive rows)
+            for (int k = 0; k < ne; ++k) {
+                double a[2], b[4];
 #pragma unroll
-            for (int i = 0; i < 2; ++i) {
-                a[i] = As[k + lk][8 * (gi + 2 * i) + lr];
-                b[i] = Bs[k + lk][8 * (gj + 2 * i) + lr];
+                for (int i = 0; i < 2; ++i) a[i] = As[k][r0 + 16 * i];
+#pragma unroll
+                for (int j = 0; j < 4; ++j) b[j] = Bs[k][c0 + 8 * j];
+#pragma unroll
+                for (int i = 0; i < 2; ++i)
+#pragma unroll
+                    for (int j = 0; j < 4; ++j)
+                        if ((r0 & ~3) + 16 * i < p.mr && 8 * j < p.nr) acc[i][j] = fma(a[i], b[j], acc[i][j]);
             }
-#pragma unroll
-            for (int i = 0; i < 2; ++i)
-#pragma unroll
-                for (int j = 0; j < 2; ++j)
-                    if (8 * (gi + 2 * i) < p.mr && 8 * (gj + 2 * j) < p.nr) mma884(acc[i][j], a[i], b[j]);
         }
     }
     double* C = bt.p[T.c_buf] + T.c_off + (int64_t)v * bt.vstride[T.c_buf];
 #pragma unroll
     for (int i = 0; i < 2; ++i)
 #pragma unroll
-        for (int j = 0; j < 2; ++j)
-#pragma unroll
-            for (int e = 0; e < 2; ++e) {
-                const int r = 8 * (gi + 2 * i) + lr, c = 8 * (gj + 2 * j) + 2 * lk + e;
-                if (r >= p.mr || c >= p.nr) continue;
-                double* dst = C + (int64_t)(p.m0 + r) * T.ldc + p.n0 + c;
-                *dst = T.mode == TILE_ATOMIC ? *dst + acc[i][j][e] : acc[i][j][e];
-            }
+        for (int j = 0; j < 4; ++j) {
+            const int r = r0 + 16 * i, c = c0 + 8 * j;
+            if (r >= p.mr || c >= p.nr) continue;
+            double* dst = C + (int64_t)(p.m0 + r) * T.ldc + p.n0 + c;
+            *dst = T.mode == TILE_ATOMIC ? *dst + acc[i][j] : acc[i][j];
+        }
 }
 }  // namespace
 
