@@ -39,8 +39,9 @@ struct Tile {
     // TMA tensor-core engine: tile width (64 or 128 columns).  Both tensor-core
     // engines of sigma: products stacked along the rows (0: none; else product i
     // holds accumulator rows i * 16 * sb ..., and its m x n block lies i * m * ldc
-    // elements behind c_off)
-    uint8_t tn, sn, sb, pad;
+    // elements behind c_off).  tr: a product that is stored transposed (TMA engine; its
+    // element (i, j) at j * ldc + i, stacked ones n * ldc apart)
+    uint8_t tn, sn, sb, tr;
 };
 static_assert(sizeof(Tile) == 48, "Tile keeps its 48-byte record");
 

@@ -461,21 +461,21 @@ __device__ __forceinline__ void epilogue_tma(const Tile& T, int v, uint32_t tacc
                                              uint32_t tempty) {
     const int row = w4 * 32 + lane;
     const int ncol = min((int)T.tn, T.n - T.n0);
-    // row of the output: of stacked products (m * ldc apart) the rows run on
+    // row r of product i of a stack
     bool any, rok;
-    int64_t r;
+    int i = 0, r = T.m0 + row;
     if (T.sn) {
-        const int i = row / (16 * T.sb), ri = row - i * 16 * T.sb;
+        i = row / (16 * T.sb);
+        r = row - i * 16 * T.sb;
         any = w4 * 32 < T.sn * 16 * T.sb;
-        rok = i < T.sn && ri < T.m;
-        r = (int64_t)i * T.m + ri;
+        rok = i < T.sn && r < T.m;
     } else {
         any = T.nst > 0 && T.m0 + w4 * 32 < T.m;
-        r = T.m0 + row;
         rok = r < T.m;
     }
     const float alpha = T.alpha;
-    const int64_t off = T.c_off + r * T.ldc + T.n0 + (int64_t)v * B.out_vstride[T.c_buf];
+    const int64_t off = T.c_off + (int64_t)v * B.out_vstride[T.c_buf] +
+                        (T.tr ? ((int64_t)i * T.n + T.n0) * T.ldc + r : ((int64_t)i * T.m + r) * T.ldc + T.n0);
     if (T.nst == 0 && T.mode == TC_STORE_SPLIT && rok) {  // a stored block without products is zero
         for (int j0 = 0; j0 < ncol; j0 += 8) {
             *(uint4*)((__nv_bfloat16*)B.out[T.c_buf] + off + j0) = make_uint4(0, 0, 0, 0);
@@ -501,6 +501,22 @@ __device__ __forceinline__ void epilogue_tma(const Tile& T, int v, uint32_t tacc
 #pragma unroll
                 for (int j = 0; j < 32; ++j)
                     if (c0 + j < ncol) atomicAdd(o + j, (double)alpha * (double)__uint_as_float(acc[j]));
+            } else if (T.tr) {  // TC_STORE_SPLIT, transposed: the lanes' elements of a column lie side by side
+                __nv_bfloat16* oh = (__nv_bfloat16*)B.out[T.c_buf] + off + (int64_t)c0 * T.ldc;
+                __nv_bfloat16* ol = (__nv_bfloat16*)B.out_lo[T.c_buf] + off + (int64_t)c0 * T.ldc;
+#pragma unroll
+                for (int j = 0; j < 32; ++j) {
+                    if (c0 + j >= ncol) break;
+                    const float x = alpha * __uint_as_float(acc[j]);
+                    const __nv_bfloat16 h = __float2bfloat16_rn(x);
+                    *oh = h;
+                    const float d = x - __bfloat162float(h);
+                    const __nv_bfloat16 l = __float2bfloat16_rn(d);
+                    if (NSPLIT >= 2) *ol = l;
+                    if (NSPLIT == 3) ol[B.out_pstride[T.c_buf]] = __float2bfloat16_rn(d - __bfloat162float(l));
+                    oh += T.ldc;
+                    ol += T.ldc;
+                }
             } else {  // TC_STORE_SPLIT: chunks of 8 (rows padded to multiples of 8)
                 __nv_bfloat16* oh = (__nv_bfloat16*)B.out[T.c_buf] + off + c0;
                 __nv_bfloat16* ol = (__nv_bfloat16*)B.out_lo[T.c_buf] + off + c0;
@@ -973,9 +989,10 @@ void launch_seg_gemm_tc(const WorkList& w, const TcBufs& b, int nvec, int nsplit
 // ---------------------------------------------------------------------------
 
 void TmaWorkList::add_block(int64_t c_off, int c_buf, int m, int n, int ldc, const std::vector<TSeg>& s, uint8_t mode,
-                            int64_t kchunk, float alpha, int tn) {
+                            int64_t kchunk, float alpha, int tn, bool tr) {
     if (m <= 0 || n <= 0) return;
     DMRG_REQUIRE(tn == 64 || tn == TN, DMRG_EINVAL, "tile width must be 64 or 128");
+    DMRG_REQUIRE(!tr || (mode == TC_STORE_SPLIT && !s.empty()), DMRG_EINVAL, "only stored products are transposed");
     std::vector<std::pair<int, int>> chunks;
     const bool atomic = (mode == TC_ATOMIC_F64 || mode == TC_ATOMIC_F32);
     if (atomic && kchunk > 0) {
@@ -1018,13 +1035,14 @@ void TmaWorkList::add_block(int64_t c_off, int c_buf, int m, int n, int ldc, con
                 t.c_buf = (uint8_t)c_buf;
                 t.mode = mode;
                 t.nst = (uint16_t)nst;
+                t.tr = tr ? 1 : 0;
                 tiles.push_back(t);
             }
     }
 }
 
 void TmaWorkList::add_stack(int64_t c_off, int c_buf, int m, int n, int ldc, const TSeg& s, float alpha, int sn, int sb,
-                            int tn) {
+                            int tn, bool tr) {
     if (m <= 0 || n <= 0 || sn <= 0) return;
     const int sbeg = (int)segs.size();
     segs.push_back(s);
@@ -1033,6 +1051,7 @@ void TmaWorkList::add_stack(int64_t c_off, int c_buf, int m, int n, int ldc, con
         t.tn = (uint8_t)tn;
         t.sn = (uint8_t)sn;
         t.sb = (uint8_t)sb;
+        t.tr = tr ? 1 : 0;
         t.alpha = alpha;
         t.c_off = c_off;
         t.ldc = ldc;

@@ -885,10 +885,8 @@ void ProductList::lower_tma(int8_t sbuf_, int8_t ibuf, int ild, int64_t cap, int
                 const double cost_qr = 2.0 * c.k1 * c.k2 * c.n + 2.0 * c.m * c.k1 * c.n;
                 it.kind = 3;
                 it.pq_first = cost_pq <= cost_qr;
-                // the operator is the product's left factor: O Psi, or R^T Psi^T (the
-                // transpose of Psi R), so that operators can be stacked along its rows
-                it.tr = it.pq_first ? c.m : c.n;
-                it.tcl = it.pq_first ? c.k2 : c.k1;
+                it.tr = it.pq_first ? c.m : c.k1;
+                it.tcl = it.pq_first ? c.k2 : c.n;
             } else {
                 if (nreal == 2) {
                     if (c.P.ident) {
@@ -918,7 +916,7 @@ void ProductList::lower_tma(int8_t sbuf_, int8_t ibuf, int ild, int64_t cap, int
                 }
             }
             int64_t need = 0;
-            if (it.kind >= 2) need = it.kind == 2 || it.pq_first ? (int64_t)it.tr * round_up(it.tcl, 8) : (int64_t)c.k1 * round_up(c.n, 8);
+            if (it.kind >= 2) need = (int64_t)it.tr * round_up(it.tcl, 8);
             if (cp.used + need > cap && cp.used > 0) break;
             cp.used += need;
             cp.items.push_back(it);
@@ -934,8 +932,13 @@ void ProductList::lower_tma(int8_t sbuf_, int8_t ibuf, int ild, int64_t cap, int
     // scratch slots.  Tiles of one 21 x 21 product each (K = 24, D = 500) used a
     // sixth of a tile's rows and loaded the sector once per operator.
     std::vector<std::vector<ProdStack>> stacks(plans.size());
-    // the operator is the product's left factor: O Psi, or R^T Psi^T (the transpose of Psi R)
+    // the operator is the computed product's left factor: O Psi, or R^T Psi^T, so that
+    // operators can be stacked along the rows.  The latter is stored transposed, as Psi R:
+    // that takes the room the cut above counted (stored as computed, k1 columns padded to
+    // eight, sectors of one to three states took up to eight times as much), and costs
+    // nothing measurable (K = 8 ... 36: 1 % either way)
     auto op_view = [&](const Contrib& c, const Item& it) { return it.pq_first ? c.P : c.R.T(); };
+    auto op_rows = [](const Item& it) { return it.pq_first ? it.tr : it.tcl; };
     // operators per tile: K-major rows are stacked 16 * sb rows apart, MN-major
     // ones in 64-wide halves
     auto stack_rows = [](const View& A, int m) { return A.tr ? 64 : box_rows(m); };
@@ -950,7 +953,7 @@ void ProductList::lower_tma(int8_t sbuf_, int8_t ibuf, int ild, int64_t cap, int
             const View A = op_view(c, it);
             k = product_key({A, c.Q, it.tr, it.tcl, 0, !it.pq_first}, it.pq_first, bits_of(std::fabs(c.alpha)));
             z = A.z;
-            most = stack_max(A, it.tr);
+            most = stack_max(A, op_rows(it));
             return true;
         });
         // scratch slots: groups of equal shape, a stack's products consecutive
@@ -1045,7 +1048,7 @@ void ProductList::lower_tma(int8_t sbuf_, int8_t ibuf, int ild, int64_t cap, int
                     u.osegs.push_back({c.out, make_tseg(lm, T, c.R, c.m, c.n, c.k2, sg, vstride, nv)});
                 } else {
                     fl += 2.0 * c.k1 * c.k2 * c.n + 2.0 * c.m * c.k1 * c.n;
-                    u.osegs.push_back({c.out, make_tseg(lm, c.P, T.T(), c.m, c.n, c.k1, sg, vstride, nv)});
+                    u.osegs.push_back({c.out, make_tseg(lm, c.P, T, c.m, c.n, c.k1, sg, vstride, nv)});
                 }
             } else if (it.kind == 2) {
                 fl += it.fl;
@@ -1068,11 +1071,12 @@ void ProductList::lower_tma(int8_t sbuf_, int8_t ibuf, int ild, int64_t cap, int
             const int64_t off = g[3] + (int64_t)it.z * g[0] * ld;
             const View A = op_view(c, it), Q = it.pq_first ? c.Q : c.Q.T();
             const int k = it.pq_first ? c.k1 : c.k2;
-            const int most = stack_max(A, it.tr);
-            TSeg s = make_tseg(lm, A, Q, it.tr, it.tcl, k, 1.0, vstride, nv, most);
-            s.swap = it.pq_first ? 0 : 1;
-            if (most > 1) p1.add_stack(off, sbuf, it.tr, it.tcl, ld, s, (float)c.alpha, sk[x].n, stack_rows(A, it.tr) / 16, tile_n);
-            else p1.add_block(off, sbuf, it.tr, it.tcl, ld, {s}, TC_STORE_SPLIT, 0, (float)c.alpha, tile_n);
+            const int rows = op_rows(it), cols = it.pq_first ? it.tcl : it.tr, most = stack_max(A, rows);
+            const bool tr = !it.pq_first;
+            TSeg s = make_tseg(lm, A, Q, rows, cols, k, 1.0, vstride, nv, most);
+            s.swap = tr ? 1 : 0;
+            if (most > 1) p1.add_stack(off, sbuf, rows, cols, ld, s, (float)c.alpha, sk[x].n, stack_rows(A, rows) / 16, tile_n, tr);
+            else p1.add_block(off, sbuf, rows, cols, ld, {s}, TC_STORE_SPLIT, 0, (float)c.alpha, tile_n, tr);
         }
         u.fl = fl;
     });

@@ -73,12 +73,14 @@ struct TmaWorkList {
     size_t cap_tiles = 0, cap_segs = 0;
     bool single = false;  // every tile has one segment (set by order_tiles)
     // output block (m x n, ld ldc) at c_off of c_buf, 128 x tn tiles (tn = 64 or
-    // 128), split into K-chunks of at most kchunk (atomic modes only)
+    // 128), split into K-chunks of at most kchunk (atomic modes only); tr: stored
+    // transposed (TC_STORE_SPLIT only)
     void add_block(int64_t c_off, int c_buf, int m, int n, int ldc, const std::vector<TSeg>& s, uint8_t mode,
-                   int64_t kchunk, float alpha, int tn = 128);
-    // sn stored products (m x n, ld ldc, m * ldc apart from c_off on) of one tile
+                   int64_t kchunk, float alpha, int tn = 128, bool tr = false);
+    // sn stored products (m x n, ld ldc, one behind another from c_off on) of one tile
     // row: product i in accumulator rows i * 16 * sb ...
-    void add_stack(int64_t c_off, int c_buf, int m, int n, int ldc, const TSeg& s, float alpha, int sn, int sb, int tn);
+    void add_stack(int64_t c_off, int c_buf, int m, int n, int ldc, const TSeg& s, float alpha, int sn, int sb, int tn,
+                   bool tr);
     void order_tiles();  // longest tiles first (stable)
     void upload(cudaStream_t st);
     void release();

@@ -44,3 +44,27 @@ def test_integrals_are_chains_of_fused_multiply_adds(tmp_path):
         plan.close()
     for x, y in zip(*out):
         assert np.array_equal(x, y)
+
+
+@pytest.mark.parametrize("K,D,width", [(14, 600, 1.0), (20, 500, 1.2)])
+def test_first_products_fit_the_scratch_that_was_allowed(tmp_path, K, D, width):
+    """Sectors of one to three states beside wide ones: a chunk's stored products stay
+    within scratch_bytes.
+
+    The renormalisation before the bond fills the scratch up to less than one product
+    (at most 190 x 192 elements of two pieces, 146 KB), and with a chunk per term sigma
+    needs no more; so a list of several full chunks may hold at most that much more."""
+    cuda_torch()
+    g = gpu_lib()
+    k, room = 4, 4 << 20
+    h, L, _, path = make_case(tmp_path, K, K, 0, D, center=k, split="gaussian", wn=width, ws=width)
+    held = []
+    for per_term in (0, 1):
+        plan = g.Plan(h, L, K, K, 0, D, path, precision=BF16X3, scratch_bytes=room, sigma_per_term=per_term)
+        plan.set_bond(k)
+        st = plan.stats()
+        held.append(st["device_bytes"])
+        if not per_term:
+            assert st["sigma_chunks"] > 1
+        plan.close()
+    assert held[0] <= held[1] + (256 << 10)
