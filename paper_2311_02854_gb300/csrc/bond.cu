@@ -1031,7 +1031,7 @@ void set_bond(Plan& P, int k) {
             ch.first.upload(P.stream);
             ch.second.upload(P.stream);
         }
-        tl.maps.encode_upload(sigma_bufs(P, k, nullptr), P.nsplit, P.stream);
+        tl.maps.encode_upload(sigma_bufs(P, k, nullptr), P.nsplit, P.stream, tl.serial);
         if (P.opt.verbose)
             fprintf(stderr, "[dmrg] bond %d sigma planning: terms %.0f ms, tuning %.0f ms, lowering %.0f ms, "
                             "counts %.0f ms, upload %.0f ms (%zu chunks)\n",
@@ -1245,10 +1245,10 @@ void sigma_fp64_units(Plan& P, const double* psi, double* out, int nvec, cudaStr
 }
 
 namespace {
-void sigma_body(Plan& P, const double* psi, double* out, int nvec, cudaStream_t st);
+void sigma_body(Plan& P, const double* psi, double* out, int nvec, cudaStream_t st, bool repeatable);
 }
 
-void sigma(Plan& P, const double* psi, double* out, int nvec, cudaStream_t st) {
+void sigma(Plan& P, const double* psi, double* out, int nvec, cudaStream_t st, bool repeatable) {
     DMRG_REQUIRE(P.bond > 0, DMRG_EINVAL, "no current bond (call dmrg_set_bond)");
     DMRG_REQUIRE(nvec >= 1, DMRG_EINVAL, "nvec must be >= 1");
     if (P.sig_pending.size() >= 64) P.collect_sigma_times(false);
@@ -1256,7 +1256,7 @@ void sigma(Plan& P, const double* psi, double* out, int nvec, cudaStream_t st) {
                          P.mixed() ? (P.stats.sigma_stages[0] + P.stats.sigma_stages[1]) * nvec : 0};
     try {
         DMRG_CHECK_CUDA(cudaEventRecord(ev.a, st));
-        sigma_body(P, psi, out, nvec, st);
+        sigma_body(P, psi, out, nvec, st, repeatable);
         DMRG_CHECK_CUDA(cudaEventRecord(ev.b, st));
     } catch (...) {
         P.ev_pool.push_back(ev.a);
@@ -1267,7 +1267,7 @@ void sigma(Plan& P, const double* psi, double* out, int nvec, cudaStream_t st) {
 }
 
 namespace {
-void sigma_body(Plan& P, const double* psi, double* out, int nvec, cudaStream_t st) {
+void sigma_body(Plan& P, const double* psi, double* out, int nvec, cudaStream_t st, bool repeatable) {
     if (!P.mixed()) {
         const int64_t per = std::max<int64_t>(P.sigma_pl.scratch_elems, 1);
         const int group = (int)std::max<int64_t>(1, std::min<int64_t>(nvec, P.n_scratch / per));
@@ -1292,12 +1292,12 @@ void sigma_body(Plan& P, const double* psi, double* out, int nvec, cudaStream_t 
                              P.ps_lo + (int64_t)v * P.dim_pad, s,
                              P.nsplit == 3 ? P.ps_lo + P.n_ppc + (int64_t)v * P.dim_pad : nullptr);
         DMRG_CHECK_CUDA(cudaMemsetAsync(o, 0, (size_t)nv * P.dim * 8, s));
-        tl.run_tma(sigma_bufs(P, P.bond, o), nv, P.nsplit, s);
+        tl.run_tma(sigma_bufs(P, P.bond, o), nv, P.nsplit, s, repeatable);
     };
     {
         const TcBufs tb = sigma_bufs(P, P.bond, nullptr);
         if (tl.maps.stale(tb)) {
-            tl.maps.encode_upload(tb, P.nsplit, st);
+            tl.maps.encode_upload(tb, P.nsplit, st, tl.serial);
             P.drop_graphs();
         }
     }
@@ -1321,7 +1321,7 @@ void sigma_body(Plan& P, const double* psi, double* out, int nvec, cudaStream_t 
         }
         double* gin = P.d_sig_io;
         double* gout = P.d_sig_io + (int64_t)G * P.dim;
-        Plan::SigmaGraph& sg = P.sigma_graphs[nv];
+        Plan::SigmaGraph& sg = P.sigma_graphs[{nv, repeatable && tl.serial}];
         if (!sg.exec) {
             // first use at this bond and vector count: capture on the plan's own stream
             const int64_t l0 = launch_counter();

@@ -97,6 +97,9 @@ constexpr int kSplitWarps = 4;  // warps of a CTA that share a part's term sum (
 }
 
 void WorkList::arrange() {
+    // lists of the bf16-piece engine keep their order: its K-chunks are added as they
+    // finish, and the rules below know the FP64 engines only
+    if (!tiles.empty() && tiles[0].mode > TILE_ATOMIC) return;
     // work of a tile: 64-deep (FP64-accurate engine: oz_stage_depth) K steps, times
     // its rows and columns to convert plus a constant (by stages alone K = 24,
     // D = 500 took 18.8 ms instead of 17.8) or its 8 x 8 groups (FP64 units)

@@ -822,6 +822,229 @@ __global__ void __launch_bounds__(THREADS3, kCtas3)
 }
 
 // ---------------------------------------------------------------------------
+// TMA-staged kernel, one tile and one stage after the other
+// ---------------------------------------------------------------------------
+//
+// The sums of short lists inside Davidson.  An output region receives one FP64 atomic
+// addition per K-chunk, and from the third chunk on their order decides the last place
+// of an element.  Davidson makes any figure of its vector out of such a place: its
+// corrections r / (theta - H_ii) lie almost in the space that it has already, and what
+// Gram-Schmidt leaves of them is normalised (K = 14, D = 600, eight steps from a random
+// vector: 1e-16 becomes 1).  tc_tma_kernel finishes chunks in an order that changes from
+// call to call in many regions; here one lane walks tile -> segment -> copies, so that a
+// tile takes a time of its own (490 ns per 64-deep stage, 245 per segment, 3.9 us),
+// repeatable to 0.3 us, and 99.4 % of all pairs of chunks keep their order: of 72
+// calls (24 problems) 6 differ from their plan's first by over 1e-9, with tc_tma_kernel
+// 17; and 100 of 108 give the vector that this schedule gave when it was the only one
+// (101 of its own repeats did).  It costs 0.41 ms per sigma there (1.45 -> 1.86).
+// Lists of more than kSerialItems products stay with tc_tma_kernel: no order repeats
+// there (K = 24, D = 500, 550 000 products: two calls differ by order one after eight
+// steps with either kernel).
+//
+// Its tiles are ordered by their stages alone and dealt in one direction, one CTA per
+// SM, fixed stages of 128 x 64 rows per piece.
+
+// 64 x 64 box of a 4-D tensor map (one piece) into shared memory, completion on an mbarrier
+__device__ __forceinline__ void tma_load4(uint32_t dst, const CUtensorMap* map, int x, int y, int z, int w,
+                                          uint32_t bar) {
+    asm volatile(
+        "cp.async.bulk.tensor.4d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3, %4, "
+        "%5}], [%6];\n" ::"r"(dst),
+        "l"(reinterpret_cast<uint64_t>(map)), "r"(x), "r"(y), "r"(z), "r"(w), "r"(bar)
+        : "memory");
+}
+
+// One 128 x 64 operand piece as (up to) two 64-row boxes, 8 KB apart.  K-major
+// (mn = 0): rows r0.. of the map at x = k0; MN-major (mn = 1): columns r0.. of the map
+// at rows k0..  halves = 1: the block ends within the first 64 (see tma_operand).
+__device__ __forceinline__ void tma_piece(uint32_t dst, const CUtensorMap* map, int mn, int r0, int k0, int z, int w,
+                                          uint32_t bar, int halves) {
+    if (!mn) {
+        tma_load4(dst, map, k0, r0, z, w, bar);
+        if (halves == 2) tma_load4(dst + 8192, map, k0, r0 + 64, z, w, bar);
+    } else {
+        tma_load4(dst, map, r0, k0, z, w, bar);
+        if (halves == 2) tma_load4(dst + 8192, map, r0 + 64, k0, z, w, bar);
+    }
+}
+
+// Roles: warps 0-3 epilogue (as in tc_seg_gemm_kernel), warp 4 lane 0 TMA
+// producer, warp 5 lane 0 MMA issuer.
+constexpr int THREADS4 = (kEpiWarps + 2) * 32;
+
+// stage record
+struct StageMeta4 {
+    uint8_t a_mn, b_mn, neg, flags;  // flags: 1 first stage of a tile, 2 last, 4 no MMA (empty tile)
+    uint8_t k16, n16, pad[2];        // 16-deep K steps holding data; MMA N / 16
+};
+
+template <int NSPLIT>
+__global__ void __launch_bounds__(THREADS4, 1)
+    tc_serial_kernel(const Tile* __restrict__ tiles, int ntiles, int nvec, const TSeg* __restrict__ segs,
+                     const CUtensorMap* __restrict__ maps, TcBufs B) {
+    using C = Cfg2<NSPLIT>;
+    constexpr int S = C::STAGES;
+    extern __shared__ uint8_t smem_raw[];
+    __shared__ __align__(8) uint64_t full_bar[S], empty_bar[S], tfull_bar[2], tempty_bar[2], drain_bar;
+    __shared__ StageMeta4 meta[S];
+    __shared__ uint32_t tmem_base_s;
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const uint32_t sbase = (smem_u32(smem_raw) + 1023u) & ~1023u;
+
+    if (warp == 0) tmem_alloc(smem_u32(&tmem_base_s), 2 * TMEM_COLS);
+    if (tid == 0) {
+        for (int s = 0; s < S; ++s) {
+            mbar_init(smem_u32(&full_bar[s]), 1);
+            mbar_init(smem_u32(&empty_bar[s]), 1);
+        }
+        for (int b = 0; b < 2; ++b) {
+            mbar_init(smem_u32(&tfull_bar[b]), 1);
+            mbar_init(smem_u32(&tempty_bar[b]), kEpiWarps);
+        }
+        mbar_init(smem_u32(&drain_bar), 1);
+        asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
+    }
+    tc_fence_before();
+    __syncthreads();
+    tc_fence_after();
+    const uint32_t tmem = tmem_base_s;
+    const int total = ntiles * nvec;
+    bool failed = false;
+
+    if (warp == kEpiWarps) {
+        // ---------------- TMA producer ----------------
+        if (lane == 0) {
+            uint32_t q = 0;
+            for (int t = blockIdx.x; t < total && !failed; t += gridDim.x) {
+                const int v = t % nvec;
+                const Tile T = tiles[t / nvec];
+                const int nst = T.nst;
+                // a second 64-row (or 64-column) half only when the block extends past the first
+                const int ncol = min((int)T.tn, T.n - T.n0);  // columns of this tile
+                const int nA = (T.m - T.m0 > 64) ? 2 : 1, nB = (ncol > 64) ? 2 : 1;
+                const int n16 = (ncol + 15) / 16;
+                if (nst == 0) {
+                    if (q >= (uint32_t)S && !mbar_wait(smem_u32(&empty_bar[q % S]), ((q / S) - 1) & 1u)) {
+                        failed = true;
+                        break;
+                    }
+                    meta[q % S] = StageMeta4{0, 0, 0, 1 | 2 | 4, 0, 0, {0, 0}};
+                    mbar_arrive(smem_u32(&full_bar[q % S]));
+                    ++q;
+                    continue;
+                }
+                int done = 0;
+                for (int s = T.seg_beg; s < T.seg_end && !failed; ++s) {
+                    const TSeg Sg = segs[s];
+                    const int a_mn = Sg.a_tr ? 1 : 0, b_mn = Sg.b_tr ? 0 : 1;
+                    const int aw = Sg.a_pv ? v : 0, bw = Sg.b_pv ? v : 0;
+                    const CUtensorMap* am = maps + NSPLIT * Sg.a_map;
+                    const CUtensorMap* bm = maps + NSPLIT * Sg.b_map;
+                    const uint32_t bytes = (uint32_t)NSPLIT * 128u * (uint32_t)(nA * Sg.a_br + nB * Sg.b_br);
+                    for (int k0 = 0; k0 < Sg.k; k0 += TK) {
+                        const uint32_t slot = q % S;
+                        if (q >= (uint32_t)S && !mbar_wait(smem_u32(&empty_bar[slot]), ((q / S) - 1) & 1u)) {
+                            failed = true;
+                            break;
+                        }
+                        const int kv = min(TK, Sg.k - k0);
+                        meta[slot] = StageMeta4{(uint8_t)a_mn, (uint8_t)b_mn, (uint8_t)(Sg.sign < 0.f ? 1 : 0),
+                                                (uint8_t)((done == 0 ? 1 : 0) | (done == nst - 1 ? 2 : 0)),
+                                                (uint8_t)((kv + 15) / 16), (uint8_t)n16, {0, 0}};
+                        const uint32_t bar = smem_u32(&full_bar[slot]);
+                        mbar_arrive_tx(bar, bytes);
+                        const uint32_t sa = sbase + slot * C::STAGE_BYTES;
+                        const uint32_t sb = sa + NSPLIT * PIECE_BYTES;
+#pragma unroll
+                        for (int pc = 0; pc < NSPLIT; ++pc) {
+                            tma_piece(sa + pc * PIECE_BYTES, am + pc, a_mn, T.m0, k0, Sg.a_z, aw, bar, nA);
+                            tma_piece(sb + pc * PIECE_BYTES, bm + pc, b_mn, T.n0, k0, Sg.b_z, bw, bar, nB);
+                        }
+                        ++q;
+                        ++done;
+                    }
+                }
+            }
+        }
+    } else if (warp == kEpiWarps + 1) {
+        // ---------------- MMA issuer ----------------
+        if (lane == 0) {
+            uint32_t q = 0, tc = 0;
+            for (int t = blockIdx.x; t < total && !failed; t += gridDim.x, ++tc) {
+                const uint32_t buf = tc & 1u, use = tc >> 1;
+                if (use > 0 && !mbar_wait(smem_u32(&tempty_bar[buf]), (use - 1) & 1u)) {
+                    failed = true;
+                    break;
+                }
+                tc_fence_after();
+                const uint32_t dt = tmem + buf * TMEM_COLS;
+                for (;;) {
+                    const uint32_t slot = q % S;
+                    if (!mbar_wait(smem_u32(&full_bar[slot]), (q / S) & 1u)) {
+                        failed = true;
+                        break;
+                    }
+                    tc_fence_after();
+                    const StageMeta4 M = meta[slot];
+                    if (!(M.flags & 4)) {
+                        const uint32_t sa = sbase + slot * C::STAGE_BYTES;
+                        const uint32_t sb = sa + NSPLIT * PIECE_BYTES;
+                        const uint32_t id = idesc_n(M.a_mn, M.b_mn, M.neg, 16 * M.n16);
+                        for (int kk = 0; kk < M.k16; ++kk) {
+#pragma unroll
+                            for (int pr = 0; pr < Prods<NSPLIT>::N; ++pr) {
+                                const int pa = prod_a(pr), pb = prod_b(pr);
+                                const uint32_t a_s = sa + pa * PIECE_BYTES;
+                                const uint32_t b_s = sb + pb * PIECE_BYTES;
+                                const uint64_t ad =
+                                    M.a_mn ? sdesc(a_s + kk * 2048, 8192, 1024) : sdesc(a_s + kk * 32, 16, 1024);
+                                const uint64_t bd =
+                                    M.b_mn ? sdesc(b_s + kk * 2048, 8192, 1024) : sdesc(b_s + kk * 32, 16, 1024);
+                                const uint32_t acc = ((M.flags & 1) && kk == 0 && pr == 0) ? 0u : 1u;
+                                mma_bf16(dt, ad, bd, id, acc);
+                            }
+                        }
+                    }
+                    mma_commit(smem_u32(&empty_bar[slot]));
+                    ++q;
+                    if (M.flags & 2) break;
+                }
+                if (failed) break;
+                mma_commit(smem_u32(&tfull_bar[buf]));
+            }
+            mma_commit(smem_u32(&drain_bar));
+            if (!mbar_wait(smem_u32(&drain_bar), 0)) failed = true;
+        }
+    } else {
+        // ---------------- epilogue ----------------
+        uint32_t tc = 0;
+        Tile Tn{};
+        if (blockIdx.x < total) Tn = tiles[blockIdx.x / nvec];
+        for (int t = blockIdx.x; t < total && !failed; t += gridDim.x, ++tc) {
+            const uint32_t buf = tc & 1u, use = tc >> 1;
+            const Tile T = Tn;  // fetched one tile ahead, while the MMAs of this one run
+            if (t + (int)gridDim.x < total) Tn = tiles[(t + gridDim.x) / nvec];
+            int ok = 1;
+            if (lane == 0) ok = mbar_wait(smem_u32(&tfull_bar[buf]), use & 1u) ? 1 : 0;
+            ok = __shfl_sync(0xffffffffu, ok, 0);  // warp-uniform (tcgen05.ld is warp-collective)
+            if (!ok) {
+                failed = true;
+                break;
+            }
+            __syncwarp();
+            tc_fence_after();
+            epilogue_tile<NSPLIT>(T, t % nvec, T.nst, tmem + buf * TMEM_COLS, warp, lane, B,
+                                  smem_u32(&tempty_bar[buf]));
+        }
+    }
+    if (failed) atomicExch(B.err, 1);
+    tc_fence_before();
+    __syncthreads();
+    tc_fence_after();
+    if (warp == 0) tmem_dealloc(tmem, 2 * TMEM_COLS);
+}
+
+// ---------------------------------------------------------------------------
 // conversions
 // ---------------------------------------------------------------------------
 
@@ -1067,30 +1290,36 @@ void TmaWorkList::add_stack(int64_t c_off, int c_buf, int m, int n, int ldc, con
     }
 }
 
-void TmaWorkList::order_tiles() {
+namespace {
+// largest work first: a stable counting sort, two linear passes instead of an n log n
+// sort of millions of records on every bond
+template <typename Work>
+std::vector<Tile> sorted_down(const std::vector<Tile>& tiles, const Work& work) {
+    int maxn = 0;
+    for (const Tile& t : tiles) maxn = std::max(maxn, work(t));
+    std::vector<size_t> pos((size_t)maxn + 2, 0);
+    for (const Tile& t : tiles) ++pos[(size_t)(maxn - work(t)) + 1];
+    for (size_t i = 1; i < pos.size(); ++i) pos[i] += pos[i - 1];
+    std::vector<Tile> sorted(tiles.size());
+    for (const Tile& t : tiles) sorted[pos[(size_t)(maxn - work(t))]++] = t;
+    return sorted;
+}
+}  // namespace
+
+void TmaWorkList::order_tiles(bool serial) {
     single = true;
     for (const Tile& t : tiles) single = single && t.seg_end - t.seg_beg == 1;
     // Longest tiles first (stages, weighted by the rows and columns they load):
     // CTAs take the tiles in turn, back and forth, so the short ones fill in at
     // the end of the launch instead of a few long ones trailing.  (By stages alone
     // and in one direction the SMs idled 19 % of a K = 14, D = 600 phase 2: sigma
-    // 1.52 -> 1.47 ms, K = 8, D = 64 199 -> 176 us.)  A stable
-    // counting sort: two linear passes instead of an n log n sort of millions of
-    // records on every bond.
-    if (tiles.size() > 1) {
-        auto work = [](const Tile& t) {
-            const int rows = t.sn ? t.sn * 16 * t.sb : std::min(t.m - t.m0, TM);
-            return (int)((int64_t)t.nst * (64 + rows + std::min<int>(t.tn, t.n - t.n0)) / 64);
-        };
-        int maxn = 0;
-        for (const Tile& t : tiles) maxn = std::max(maxn, work(t));
-        std::vector<size_t> pos((size_t)maxn + 2, 0);
-        for (const Tile& t : tiles) ++pos[(size_t)(maxn - work(t)) + 1];
-        for (size_t i = 1; i < pos.size(); ++i) pos[i] += pos[i - 1];
-        std::vector<Tile> sorted(tiles.size());
-        for (const Tile& t : tiles) sorted[pos[(size_t)(maxn - work(t))]++] = t;
-        tiles.swap(sorted);
-    }
+    // 1.52 -> 1.47 ms, K = 8, D = 64 199 -> 176 us.)
+    by_stages.clear();
+    if (serial) by_stages = sorted_down(tiles, [](const Tile& t) { return (int)t.nst; });
+    tiles = sorted_down(tiles, [](const Tile& t) {
+        const int rows = t.sn ? t.sn * 16 * t.sb : std::min(t.m - t.m0, TM);
+        return (int)((int64_t)t.nst * (64 + rows + std::min<int>(t.tn, t.n - t.n0)) / 64);
+    });
 }
 
 void TmaWorkList::upload(cudaStream_t st) {
@@ -1104,6 +1333,14 @@ void TmaWorkList::upload(cudaStream_t st) {
         cap_segs = segs.size() + 16;
         DMRG_CHECK_CUDA(cudaMalloc(&d_segs, cap_segs * sizeof(TSeg)));
     }
+    if (by_stages.size() > cap_stages) {
+        if (d_by_stages) cudaFree(d_by_stages);
+        cap_stages = by_stages.size() + 16;
+        DMRG_CHECK_CUDA(cudaMalloc(&d_by_stages, cap_stages * sizeof(Tile)));
+    }
+    if (!by_stages.empty())
+        DMRG_CHECK_CUDA(cudaMemcpyAsync(d_by_stages, by_stages.data(), by_stages.size() * sizeof(Tile),
+                                        cudaMemcpyHostToDevice, st));
     if (!tiles.empty())
         DMRG_CHECK_CUDA(cudaMemcpyAsync(d_tiles, tiles.data(), tiles.size() * sizeof(Tile), cudaMemcpyHostToDevice, st));
     if (!segs.empty())
@@ -1113,9 +1350,11 @@ void TmaWorkList::upload(cudaStream_t st) {
 void TmaWorkList::release() {
     if (d_tiles) cudaFree(d_tiles);
     if (d_segs) cudaFree(d_segs);
+    if (d_by_stages) cudaFree(d_by_stages);
     d_tiles = nullptr;
     d_segs = nullptr;
-    cap_tiles = cap_segs = 0;
+    d_by_stages = nullptr;
+    cap_tiles = cap_segs = cap_stages = 0;
 }
 
 int MapTable::get(const MapKey& k) {
@@ -1149,10 +1388,18 @@ EncodeTiledFn encode_fn() {
 }
 }  // namespace
 
-void MapTable::encode_upload(const TcBufs& tb, int nsplit, cudaStream_t st) {
+void MapTable::encode_upload(const TcBufs& tb, int nsplit, cudaStream_t st, bool serial) {
     const size_t n = kMapsPerKey * keys.size();
     std::vector<CUtensorMap> h(std::max<size_t>(n, 1));
     EncodeTiledFn fn = encode_fn();
+    const auto encode = [fn](CUtensorMap& map, int nd, const __nv_bfloat16* base, const cuuint64_t* dims,
+                             const cuuint64_t* strides, const cuuint32_t* box) {
+        const cuuint32_t estr[5] = {1, 1, 1, 1, 1};
+        const CUresult r = fn(&map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, nd, (void*)base, dims, strides, box, estr,
+                              CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+                              CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+        DMRG_REQUIRE(r == CUDA_SUCCESS, DMRG_ECUDA, "cuTensorMapEncodeTiled failed (" + std::to_string((int)r) + ")");
+    };
     for (size_t i = 0; i < keys.size(); ++i) {
         const MapKey& k = keys[i];
         for (int m = 0; m < kMapsPerKey; ++m) {
@@ -1173,13 +1420,29 @@ void MapTable::encode_upload(const TcBufs& tb, int nsplit, cudaStream_t st) {
                                            (cuuint64_t)pst * 2};
             const cuuint32_t box[5] = {64, tall ? 128u : (cuuint32_t)box_rows(k.rows), (cuuint32_t)k.bz, 1,
                                        (cuuint32_t)pieces};
-            const cuuint32_t estr[5] = {1, 1, 1, 1, 1};
-            const CUresult r = fn(&h[kMapsPerKey * i + m], CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 5, (void*)(base + k.off), dims,
-                                  strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
-                                  CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
-            DMRG_REQUIRE(r == CUDA_SUCCESS, DMRG_ECUDA, "cuTensorMapEncodeTiled failed (" + std::to_string((int)r) + ")");
+            encode(h[kMapsPerKey * i + m], 5, base + k.off, dims, strides, box);
         }
     }
+    // one piece per map, for launch_seg_gemm_serial (which runs no stacked products)
+    std::vector<CUtensorMap> h1(serial ? (size_t)nsplit * keys.size() : 0);
+    for (size_t i = 0; serial && i < keys.size(); ++i) {
+        const MapKey& k = keys[i];
+        if (k.bz > 1) continue;
+        const cuuint64_t dims[4] = {(cuuint64_t)k.cols, (cuuint64_t)k.rows, (cuuint64_t)k.nz, (cuuint64_t)k.nv};
+        const cuuint64_t strides[3] = {(cuuint64_t)k.ld * 2, (cuuint64_t)k.zstride * 2, (cuuint64_t)k.vstride * 2};
+        const cuuint32_t box[4] = {64, (cuuint32_t)box_rows(k.rows), 1, 1};
+        for (int pc = 0; pc < nsplit; ++pc) {
+            const __nv_bfloat16* base = pc == 0 ? tb.hi[k.buf] : tb.lo[k.buf] + (pc == 2 ? tb.pstride[k.buf] : 0);
+            encode(h1[(size_t)nsplit * i + pc], 4, base + k.off, dims, strides, box);
+        }
+    }
+    if (h1.size() > cap1) {
+        if (d_maps1) cudaFree(d_maps1);
+        cap1 = h1.size() + 64;
+        DMRG_CHECK_CUDA(cudaMalloc(&d_maps1, cap1 * sizeof(CUtensorMap)));
+    }
+    if (!h1.empty())
+        DMRG_CHECK_CUDA(cudaMemcpyAsync(d_maps1, h1.data(), h1.size() * sizeof(CUtensorMap), cudaMemcpyHostToDevice, st));
     if (n > cap) {
         if (d_maps) cudaFree(d_maps);
         cap = n + 64;
@@ -1205,8 +1468,9 @@ bool MapTable::stale(const TcBufs& tb) const {
 
 void MapTable::release() {
     if (d_maps) cudaFree(d_maps);
-    d_maps = nullptr;
-    cap = 0;
+    if (d_maps1) cudaFree(d_maps1);
+    d_maps = d_maps1 = nullptr;
+    cap = cap1 = 0;
     clear();
 }
 
@@ -1215,10 +1479,13 @@ void tc_prepare(int nsplit) {
     if (nsplit < 1 || nsplit > 3 || done[nsplit]) return;
     if (nsplit == 1) {
         DMRG_CHECK_CUDA(cudaFuncSetAttribute(tc_tma_kernel<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, Cfg3<1>::SMEM));
+        DMRG_CHECK_CUDA(cudaFuncSetAttribute(tc_serial_kernel<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, Cfg2<1>::SMEM));
     } else if (nsplit == 2) {
         DMRG_CHECK_CUDA(cudaFuncSetAttribute(tc_tma_kernel<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, Cfg3<2>::SMEM));
+        DMRG_CHECK_CUDA(cudaFuncSetAttribute(tc_serial_kernel<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, Cfg2<2>::SMEM));
     } else {
         DMRG_CHECK_CUDA(cudaFuncSetAttribute(tc_tma_kernel<3>, cudaFuncAttributeMaxDynamicSharedMemorySize, Cfg3<3>::SMEM));
+        DMRG_CHECK_CUDA(cudaFuncSetAttribute(tc_serial_kernel<3>, cudaFuncAttributeMaxDynamicSharedMemorySize, Cfg2<3>::SMEM));
     }
     done[nsplit] = true;
 }
@@ -1242,6 +1509,21 @@ void launch_seg_gemm_tma(const TmaWorkList& w, const MapTable& maps, const TcBuf
         tc_tma_kernel<1><<<grid, THREADS3, Cfg3<1>::SMEM, st>>>(w.d_tiles, (int)w.tiles.size(), nvec, w.d_segs,
                                                                 maps.d_maps, single, b);
     }
+    ++launch_counter();
+    DMRG_CHECK_CUDA(cudaGetLastError());
+}
+
+void launch_seg_gemm_serial(const TmaWorkList& w, const MapTable& maps, const TcBufs& b, int nvec, int nsplit,
+                            cudaStream_t st) {
+    tc_prepare(nsplit);
+    if (w.by_stages.empty()) return;
+    const int64_t total = (int64_t)w.by_stages.size() * nvec;
+    DMRG_REQUIRE(total < (1LL << 30), DMRG_EINVAL, "tensor-core work list too large");
+    DMRG_REQUIRE(maps.d_maps1 != nullptr, DMRG_EINVAL, "tensor maps not uploaded");
+    const int grid = (int)std::min<int64_t>(total, tc_num_sms()), n = (int)w.by_stages.size();
+    if (nsplit == 3) tc_serial_kernel<3><<<grid, THREADS4, Cfg2<3>::SMEM, st>>>(w.d_by_stages, n, nvec, w.d_segs, maps.d_maps1, b);
+    else if (nsplit == 2) tc_serial_kernel<2><<<grid, THREADS4, Cfg2<2>::SMEM, st>>>(w.d_by_stages, n, nvec, w.d_segs, maps.d_maps1, b);
+    else tc_serial_kernel<1><<<grid, THREADS4, Cfg2<1>::SMEM, st>>>(w.d_by_stages, n, nvec, w.d_segs, maps.d_maps1, b);
     ++launch_counter();
     DMRG_CHECK_CUDA(cudaGetLastError());
 }

@@ -841,6 +841,7 @@ void ProductList::lower_tma(int8_t sbuf_, int8_t ibuf, int ild, int64_t cap, int
     flops = 0.0;
     scratch_elems = 0;
     tc = true;
+    serial = cs.size() <= kSerialItems;
     View I;
     I.buf = ibuf;
     I.off = 0;
@@ -1141,7 +1142,7 @@ void ProductList::lower_tma(int8_t sbuf_, int8_t ibuf, int ild, int64_t cap, int
             p2.add_block(ob.off, ob.buf, ob.m, ob.n, ob.ldc, segs[o], out_mode, kchunk, 1.0f, tile_n);
         }
         p1.order_tiles();
-        p2.order_tiles();
+        p2.order_tiles(serial);
     });
     for (size_t ch = 0; ch < nch; ++ch) {
         flops += cfl[ch];
@@ -1155,12 +1156,13 @@ void ProductList::lower_tma(int8_t sbuf_, int8_t ibuf, int ild, int64_t cap, int
     maps.index.clear();
 }
 
-void ProductList::run_tma(const TcBufs& tb, int nvec, int nsplit, cudaStream_t st) {
+void ProductList::run_tma(const TcBufs& tb, int nvec, int nsplit, cudaStream_t st, bool repeatable) {
     for (auto& c : tchunks) {
         DMRG_REQUIRE(c.first.tiles.empty() || (sbuf >= 0 && tb.out[sbuf]), DMRG_EINVAL,
                      "tensor-core product list run without its scratch buffer");
         launch_seg_gemm_tma(c.first, maps, tb, nvec, nsplit, st);
-        launch_seg_gemm_tma(c.second, maps, tb, nvec, nsplit, st);
+        if (serial && repeatable) launch_seg_gemm_serial(c.second, maps, tb, nvec, nsplit, st);
+        else launch_seg_gemm_tma(c.second, maps, tb, nvec, nsplit, st);
     }
 }
 

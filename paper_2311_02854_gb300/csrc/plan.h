@@ -114,7 +114,9 @@ struct ProductList {
     // nv copies); the maps are encoded later by maps.encode_upload.
     void lower_tma(int8_t scratch_buf, int8_t ident_buf, int ident_ld, int64_t scratch_cap, int64_t kchunk,
                    uint8_t out_mode, const int64_t* vstride, int nv, int tile_n = 128);
-    void run_tma(const TcBufs& tb, int nvec, int nsplit, cudaStream_t st);
+    // repeatable: the K-chunks of short lists in an order that repeats (tc_serial_kernel)
+    void run_tma(const TcBufs& tb, int nvec, int nsplit, cudaStream_t st, bool repeatable = false);
+    bool serial = false;  // lower_tma: a list of up to kSerialItems products
     std::vector<std::pair<TmaWorkList, TmaWorkList>> tchunks;
     MapTable maps;
     void release();
@@ -222,7 +224,7 @@ struct Plan {
         cudaGraphExec_t exec = nullptr;
         int64_t launches = 0;
     };
-    std::map<int, SigmaGraph> sigma_graphs;
+    std::map<std::pair<int, bool>, SigmaGraph> sigma_graphs;  // (vectors, repeatable)
     cudaStream_t cap_stream = nullptr;
     double* d_sig_io = nullptr;  // [G x dim in | G x dim out]
     int64_t n_sig_io = 0;

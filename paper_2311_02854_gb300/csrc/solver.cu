@@ -172,7 +172,7 @@ void davidson_run(Plan& P, double* psi, int nr, double tol, int max_iter, int pr
     std::vector<double> ha((size_t)std::max(nr, 1) * 3);
     auto apply = [&](const double* Vb, double* Wb, int cnt) {
         if (!corr) {
-            sigma(P, Vb, Wb, cnt, st);
+            sigma(P, Vb, Wb, cnt, st, true);
             return;
         }
         const int q = corr->nr;
@@ -186,7 +186,7 @@ void davidson_run(Plan& P, double* psi, int nr, double tol, int max_iter, int pr
             dev_combine(corr->X, n, q, dco, n, tmp, st);
             dev_axpby(-1.0, tmp, 1.0, corr->proj + (int64_t)j * n, n, st);
         }
-        sigma(P, corr->proj, Wb, cnt, st);
+        sigma(P, corr->proj, Wb, cnt, st, true);
         for (int j = 0; j < cnt; ++j) {
             const double* v = Vb + (int64_t)j * n;
             double* w = Wb + (int64_t)j * n;

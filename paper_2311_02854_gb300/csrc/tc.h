@@ -72,6 +72,10 @@ struct TmaWorkList {
     TSeg* d_segs = nullptr;
     size_t cap_tiles = 0, cap_segs = 0;
     bool single = false;  // every tile has one segment (set by order_tiles)
+    // the tiles by stages alone, for launch_seg_gemm_serial (empty where that is not used)
+    std::vector<Tile> by_stages;
+    Tile* d_by_stages = nullptr;
+    size_t cap_stages = 0;
     // output block (m x n, ld ldc) at c_off of c_buf, 128 x tn tiles (tn = 64 or
     // 128), split into K-chunks of at most kchunk (atomic modes only); tr: stored
     // transposed (TC_STORE_SPLIT only)
@@ -81,7 +85,7 @@ struct TmaWorkList {
     // row: product i in accumulator rows i * 16 * sb ...
     void add_stack(int64_t c_off, int c_buf, int m, int n, int ldc, const TSeg& s, float alpha, int sn, int sb, int tn,
                    bool tr);
-    void order_tiles();  // longest tiles first (stable)
+    void order_tiles(bool serial = false);  // longest tiles first (stable); serial: by_stages too
     void upload(cudaStream_t st);
     void release();
 };
@@ -117,13 +121,15 @@ struct MapKeyEq {
 struct MapTable {
     std::vector<MapKey> keys;
     std::unordered_map<MapKey, int, MapKeyHash, MapKeyEq> index;
-    CUtensorMap* d_maps = nullptr;
-    size_t cap = 0;
+    CUtensorMap* d_maps = nullptr;   // kMapsPerKey per key
+    CUtensorMap* d_maps1 = nullptr;  // 4-D, one per piece and key (launch_seg_gemm_serial)
+    size_t cap = 0, cap1 = 0;
     const void* enc_ptr[kMaxBufs][3] = {};  // piece pointers the device maps were encoded with
     int get(const MapKey& k);  // validates alignment; returns the key index
     bool stale(const TcBufs& tb) const;  // a piece pointer moved since the last encode
-    // encode the maps of every key and copy them to the device
-    void encode_upload(const TcBufs& tb, int nsplit, cudaStream_t st);
+    // encode the maps of every key (serial: those of launch_seg_gemm_serial too) and copy
+    // them to the device
+    void encode_upload(const TcBufs& tb, int nsplit, cudaStream_t st, bool serial);
     void clear() {
         keys.clear();
         index.clear();
@@ -134,6 +140,11 @@ struct MapTable {
 // Launch the TMA-staged kernel over the tiles of `w` (maps on the device).
 void launch_seg_gemm_tma(const TmaWorkList& w, const MapTable& maps, const TcBufs& b, int nvec, int nsplit,
                          cudaStream_t st);
+// The same for the phase-2 tiles of lists of up to kSerialItems products, in an order of
+// arrival that repeats from call to call (see tc_serial_kernel).
+constexpr size_t kSerialItems = 1 << 18;
+void launch_seg_gemm_serial(const TmaWorkList& w, const MapTable& maps, const TcBufs& b, int nvec, int nsplit,
+                            cudaStream_t st);
 
 // FP64 -> bf16 pieces (hi, lo, optionally lo2), same layout, n elements, then
 // zeros up to n_pad (0: none); lo2 receives the third piece x - hi - lo

@@ -68,3 +68,66 @@ def test_first_products_fit_the_scratch_that_was_allowed(tmp_path, K, D, width):
             assert st["sigma_chunks"] > 1
         plan.close()
     assert held[0] <= held[1] + (256 << 10)
+
+
+def test_davidson_calls_repeat_and_match_fp64(tmp_path):
+    """Mixed Davidson on a short list: eight steps from a random vector, stopped unconverged.
+
+    Such a call makes any figure of its vector out of the last place of a sum, and the
+    FP64 additions of K-chunks come in an order that repeats, not in a fixed one: with the
+    schedule of short lists 1 call in 16 falls out (6 of 72 from its first call), with that
+    of long lists 1 in 4 (17 of 72).  Of 48 calls (six problems, eight each, every one
+    against the vector that most of its problem's calls agree on) 3 and 12 are expected;
+    7 may.  The energy is that of the vector in FP64 arithmetic: to 4.6e-5 of |H x|, the
+    bound of the mixed sigma."""
+    torch = cuda_torch()
+    g = gpu_lib()
+    K, D, k = 14, 600, 7
+    out = 0
+    for seed in (20, 27, 28, 30, 32, 39):
+        h, L = si.make_integrals(K, 4 * K, seed=2 * seed)
+        mps = si.random_mps(K, K, 0, si.bond_sectors(K, K, 0, D, "gaussian", 1.0, 1.0), center=k, seed=2 * seed + 1)
+        path = str(tmp_path / f"mps_{seed}.bin")
+        si.write_mps(path, mps)
+        plan = g.Plan(h, L, K, K, 0, D, path, precision=BF16X3, tc_kchunk=1024)
+        plan.set_bond(k)
+        gen = torch.Generator(device="cuda").manual_seed(seed)
+        x = torch.randn(plan.dim, dtype=torch.float64, device="cuda", generator=gen)
+        x /= x.norm()
+        got = []
+        for _ in range(8):
+            y = x.clone()
+            e, _, _ = plan.davidson(y, 1, tol=1e-10, max_iter=8)
+            got.append(y)
+        off = [sum(float((a - b).norm()) > 1e-9 for b in got) for a in got]
+        out += min(off)
+        hy = torch.empty_like(y)
+        plan.sigma_fp64(y, hy)
+        assert abs(e[0] - float(y @ hy)) <= 4.6e-5 * float(hy.norm())
+        plan.close()
+    print(f"{out} of 48 calls off")
+    assert out <= 7
+
+
+def test_short_and_long_lists_of_all_piece_counts(tmp_path):
+    """Davidson's own schedule of short lists against the one of dmrg_sigma: two steps from
+    a vector with every sector filled give Ritz values of the same matrix, each off by at
+    most the bound of the mixed sigma (4.6e-5 of |H x|; one piece 3e-2)."""
+    torch = cuda_torch()
+    g = gpu_lib()
+    for precision, bound in ((1, 4.6e-5), (2, 3e-2), (3, 1.5e-5)):
+        for K, D, k, tile_n in ((8, 64, 2, 0), (10, 100, 5, 64), (14, 600, 7, 0)):
+            h, L, _, path = make_case(tmp_path, K, K, 0, D, center=k, split="gaussian", wn=1.0, ws=1.0)
+            plan = g.Plan(h, L, K, K, 0, D, path, precision=precision, sigma_tile_n=tile_n)
+            plan.set_bond(k)
+            y = torch.from_numpy(si.random_vector(plan.dim, seed=3)).cuda()
+            hy = torch.empty_like(y)
+            y /= y.norm()
+            plan.sigma(y, hy)
+            z = y.clone()
+            e, _, _ = plan.davidson(z, 1, tol=1e-10, max_iter=1)  # the Ritz value of one vector: x H x
+            assert abs(e[0] - float(y @ hy)) <= 2 * bound * float(hy.norm())
+            e, _, _ = plan.davidson(z, 1, tol=1e-10, max_iter=2)
+            plan.sigma(z, hy)
+            assert abs(e[0] - float(z @ hy) / float(z @ z)) <= 2 * bound * float(hy.norm())
+            plan.close()
