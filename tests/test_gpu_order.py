@@ -131,3 +131,24 @@ def test_short_and_long_lists_of_all_piece_counts(tmp_path):
             plan.sigma(z, hy)
             assert abs(e[0] - float(z @ hy) / float(z @ z)) <= 2 * bound * float(hy.norm())
             plan.close()
+
+
+@pytest.mark.parametrize("K,D,width", [(12, 300, 1.0), (20, 300, 1.2)])
+def test_fp64_accurate_sigma_repeats(tmp_path, K, D, width):
+    """FP64_TC: sums up to 16384 deep are one addition, twice that two, in either order."""
+    torch = cuda_torch()
+    g = gpu_lib()
+    k = K // 2
+    h, L, _, path = make_case(tmp_path, K, K, 0, D, center=k, split="gaussian", wn=width, ws=width)
+    plan = g.Plan(h, L, K, K, 0, D, path, precision=FP64_TC)
+    plan.set_bond(k)
+    rng = np.random.default_rng(1)
+    x = np.ldexp(rng.standard_normal(plan.dim), rng.integers(-45, 1, plan.dim))  # partial sums of unlike size
+    x = torch.from_numpy(x).cuda()
+    first = None
+    for _ in range(12):
+        y = torch.empty_like(x)
+        plan.sigma(x, y)
+        first = y if first is None else first
+        assert torch.equal(y, first)
+    plan.close()
