@@ -112,8 +112,8 @@ typedef struct {
                                (tile width 128 or 64, phase-2 K-chunk) is picked per bond by
                                the estimated time of each candidate on a sample of the bond's
                                own work (every 8th output block with all of its products), so
-                               that a bond always gets the same shape; choices are cached by
-                               the bond's sector-size histogram; ignored when tc_kchunk > 0
+                               that a bond with the same sectors always gets the same shape
+                               (kept per bond for its last layout); ignored when tc_kchunk > 0
                                or sigma_tile_n > 0, and for lists of over 2^20 products (which
                                keep tile width 128 and the full K-chunk, the measured winner
                                there); default 1 */
@@ -196,10 +196,10 @@ typedef struct {
     int decim_sweeps32_last;      /* last decimation: FP32 sweeps before the FP64 ones (0: FP64 only) */
     int sigma_tile_n;             /* mixed sigma: tile width of the current bond's work lists */
     int64_t sigma_kchunk;         /* mixed sigma: phase-2 K-chunk of the current bond */
-    int64_t tunes;                /* autotuner runs (histograms not seen before) */
-    int64_t tune_hits;            /* bonds whose histogram was already tuned */
+    int64_t tunes;                /* estimates of the tile shape (new bonds or new sectors) */
+    int64_t tune_hits;            /* bonds set again with the sectors of the last estimate */
     double ms_tune;               /* wall time of all autotuner runs */
-    double tune_cand_ms[4];       /* last autotuner run: estimated sample time per candidate
+    double tune_cand_ms[4];       /* the last bond's estimated sample time per candidate
                                      (128 / K-chunk, 64 / K-chunk, 128 / half K-chunk, 64 / half) */
     double sigma_load_bytes[2][2];/* mixed sigma, one vector: operand bytes the tensor-core tiles
                                      load through TMA, [phase 1 / 2][other operands / phase-1

@@ -161,40 +161,16 @@ TcBufs sigma_bufs(Plan& P, int k, double* out) {
 // Tile-shape autotuner of the mixed sigma
 // ---------------------------------------------------------------------------
 
-// Key of the bond's sector-size histogram, coarse enough that the bonds of one
-// region of a sweep share it: the size classes (limits 16 ... 384) of the
-// largest row and column sector, the number of sectors, of psi elements and
-// of terms on a log2 scale, the piece count and the vectors per launch.
-uint64_t sector_histogram_key(const Plan& P, int G) {
-    static const int cuts[7] = {16, 32, 64, 128, 192, 256, 384};
-    auto cls = [&](int d) {
-        int c = 0;
-        while (c < 7 && d > cuts[c]) ++c;
-        return c;
-    };
-    auto lg = [](int64_t x) {
-        int l = 0;
-        while (((int64_t)1 << l) <= x) ++l;
-        return l;
-    };
-    int dl = 0, dr = 0;
-    for (const Plan::Sector& s : P.layout) {
-        dl = std::max(dl, s.dl);
-        dr = std::max(dr, s.dr);
+// What the estimate depends on at a bond of this plan: the sectors of the two blocks and
+// of psi (the terms are those of the bond, the vectors per launch the plan's).
+std::vector<int> shape_key(const Plan& P, int k) {
+    std::vector<int> key;
+    for (int at : {k - 1, k + 1}) {
+        for (const auto& b : P.mps.bonds[at]) key.insert(key.end(), b.begin(), b.end());
+        key.push_back(-1);
     }
-    uint64_t h = 1469598103934665603ull;
-    auto mix = [&](uint64_t x) {
-        h ^= x;
-        h *= 1099511628211ull;
-    };
-    mix((uint64_t)P.nsplit);
-    mix((uint64_t)G);
-    mix((uint64_t)cls(dl));
-    mix((uint64_t)cls(dr));
-    mix((uint64_t)lg((int64_t)P.layout.size()));
-    mix((uint64_t)lg(P.dim));
-    mix((uint64_t)lg((int64_t)P.sp.terms.size()));
-    return h;
+    for (const Plan::Sector& s : P.layout) key.insert(key.end(), {s.il, s.y, s.ir, s.dl, s.dr});
+    return key;
 }
 
 struct SigmaShape {
@@ -214,12 +190,13 @@ struct SigmaShape {
 // bond, and near a tie it chose by noise, so that one bond's sigma differed by
 // the FP32 rounding of the other chain length (3e-6) from run to run.  The
 // fastest wins, the default (128, kmax) unless another is 0.5 % faster.
-SigmaShape tune_sigma_shape(Plan& P, const ProductList& tl, int64_t kmax, int G) {
-    const uint64_t key = sector_histogram_key(P, G);
-    auto f = P.tune_cache.find(key);
-    if (f != P.tune_cache.end()) {
+SigmaShape tune_sigma_shape(Plan& P, int bond, const ProductList& tl, int64_t kmax) {
+    Plan::TunedShape& f = P.tuned[bond];
+    std::vector<int> key = shape_key(P, bond);
+    if (f.layout == key) {
         ++P.stats.tune_hits;
-        return {f->second.first, f->second.second};
+        std::copy(f.cand_ms, f.cand_ms + 4, P.stats.tune_cand_ms);
+        return {f.tn, f.kchunk};
     }
     const auto t0 = std::chrono::steady_clock::now();
     constexpr int kSMs = 152;
@@ -286,7 +263,10 @@ SigmaShape tune_sigma_shape(Plan& P, const ProductList& tl, int64_t kmax, int G)
             bi = x;
         }
     }
-    P.tune_cache[key] = {cand[bi].tn, cand[bi].kchunk};
+    f.layout = std::move(key);
+    f.tn = cand[bi].tn;
+    f.kchunk = cand[bi].kchunk;
+    std::copy(P.stats.tune_cand_ms, P.stats.tune_cand_ms + 4, f.cand_ms);
     ++P.stats.tunes;
     P.stats.ms_tune += std::chrono::duration<double, std::milli>(std::chrono::steady_clock::now() - t0).count();
     return cand[bi];
@@ -1022,7 +1002,7 @@ void set_bond(Plan& P, int k) {
         double t_tune = 0.0;
         if (tune_later) {
             const auto c0 = std::chrono::steady_clock::now();
-            shape = tune_sigma_shape(P, tl, shape.kchunk, G);
+            shape = tune_sigma_shape(P, k, tl, shape.kchunk);
             t_tune = host_ms_since(c0);
             lower_and_count();
         }

@@ -238,8 +238,14 @@ struct Plan {
         int64_t stages;
     };
     std::vector<SigmaEvents> sig_pending;
-    // tile-shape autotuner: sector-size histogram key -> (tile width, phase-2 K-chunk)
-    std::map<uint64_t, std::pair<int, int64_t>> tune_cache;
+    // tile-shape estimate of a bond's last layout (what the estimate depends on)
+    struct TunedShape {
+        std::vector<int> layout;
+        int tn;
+        int64_t kchunk;
+        double cand_ms[4];
+    };
+    std::map<int, TunedShape> tuned;  // by bond
     std::vector<cudaEvent_t> ev_pool;
     cudaEvent_t take_event();
     void collect_sigma_times(bool wait);

@@ -152,3 +152,29 @@ def test_fp64_accurate_sigma_repeats(tmp_path, K, D, width):
         first = y if first is None else first
         assert torch.equal(y, first)
     plan.close()
+
+
+@pytest.mark.parametrize("K,D,width", [(10, 60, 1.0), (14, 400, 1.2)])
+def test_tile_shape_does_not_depend_on_the_way_to_a_bond(tmp_path, K, D, width):
+    """A plan that has come through the chain and a new one at the same bond (same sectors)
+    choose the same tile shape, and say the same of the candidates."""
+    torch = cuda_torch()
+    g = gpu_lib()
+    h, L, _, path = make_case(tmp_path, K, K, 0, D, center=2, split="gaussian", wn=width, ws=width)
+    plan = g.Plan(h, L, K, K, 0, D, path, precision=BF16X3)
+    plan.set_bond(2)
+    for k in range(2, K - 2):
+        x = torch.from_numpy(si.random_vector(plan.dim, seed=k)).cuda()
+        room = torch.zeros(8 * plan.dim + 65536, dtype=torch.float64, device="cuda")
+        plan.decimate(x, 1, D, True, next_psi=room, next_cap=room.numel())
+        plan.set_bond(k + 1)
+        here = str(tmp_path / "here.bin")
+        plan.save_mps(here)
+        fresh = g.Plan(h, L, K, K, 0, D, here, precision=BF16X3)
+        fresh.set_bond(k + 1)
+        a, b = plan.stats(), fresh.stats()
+        assert plan.dim == fresh.dim
+        for name in ("sigma_tile_n", "sigma_kchunk", "tune_cand_ms"):
+            assert a[name] == b[name], (k + 1, name)
+        fresh.close()
+    plan.close()
