@@ -99,18 +99,10 @@ double host_ms_since(std::chrono::steady_clock::time_point t0) {
     return std::chrono::duration<double, std::milli>(std::chrono::steady_clock::now() - t0).count();
 }
 
-void ensure_counter(Plan& P) {
-    if (!P.d_ctr) {
-        DMRG_CHECK_CUDA(cudaMalloc(&P.d_ctr, 2 * sizeof(int)));
-        DMRG_CHECK_CUDA(cudaMemset(P.d_ctr, 0, 2 * sizeof(int)));
-    }
-}
-
 TcBufs tc_base(Plan& P) {
-    ensure_counter(P);
     TcBufs tb{};
+    tb.err = P.error_word();
     tb.counter = P.d_ctr;
-    tb.err = P.d_ctr + 1;
     return tb;
 }
 
@@ -428,6 +420,7 @@ void form_interms(Plan& P, Interms& im, const Block* blocks[2], IntermStore& S, 
         bt.p[BUF_R] = blocks[1] ? blocks[1]->d : nullptr;
         bt.p[BUF_INT] = S.d;
         bt.p[BUF_W] = P.d_wcoef;
+        bt.err = P.error_word();
         launch_seg_gemm_f64(wl, bt, 1, P.stream);
         if (P.mixed()) dev_split_f64_flat(S.d, S.n, S.h, S.l, P.stream, P.lo2(S.l, S.n));
     }
@@ -692,6 +685,7 @@ std::unique_ptr<Block> renormalise(Plan& P, const Block& X, int m, bool forward)
         bt.p[BUF_PSI] = A.d;
         bt.p[BUF_SCR] = P.d_scratch;
         bt.p[BUF_ID] = P.d_ident;
+        bt.err = P.error_word();
         pl.run(bt, 1, P.stream);
         if (P.mixed()) {  // bf16 pieces of the FP64 store for the tensor-core sigma
             P.alloc_pieces(out->n, out->h, out->l);
@@ -1131,6 +1125,7 @@ void set_bond(Plan& P, int k) {
     }
     P.stats.ms_host_plan += plan_ms + host_ms_since(hs0);
     P.drop_graphs();  // captured for the previous bond's work lists
+    P.check_device_error();
     P.bond = k;
     DMRG_CHECK_CUDA(cudaStreamSynchronize(P.stream));
 }
@@ -1162,6 +1157,7 @@ BufTable bond_buffers(Plan& P, const double* psi, double* out) {
     bt.p[BUF_SCR] = P.d_scratch;
     bt.p[BUF_ID] = P.d_ident;
     bt.p[BUF_OUT] = out;
+    bt.err = P.error_word();
     bt.vstride[BUF_PSI] = P.dim;
     bt.vstride[BUF_OUT] = P.dim;
     bt.vstride[BUF_SCR] = P.sigma_pl.scratch_elems;
@@ -1194,6 +1190,7 @@ void sigma_fp64(Plan& P, const double* psi, double* out, int nvec, cudaStream_t 
     cudaEventElapsedTime(&ms, e0, e1);
     P.ev_pool.push_back(e0);
     P.ev_pool.push_back(e1);
+    if (P.oz) P.check_device_error();
     P.stats.sigma_acc_calls += nvec;
     P.stats.ms_sigma_acc += ms;
     P.stats.sigma_acc_flops += P.sigma_pl.flops * nvec;

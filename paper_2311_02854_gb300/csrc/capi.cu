@@ -704,10 +704,15 @@ dmrg_status dmrg_grouped_gemm(int precision, int n_out, const int* m, const int*
         bt.p[0] = const_cast<double*>(a);
         bt.p[1] = const_cast<double*>(b);
         bt.p[2] = c;
+        int err = 0;
+        if (precision == DMRG_FP64_TC) {  // the call's own word: calls of other threads have theirs
+            bt.err = ar.get<int>(1);
+            DMRG_CHECK_CUDA(cudaMemsetAsync(bt.err, 0, sizeof(int), st));
+        }
         launch_seg_gemm_f64(wl, bt, 1, st);
+        if (bt.err) DMRG_CHECK_CUDA(cudaMemcpyAsync(&err, bt.err, sizeof(int), cudaMemcpyDeviceToHost, st));
         DMRG_CHECK_CUDA(cudaStreamSynchronize(st));
-        if (precision == DMRG_FP64_TC && oz_take_error(st))
-            return fail(nullptr, DMRG_ETIMEOUT, "the FP64 tensor-core engine gave up waiting");
+        if (err) return fail(nullptr, DMRG_ETIMEOUT, "the FP64 tensor-core engine gave up waiting");
         return DMRG_OK;
     } catch (const Error& e) {
         return fail(nullptr, e.code, e.what());

@@ -56,6 +56,7 @@ struct BufTable {
     const void* lo[kMaxBufs];
     int64_t pstride[kMaxBufs];  // three pieces: piece 2 at lo + pstride (0: none)
     uint32_t pmask;
+    int* err;  // FP64-accurate tensor-core lists: the word set when a bounded wait gives up
 };
 
 // A work list in host memory plus its device copy.
@@ -97,14 +98,10 @@ struct WorkList {
 void launch_seg_gemm_f64(const WorkList& w, const BufTable& bt, int nvec, cudaStream_t st);
 // FP64-accurate products on the bf16 tensor cores (kernels_oz.cu): work lists
 // lowered with oz_tile_rows() x oz_tile_cols() tiles over FP64 buffers
-void launch_seg_gemm_oz(const WorkList& w, const BufTable& bt, int nvec, int* d_err, cudaStream_t st);
+void launch_seg_gemm_oz(const WorkList& w, const BufTable& bt, int nvec, cudaStream_t st);
 int oz_tile_rows();
 int oz_tile_cols();
 int oz_stage_depth();
-// device error word of the FP64 tensor-core engine (set when a bounded wait
-// gave up); oz_take_error reads and clears it (synchronises the stream)
-int* oz_error_word();
-bool oz_take_error(cudaStream_t st);
 // FP64 grouped GEMM with the work list in a static device array (noalloc.cu);
 // a, b, c as buffers 0, 1, 2 of the work list
 void grouped_gemm_f64_noalloc(WorkList& host_wl, const double* a, const double* b, double* c, cudaStream_t st);

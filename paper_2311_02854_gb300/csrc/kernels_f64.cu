@@ -483,7 +483,7 @@ __global__ void __launch_bounds__(2 * kOuter)
 void launch_seg_gemm_f64(const WorkList& w, const BufTable& bt, int nvec, cudaStream_t st) {
     if (w.tiles.empty()) return;
     if (w.tile_m == oz_tile_rows() && !w.rank1) {
-        launch_seg_gemm_oz(w, bt, nvec, oz_error_word(), st);
+        launch_seg_gemm_oz(w, bt, nvec, st);
         return;
     }
     DMRG_REQUIRE(w.tile_m == 0, DMRG_EINVAL, "work list tile shape not runnable on the FP64 engine");

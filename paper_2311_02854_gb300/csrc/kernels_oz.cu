@@ -155,7 +155,7 @@ __device__ __forceinline__ float pow2f(int k) {
 
 __global__ void __launch_bounds__(OZ_THREADS, 1)
     oz_gemm_kernel(const Tile* __restrict__ tiles, int ntiles, int nvec, int single, const Seg* __restrict__ segs,
-                   BufTable bt, int* err) {
+                   BufTable bt) {
     extern __shared__ uint8_t smem_raw[];
     // full[h]: loaders -> MMA (slices of K half h and the stage record written);
     // rec[h]: MMA -> epilogue (record visible); done[h]: MMA completion -> loaders
@@ -467,7 +467,7 @@ __global__ void __launch_bounds__(OZ_THREADS, 1)
             }
         }
     }
-    if (failed) atomicExch(err, 1);
+    if (failed) atomicExch(bt.err, 1);
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
@@ -480,28 +480,11 @@ int oz_tile_rows() { return OTM; }
 int oz_tile_cols() { return OTN; }
 int oz_stage_depth() { return OTK; }
 
-int* oz_error_word() {
-    static int* d = nullptr;
-    if (!d) {
-        DMRG_CHECK_CUDA(cudaMalloc(&d, sizeof(int)));
-        DMRG_CHECK_CUDA(cudaMemset(d, 0, sizeof(int)));
-    }
-    return d;
-}
-
-bool oz_take_error(cudaStream_t st) {
-    int* d = oz_error_word();
-    int h = 0;
-    DMRG_CHECK_CUDA(cudaMemcpyAsync(&h, d, sizeof(int), cudaMemcpyDeviceToHost, st));
-    DMRG_CHECK_CUDA(cudaStreamSynchronize(st));
-    if (h) DMRG_CHECK_CUDA(cudaMemsetAsync(d, 0, sizeof(int), st));
-    return h != 0;
-}
-
-void launch_seg_gemm_oz(const WorkList& w, const BufTable& bt, int nvec, int* d_err, cudaStream_t st) {
+void launch_seg_gemm_oz(const WorkList& w, const BufTable& bt, int nvec, cudaStream_t st) {
     if (w.tiles.empty()) return;
     DMRG_REQUIRE(w.tile_m == OTM && w.tile_n == OTN, DMRG_EINVAL, "work list not lowered for the FP64 tensor-core engine");
     DMRG_REQUIRE(bt.pmask == 0, DMRG_EINVAL, "the FP64 tensor-core engine reads FP64 buffers only");
+    DMRG_REQUIRE(bt.err != nullptr, DMRG_EINVAL, "the FP64 tensor-core engine needs an error word");
     const int64_t total = (int64_t)w.tiles.size() * nvec;
     DMRG_REQUIRE(total < (1LL << 31), DMRG_EINVAL, "work list too large for one launch");
     static bool attr = false;
@@ -513,8 +496,7 @@ void launch_seg_gemm_oz(const WorkList& w, const BufTable& bt, int nvec, int* d_
     DMRG_CHECK_CUDA(cudaGetDevice(&dev));
     DMRG_CHECK_CUDA(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev));
     const int grid = (int)std::min<int64_t>(total, std::max(nsm, 1));
-    oz_gemm_kernel<<<grid, OZ_THREADS, OZ_SMEM, st>>>(w.d_tiles, (int)w.tiles.size(), nvec, (int)w.single, w.d_segs, bt,
-                                                       d_err);
+    oz_gemm_kernel<<<grid, OZ_THREADS, OZ_SMEM, st>>>(w.d_tiles, (int)w.tiles.size(), nvec, (int)w.single, w.d_segs, bt);
     ++launch_counter();
     DMRG_CHECK_CUDA(cudaGetLastError());
 }

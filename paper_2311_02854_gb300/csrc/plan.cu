@@ -227,9 +227,15 @@ void Plan::free_bf16(__nv_bfloat16*& p, int64_t n) {
     p = nullptr;
 }
 
+int* Plan::error_word() {
+    if (!d_ctr) {
+        DMRG_CHECK_CUDA(cudaMalloc(&d_ctr, 2 * sizeof(int)));
+        DMRG_CHECK_CUDA(cudaMemsetAsync(d_ctr, 0, 2 * sizeof(int), stream));
+    }
+    return d_ctr + 1;
+}
+
 void Plan::check_device_error() {
-    if (oz && oz_take_error(stream))
-        throw Error(DMRG_ETIMEOUT, "the FP64 tensor-core engine gave up waiting (device error word set)");
     if (!d_ctr) return;
     int err = 0;
     DMRG_CHECK_CUDA(cudaMemcpyAsync(&err, d_ctr + 1, sizeof(int), cudaMemcpyDeviceToHost, stream));

@@ -215,7 +215,7 @@ struct Plan {
     int64_t n_wpc = 0;
     SplitJob* d_psi_jobs = nullptr;
     int n_psi_jobs = 0;
-    int* d_ctr = nullptr;  // [0] tile counter, [1] device error word
+    int* d_ctr = nullptr;  // [0] tile counter, [1] device error word (all tensor-core engines)
     bool sigma_fp64_ready = false;
 
     // CUDA graphs of the mixed sigma, per number of vectors in a launch, for the
@@ -296,7 +296,8 @@ struct Plan {
     }
     // piece 2 of a lo array of n elements per piece (null unless three pieces)
     __nv_bfloat16* lo2(__nv_bfloat16* lo, int64_t n) const { return (nsplit == 3 && lo) ? lo + n : nullptr; }
-    void check_device_error();
+    int* error_word();  // d_ctr + 1, allocated on first use
+    void check_device_error();  // waits for the stream; throws if a kernel of the plan gave up waiting
     ~Plan();
 };
 

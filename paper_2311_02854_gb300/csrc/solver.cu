@@ -173,6 +173,7 @@ void davidson_run(Plan& P, double* psi, int nr, double tol, int max_iter, int pr
     auto apply = [&](const double* Vb, double* Wb, int cnt) {
         if (!corr) {
             sigma(P, Vb, Wb, cnt, st, true);
+            if (P.oz && !P.mixed()) P.check_device_error();  // (a mixed sigma has done so)
             return;
         }
         const int q = corr->nr;
@@ -661,6 +662,7 @@ void decimate(Plan& P, const double* psi, int nr, int Dmax, bool forward, double
     BufTable bt{};
     bt.p[BUF_PSI] = const_cast<double*>(psi);
     bt.p[BUF_OUT] = d_rho;
+    bt.err = P.error_word();
     const auto hd0 = std::chrono::steady_clock::now();
     launch_seg_gemm_f64(wl, bt, 1, st);
     DMRG_CHECK_CUDA(cudaStreamSynchronize(st));
@@ -925,6 +927,7 @@ void decimate(Plan& P, const double* psi, int nr, int Dmax, bool forward, double
         b2.p[BUF_SCR] = P.d_scratch;
         b2.p[BUF_ID] = P.d_ident;
         b2.p[BUF_OUT] = next_psi;
+        b2.err = P.error_word();
         b2.vstride[BUF_PSI] = old_dim;
         b2.vstride[BUF_OUT] = ndim;
         b2.vstride[BUF_SCR] = std::max<int64_t>(pl.scratch_elems, 1);
@@ -1003,6 +1006,7 @@ void two_site_guess(Plan& P, double* out) {
     bt.p[BUF_L] = da;
     bt.p[BUF_R] = db;
     bt.p[BUF_OUT] = out;
+    bt.err = P.error_word();
     launch_seg_gemm_f64(wl, bt, 1, st);
     DMRG_CHECK_CUDA(cudaStreamSynchronize(st));
     wl.release();

@@ -1,4 +1,6 @@
 """Sums whose order is part of the result, and the resources a call may take."""
+import subprocess
+import sys
 from fractions import Fraction
 
 import numpy as np
@@ -178,3 +180,35 @@ def test_tile_shape_does_not_depend_on_the_way_to_a_bond(tmp_path, K, D, width):
             assert a[name] == b[name], (k + 1, name)
         fresh.close()
     plan.close()
+
+
+FIRST_CALLS = """
+import sys, threading
+import numpy as np, torch
+import paper_2311_02854_gb300 as g
+rng = np.random.default_rng(4)
+A, B = (torch.from_numpy(rng.standard_normal(48 * 96)).cuda() for _ in range(2))
+blocks = [(48, 48, 0, [(96, 0, 96, 0, 0, 48, 0, 1.0)])]
+C = [torch.full((48 * 48,), float("nan"), dtype=torch.float64, device="cuda") for _ in range(6)]
+torch.cuda.synchronize()
+start = threading.Barrier(6)
+def run(i):
+    st = torch.cuda.Stream()
+    start.wait()
+    for _ in range(20):
+        g.grouped_gemm(4, blocks, A, B, C[i], stream=st)
+ts = [threading.Thread(target=run, args=(i,)) for i in range(6)]
+[t.start() for t in ts], [t.join() for t in ts]
+want = A.view(48, 96) @ B.view(96, 48)
+for c in C:
+    assert torch.equal(c, C[0])
+    assert float((c.view(48, 48) - want).norm() / want.norm()) < 1e-12
+print("ok")
+"""
+
+
+def test_first_fp64_accurate_products_of_several_threads():
+    """Each call has an error word of its own: nothing is set up by whoever comes first."""
+    cuda_torch()
+    r = subprocess.run([sys.executable, "-c", FIRST_CALLS], capture_output=True, text=True, timeout=300)
+    assert r.returncode == 0 and r.stdout.strip() == "ok", r.stderr[-2000:]
