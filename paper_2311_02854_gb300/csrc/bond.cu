@@ -1020,7 +1020,7 @@ void set_bond(Plan& P, int k) {
             jobs.push_back({s.off, s.poff, s.dl, s.dr, s.dr, (int)round_up(s.dr, 8)});
         if (P.d_psi_jobs) cudaFree(P.d_psi_jobs);
         P.n_psi_jobs = (int)jobs.size();
-        DMRG_CHECK_CUDA(cudaMalloc(&P.d_psi_jobs, std::max<size_t>(jobs.size(), 1) * sizeof(SplitJob)));
+        DMRG_CHECK_CUDA(dev_malloc(&P.d_psi_jobs, std::max<size_t>(jobs.size(), 1) * sizeof(SplitJob)));
         if (!jobs.empty())
             DMRG_CHECK_CUDA(cudaMemcpyAsync(P.d_psi_jobs, jobs.data(), jobs.size() * sizeof(SplitJob),
                                             cudaMemcpyHostToDevice, P.stream));
@@ -1116,8 +1116,8 @@ void set_bond(Plan& P, int k) {
         cudaFree(m.d_sec_off);
         cudaFree(m.d_sec_q);
         m.n_sec = (int)std::max<size_t>(P.layout.size(), 1);
-        DMRG_CHECK_CUDA(cudaMalloc(&m.d_sec_off, off.size() * sizeof(int64_t)));
-        DMRG_CHECK_CUDA(cudaMalloc(&m.d_sec_q, q.size() * sizeof(float)));
+        DMRG_CHECK_CUDA(dev_malloc(&m.d_sec_off, off.size() * sizeof(int64_t)));
+        DMRG_CHECK_CUDA(dev_malloc(&m.d_sec_q, q.size() * sizeof(float)));
         DMRG_CHECK_CUDA(cudaMemcpyAsync(m.d_sec_off, off.data(), off.size() * sizeof(int64_t), cudaMemcpyHostToDevice,
                                         P.stream));
         DMRG_CHECK_CUDA(

@@ -256,6 +256,7 @@ dmrg_status dmrg_plan(const double* h, const double* chol, int n_chol, double e_
             P.mps.bonds[K][0][1] != twoS)
             throw Error(DMRG_EINVAL, "MPS boundary sectors do not match the quantum numbers");
         size_t freeb = 0, totb = 0;
+        trim_product_pool();
         DMRG_CHECK_CUDA(cudaMemGetInfo(&freeb, &totb));
         P.budget = P.opt.mem_budget > 0 ? P.opt.mem_budget : (int64_t)(0.9 * (double)freeb);
         const int64_t K2 = (int64_t)K * K;

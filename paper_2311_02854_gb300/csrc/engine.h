@@ -136,11 +136,18 @@ void dev_perturb(double* x, int64_t n, uint32_t seed, double amp, cudaStream_t s
 void dev_identity(double* x, int n, cudaStream_t st);
 int64_t& launch_counter();
 // Pool of the grouped products' device memory on the current device: it keeps up
-// to kPoolKeep bytes between calls (any stream, any thread) and gives them back
-// when an allocation of a plan fails (trim_product_pool)
+// to kPoolKeep bytes between calls (any stream, any thread).  It gives them back
+// (trim_product_pool) when a plan is made, before the plan's budget is taken from the
+// free memory, and when any device allocation of a plan fails (dev_malloc).
 constexpr uint64_t kPoolKeep = 1ull << 30;
 cudaMemPool_t product_pool();
 void trim_product_pool();
+// cudaMalloc, once more without what the pool keeps if it fails
+cudaError_t dev_malloc_bytes(void** p, size_t bytes);
+template <typename T>
+cudaError_t dev_malloc(T** p, size_t bytes) {
+    return dev_malloc_bytes((void**)p, bytes);
+}
 // selftest.cu: one bounded mbarrier wait (arrived on or not); false if it gave up
 bool wait_selftest(double seconds, bool arrive, cudaStream_t st);
 

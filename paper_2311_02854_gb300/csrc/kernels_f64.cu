@@ -166,12 +166,12 @@ void WorkList::upload(cudaStream_t st) {
     if (tiles.size() > cap_tiles) {
         if (d_tiles) cudaFree(d_tiles);
         cap_tiles = tiles.size() + tiles.size() / 4 + 16;
-        DMRG_CHECK_CUDA(cudaMalloc(&d_tiles, cap_tiles * sizeof(Tile)));
+        DMRG_CHECK_CUDA(dev_malloc(&d_tiles, cap_tiles * sizeof(Tile)));
     }
     if (segs.size() > cap_segs) {
         if (d_segs) cudaFree(d_segs);
         cap_segs = segs.size() + segs.size() / 4 + 16;
-        DMRG_CHECK_CUDA(cudaMalloc(&d_segs, cap_segs * sizeof(Seg)));
+        DMRG_CHECK_CUDA(dev_malloc(&d_segs, cap_segs * sizeof(Seg)));
     }
     if (!tiles.empty())
         DMRG_CHECK_CUDA(cudaMemcpyAsync(d_tiles, tiles.data(), tiles.size() * sizeof(Tile),

@@ -266,10 +266,10 @@ void Mlp::release() {
 
 void mlp_init(Mlp& m, uint32_t seed, cudaStream_t st) {
     if (!m.d_w) {
-        DMRG_CHECK_CUDA(cudaMalloc(&m.d_w, kMlpParams * sizeof(float)));
-        DMRG_CHECK_CUDA(cudaMalloc(&m.d_wb, kMlpParams * sizeof(__nv_bfloat16)));
-        DMRG_CHECK_CUDA(cudaMalloc(&m.d_adam, 2 * kMlpParams * sizeof(float)));
-        DMRG_CHECK_CUDA(cudaMalloc(&m.d_grad, (kMlpParams + 1) * sizeof(float)));
+        DMRG_CHECK_CUDA(dev_malloc(&m.d_w, kMlpParams * sizeof(float)));
+        DMRG_CHECK_CUDA(dev_malloc(&m.d_wb, kMlpParams * sizeof(__nv_bfloat16)));
+        DMRG_CHECK_CUDA(dev_malloc(&m.d_adam, 2 * kMlpParams * sizeof(float)));
+        DMRG_CHECK_CUDA(dev_malloc(&m.d_grad, (kMlpParams + 1) * sizeof(float)));
     }
     // uniform draws from a counter-based generator (splitmix64 of seed and index)
     std::vector<float> w(kMlpParams, 0.f);
@@ -312,7 +312,7 @@ void ensure_work(Mlp& m, int64_t B) {
     if (B <= m.cap_work) return;
     cudaFree(m.d_work);
     m.cap_work = B;
-    DMRG_CHECK_CUDA(cudaMalloc(&m.d_work, (size_t)B * kWorkRow * sizeof(float)));
+    DMRG_CHECK_CUDA(dev_malloc(&m.d_work, (size_t)B * kWorkRow * sizeof(float)));
 }
 
 void gradient_batch(Mlp& m, const float* x, const float* y, const float* wt, int64_t n_set, int64_t B,
@@ -386,9 +386,9 @@ int64_t mlp_collect(Mlp& m, const double* hd, const double* r, const double* t, 
     if (m.n_set + take > m.cap_set) {  // grow the set
         const int64_t cap = std::max<int64_t>(2 * m.cap_set, m.n_set + take);
         float *nx = nullptr, *ny = nullptr, *nw = nullptr;
-        DMRG_CHECK_CUDA(cudaMalloc(&nx, (size_t)cap * kMlpIn * sizeof(float)));
-        DMRG_CHECK_CUDA(cudaMalloc(&ny, (size_t)cap * sizeof(float)));
-        DMRG_CHECK_CUDA(cudaMalloc(&nw, (size_t)cap * sizeof(float)));
+        DMRG_CHECK_CUDA(dev_malloc(&nx, (size_t)cap * kMlpIn * sizeof(float)));
+        DMRG_CHECK_CUDA(dev_malloc(&ny, (size_t)cap * sizeof(float)));
+        DMRG_CHECK_CUDA(dev_malloc(&nw, (size_t)cap * sizeof(float)));
         if (m.n_set > 0) {
             DMRG_CHECK_CUDA(cudaMemcpyAsync(nx, m.d_x, (size_t)m.n_set * kMlpIn * sizeof(float),
                                             cudaMemcpyDeviceToDevice, st));
@@ -406,8 +406,8 @@ int64_t mlp_collect(Mlp& m, const double* hd, const double* r, const double* t, 
     }
     int* flag = nullptr;
     float *xs = nullptr, *ys = nullptr, *ws = nullptr;
-    DMRG_CHECK_CUDA(cudaMalloc(&flag, (size_t)take * 2 * sizeof(int)));
-    DMRG_CHECK_CUDA(cudaMalloc(&xs, (size_t)take * (kMlpIn + 2) * sizeof(float)));
+    DMRG_CHECK_CUDA(dev_malloc(&flag, (size_t)take * 2 * sizeof(int)));
+    DMRG_CHECK_CUDA(dev_malloc(&xs, (size_t)take * (kMlpIn + 2) * sizeof(float)));
     ys = xs + (size_t)take * kMlpIn;
     ws = ys + take;
     const int blocks = (int)((take + NT - 1) / NT);

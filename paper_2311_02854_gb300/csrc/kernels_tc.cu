@@ -1326,17 +1326,17 @@ void TmaWorkList::upload(cudaStream_t st) {
     if (tiles.size() > cap_tiles) {
         if (d_tiles) cudaFree(d_tiles);
         cap_tiles = tiles.size() + 16;
-        DMRG_CHECK_CUDA(cudaMalloc(&d_tiles, cap_tiles * sizeof(Tile)));
+        DMRG_CHECK_CUDA(dev_malloc(&d_tiles, cap_tiles * sizeof(Tile)));
     }
     if (segs.size() > cap_segs) {
         if (d_segs) cudaFree(d_segs);
         cap_segs = segs.size() + 16;
-        DMRG_CHECK_CUDA(cudaMalloc(&d_segs, cap_segs * sizeof(TSeg)));
+        DMRG_CHECK_CUDA(dev_malloc(&d_segs, cap_segs * sizeof(TSeg)));
     }
     if (by_stages.size() > cap_stages) {
         if (d_by_stages) cudaFree(d_by_stages);
         cap_stages = by_stages.size() + 16;
-        DMRG_CHECK_CUDA(cudaMalloc(&d_by_stages, cap_stages * sizeof(Tile)));
+        DMRG_CHECK_CUDA(dev_malloc(&d_by_stages, cap_stages * sizeof(Tile)));
     }
     if (!by_stages.empty())
         DMRG_CHECK_CUDA(cudaMemcpyAsync(d_by_stages, by_stages.data(), by_stages.size() * sizeof(Tile),
@@ -1439,14 +1439,14 @@ void MapTable::encode_upload(const TcBufs& tb, int nsplit, cudaStream_t st, bool
     if (h1.size() > cap1) {
         if (d_maps1) cudaFree(d_maps1);
         cap1 = h1.size() + 64;
-        DMRG_CHECK_CUDA(cudaMalloc(&d_maps1, cap1 * sizeof(CUtensorMap)));
+        DMRG_CHECK_CUDA(dev_malloc(&d_maps1, cap1 * sizeof(CUtensorMap)));
     }
     if (!h1.empty())
         DMRG_CHECK_CUDA(cudaMemcpyAsync(d_maps1, h1.data(), h1.size() * sizeof(CUtensorMap), cudaMemcpyHostToDevice, st));
     if (n > cap) {
         if (d_maps) cudaFree(d_maps);
         cap = n + 64;
-        DMRG_CHECK_CUDA(cudaMalloc(&d_maps, cap * sizeof(CUtensorMap)));
+        DMRG_CHECK_CUDA(dev_malloc(&d_maps, cap * sizeof(CUtensorMap)));
     }
     if (n > 0) DMRG_CHECK_CUDA(cudaMemcpyAsync(d_maps, h.data(), n * sizeof(CUtensorMap), cudaMemcpyHostToDevice, st));
     DMRG_CHECK_CUDA(cudaStreamSynchronize(st));

@@ -165,18 +165,23 @@ void trim_product_pool() {
     if (g_pools[dev]) cudaMemPoolTrimTo(g_pools[dev], 0);
 }
 
+cudaError_t dev_malloc_bytes(void** p, size_t bytes) {
+    cudaError_t e = cudaMalloc(p, bytes);
+    if (e != cudaSuccess) {
+        cudaGetLastError();
+        trim_product_pool();
+        e = cudaMalloc(p, bytes);
+    }
+    return e;
+}
+
 double* Plan::alloc(int64_t n) {
     if (n <= 0) return nullptr;
     int64_t bytes = n * 8;
     DMRG_REQUIRE(budget <= 0 || dev_bytes + bytes <= budget, DMRG_ENOMEM,
                  "device budget exceeded (" + std::to_string((dev_bytes + bytes) >> 20) + " MiB)");
     void* p = nullptr;
-    cudaError_t e = cudaMalloc(&p, bytes);
-    if (e != cudaSuccess) {  // once more without what the grouped products keep
-        cudaGetLastError();
-        trim_product_pool();
-        e = cudaMalloc(&p, bytes);
-    }
+    cudaError_t e = dev_malloc(&p, bytes);
     if (e != cudaSuccess) {
         cudaGetLastError();
         throw Error(DMRG_ENOMEM, "cudaMalloc of " + std::to_string(bytes >> 20) + " MiB failed");
@@ -202,12 +207,7 @@ __nv_bfloat16* Plan::alloc_bf16(int64_t n) {
     DMRG_REQUIRE(budget <= 0 || dev_bytes + bytes <= budget, DMRG_ENOMEM,
                  "device budget exceeded (" + std::to_string((dev_bytes + bytes) >> 20) + " MiB)");
     void* p = nullptr;
-    cudaError_t e = cudaMalloc(&p, bytes);
-    if (e != cudaSuccess) {  // once more without what the grouped products keep
-        cudaGetLastError();
-        trim_product_pool();
-        e = cudaMalloc(&p, bytes);
-    }
+    cudaError_t e = dev_malloc(&p, bytes);
     if (e != cudaSuccess) {
         cudaGetLastError();
         throw Error(DMRG_ENOMEM, "cudaMalloc of " + std::to_string(bytes >> 20) + " MiB failed");
@@ -229,7 +229,7 @@ void Plan::free_bf16(__nv_bfloat16*& p, int64_t n) {
 
 int* Plan::error_word() {
     if (!d_ctr) {
-        DMRG_CHECK_CUDA(cudaMalloc(&d_ctr, 2 * sizeof(int)));
+        DMRG_CHECK_CUDA(dev_malloc(&d_ctr, 2 * sizeof(int)));
         DMRG_CHECK_CUDA(cudaMemsetAsync(d_ctr, 0, 2 * sizeof(int), stream));
     }
     return d_ctr + 1;

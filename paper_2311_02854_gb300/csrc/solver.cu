@@ -223,7 +223,7 @@ void davidson_run(Plan& P, double* psi, int nr, double tol, int max_iter, int pr
     bool conv = false, stalled = false;
     EigJob job;
     EigJob* d_job = nullptr;
-    DMRG_CHECK_CUDA(cudaMalloc(&d_job, sizeof(EigJob)));
+    DMRG_CHECK_CUDA(dev_malloc(&d_job, sizeof(EigJob)));
     struct JobFree {
         EigJob*& p;
         ~JobFree() {
@@ -369,7 +369,7 @@ void davidson_run(Plan& P, double* psi, int nr, double tol, int max_iter, int pr
         if (use_mlp && P.n_mlp_feat < 6 * n) {
             if (P.d_mlp_feat) cudaFree(P.d_mlp_feat);
             P.n_mlp_feat = 6 * n;
-            DMRG_CHECK_CUDA(cudaMalloc(&P.d_mlp_feat, P.n_mlp_feat * sizeof(float)));
+            DMRG_CHECK_CUDA(dev_malloc(&P.d_mlp_feat, P.n_mlp_feat * sizeof(float)));
         }
         for (int i = 0; i < nr; ++i) {
             double* ri = T + (int64_t)i * n;

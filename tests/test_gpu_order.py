@@ -212,3 +212,24 @@ def test_first_fp64_accurate_products_of_several_threads():
     cuda_torch()
     r = subprocess.run([sys.executable, "-c", FIRST_CALLS], capture_output=True, text=True, timeout=300)
     assert r.returncode == 0 and r.stdout.strip() == "ok", r.stderr[-2000:]
+
+
+def test_a_new_plan_takes_back_what_grouped_products_keep(tmp_path):
+    """The pool of dmrg_grouped_gemm keeps memory between calls, but not from a plan."""
+    torch = cuda_torch()
+    g = gpu_lib()
+    h, L, _, path = make_case(tmp_path, 6, 6, 0, 20, center=3)
+
+    def plan():
+        g.Plan(h, L, 6, 6, 0, 20, path).close()
+        torch.cuda.synchronize()
+        return torch.cuda.mem_get_info()[0]
+
+    n = 4096
+    a, b, c = (torch.ones(n * n, dtype=torch.float64, device="cuda") for _ in range(3))
+    free = plan()
+    g.grouped_gemm(BF16X3, [(n, n, 0, [(n, 0, n, 0, 0, n, 0, 1.0)])], a, b, c)
+    torch.cuda.synchronize()
+    assert float(c[0]) == n
+    assert torch.cuda.mem_get_info()[0] <= free - (100 << 20)  # the pieces of a and b: 128 MB
+    assert plan() >= free - (16 << 20)
