@@ -116,7 +116,8 @@ typedef struct {
                                (kept per bond for its last layout); ignored when tc_kchunk > 0
                                or sigma_tile_n > 0, and for lists of over 2^20 products (which
                                keep tile width 128 and the full K-chunk, the measured winner
-                               there); default 1 */
+                               there).  The K-chunk moves sigma by its FP32 rounding, about
+                               3e-6; default 1 */
     int sigma_tile_n;       /* mixed modes: 64 or 128 fixes the tile width of the sigma work
                                lists (no tuning); 0 = tuned or 128; default 0 */
     int refine;             /* mixed modes: 1 = FP64 residual correction of Davidson (a defect
@@ -199,7 +200,8 @@ typedef struct {
     int64_t tunes;                /* estimates of the tile shape (new bonds or new sectors) */
     int64_t tune_hits;            /* bonds set again with the sectors of the last estimate */
     double ms_tune;               /* wall time of all autotuner runs */
-    double tune_cand_ms[4];       /* the last bond's estimated sample time per candidate
+    double tune_cand_ms[4];       /* the last bond's estimated sample time per candidate (to be
+                                     compared with each other: the kernels take about half)
                                      (128 / K-chunk, 64 / K-chunk, 128 / half K-chunk, 64 / half) */
     double sigma_load_bytes[2][2];/* mixed sigma, one vector: operand bytes the tensor-core tiles
                                      load through TMA, [phase 1 / 2][other operands / phase-1
@@ -301,7 +303,11 @@ dmrg_status dmrg_hdiag(dmrg_plan_t plan, double* diag_dev, void* stream);
  *  iters    out (host): iterations used (may be NULL).
  *  precond  dmrg_precond; MLP falls back to Jacobi (counted in stats) if its
  *           correction is not finite or not a descent direction.
- * Returns DMRG_ENOTCONV if max_iter is reached above tol (energies filled). */
+ * Returns DMRG_ENOTCONV if max_iter is reached above tol (energies filled).  A
+ * call that stops unconverged makes any figure of its vector out of the last
+ * place of sigma.  In the mixed modes that place depends on the order in which
+ * the sums of an element arrive: it repeats, nearly always, at bonds of up to
+ * 2^18 products (dmrg_stats n_items), beyond them it does not. */
 dmrg_status dmrg_davidson(dmrg_plan_t plan, double* psi_dev, int n_roots, double tol, int max_iter,
                           int precond, double* energies, int* iters, void* stream);
 

@@ -172,16 +172,18 @@ struct SigmaShape {
 
 // Estimates the time of the candidate shapes (tile width 128 / 64, phase-2
 // K-chunk kmax / kmax/2) on a sample of the bond's work list: every 8th output
-// block with all of its products, cut into tiles and K-chunks as the list would
-// be and dealt to the SMs longest first.  In units of a 64-deep K stage of phase
-// 2: 16 for the launches, 1.6 per phase-1 stage of an SM, and for phase 2 the
-// largest SM's stages plus 4 per tile (its drain).  The weights are fitted to
-// timings of 420 bonds (K = 7 to 32, D = 30 to 900; one, two and three bf16
-// pieces), of which the estimate picks the faster K-chunk in all but 23, half of
-// those within 2 % either way.  Timing the sample instead took 8 to 60 ms per new
-// bond, and near a tie it chose by noise, so that one bond's sigma differed by
-// the FP32 rounding of the other chain length (3e-6) from run to run.  The
-// fastest wins, the default (128, kmax) unless another is 0.5 % faster.
+// block with all of its products, cut into tiles and K-chunks and dealt to 152 SMs
+// longest first, every first product a tile of its own.  In units of a 64-deep K stage
+// of phase 2: 16 for the launches, 1.6 per phase-1 stage of an SM, and for phase 2 the
+// largest SM's stages plus 4 per tile (its drain).  That describes the kernel on which
+// the weights were fitted (one CTA per SM, products neither shared nor stacked; 420
+// bonds, K = 7 to 32, D = 30 to 900, one, two and three bf16 pieces), where it picks
+// the K-chunk that timing the sample chose in all but 23; width 64 was never the
+// faster one there.  The times are about twice those of the present kernels.  The
+// weights are kept because the K-chunk is part of the result: the two chain lengths
+// differ by the FP32 rounding of sigma (3e-6), and timing the sample, 8 to 60 ms per
+// new bond, chose by noise near a tie.  The fastest wins, the default (128, kmax)
+// unless another is 0.5 % faster.
 SigmaShape tune_sigma_shape(Plan& P, int bond, const ProductList& tl, int64_t kmax) {
     Plan::TunedShape& f = P.tuned[bond];
     std::vector<int> key = shape_key(P, bond);
@@ -646,8 +648,9 @@ std::unique_ptr<Block> renormalise(Plan& P, const Block& X, int m, bool forward)
     const int64_t cap = P.tc_store() ? scratch_cap(P) : scratch_cap_f64(P);
     if (P.tc_store()) {
         // the cp.async-staged engine: renormalisation lists hold many short
-        // products (K-chunks of 256), where it measured faster than the
-        // TMA-staged engine of sigma (map encoding and lowering cost included)
+        // products (K-chunks of 256), where it measured faster than the TMA-staged
+        // engine of sigma with one CTA per SM (map encoding and lowering cost
+        // included); the present one has not been compared
         pl.lower_tc(BUF_SCR, BUF_ID, P.id_n, cap, kChunkTC, TC_ATOMIC_F64);
         host_lower_ms = host_ms_since(host0);
         P.stats.ms_host_plan += host_lower_ms;
@@ -941,8 +944,8 @@ void set_bond(Plan& P, int k) {
             });
             t_terms = host_ms_since(h0);
             // lists of over a million products keep the default shape: it won every
-            // measurement at that size (K = 54 and K = 73 middle bonds), and the
-            // timing of the candidates costs 0.3-1 s per new bond there
+            // measurement at that size (K = 54 and K = 73 middle bonds), and the fit of
+            // the estimate has no such list
             tune_later = P.opt.sigma_tile_n <= 0 && P.opt.sigma_tune && P.opt.tc_kchunk <= 0 &&
                          !P.opt.sigma_per_term && tl.cs.size() <= ((size_t)1 << 20);
             if (!tune_later) lower_and_count();

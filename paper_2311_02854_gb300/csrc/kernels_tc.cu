@@ -411,10 +411,10 @@ __device__ __forceinline__ void tma_operand(uint32_t dst, const CUtensorMap* map
 // Roles: warps 0-7 epilogue in two groups of four that take the CTA's tiles
 // alternately, warp 8 TMA producer (all lanes), warp 9 lane 0 MMA issuer.
 //
-// Bound: not by data.  The producer and the MMA lane are each busy ~1000 cycles
-// per stage with issuing (waits, descriptors, copies, 6 to 12 MMAs,
-// commits), whatever the stage holds, so two CTAs share an SM, half of shared
-// and tensor memory each, and issue in parallel (one CTA with everything:
+// Bound: not by data.  The producer and the MMA lane spend their time issuing (waits,
+// descriptors, copies, 6 to 12 MMAs, commits; ~1000 cycles per stage each, counted with
+// one CTA per SM and a copy per piece), whatever the stage holds, so two CTAs share an
+// SM, half of shared and tensor memory each, and issue in parallel (one CTA with everything:
 // K = 24, D = 500, four vectors 20.4 ms, two: 11.6 ms; K = 36, D = 1000
 // 16.4 -> 13.5 ms), and one copy brings all pieces of an operand (two per small
 // stage instead of four: K = 8, D = 64 233 -> 185 us, K = 24 8.5 -> 7.7 ms).
