@@ -1258,7 +1258,7 @@ void sigma_body(Plan& P, const double* psi, double* out, int nvec, cudaStream_t 
             DMRG_CHECK_CUDA(cudaMemsetAsync(out + (int64_t)v0 * P.dim, 0, (size_t)nv * P.dim * 8, st));
             BufTable bt = bond_buffers(P, psi + (int64_t)v0 * P.dim, out + (int64_t)v0 * P.dim);
             bt.vstride[BUF_SCR] = per;
-            P.sigma_pl.run(bt, nv, st);
+            P.sigma_pl.run(bt, nv, st, repeatable);
         }
         P.stats.sigma_calls += nvec;
         return;

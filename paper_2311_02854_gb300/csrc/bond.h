@@ -25,8 +25,9 @@ void build_layout(Plan& P, int k);
 void set_bond(Plan& P, int k);
 BufTable bond_buffers(Plan& P, const double* psi, double* out);
 // sigma with the plan's engine (tensor cores in mixed precision)
-// repeatable (Davidson): short lists add their K-chunks in an order that repeats from
-// call to call, where the mixed sigma otherwise adds them as they finish
+// repeatable (Davidson): short lists of a mixed sigma add their K-chunks in an order that
+// repeats from call to call instead of as they finish, the FP64 units sum in one chain
+// per element instead of sharing sums
 void sigma(Plan& P, const double* psi, double* out, int nvec, cudaStream_t st, bool repeatable = false);
 // sigma in FP64 arithmetic over the stored operators (either precision)
 void sigma_fp64(Plan& P, const double* psi, double* out, int nvec, cudaStream_t st);

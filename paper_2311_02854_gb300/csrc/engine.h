@@ -73,6 +73,9 @@ struct WorkList {
     // it), by K-blocks of every segment (byk) or by segments
     int part = 64, split = 0;
     bool byk = false;
+    // chains on the FP64 units, set by arrange: columns of a part (a warp's; 32, 16, 8, or
+    // 4 of 8 rows) and the parts along a tile; depth at which a chain is cut (0: never)
+    int chain_part = 32, sub_m = 2, sub_n = 2, kchunk = 0;
     bool single = false;  // every tile has one segment (FP64-accurate tensor-core engine, set by arrange)
     // tile shape of add_block when nonzero (rows, columns); 128 x 64 lists run on
     // the FP64-accurate tensor-core engine (launch_seg_gemm_f64 dispatches on it)
@@ -95,7 +98,8 @@ struct WorkList {
     void release();
 };
 
-void launch_seg_gemm_f64(const WorkList& w, const BufTable& bt, int nvec, cudaStream_t st);
+// chains: one chain of fused multiply-adds per element (FP64 units only)
+void launch_seg_gemm_f64(const WorkList& w, const BufTable& bt, int nvec, cudaStream_t st, bool chains = false);
 // FP64-accurate products on the bf16 tensor cores (kernels_oz.cu): work lists
 // lowered with oz_tile_rows() x oz_tile_cols() tiles over FP64 buffers
 void launch_seg_gemm_oz(const WorkList& w, const BufTable& bt, int nvec, cudaStream_t st);

@@ -149,6 +149,26 @@ void WorkList::arrange() {
         if ((few || longest) && (byk || segsum >= 8 * nt)) split = 1;
         if (split && !byk && parts * kSplitWarps < kSlots && segsum >= 64 * nt) split = 8;
     }
+    // chains (seg_chain_f64_kernel): parts of 32 x 32, or smaller ones (16 x 16, 8 x 8,
+    // 8 x 4) where that leaves the SMs without warps (fewer parts than kFill) or one warp
+    // with a sum that outlasts its SM's share of the launch
+    chain_part = 32;
+    if (!oz && !rank1) {
+        constexpr int64_t kSMs = 152, kFill = 8 * kSMs;
+        for (; chain_part > 4; chain_part /= 2) {
+            const int rows = std::max(chain_part, 8);
+            int64_t np_all = 0, worst = 0;
+            for (size_t i = 0; i < tiles.size(); ++i) {
+                const int m = std::min(tiles[i].m - tiles[i].m0, 64), n = std::min(tiles[i].n - tiles[i].n0, 64);
+                const int64_t np = (int64_t)((m + rows - 1) / rows) * ((n + chain_part - 1) / chain_part);
+                np_all += np;
+                worst = std::max(worst, cost[i] / np);
+            }
+            if (np_all >= kFill && worst * kSMs <= total) break;
+        }
+    }
+    sub_m = (mmax + std::max(chain_part, 8) - 1) / std::max(chain_part, 8);
+    sub_n = (nmax + chain_part - 1) / chain_part;
     if ((oz || split) && tiles.size() > 1) {
         // longest first (stable counting sort), so that short tiles fill in at the
         // end instead of a few long ones trailing
@@ -407,6 +427,150 @@ __global__ void __launch_bounds__(32 * kSplit, GR == 2 ? 5 : 3)
     if (warp == 0 && rank == 0) store_part<GR>(T, bt, v, p, acc);
 }
 
+// The same product with one chain of fused multiply-adds per element, segment after
+// segment and k after k (cut where its depth reaches the list's K-chunk, the pieces
+// added in order): the sigma inside an FP64 Davidson call, which makes any figure of its
+// vector out of a last place (see seg_outer_f64_kernel; products of four k's on the
+// mma units with long sums shared among warps are off by 2e-15 of a sigma, and eight
+// steps turned that into 1e-7 to 1e-2 of the vector in three of four problems).
+//
+// Bound: the FP64 units (89 % busy on K = 14, D = 600 first products), or for small
+// bonds the longest chain, 63 ns per k.  What is shared among warps is the elements of a
+// sum: a warp owns a part of 32 x 32 down to 8 x 4 of a tile.  Lane l = 4 r + c sums rows
+// 8 i + r of columns 4 j + c.  Batches of KU k's, the next one in flight: of their operand
+// elements a lane loads (and scales) KA of A and KB of B, one row and one column of its
+// own at every few k's, and the lanes hand them to each other, so that a multiply-add
+// comes with one or two other instructions (eighteen where each lane loaded all of its
+// operands: sigma K = 14, D = 600 173 ms, now 93; 89 on the mma units).  Rows and columns
+// outside the part read its last one and are dropped.
+template <int GI, int GJ, int KU>
+__global__ void __launch_bounds__(32, GI == 4 ? 12 : 20)
+    seg_chain_f64_kernel(const Tile* __restrict__ tiles, int sub_m, int sub_n, int kchunk, const Seg* __restrict__ segs,
+                        BufTable bt) {
+    constexpr int UA = 4 / GI, UB = 8 / GJ;  // a lane's elements of A (B) are UA (UB) k's apart
+    constexpr int KA = KU / UA, KB = KU / UB;
+    const int subs = sub_m * sub_n;
+    const Tile T = tiles[blockIdx.x / subs];
+    const int sub = (int)(blockIdx.x % subs);
+    Part p;
+    p.m0 = T.m0 + sub / sub_n * 8 * GI;
+    p.n0 = T.n0 + sub % sub_n * 4 * GJ;
+    p.mr = min(8 * GI, min(T.m, T.m0 + 64) - p.m0);
+    p.nr = min(4 * GJ, min(T.n, T.n0 + 64) - p.n0);
+    if (p.mr <= 0 || p.nr <= 0) return;
+    const int v = blockIdx.y, lane = threadIdx.x & 31, lr = lane >> 2, lc = lane & 3;
+    const int arow = min(8 * (lc % GI) + lr, p.mr - 1), au = lc / GI;  // the lane's row of A, its first k
+    const int bcol = min(4 * (lr % GJ) + lc, p.nr - 1), bu = lr / GJ;  // column of B
+    double acc[GI][GJ] = {};
+    // the chain so far to the output.  TILE_ATOMIC: added without atomics (one warp owns
+    // the elements, and lists that add to the same output run one after the other)
+    auto flush = [&]() {
+        double* C = bt.p[T.c_buf] + T.c_off + (int64_t)v * bt.vstride[T.c_buf] + (int64_t)(p.m0 + lr) * T.ldc + p.n0 + lc;
+#pragma unroll
+        for (int i = 0; i < GI; ++i)
+#pragma unroll
+            for (int j = 0; j < GJ; ++j)
+                if (8 * i + lr < p.mr && 4 * j + lc < p.nr) {
+                    double* c = C + (int64_t)8 * i * T.ldc + 4 * j;
+                    *c = T.mode == TILE_ATOMIC ? *c + acc[i][j] : acc[i][j];
+                }
+    };
+    struct Batch {
+        double a[KA], b[KB], alpha;
+        int n;       // k's
+        bool first;  // a new chain begins with it
+    };
+    // cursor: segment s (records one ahead in N), k's left of it, depth of the chain
+    int s = T.seg_beg, left = 0, depth = 0;
+    Seg N{};
+    if (s < T.seg_end) N = segs[s];
+    const double *pa = nullptr, *pb = nullptr;
+    int64_t ka = 0, kb = 0;
+    double alpha = 0.0;
+    bool cut = false;
+    auto open = [&]() {  // the next segment with products, if any
+        left = 0;
+        while (s < T.seg_end) {
+            const Seg S = N;
+            if (s + 1 < T.seg_end) N = segs[s + 1];
+            if (kchunk > 0 && depth > 0 && depth + S.k > kchunk) {
+                cut = true;
+                depth = 0;
+            }
+            depth += S.k;
+            if (S.k <= 0) {
+                ++s;
+                continue;
+            }
+            // element (row, k) of op(A) at A + row * ra + k * ka, (k, col) of op(B) at B + k * kb + col * cb
+            const int64_t ra = S.a_tr ? 1 : S.lda, cb = S.b_tr ? S.ldb : 1;
+            ka = S.a_tr ? S.lda : 1;
+            kb = S.b_tr ? 1 : S.ldb;
+            pa = bt.p[S.a_buf] + S.a_off + (int64_t)v * bt.vstride[S.a_buf] + (p.m0 + arow) * ra + au * ka;
+            pb = bt.p[S.b_buf] + S.b_off + (int64_t)v * bt.vstride[S.b_buf] + (p.n0 + bcol) * cb + bu * kb;
+            alpha = S.alpha;
+            left = S.k;
+            break;
+        }
+    };
+    auto fetch = [&](Batch& x) {
+        x.n = min(KU, left);
+        x.first = cut;
+        x.alpha = alpha;
+        cut = false;
+        if (left <= 0) return;
+#pragma unroll
+        for (int q = 0; q < KA; ++q) {
+            x.a[q] = au + q * UA < left ? *pa : 0.0;
+            pa += UA * ka;
+        }
+#pragma unroll
+        for (int q = 0; q < KB; ++q) {
+            x.b[q] = bu + q * UB < left ? *pb : 0.0;
+            pb += UB * kb;
+        }
+        left -= KU;
+        if (left <= 0) {
+            ++s;
+            open();
+        }
+    };
+    Batch next;
+    open();
+    fetch(next);
+    while (next.n > 0) {
+        Batch x = next;
+        fetch(next);
+        if (x.first) {
+            flush();
+#pragma unroll
+            for (int i = 0; i < GI; ++i)
+#pragma unroll
+                for (int j = 0; j < GJ; ++j) acc[i][j] = 0.0;
+        }
+        if (x.alpha != 1.0) {
+#pragma unroll
+            for (int q = 0; q < KA; ++q) x.a[q] *= x.alpha;
+        }
+#pragma unroll
+        for (int u = 0; u < KU; ++u) {
+            if (u >= x.n) break;
+            double b[GJ];
+#pragma unroll
+            for (int j = 0; j < GJ; ++j) b[j] = __shfl_sync(0xffffffffu, x.b[u / UB], ((u % UB) * GJ + j) * 4 + lc);
+#pragma unroll
+            for (int i = 0; i < GI; ++i) {
+                const double a = __shfl_sync(0xffffffffu, x.a[u / UA], (lane & 28) | ((u % UA) * GI + i));
+                if (i > 0 && 8 * i >= p.mr) break;
+#pragma unroll
+                for (int j = 0; j < GJ; ++j)
+                    if (j == 0 || 4 * j < p.nr) acc[i][j] = fma(a, b[j], acc[i][j]);
+            }
+        }
+    }
+    flush();
+}
+
 // The same product for lists whose segments all have K = 1 (rank-1 updates:
 // the diagonal of H_eff as sums of diag(O_L) diag(O_R)^T, the two-electron
 // integrals as a sum over Cholesky vectors).  Every element is one chain of fused
@@ -480,7 +644,15 @@ __global__ void __launch_bounds__(2 * kOuter)
 }
 }  // namespace
 
-void launch_seg_gemm_f64(const WorkList& w, const BufTable& bt, int nvec, cudaStream_t st) {
+static void launch_chains(const WorkList& w, dim3 grid, const Tile* tiles, const BufTable& bt, cudaStream_t st) {
+    auto kernel = w.chain_part == 32   ? seg_chain_f64_kernel<4, 8, 4>
+                  : w.chain_part == 16 ? seg_chain_f64_kernel<2, 4, 4>
+                  : w.chain_part == 8  ? seg_chain_f64_kernel<1, 2, 16>
+                                       : seg_chain_f64_kernel<1, 1, 16>;
+    kernel<<<grid, 32, 0, st>>>(tiles, w.sub_m, w.sub_n, w.kchunk, w.d_segs, bt);
+}
+
+void launch_seg_gemm_f64(const WorkList& w, const BufTable& bt, int nvec, cudaStream_t st, bool chains) {
     if (w.tiles.empty()) return;
     if (w.tile_m == oz_tile_rows() && !w.rank1) {
         launch_seg_gemm_oz(w, bt, nvec, st);
@@ -488,9 +660,11 @@ void launch_seg_gemm_f64(const WorkList& w, const BufTable& bt, int nvec, cudaSt
     }
     DMRG_REQUIRE(w.tile_m == 0, DMRG_EINVAL, "work list tile shape not runnable on the FP64 engine");
     DMRG_REQUIRE(nvec <= 65535, DMRG_EINVAL, "too many vectors for one launch");
-    const int subs = w.part == 64 ? 4 : 1;
+    chains = chains && !w.rank1;
+    DMRG_REQUIRE(!chains || bt.pmask == 0, DMRG_EINVAL, "chains are summed over FP64 buffers only");
+    const int subs = chains ? w.sub_m * w.sub_n : (w.part == 64 ? 4 : 1);
     const bool tiny = w.part == 16;
-    const int nrank = w.split ? w.split : 1;
+    const int nrank = w.split && !chains ? w.split : 1;
     const int64_t n = (int64_t)w.tiles.size(), maxt = 2147483647LL / (subs * nrank);
     for (int64_t t0 = 0; t0 < n; t0 += maxt) {
         const int64_t nt = std::min(n - t0, maxt);
@@ -498,6 +672,8 @@ void launch_seg_gemm_f64(const WorkList& w, const BufTable& bt, int nvec, cudaSt
         const Tile* tl = w.d_tiles + t0;
         if (w.rank1) {
             seg_outer_f64_kernel<<<grid, 2 * kOuter, 0, st>>>(tl, subs, w.d_segs, bt);
+        } else if (chains) {
+            launch_chains(w, grid, tl, bt, st);
         } else if (w.split) {
             cudaLaunchConfig_t cfg{};
             cfg.gridDim = grid;

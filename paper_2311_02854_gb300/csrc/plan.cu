@@ -591,10 +591,11 @@ void ProductList::lower(int8_t sbuf_, int8_t ibuf, int ild, int64_t cap, int64_t
                 flops += 2.0 * c.m * c.n;
             }
         }
+        // the FP64 units' kernels share a long term sum among the CTAs of a cluster, or cut
+        // its chains themselves, and add without atomics: one tile per output region
+        if (!oz) p2.kchunk = (int)kchunk;
         for (int o : order) {
             const OutBlock& ob = outs[o];
-            // the FP64 units' kernels share a long term sum among the CTAs of a cluster
-            // and add without atomics: one tile per output region, no K-chunks
             p2.add_block(ob.off, ob.buf, ob.m, ob.n, ob.ldc, segs[o], TILE_ATOMIC, oz ? kchunk : 0);
         }
         scratch_elems = std::max(scratch_elems, used);
@@ -1188,12 +1189,12 @@ void ProductList::upload(cudaStream_t st) {
     }
 }
 
-void ProductList::run(const BufTable& bt, int nvec, cudaStream_t st) {
+void ProductList::run(const BufTable& bt, int nvec, cudaStream_t st, bool chains) {
     for (auto& c : chunks) {
         DMRG_REQUIRE(c.first.tiles.empty() || (sbuf >= 0 && bt.p[sbuf]), DMRG_EINVAL,
                      "product list run without its scratch buffer");
-        launch_seg_gemm_f64(c.first, bt, nvec, st);
-        launch_seg_gemm_f64(c.second, bt, nvec, st);
+        launch_seg_gemm_f64(c.first, bt, nvec, st, chains);
+        launch_seg_gemm_f64(c.second, bt, nvec, st, chains);
     }
 }
 

@@ -106,7 +106,8 @@ struct ProductList {
     void lower_tc(int8_t scratch_buf, int8_t ident_buf, int ident_ld, int64_t scratch_cap, int64_t kchunk,
                   uint8_t out_mode);
     void upload(cudaStream_t st);
-    void run(const BufTable& bt, int nvec, cudaStream_t st);
+    // chains: every sum of the FP64 units in one order (seg_chain_f64_kernel)
+    void run(const BufTable& bt, int nvec, cudaStream_t st, bool chains = false);
     void run_tc(const TcBufs& tb, int nvec, int nsplit, cudaStream_t st);
     // TMA-staged tensor-core engine: as lower_tc, with every operand read through
     // a tensor map (maps); phase-1 products of equal shape share a 3-D scratch

@@ -233,3 +233,37 @@ def test_a_new_plan_takes_back_what_grouped_products_keep(tmp_path):
     assert float(c[0]) == n
     assert torch.cuda.mem_get_info()[0] <= free - (100 << 20)  # the pieces of a and b: 128 MB
     assert plan() >= free - (16 << 20)
+
+
+@pytest.mark.parametrize("K,D,k,n_roots", [(4, 8, 1, 1), (6, 20, 3, 2), (8, 64, 4, 1), (10, 100, 5, 3), (12, 300, 4, 1),
+                                           (14, 600, 7, 1)])
+def test_fp64_davidson_sums_in_chains(tmp_path, K, D, k, n_roots):
+    """The sigma inside an FP64 Davidson call (one chain per element, parts of every size,
+    chains cut at 16384: the last case sums to 40 000) against dmrg_sigma: one step from
+    orthonormal vectors gives the eigenvalues of X H X^T.  A sum of n terms is off by at most
+    n u of the sum of their magnitudes on either side; 1e-12 of |H x| holds that at n = 4000
+    with room for the sums' cancellation, the bar of the FP64 tests.  Calls repeat."""
+    torch = cuda_torch()
+    g = gpu_lib()
+    h, L, _, path = make_case(tmp_path, K, K, 0, D, center=k, split="gaussian", wn=1.0, ws=1.0)
+    plan = g.Plan(h, L, K, K, 0, D, path, precision=FP64, n_roots=n_roots)
+    plan.set_bond(k)
+    n_roots = min(n_roots, plan.dim)
+    x = np.linalg.qr(si.random_vector(plan.dim, seed=1, nvec=n_roots).reshape(n_roots, plan.dim).T)[0].T.copy()
+    x = torch.from_numpy(x).cuda()
+    hx = torch.empty_like(x)
+    plan.sigma(x, hx, nvec=n_roots)
+    want = torch.linalg.eigvalsh((x @ hx.T + hx @ x.T) / 2).cpu().numpy()
+    got = []
+    for _ in range(2):
+        y = x.clone()
+        e, _, _ = plan.davidson(y, n_roots, tol=1e-14, max_iter=1)
+        got.append((e, y))
+    assert np.abs(np.sort(got[0][0]) - want).max() <= 1e-12 * float(hx.norm(dim=1).max()) * n_roots
+    assert np.array_equal(got[0][0], got[1][0]) and torch.equal(got[0][1], got[1][1])
+    z = x.clone()
+    e, _, _ = plan.davidson(z, n_roots, tol=1e-14, max_iter=6)
+    plan.sigma(z, hx, nvec=n_roots)  # of Ritz vectors
+    for i in range(n_roots):
+        assert abs(e[i] - float(z[i] @ hx[i])) <= 1e-11 * float(hx[i].norm())
+    plan.close()
